@@ -91,7 +91,8 @@ typedef struct aded_weights {
 typedef struct aded_trigram_config {
     int32_t vocab;            /* token ids are 0 .. vocab-1 */
     int32_t log2_buckets;     /* 2^log2_buckets home buckets (one per two-token context), 4..28 */
-    int32_t overflow_buckets; /* extra buckets for contexts with more than 6 continuations */
+    int32_t overflow_buckets; /* extra buckets (six entries each) for contexts with more than 6 continuations;
+                                 they and their index take 272-400 bytes of device memory each */
     uint32_t cap;             /* counts saturate here (Algorithm 2's maximum); 0 = 2^31 - 1, which is also the largest allowed */
     uint32_t min_count;       /* top-k skips entries below this count; 0 = off */
 } aded_trigram_config;

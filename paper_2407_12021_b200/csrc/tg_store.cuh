@@ -1,0 +1,386 @@
+// The tri-gram store in device memory: layout, insertion and lookup (device code shared by the kernels of trigram.cu).
+//
+// Three arrays:
+//   * home buckets (64 bytes, 2^log2_buckets of them), found by hashing the two-token context (a, b) and probing
+//     linearly; a bucket holds its context, six (token, count) entries that fill front to back, and where the
+//     context's further entries are;
+//   * a pool of (token, count) entries in units of six (48 bytes).  A context's entries beyond six lie in extents of
+//     1, 2, 4, ... units, each contiguous, handed out by a bump allocator when the extent before is full; the first
+//     extent starts with a directory of the others.  Every entry of a context, however many there are, is therefore two
+//     dependent reads behind its home bucket, and a lookup reads them with coalesced 16-byte loads that are all
+//     independent.  (Chains of single buckets, as before, cost one dependent read per six entries: a lookup of a
+//     frequent context -- thousands of continuations -- was a chain of hundreds to thousands of memory round trips.)
+//   * an index over the pool entries: (home bucket, token) -> entry, open addressing, at most three quarters full.
+//     Raising a count is one probe of the home buckets, one of the index and one atomic add, wherever the entry is.
+//     Measured, 10^6 tokens into an empty table: 13.6 ms with chains that every insertion walked from the front.
+//
+// Entries are never moved or removed.  The configured number of overflow buckets limits units of six entries in use
+// exactly as it limited chain buckets; the pool has room for the unused ends of the extents on top (a context with d units
+// takes at most 3 d).
+#pragma once
+
+#include "aded_internal.cuh"
+
+namespace aded {
+
+struct TgSlot { int32_t tok; uint32_t cnt; };
+struct __align__(64) Bucket {
+    unsigned long long key;   // context
+    uint32_t more;            // first extent: pool unit + 1 (0 none yet, TG_FAILED: there was no room for it)
+    uint32_t n_more;          // entries beyond six; bit 31 (TG_CLOSED): no room for further ones
+    TgSlot e[6];
+};
+static_assert(sizeof(Bucket) == 64, "bucket must be 64 bytes");
+struct __align__(16) TgIndexSlot {
+    unsigned long long key;   // home bucket and token (tg_index_key), 0 empty
+    unsigned long long at;    // pool entry + 1; 0 while its thread is still placing it, TG_DEAD: there was no room
+};
+
+constexpr unsigned long long TG_EMPTY = ~0ull, TG_DEAD = ~0ull;
+constexpr int TG_MAX_PROBE = 4096;
+constexpr uint32_t TG_FAILED = 0xFFFFFFFFu, TG_CLOSED = 0x80000000u;
+constexpr int TG_MAX_SPIN = 1 << 20;
+constexpr int TG_UNIT = 6;            // entries of a pool unit
+constexpr int TG_LINKS = 24;          // directory words: extent s (2^s units) is links[s], s >= 1
+constexpr int TG_DIR_UNITS = 2;       // units the directory takes in front of the first extent's entries
+static_assert(TG_LINKS * 4 == TG_DIR_UNITS * TG_UNIT * 8, "the directory fills whole units");
+
+struct TgView {
+    Bucket* buckets;
+    TgSlot* pool;                // [n_units][TG_UNIT]
+    TgIndexSlot* index;
+    uint32_t n_home_mask;
+    uint32_t n_home;
+    uint32_t n_over;             // configured limit on units of entries in use
+    uint32_t n_units;            // units the pool has
+    unsigned long long index_mask;
+    uint32_t* used;              // [0] units of entries in use (counts on past n_over), [1] pool units handed out
+    int32_t* status;
+    int32_t vocab;
+    uint32_t cap;
+    uint32_t min_count;
+};
+
+// Pool units for a limit of n_over units in use: a context using d units has extents of 1 + 2 + .. < 2 d units and a directory.
+__host__ __device__ constexpr unsigned long long tg_pool_units(unsigned long long n_over) { return 3 * n_over; }
+
+__device__ __forceinline__ uint32_t tg_hash(unsigned long long k) {
+    k ^= k >> 30; k *= 0xBF58476D1CE4E5B9ull;
+    k ^= k >> 27; k *= 0x94D049BB133111EBull;
+    k ^= k >> 31;
+    return (uint32_t)k;
+}
+__device__ __forceinline__ unsigned long long tg_key(int a, int b) {
+    return ((unsigned long long)(uint32_t)a << 32) | (uint32_t)b;
+}
+// Home buckets number at most 2^28 and tokens are below 2^31: exact, and never 0.
+__device__ __forceinline__ unsigned long long tg_index_key(uint32_t home, int tok) {
+    return (((unsigned long long)home << 31) | (uint32_t)tok) + 1ull;
+}
+__device__ __forceinline__ unsigned long long tg_index_start(unsigned long long key) {
+    key ^= key >> 29; key *= 0x9E3779B97F4A7C15ull;
+    key ^= key >> 32; key *= 0xBF58476D1CE4E5B9ull;
+    return key ^ (key >> 31);
+}
+// Extent of the unit with ordinal m (0-based among a context's units beyond the home bucket): 2^s units from ordinal 2^s - 1.
+__device__ __forceinline__ int tg_extent(uint32_t m) { return 31 - __clz((int)(m + 1)); }
+
+// Home bucket of a context; claims an empty one when `insert`.  Returns -1 if absent / no room.
+__device__ __forceinline__ int64_t tg_find_home(const TgView& t, unsigned long long key, bool insert) {
+    const uint32_t h = tg_hash(key);
+    const int limit = t.n_home < (uint32_t)TG_MAX_PROBE ? (int)t.n_home : TG_MAX_PROBE;
+    for (int probe = 0; probe < limit; ++probe) {
+        const uint32_t idx = (h + probe) & t.n_home_mask;
+        unsigned long long k = *reinterpret_cast<volatile unsigned long long*>(&t.buckets[idx].key);
+        if (k == key) return idx;
+        if (k == TG_EMPTY) {
+            if (!insert) return -1;
+            k = atomicCAS(&t.buckets[idx].key, TG_EMPTY, key);
+            if (k == TG_EMPTY || k == key) return idx;
+        }
+    }
+    return -1;
+}
+
+// ---- insertion ------------------------------------------------------------------------------------------------------
+__device__ __forceinline__ void tg_report(const TgView& t, int what) { atomicCAS(t.status, 0, what); }
+
+// Raises an entry's count by inc (>= 1), saturating at the cap.  `windows`: the increments of the launch number the
+// windows of one span.
+__device__ __forceinline__ void tg_raise(const TgView& t, uint32_t* cnt, uint32_t inc, bool windows) {
+    if (windows || inc == 1) {
+        // cap <= 2^31 - 1 and a span has fewer than 2^31 windows: even if all of them are added before the minimum
+        // below takes effect, the 32-bit count cannot wrap
+        const uint32_t old = atomicAdd(cnt, inc);
+        if (old + inc > t.cap) atomicMin(cnt, t.cap);
+        return;
+    }
+    // imports add arbitrary counts: saturate in one step, so that two large additions to one
+    // tri-gram cannot carry the count past 2^32 between an add and a later minimum
+    uint32_t seen = *reinterpret_cast<volatile uint32_t*>(cnt);
+    for (;;) {
+        const uint32_t want = seen >= t.cap || inc > t.cap - seen ? t.cap : seen + inc;
+        const uint32_t prev = atomicCAS(cnt, seen, want);
+        if (prev == seen) break;
+        seen = prev;      // (another thread moved the count; every retry follows a change made by someone else)
+    }
+}
+
+// Waits (bounded) until another thread has published a link of a directory; 0 when the wait ran out.
+__device__ __forceinline__ uint32_t tg_wait_link(const uint32_t* link) {
+    uint32_t v = *reinterpret_cast<const volatile uint32_t*>(link);
+    for (int spin = 0; v == 0 && spin < TG_MAX_SPIN; ++spin) {
+        __nanosleep(32);
+        v = *reinterpret_cast<const volatile uint32_t*>(link);
+    }
+    __threadfence();
+    return v;
+}
+
+// Takes the next entry of a context beyond its home bucket and writes the token with count 0.  Returns the entry's
+// number in the pool plus one, or 0 (reported) when there is no room.  The thread that takes the first entry of an
+// extent allocates the extent and publishes it; the others of that extent wait for it.  Threads only ever wait for owners
+// of earlier entries, so the waits cannot form a cycle.
+__device__ __forceinline__ unsigned long long tg_place(const TgView& t, Bucket* bk, int c) {
+    const uint32_t p = atomicAdd(&bk->n_more, 1u) & ~TG_CLOSED;
+    const uint32_t m = p / TG_UNIT, e = p % TG_UNIT;
+    const int s = tg_extent(m);
+    const uint32_t in_extent = m + 1 - (1u << s);             // the unit's place in its extent
+    const bool room = e != 0 || atomicAdd(&t.used[0], 1u) < t.n_over;
+    uint32_t base = TG_FAILED;                                // extent's first unit + 1
+    if (s < TG_LINKS) {
+        uint32_t* link = &bk->more;
+        if (s > 0) {
+            const uint32_t first = tg_wait_link(&bk->more);
+            link = first == 0 || first == TG_FAILED ? nullptr : reinterpret_cast<uint32_t*>(t.pool + (size_t)(first - 1) * TG_UNIT) + s;
+            if (first == 0) { tg_report(t, (int)ADED_ERR_TIMEOUT); return 0; }
+        }
+        if (link && e == 0 && in_extent == 0) {
+            if (room) {
+                const uint32_t units = s == 0 ? TG_DIR_UNITS + 1 : 1u << s;
+                const uint32_t at = atomicAdd(&t.used[1], units);
+                if (ADED_IN_RANGE((unsigned long long)at + units <= t.n_units, t.status)) {   // (the pool is sized so that this holds)
+                    base = at + 1;
+                    if (s == 0) {
+                        uint4* dir = reinterpret_cast<uint4*>(t.pool + (size_t)at * TG_UNIT);
+                        for (int i = 0; i < TG_LINKS / 4; ++i) dir[i] = make_uint4(0u, 0u, 0u, 0u);
+                    }
+                }
+            }
+            __threadfence();
+            atomicExch(link, base);
+        } else if (link) {
+            base = tg_wait_link(link);
+            if (base == 0) { tg_report(t, (int)ADED_ERR_TIMEOUT); return 0; }
+        }
+    }
+    if (base == TG_FAILED) {
+        atomicOr(&bk->n_more, TG_CLOSED);
+        tg_report(t, (int)ADED_ERR_TABLE_FULL);
+        return 0;
+    }
+    const unsigned long long at = ((unsigned long long)(base - 1) + (s == 0 ? TG_DIR_UNITS : 0) + in_extent) * TG_UNIT + e;
+    if (!ADED_IN_RANGE(at < (unsigned long long)t.n_units * TG_UNIT, t.status)) return 0;
+    t.pool[at] = TgSlot{room ? c : -1, 0u};                   // (an entry without a token is skipped by every reader)
+    if (room) return at + 1;
+    atomicOr(&bk->n_more, TG_CLOSED);
+    tg_report(t, (int)ADED_ERR_TABLE_FULL);
+    return 0;
+}
+
+// Raises the count of tri-gram (a, b, c) by `inc` (see tg_raise), inserting it if absent; counts
+// saturate at the cap.  Independent atomic adds: the result does not depend on the thread order.
+__device__ __forceinline__ void tg_add(const TgView& t, int a, int b, int c, uint32_t inc, bool windows) {
+    const int64_t home = tg_find_home(t, tg_key(a, b), true);
+    if (home < 0) { tg_report(t, (int)ADED_ERR_TABLE_FULL); return; }
+    if (!ADED_IN_RANGE((uint64_t)home < (uint64_t)t.n_home, t.status)) return;
+    Bucket* bk = t.buckets + home;
+    // the six tokens at once (they are only ever written from -1 to their final value)
+    const int4 e01 = __ldcg(reinterpret_cast<const int4*>(bk) + 1), e23 = __ldcg(reinterpret_cast<const int4*>(bk) + 2), e45 = __ldcg(reinterpret_cast<const int4*>(bk) + 3);
+    const int32_t seen[6] = {e01.x, e01.z, e23.x, e23.z, e45.x, e45.z};
+#pragma unroll
+    for (int e = 0; e < 6; ++e) {
+        int32_t have = seen[e];
+        if (have == -1) {
+            have = atomicCAS(&bk->e[e].tok, -1, c);
+            if (have == -1) have = c;
+        }
+        if (have == c) { tg_raise(t, &bk->e[e].cnt, inc, windows); return; }
+    }
+    const unsigned long long key = tg_index_key((uint32_t)home, c);
+    unsigned long long at_index = tg_index_start(key) & t.index_mask;
+    const int limit = t.index_mask < TG_MAX_PROBE ? (int)t.index_mask + 1 : TG_MAX_PROBE;
+    for (int probe = 0; probe < limit; ++probe, at_index = (at_index + 1) & t.index_mask) {
+        TgIndexSlot* slot = t.index + at_index;
+        unsigned long long k = *reinterpret_cast<volatile unsigned long long*>(&slot->key);
+        if (k == 0) {
+            // A context that could not grow stays as it is (and takes no index slot for what it refuses).
+            const uint32_t n = *reinterpret_cast<volatile uint32_t*>(&bk->n_more);
+            if ((n & TG_CLOSED) || (n % TG_UNIT == 0 && *reinterpret_cast<volatile uint32_t*>(&t.used[0]) >= t.n_over)) {
+                tg_report(t, (int)ADED_ERR_TABLE_FULL);
+                return;
+            }
+            k = atomicCAS(&slot->key, 0ull, key);
+            if (k == 0) {
+                const unsigned long long at = tg_place(t, bk, c);
+                __threadfence();
+                atomicExch(&slot->at, at ? at : TG_DEAD);
+                if (at) tg_raise(t, &t.pool[at - 1].cnt, inc, windows);
+                return;
+            }
+        }
+        if (k == key) {
+            unsigned long long at = *reinterpret_cast<volatile unsigned long long*>(&slot->at);
+            for (int spin = 0; at == 0 && spin < TG_MAX_SPIN; ++spin) {
+                __nanosleep(32);
+                at = *reinterpret_cast<volatile unsigned long long*>(&slot->at);
+            }
+            if (at == 0) { tg_report(t, (int)ADED_ERR_TIMEOUT); return; }
+            if (at == TG_DEAD) { tg_report(t, (int)ADED_ERR_TABLE_FULL); return; }
+            __threadfence();
+            tg_raise(t, &t.pool[at - 1].cnt, inc, windows);
+            return;
+        }
+    }
+    tg_report(t, (int)ADED_ERR_TABLE_FULL);
+}
+
+// ---- lookup ---------------------------------------------------------------------------------------------------------
+// A context's entries as one warp holds them.
+struct TgWalk {
+    uint4 part;            // lanes 0..3: the home bucket's 16-byte parts (header, then two entries each); elsewhere no entries
+    uint32_t n;            // entries beyond the home bucket
+    uint32_t extent;       // lane s: where extent s has its entries (first unit + 1, 0 none)
+    bool found;            // the context is stored
+};
+
+// Lane s gets extent s of the context whose home bucket `w.part` holds.
+__device__ __forceinline__ void tg_open_extents(const TgView& t, TgWalk& w, int lane) {
+    const uint32_t more = __shfl_sync(0xffffffffu, w.part.z, 0), n = __shfl_sync(0xffffffffu, w.part.w, 0);
+    if (lane == 0 || lane > 3) { w.part.x = 0xFFFFFFFFu; w.part.y = 0u; w.part.z = 0xFFFFFFFFu; w.part.w = 0u; }
+    w.n = 0;
+    w.extent = 0;
+    if (more == 0 || more == TG_FAILED) return;
+    w.n = n & ~TG_CLOSED;
+    if (lane == 0) {
+        w.extent = more + TG_DIR_UNITS;
+    } else if (lane < TG_LINKS && w.n > (uint32_t)TG_UNIT * ((1u << lane) - 1u)) {
+        const uint32_t link = reinterpret_cast<const uint32_t*>(t.pool + (size_t)(more - 1) * TG_UNIT)[lane];
+        w.extent = link == TG_FAILED ? 0u : link;
+    }
+}
+
+// By home bucket (all lanes the same, stored).
+__device__ __forceinline__ TgWalk tg_open(const TgView& t, uint32_t home, int lane) {
+    TgWalk w;
+    w.found = ADED_IN_RANGE(home < t.n_home, t.status);
+    w.part = make_uint4(0u, 0u, 0u, 0u);
+    if (w.found && lane < 4) w.part = reinterpret_cast<const uint4*>(t.buckets + home)[lane];
+    tg_open_extents(t, w, lane);
+    return w;
+}
+
+// By context (all lanes the same): a bucket's key and entries come with one read.
+__device__ __forceinline__ TgWalk tg_open(const TgView& t, int a, int b, int lane) {
+    TgWalk w;
+    w.part = make_uint4(0u, 0u, 0u, 0u);
+    w.found = false;
+    if (a >= 0 && b >= 0 && a < t.vocab && b < t.vocab) {
+        const unsigned long long key = tg_key(a, b);
+        const uint32_t h = tg_hash(key);
+        const int limit = t.n_home < (uint32_t)TG_MAX_PROBE ? (int)t.n_home : TG_MAX_PROBE;
+        for (int probe = 0; probe < limit; ++probe) {
+            const uint32_t idx = (h + probe) & t.n_home_mask;
+            if (lane < 4) w.part = reinterpret_cast<const uint4*>(t.buckets + idx)[lane];
+            const unsigned long long k = ((unsigned long long)__shfl_sync(0xffffffffu, w.part.y, 0) << 32) | __shfl_sync(0xffffffffu, w.part.x, 0);
+            w.found = k == key;
+            if (k == key || k == TG_EMPTY) break;
+        }
+    }
+    if (!w.found) w.part = make_uint4(0u, 0u, 0u, 0u);
+    tg_open_extents(t, w, lane);
+    return w;
+}
+
+// The best entries of a context, largest packed (count, ~token) first: lane r holds the r-th, lanes from k on nothing of use.
+// Packed keys are distinct (a context holds a token once); 0 = none.
+__device__ __forceinline__ unsigned long long tg_pack(const TgView& t, int32_t tok, uint32_t cnt) {
+    return tok >= 0 && cnt > 0 && cnt >= t.min_count ? ((unsigned long long)cnt << 32) | (0xFFFFFFFFu - (uint32_t)tok) : 0ull;
+}
+__device__ __forceinline__ int32_t tg_packed_tok(unsigned long long key) { return key ? (int32_t)(0xFFFFFFFFu - (uint32_t)key) : -1; }
+__device__ __forceinline__ uint32_t tg_packed_cnt(unsigned long long key) { return (uint32_t)(key >> 32); }
+
+// Every lane offers one key; those that beat the k-th best so far are inserted one by one, which is rare after the first
+// few (entries lie in order of first appearance, so the frequent tokens come early).
+__device__ __forceinline__ void tg_offer(unsigned long long cand, int k, int lane, unsigned long long& best) {
+    unsigned m = __ballot_sync(0xffffffffu, cand > __shfl_sync(0xffffffffu, best, k - 1));
+    while (m) {
+        const unsigned long long c = __shfl_sync(0xffffffffu, cand, __ffs((int)m) - 1);
+        const int rank = __popc(__ballot_sync(0xffffffffu, lane < k && best > c));
+        const unsigned long long up = __shfl_up_sync(0xffffffffu, best, 1);
+        if (lane == rank) best = c;
+        else if (lane > rank) best = up;
+        m &= m - 1;
+        m &= __ballot_sync(0xffffffffu, cand > __shfl_sync(0xffffffffu, best, k - 1));
+    }
+}
+
+// Two entries per lane (token -1: none) into the running list and sum.
+__device__ __forceinline__ void tg_take(const TgView& t, uint4 v, int k, int lane, unsigned long long& best, uint32_t& total) {
+    if ((int32_t)v.x >= 0) total += v.y;
+    if ((int32_t)v.z >= 0) total += v.w;
+    const unsigned long long c0 = tg_pack(t, (int32_t)v.x, v.y), c1 = tg_pack(t, (int32_t)v.z, v.w);
+    if (__any_sync(0xffffffffu, (c0 > c1 ? c0 : c1) > __shfl_sync(0xffffffffu, best, k - 1))) {
+        tg_offer(c0, k, lane, best);
+        tg_offer(c1, k, lane, best);
+    }
+}
+
+// Part `part` of `parts` of a context's entries (each part by one warp, all lanes): the k <= 32 best of them in `best`, and this
+// lane's share of the sum of the counts in `total` (both are carried on from the caller's values).
+__device__ __forceinline__ void tg_scan(const TgView& t, const TgWalk& w, int part, int parts, int k, int lane, unsigned long long& best, uint32_t& total) {
+    if (part == 0) tg_take(t, w.part, k, lane, best, total);
+    // The entries beyond, two per lane and load, BATCH loads in flight.  Pair g is the (g % 3)-th of the unit with ordinal g / 3.
+    constexpr int BATCH = 4;
+    const uint32_t pairs = (w.n + 1) / 2;
+    for (uint32_t g0 = (uint32_t)part * 32; g0 < pairs; g0 += (uint32_t)parts * 32 * BATCH) {
+        uint4 v[BATCH];
+#pragma unroll
+        for (int i = 0; i < BATCH; ++i) {
+            const uint32_t g = g0 + (uint32_t)i * parts * 32 + lane;
+            const uint32_t m = g / 3;
+            const int s = tg_extent(m);
+            const uint32_t base = __shfl_sync(0xffffffffu, w.extent, s & 31);
+            v[i] = make_uint4(0xFFFFFFFFu, 0u, 0xFFFFFFFFu, 0u);
+            if (g < pairs && base != 0) {
+                const size_t unit = (size_t)(base - 1) + (m + 1 - (1u << s));
+                if (ADED_IN_RANGE(unit < t.n_units, t.status)) v[i] = reinterpret_cast<const uint4*>(t.pool + unit * TG_UNIT)[g % 3];
+                if (2 * g + 1 >= w.n) { v[i].z = 0xFFFFFFFFu; v[i].w = 0u; }
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < BATCH; ++i) tg_take(t, v[i], k, lane, best, total);
+    }
+}
+
+// Count cell of a stored tri-gram, or NULL.
+__device__ __forceinline__ const uint32_t* tg_find(const TgView& t, int a, int b, int c) {
+    const int64_t home = tg_find_home(t, tg_key(a, b), false);
+    if (home < 0) return nullptr;
+    const Bucket* bk = t.buckets + home;
+    for (int e = 0; e < 6; ++e)
+        if (bk->e[e].tok == c) return &bk->e[e].cnt;
+    const unsigned long long key = tg_index_key((uint32_t)home, c);
+    unsigned long long i = tg_index_start(key) & t.index_mask;
+    const int limit = t.index_mask < TG_MAX_PROBE ? (int)t.index_mask + 1 : TG_MAX_PROBE;
+    for (int probe = 0; probe < limit; ++probe, i = (i + 1) & t.index_mask) {
+        if (t.index[i].key == 0) return nullptr;
+        if (t.index[i].key == key) {
+            const unsigned long long at = t.index[i].at;
+            return at == 0 || at == TG_DEAD ? nullptr : &t.pool[at - 1].cnt;
+        }
+    }
+    return nullptr;
+}
+
+}  // namespace aded

@@ -1,12 +1,6 @@
 // Tri-gram store on the GPU (Eq. 1 counts, Algorithm 2 update, top-k continuation lookup).
 //
-// Layout: an array of 64-byte buckets.  The first 2^log2_buckets are "home" buckets, found by
-// hashing the two-token context (a, b) and probing linearly; a context owns its home bucket and,
-// when it has more than six continuations, a chain of overflow buckets taken from a bump
-// allocator.  A bucket holds the context key, the index of the next bucket of the chain (0 = none)
-// and six (token, count) entries that fill front to back and are never removed.  All contexts'
-// continuations are therefore reachable from one hash probe, which is what top-k needs, and an
-// update is one probe plus one atomic add.
+// The table itself -- layout, insertion, lookup -- is in tg_store.cuh; here are the kernels over it and the entry points.
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -14,137 +8,15 @@
 #include <vector>
 
 #include "aded_internal.cuh"
+#include "tg_store.cuh"
 
 namespace aded {
 
-struct TgSlot { int32_t tok; uint32_t cnt; };
-struct __align__(64) Bucket {
-    unsigned long long key;
-    uint32_t next;
-    uint32_t pad;
-    TgSlot e[6];
-};
-static_assert(sizeof(Bucket) == 64, "bucket must be 64 bytes");
-
-constexpr unsigned long long TG_EMPTY = ~0ull;
-constexpr int TG_MAX_PROBE = 4096;
-constexpr uint32_t TG_LOCKED = 0xFFFFFFFFu;   // `next` while its chain is being extended
-constexpr int TG_MAX_SPIN = 1 << 20;
-
-struct TgView {
-    Bucket* buckets;
-    uint32_t n_home_mask;
-    uint32_t n_home;
-    uint32_t n_over;
-    uint32_t* over_used;
-    int32_t* status;
-    int32_t vocab;
-    uint32_t cap;
-    uint32_t min_count;
-};
-
-__device__ __forceinline__ uint32_t tg_hash(unsigned long long k) {
-    k ^= k >> 30; k *= 0xBF58476D1CE4E5B9ull;
-    k ^= k >> 27; k *= 0x94D049BB133111EBull;
-    k ^= k >> 31;
-    return (uint32_t)k;
-}
-
-__device__ __forceinline__ unsigned long long tg_key(int a, int b) {
-    return ((unsigned long long)(uint32_t)a << 32) | (uint32_t)b;
-}
-
-// Home bucket of a context; claims an empty one when `insert`.  Returns -1 if absent / no room.
-__device__ __forceinline__ int64_t tg_find_home(const TgView& t, unsigned long long key, bool insert) {
-    const uint32_t h = tg_hash(key);
-    const int limit = t.n_home < (uint32_t)TG_MAX_PROBE ? (int)t.n_home : TG_MAX_PROBE;
-    for (int probe = 0; probe < limit; ++probe) {
-        const uint32_t idx = (h + probe) & t.n_home_mask;
-        unsigned long long k = *reinterpret_cast<volatile unsigned long long*>(&t.buckets[idx].key);
-        if (k == key) return idx;
-        if (k == TG_EMPTY) {
-            if (!insert) return -1;
-            k = atomicCAS(&t.buckets[idx].key, TG_EMPTY, key);
-            if (k == TG_EMPTY || k == key) return idx;
-        }
-    }
-    return -1;
-}
-
-__global__ void k_tg_init(Bucket* b, size_t n) {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        Bucket z;
-        z.key = TG_EMPTY;
-        z.next = 0;
-        z.pad = 0;
-        for (int e = 0; e < 6; ++e) { z.e[e].tok = -1; z.e[e].cnt = 0; }
-        b[i] = z;
-    }
-}
-
-// Raises the count of tri-gram (a, b, c) by `inc` (1 <= inc <= cap), inserting it if absent; counts
-// saturate at the cap.  Independent atomic adds: the result does not depend on the thread order.
-__device__ __forceinline__ void tg_add(const TgView& t, int a, int b, int c, uint32_t inc) {
-    const unsigned long long key = tg_key(a, b);
-    int64_t cur = tg_find_home(t, key, true);
-    if (cur < 0) { atomicCAS(t.status, 0, (int)ADED_ERR_TABLE_FULL); return; }
-    // a chain can never be longer than every overflow bucket plus the home bucket
-    for (uint32_t hop = 0; hop <= t.n_over; ++hop) {
-        if (!ADED_IN_RANGE(cur >= 0 && (uint64_t)cur < (uint64_t)t.n_home + t.n_over, t.status)) return;
-        Bucket* bk = t.buckets + cur;
-        for (int e = 0; e < 6; ++e) {
-            int32_t have = *reinterpret_cast<volatile int32_t*>(&bk->e[e].tok);
-            if (have == -1) have = atomicCAS(&bk->e[e].tok, -1, c) == -1 ? c : *reinterpret_cast<volatile int32_t*>(&bk->e[e].tok);
-            if (have == c) {
-                if (inc == 1) {
-                    // the per-step update: cap <= 2^31 - 1 and at most 2^31 threads add 1 before the minimum below
-                    // takes effect, so the 32-bit count cannot wrap
-                    const uint32_t old = atomicAdd(&bk->e[e].cnt, 1u);
-                    if (old >= t.cap) atomicMin(&bk->e[e].cnt, t.cap);
-                } else {
-                    // imports add arbitrary counts: saturate in one step, so that two large additions to one
-                    // tri-gram cannot carry the count past 2^32 between an add and a later minimum
-                    uint32_t seen = *reinterpret_cast<volatile uint32_t*>(&bk->e[e].cnt);
-                    for (;;) {
-                        const uint32_t want = seen >= t.cap || inc > t.cap - seen ? t.cap : seen + inc;
-                        const uint32_t prev = atomicCAS(&bk->e[e].cnt, seen, want);
-                        if (prev == seen) break;
-                        seen = prev;      // (another thread moved the count; every retry follows a change made by someone else)
-                    }
-                }
-                return;
-            }
-        }
-        // Extend the chain under a one-word lock so that concurrent inserts into a hot context do
-        // not each take a bucket: the thread that swings `next` from 0 to TG_LOCKED allocates and
-        // publishes the index; the others wait for it, for a bounded number of polls.
-        uint32_t nxt = *reinterpret_cast<volatile uint32_t*>(&bk->next);
-        if (nxt == 0) {
-            const uint32_t prev = atomicCAS(&bk->next, 0u, TG_LOCKED);
-            if (prev == 0) {
-                const uint32_t fresh = atomicAdd(t.over_used, 1u);
-                if (fresh >= t.n_over) {
-                    atomicExch(&bk->next, 0u);
-                    atomicCAS(t.status, 0, (int)ADED_ERR_TABLE_FULL);
-                    return;
-                }
-                nxt = t.n_home + fresh;
-                t.buckets[nxt].key = key;
-                __threadfence();
-                atomicExch(&bk->next, nxt);
-            } else {
-                nxt = prev;
-            }
-        }
-        for (int spin = 0; nxt == TG_LOCKED && spin < TG_MAX_SPIN; ++spin) {
-            __nanosleep(64);
-            nxt = *reinterpret_cast<volatile uint32_t*>(&bk->next);
-        }
-        if (nxt == TG_LOCKED) { atomicCAS(t.status, 0, (int)ADED_ERR_TIMEOUT); return; }
-        if (nxt == 0) return;   // the allocating thread ran out of buckets and has reported it
-        cur = nxt;
-    }
-    atomicCAS(t.status, 0, (int)ADED_ERR_TIMEOUT);
+// Empty home buckets: one 16-byte part per thread and step (header, or two entries), so that a warp's stores are whole lines
+// (a thread per bucket wrote 128 MB in 52 us; with the index, 192 MB: 77 us then, 45 now).
+__global__ void k_tg_init(uint4* b, size_t parts) {
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < parts; i += (size_t)gridDim.x * blockDim.x)
+        b[i] = (i & 3) == 0 ? make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0u, 0u) : make_uint4(0xFFFFFFFFu, 0u, 0xFFFFFFFFu, 0u);
 }
 
 // Algorithm 2, one thread per window.  Duplicate windows inside one call are independent atomic
@@ -159,28 +31,94 @@ __global__ void k_tg_update(TgView t, const int32_t* __restrict__ tok, int n, co
         atomicCAS(t.status, 0, (int)ADED_ERR_INVALID_ARG);
         return;
     }
-    tg_add(t, a, b, c, 1u);
+    tg_add(t, a, b, c, 1u, true);
+}
+
+// The same for a long span: a block first adds up equal windows of its BULK_WINDOWS in a hash table in shared memory and then
+// raises every distinct tri-gram once.  In text a few tri-grams are a large share of all windows (one in twenty of the
+// synthetic text's), and a count takes one atomic add at a time.  Sums are the same whatever the order; no count can wrap, as the
+// increments of a launch add up to fewer than 2^31.  `n` windows begin at tok[0].
+// Measured, one thread per window against this (an empty table / one that holds the span already), us: 131,000 tokens 87 / 36
+// against 88 / 39, 262,000 154 / 64 against 117 / 50, 10^6 406 / 255 against 287 / 139, 4 x 10^6 1284 / 1044 against 824 / 499:
+// the line is at BULK_MIN; below, blocks of this size leave the device idle (20,000: 37 / 19 against 68 / 35).  What bounds it
+// then is random access to the home buckets and the index (about 7 x 10^9 windows a second), and when filling the hand-overs of
+// new entries.  Blocks of 512 threads and 1024 windows: 291 / 149 at 10^6.
+constexpr int BULK_THREADS = 1024, BULK_WINDOWS = 2048, BULK_SLOTS = 4096, BULK_MIN = 1 << 17;
+__global__ void __launch_bounds__(BULK_THREADS) k_tg_update_bulk(TgView t, const int32_t* __restrict__ tok, int n) {
+    extern __shared__ int32_t bulk_smem[];
+    int32_t* s_tok = bulk_smem;                               // [BULK_WINDOWS + 2]
+    int32_t* s_first = s_tok + BULK_WINDOWS + 2;              // [BULK_SLOTS] window that stands for the slot's tri-gram, -1 empty
+    int32_t* s_count = s_first + BULK_SLOTS;                  // [BULK_SLOTS]
+    __shared__ int s_stop;
+    if (threadIdx.x == 0) s_stop = *t.status != 0;
+    __syncthreads();
+    if (s_stop) return;
+    const int w0 = blockIdx.x * BULK_WINDOWS, nw = min(BULK_WINDOWS, n - w0);
+    for (int i = threadIdx.x; i < nw + 2; i += BULK_THREADS) s_tok[i] = tok[w0 + i];
+    for (int i = threadIdx.x; i < BULK_SLOTS; i += BULK_THREADS) { s_first[i] = -1; s_count[i] = 0; }
+    __syncthreads();
+    for (int i = threadIdx.x; i < nw; i += BULK_THREADS) {
+        const int a = s_tok[i], b = s_tok[i + 1], c = s_tok[i + 2];
+        if (a < 0 || b < 0 || c < 0 || a >= t.vocab || b >= t.vocab || c >= t.vocab) {
+            tg_report(t, (int)ADED_ERR_INVALID_ARG);
+            continue;
+        }
+        int at = (int)(tg_hash(tg_key(a, b) * 31ull + (uint32_t)c) & (BULK_SLOTS - 1));
+        for (;;) {                                            // (twice as many slots as windows: ends)
+            const int have = atomicCAS(&s_first[at], -1, i);
+            if (have == -1 || (s_tok[have] == a && s_tok[have + 1] == b && s_tok[have + 2] == c)) break;
+            at = (at + 1) & (BULK_SLOTS - 1);
+        }
+        atomicAdd(&s_count[at], 1);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < BULK_SLOTS; i += BULK_THREADS) {
+        const int w = s_first[i];
+        if (w >= 0) tg_add(t, s_tok[w], s_tok[w + 1], s_tok[w + 2], (uint32_t)s_count[i], true);
+    }
 }
 
 // Every stored tri-gram with count >= min_count as (a, b, c) and its count, in no particular order;
-// *n_out counts all of them, only the first `max_entries` are written.
+// *n_out counts all of them, only the first `max_entries` are written.  A warp takes 32 home buckets at a time, a lane each,
+// and then together the further entries of those that have any.
+__device__ __forceinline__ void tg_export_one(unsigned long long key, int32_t tok, uint32_t cnt, bool take, int lane, int32_t* keys, uint32_t* counts,
+                                              unsigned long long max_entries, unsigned long long* n_out) {
+    const unsigned m = __ballot_sync(0xffffffffu, take);
+    if (m == 0) return;
+    unsigned long long at = 0;
+    if (lane == 0) at = atomicAdd(n_out, (unsigned long long)__popc(m));
+    at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << lane) - 1u));
+    if (take && at < max_entries) {
+        keys[3 * at + 0] = (int32_t)(key >> 32);
+        keys[3 * at + 1] = (int32_t)(key & 0xFFFFFFFFu);
+        keys[3 * at + 2] = tok;
+        counts[at] = cnt;
+    }
+}
 __global__ void k_tg_export(TgView t, uint32_t min_count, int32_t* __restrict__ keys, uint32_t* __restrict__ counts,
                             unsigned long long max_entries, unsigned long long* n_out) {
-    const size_t n = (size_t)t.n_home + t.n_over;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const Bucket* bk = t.buckets + i;
-        const unsigned long long key = bk->key;
-        if (key == TG_EMPTY) continue;
+    const int lane = threadIdx.x & 31;
+    const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
+    for (uint32_t g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; g < (t.n_home + 31) / 32; g += warps) {
+        const uint32_t mine = g * 32 + lane;
+        const unsigned long long key = mine < t.n_home ? t.buckets[mine].key : TG_EMPTY;
+        const bool used = key != TG_EMPTY;
+        if (!__any_sync(0xffffffffu, used)) continue;
         for (int e = 0; e < 6; ++e) {
-            const int32_t tk = bk->e[e].tok;
-            const uint32_t cn = bk->e[e].cnt;
-            if (tk < 0 || cn < min_count || cn == 0) continue;
-            const unsigned long long at = atomicAdd(n_out, 1ull);
-            if (at < max_entries) {
-                keys[3 * at + 0] = (int32_t)(key >> 32);
-                keys[3 * at + 1] = (int32_t)(key & 0xFFFFFFFFu);
-                keys[3 * at + 2] = tk;
-                counts[at] = cn;
+            const TgSlot s = used ? t.buckets[mine].e[e] : TgSlot{-1, 0u};
+            tg_export_one(key, s.tok, s.cnt, s.tok >= 0 && s.cnt >= min_count && s.cnt != 0, lane, keys, counts, max_entries, n_out);
+        }
+        for (unsigned more = __ballot_sync(0xffffffffu, used && t.buckets[mine].more != 0); more; more &= more - 1) {
+            const int src = __ffs((int)more) - 1;
+            const TgWalk w = tg_open(t, g * 32 + src, lane);
+            const unsigned long long k = __shfl_sync(0xffffffffu, key, src);
+            for (uint32_t i0 = 0; i0 < w.n; i0 += 32) {
+                const uint32_t m = (i0 + lane) / TG_UNIT;
+                const int x = tg_extent(m);
+                const uint32_t base = __shfl_sync(0xffffffffu, w.extent, x & 31);
+                TgSlot s = {-1, 0u};
+                if (i0 + lane < w.n && base != 0) s = t.pool[((size_t)(base - 1) + (m + 1 - (1u << x))) * TG_UNIT + (i0 + lane) % TG_UNIT];
+                tg_export_one(k, s.tok, s.cnt, s.tok >= 0 && s.cnt >= min_count && s.cnt != 0, lane, keys, counts, max_entries, n_out);
             }
         }
     }
@@ -198,139 +136,115 @@ __global__ void k_tg_import(TgView t, const int32_t* __restrict__ keys, const ui
     }
     if (inc == 0) return;
     if (inc > t.cap) inc = t.cap;
-    tg_add(t, a, b, c, inc);
+    tg_add(t, a, b, c, inc, false);
 }
 
-// One selection round of a warp over the chain that starts at `home`: the largest packed
-// (count, ~token) strictly below `prev`, or 0 when nothing is left; `total` = sum of the counts.
-__device__ __forceinline__ unsigned long long tg_select_round(const TgView& t, int64_t home, unsigned long long prev,
-                                                              int lane, uint32_t* total_out) {
-    unsigned long long best = 0;
-    uint32_t total = 0;
-    int64_t cur = home;
-    for (uint32_t hop = 0; cur >= 0 && hop <= t.n_over; ++hop) {
-        const Bucket* bk = t.buckets + cur;
-        if (lane < 6) {
-            const int32_t tk = bk->e[lane].tok;
-            const uint32_t cn = bk->e[lane].cnt;
-            if (tk >= 0) {
-                total += cn;
-                const unsigned long long key = ((unsigned long long)cn << 32) | (0xFFFFFFFFu - (uint32_t)tk);
-                if (cn >= t.min_count && cn > 0 && key < prev && key > best) best = key;
-            }
-        }
-        const uint32_t nxt = bk->next;
-        cur = nxt == 0 ? -1 : (int64_t)nxt;
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long ob = __shfl_xor_sync(0xffffffffu, best, o);
-        if (ob > best) best = ob;
-        total += __shfl_xor_sync(0xffffffffu, total, o);
-    }
-    if (total_out) *total_out = total;
-    return best;
-}
+// Top-k lists of q contexts.  A block takes `per_block` queries.  Its threads first look up the home buckets, one query each,
+// and hang queries of the same context on one entry of a hash table in shared memory: in text, frequent contexts are asked for
+// again and again, and they are the ones with thousands of continuations.  Every distinct context is then scanned once per
+// block, by one warp -- or, while at most TOPK_WIDE contexts of the block have more than TOPK_LONG entries, those by the whole
+// block -- and the list is written to all queries that asked for it.
+// Measured (2^20 queries drawn from a 16-million-token text, k = 4; 4.9e9 entries on the contexts of all queries, 0.2-0.5e9 on
+// the distinct ones of each block): bound by the L2 reads of the entries.
+constexpr int TOPK_THREADS = 512, TOPK_WARPS = TOPK_THREADS / 32, TOPK_MAX_QUERIES = 3072;
+constexpr uint32_t TOPK_LONG = 2048;
+constexpr int TOPK_WIDE = 4;
 
-// The k <= TG_LIST largest packed (count, ~token) keys of the chain that starts at `home`, in descending order
-// (count descending, token ascending among equals), in ONE walk over the chain: lanes 0..5 each keep the best
-// TG_LIST keys of their entry slot of every bucket in registers (sorted insertion); afterwards the six lists
-// are merged by k warp-wide maxima, the lane that held a maximum dropping it.  Keys are distinct (a context
-// holds a token once).  Every lane returns the same list in `out` (0 = nothing left); `total` = sum of the counts.
-constexpr int TG_LIST = 8;
-static_assert(TG_LIST >= ADED_DRAFT_MAX_K, "the draft tree takes its lists in one walk");
-__device__ __forceinline__ void tg_select_list(const TgView& t, int64_t home, int k, int lane,
-                                               unsigned long long (&out)[TG_LIST], uint32_t* total_out) {
-    unsigned long long loc[TG_LIST];
-#pragma unroll
-    for (int i = 0; i < TG_LIST; ++i) loc[i] = 0;
-    uint32_t total = 0;
-    int64_t cur = home;
-    for (uint32_t hop = 0; cur >= 0 && hop <= t.n_over; ++hop) {
-        const Bucket* bk = t.buckets + cur;
-        if (lane < 6) {
-            const int32_t tk = bk->e[lane].tok;
-            const uint32_t cn = bk->e[lane].cnt;
-            if (tk >= 0) {
-                total += cn;
-                unsigned long long key = ((unsigned long long)cn << 32) | (0xFFFFFFFFu - (uint32_t)tk);
-                if (cn >= t.min_count && cn > 0 && key > loc[TG_LIST - 1]) {
-#pragma unroll
-                    for (int i = 0; i < TG_LIST; ++i) {       // sorted insertion: the key sinks to its place
-                        if (key > loc[i]) { const unsigned long long tmp = loc[i]; loc[i] = key; key = tmp; }
-                    }
-                }
-            }
+// Slots of the block's hash table: a power of two, at most four fifths full.
+static __host__ __device__ int topk_slots(int per_block) {
+    int n = 32;
+    while (n < per_block + per_block / 4) n *= 2;
+    return n;
+}
+static size_t topk_smem(int per_block) { return (size_t)topk_slots(per_block) * 8 + (size_t)per_block * 8; }
+
+__global__ void __launch_bounds__(TOPK_THREADS, 3)
+k_tg_topk(TgView t, const int32_t* __restrict__ ctx, int q, int k, int per_block, int32_t* __restrict__ out_tok,
+          uint32_t* __restrict__ out_cnt, uint32_t* __restrict__ out_total) {
+    extern __shared__ int32_t topk_smem_raw[];
+    const int slots = topk_slots(per_block);
+    int32_t* s_key = topk_smem_raw;                 // [slots] home bucket, -1 empty
+    int32_t* s_head = s_key + slots;                // [slots] last query (index in the block) hung on it, -1 none
+    int32_t* s_next = s_head + slots;               // [per_block]
+    int32_t* s_order = s_next + per_block;          // [per_block] the slots in use, long contexts from the back
+    __shared__ int s_n, s_long, s_cursor;
+    __shared__ unsigned long long s_best[TOPK_WARPS * 32];
+    __shared__ uint32_t s_total[TOPK_WARPS];
+    const int q0 = blockIdx.x * per_block, nq = min(per_block, q - q0);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int i = threadIdx.x; i < slots; i += TOPK_THREADS) { s_key[i] = -1; s_head[i] = -1; }
+    if (threadIdx.x == 0) { s_n = 0; s_long = 0; s_cursor = 0; }
+    __syncthreads();
+    for (int i = threadIdx.x; i < nq; i += TOPK_THREADS) {
+        const int a = ctx[2 * (size_t)(q0 + i)], b = ctx[2 * (size_t)(q0 + i) + 1];
+        int64_t home = -1;
+        if (a >= 0 && b >= 0 && a < t.vocab && b < t.vocab) home = tg_find_home(t, tg_key(a, b), false);
+        if (home < 0) {
+            for (int r = 0; r < k; ++r) { out_tok[(size_t)(q0 + i) * k + r] = -1; out_cnt[(size_t)(q0 + i) * k + r] = 0; }
+            if (out_total) out_total[q0 + i] = 0;
+            continue;
         }
-        const uint32_t nxt = bk->next;
-        cur = nxt == 0 ? -1 : (int64_t)nxt;
+        int at = (int)(((uint32_t)home * 0x9E3779B1u) >> 8) & (slots - 1);
+        for (;;) {                                  // (more slots than queries: ends)
+            const int have = atomicCAS(&s_key[at], -1, (int)home);
+            if (have == -1) {
+                if ((t.buckets[home].n_more & ~TG_CLOSED) > TOPK_LONG) s_order[per_block - 1 - atomicAdd(&s_long, 1)] = at;
+                else s_order[atomicAdd(&s_n, 1)] = at;
+            }
+            if (have == -1 || have == (int)home) break;
+            at = (at + 1) & (slots - 1);
+        }
+        s_next[i] = atomicExch(&s_head[at], i);
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
-    if (total_out) *total_out = total;
-#pragma unroll
-    for (int r = 0; r < TG_LIST; ++r) {
+    __syncthreads();
+    auto write = [&](int slot, unsigned long long best, uint32_t total) {
+        for (int i = s_head[slot]; i >= 0; i = s_next[i]) {
+            const size_t row = (size_t)(q0 + i);
+            if (lane < k) {
+                out_tok[row * k + lane] = tg_packed_tok(best);
+                out_cnt[row * k + lane] = tg_packed_cnt(best);
+            }
+            if (lane == 0 && out_total) out_total[row] = total;
+        }
+    };
+    const int n_long = s_long, n_short = s_n;
+    const bool wide = n_long <= TOPK_WIDE;
+    for (int j = 0; wide && j < n_long; ++j) {
+        const int slot = s_order[per_block - 1 - j];
         unsigned long long best = 0;
-        if (r < k) {
-            best = loc[0];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const unsigned long long ob = __shfl_xor_sync(0xffffffffu, best, o);
-                if (ob > best) best = ob;
-            }
-            if (best != 0 && loc[0] == best) {                // this lane held it: drop it
-#pragma unroll
-                for (int i = 0; i + 1 < TG_LIST; ++i) loc[i] = loc[i + 1];
-                loc[TG_LIST - 1] = 0;
-            }
+        uint32_t total = 0;
+        tg_scan(t, tg_open(t, (uint32_t)s_key[slot], lane), warp, TOPK_WARPS, k, lane, best, total);
+        s_best[warp * 32 + lane] = lane < k ? best : 0ull;
+        total = __reduce_add_sync(0xffffffffu, total);
+        if (lane == 0) s_total[warp] = total;
+        __syncthreads();
+        if (warp == 0) {
+            for (int w = 1; w < TOPK_WARPS; ++w) tg_offer(s_best[w * 32 + lane], k, lane, best);
+            total = __reduce_add_sync(0xffffffffu, lane < TOPK_WARPS ? s_total[lane] : 0u);
+            write(slot, best, total);
         }
-        out[r] = best;
+        __syncthreads();
     }
-}
-
-// One warp per query.  Up to TG_LIST continuations: one walk over the context's chain (tg_select_list).  Longer
-// lists: k selection rounds, a round picking the largest packed (count, ~token) strictly below the previous
-// pick, which yields count descending, token ascending among equals, without storing the list.
-__global__ void k_tg_topk(TgView t, const int32_t* __restrict__ ctx, int q, int k, int32_t* __restrict__ out_tok,
-                          uint32_t* __restrict__ out_cnt, uint32_t* __restrict__ out_total) {
-    const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (w >= q) return;
-    const int a = ctx[2 * w], b = ctx[2 * w + 1];
-    int64_t home = -1;
-    if (a >= 0 && b >= 0 && a < t.vocab && b < t.vocab) home = tg_find_home(t, tg_key(a, b), false);
-    if (k <= TG_LIST) {
-        unsigned long long list[TG_LIST];
-        uint32_t total;
-        tg_select_list(t, home, k, lane, list, &total);
-        if (lane == 0) {
-#pragma unroll
-            for (int r = 0; r < TG_LIST; ++r) {
-                if (r < k) {
-                    out_tok[(size_t)w * k + r] = list[r] ? (int32_t)(0xFFFFFFFFu - (uint32_t)list[r]) : -1;
-                    out_cnt[(size_t)w * k + r] = (uint32_t)(list[r] >> 32);
-                }
-            }
-            if (out_total) out_total[w] = total;
-        }
-        return;
-    }
-    unsigned long long prev = ~0ull;
-    for (int round = 0; round < k; ++round) {
-        uint32_t total;
-        const unsigned long long best = tg_select_round(t, home, prev, lane, &total);
-        if (lane == 0) {
-            out_tok[(size_t)w * k + round] = best ? (int32_t)(0xFFFFFFFFu - (uint32_t)best) : -1;
-            out_cnt[(size_t)w * k + round] = (uint32_t)(best >> 32);
-            if (round == 0 && out_total) out_total[w] = total;
-        }
-        prev = best ? best : 0;   // nothing left: later rounds find nothing either
+    // the rest, longest first as far as they are sorted
+    const int first = wide ? n_long : 0, jobs = n_long - first + n_short;
+    for (;;) {
+        int j = 0;
+        if (lane == 0) j = atomicAdd(&s_cursor, 1);
+        j = __shfl_sync(0xffffffffu, j, 0);
+        if (j >= jobs) break;
+        const int slot = j < n_long - first ? s_order[per_block - 1 - first - j] : s_order[j - (n_long - first)];
+        unsigned long long best = 0;
+        uint32_t total = 0;
+        tg_scan(t, tg_open(t, (uint32_t)s_key[slot], lane), 0, 1, k, lane, best, total);
+        write(slot, best, __reduce_add_sync(0xffffffffu, total));
     }
 }
 
 // Draft tree of n_nodes nodes for the context (ctx[0], ctx[1]); one block of 32 warps.
-// Level by level: every node of the current level gets its top-k list (one warp per node), then
-// one thread appends the lists in node order, rank order -- the same tree as visiting the nodes in
-// index order.  The filler pass (one thread; child lists kept in shared memory) hangs caller-
+// Level by level: every node of the current level gets its top-k list -- the block's warps are shared out evenly, so that
+// the first levels' few nodes, whose contexts may have thousands of continuations, are scanned by several warps each --
+// then one warp appends the lists in node order, rank order: the same tree as visiting the nodes in index order.
+// Latency-bound: a level is the chain home bucket -> directory -> entries -> merge.  The filler pass (one thread; child lists kept in shared memory) hangs caller-
 // supplied tokens under nodes with room, round-robin, until the tree is full.
 constexpr int DRAFT_MAX_FILLER = 4 * ADED_MAX_NODES;
 
@@ -365,7 +279,7 @@ __device__ __forceinline__ int draft_fill(int32_t* tok, int32_t* par, int32_t* d
             *fail = true;
             break;
         }
-        p = (p + 1) % n;
+        if (++p >= n) p = 0;
     }
     return n;
 }
@@ -377,6 +291,7 @@ k_draft_tree(TgView t, const int32_t* __restrict__ ctx, int n_nodes, int max_dep
     __shared__ int32_t s_tok[ADED_MAX_NODES], s_par[ADED_MAX_NODES], s_dep[ADED_MAX_NODES], s_nkid[ADED_MAX_NODES];
     __shared__ int32_t s_cand[ADED_MAX_NODES * ADED_DRAFT_MAX_K];   // top-k lists, later the child tokens of every node
     __shared__ int32_t s_fill[DRAFT_MAX_FILLER];
+    __shared__ unsigned long long s_part[32 * ADED_DRAFT_MAX_K];    // the lists of the warps that share a node
     __shared__ int s_n, s_lo, s_hi, s_fail;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int prev_token = ctx[0];
@@ -395,35 +310,52 @@ k_draft_tree(TgView t, const int32_t* __restrict__ ctx, int n_nodes, int max_dep
     for (int d = 0; d < max_depth; ++d) {
         const int lo = s_lo, hi = s_hi;
         if (lo >= hi || s_n >= n_nodes) break;
-        for (int node = lo + warp; node < hi; node += 32) {
+        int parts = 1;                                  // warps per node
+        while (parts * 2 * (hi - lo) <= 32) parts *= 2;
+        for (int node = lo + warp / parts; node < hi; node += 32 / parts) {
             const int u = node == 0 ? prev_token : s_tok[s_par[node]], w = s_tok[node];
-            int64_t home = -1;
-            if (u >= 0 && w >= 0 && u < t.vocab && w < t.vocab) home = tg_find_home(t, tg_key(u, w), false);
-            unsigned long long list[TG_LIST];          // (k <= ADED_DRAFT_MAX_K = TG_LIST: one walk over the chain)
-            tg_select_list(t, home, k, lane, list, nullptr);
-            if (lane == 0) {
-#pragma unroll
-                for (int r = 0; r < TG_LIST; ++r)
-                    if (r < k) s_cand[node * ADED_DRAFT_MAX_K + r] = list[r] ? (int32_t)(0xFFFFFFFFu - (uint32_t)list[r]) : -1;
+            unsigned long long best = 0;
+            uint32_t total = 0;
+            tg_scan(t, tg_open(t, u, w, lane), warp % parts, parts, k, lane, best, total);
+            if (lane < k) {
+                if (parts == 1) s_cand[node * ADED_DRAFT_MAX_K + lane] = tg_packed_tok(best);
+                else s_part[warp * ADED_DRAFT_MAX_K + lane] = best;
             }
         }
         __syncthreads();
-        if (threadIdx.x == 0) {
-            int n = s_n;
-            for (int node = lo; node < hi && n < n_nodes; ++node) {
-                for (int j = 0; j < k && n < n_nodes; ++j) {
-                    const int32_t c = s_cand[node * ADED_DRAFT_MAX_K + j];
-                    if (c < 0) break;
-                    s_tok[n] = c;
-                    s_par[n] = node;
-                    s_dep[n] = d + 1;
-                    s_nkid[node] = j + 1;    // s_cand[node][0 .. j] are this node's child tokens
-                    ++n;
-                }
+        if (parts > 1 && warp < hi - lo) {
+            unsigned long long best = 0;
+            for (int i = 0; i < parts; i += 32 / ADED_DRAFT_MAX_K) {      // four warps' lists at a time
+                const int from = i + lane / ADED_DRAFT_MAX_K, r = lane % ADED_DRAFT_MAX_K;
+                tg_offer(from < parts && r < k ? s_part[(warp * parts + from) * ADED_DRAFT_MAX_K + r] : 0ull, k, lane, best);
             }
-            s_lo = hi;
-            s_hi = n;
-            s_n = n;
+            if (lane < k) s_cand[(lo + warp) * ADED_DRAFT_MAX_K + lane] = tg_packed_tok(best);
+        }
+        __syncthreads();
+        if (warp == 0) {
+            int n = s_n;
+            for (int node0 = lo; node0 < hi && n < n_nodes; node0 += 32) {
+                const int node = node0 + lane;
+                int mine = 0;                               // this node's children (valid entries come first)
+                if (node < hi)
+                    while (mine < k && s_cand[node * ADED_DRAFT_MAX_K + mine] >= 0) ++mine;
+                int upto = mine;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int other = __shfl_up_sync(0xffffffffu, upto, o);
+                    if (lane >= o) upto += other;
+                }
+                const int at = n + upto - mine;
+                const int kept = max(0, min(mine, n_nodes - at));
+                for (int j = 0; j < kept; ++j) {
+                    s_tok[at + j] = s_cand[node * ADED_DRAFT_MAX_K + j];
+                    s_par[at + j] = node;
+                    s_dep[at + j] = d + 1;
+                }
+                if (kept > 0) s_nkid[node] = kept;          // s_cand[node][0 .. kept) are this node's child tokens
+                n = min(n_nodes, n + __shfl_sync(0xffffffffu, upto, 31));
+            }
+            if (lane == 0) { s_lo = hi; s_hi = n; s_n = n; }
         }
         __syncthreads();
     }
@@ -470,24 +402,36 @@ __global__ void k_decode_advance(const int32_t* __restrict__ out_tok, int32_t* _
 __global__ void k_tg_get(TgView t, int a, int b, int c, uint32_t* out) {
     *out = 0;
     if (a < 0 || b < 0 || c < 0 || a >= t.vocab || b >= t.vocab || c >= t.vocab) return;
-    int64_t cur = tg_find_home(t, tg_key(a, b), false);
-    for (uint32_t hop = 0; cur >= 0 && hop <= t.n_over; ++hop) {
-        const Bucket* bk = t.buckets + cur;
-        for (int e = 0; e < 6; ++e)
-            if (bk->e[e].tok == c) { *out = bk->e[e].cnt; return; }
-        cur = bk->next == 0 ? -1 : (int64_t)bk->next;
-    }
+    const uint32_t* cnt = tg_find(t, a, b, c);
+    if (cnt) *out = *cnt;
 }
 
+// Stored tri-grams, and buckets in use (home buckets and units of six further entries).
 __global__ void k_tg_stats(TgView t, unsigned long long* out) {
     unsigned long long entries = 0, used = 0;
-    const size_t n = (size_t)t.n_home + t.n_over;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < t.n_home; i += gridDim.x * blockDim.x) {
         const Bucket* bk = t.buckets + i;
-        int here = 0;
-        for (int e = 0; e < 6; ++e) here += bk->e[e].tok >= 0;
-        entries += here;
-        used += bk->key != TG_EMPTY;
+        if (bk->key == TG_EMPTY) continue;
+        ++used;
+        for (int e = 0; e < 6; ++e) entries += bk->e[e].tok >= 0;
+        if (bk->more == 0 || bk->more == TG_FAILED) continue;
+        const uint32_t n = bk->n_more & ~TG_CLOSED;
+        if (!(bk->n_more & TG_CLOSED)) {
+            entries += n;
+            used += (n + TG_UNIT - 1) / TG_UNIT;
+            continue;
+        }
+        const uint32_t* dir = reinterpret_cast<const uint32_t*>(t.pool + (size_t)(bk->more - 1) * TG_UNIT);
+        for (uint32_t m = 0; m * TG_UNIT < n; ++m) {       // a context that ran out of room: some of its entries are not there
+            const int x = tg_extent(m);
+            const uint32_t base = x == 0 ? bk->more + TG_DIR_UNITS : x < TG_LINKS ? dir[x] : 0;
+            if (base == 0 || base == TG_FAILED) continue;
+            int here = 0;
+            for (uint32_t e = 0; e < TG_UNIT && m * TG_UNIT + e < n; ++e)
+                here += t.pool[((size_t)(base - 1) + (m + 1 - (1u << x))) * TG_UNIT + e].tok >= 0;
+            entries += here;
+            used += here > 0;
+        }
     }
     atomicAdd(out, entries);
     atomicAdd(out + 1, used);
@@ -496,14 +440,12 @@ __global__ void k_tg_stats(TgView t, unsigned long long* out) {
 
 // ---- draft maker: Monte Carlo tree search (Eq. 2-3, Algorithm 1) -----------------------------------
 // One warp runs the search; every lane executes the same scalar logic on the tree in shared memory
-// (lane 0 alone writes), the lanes cooperate only in the table lookups.  A lookup reads the context's
-// chain once into shared memory and then selects the k best entries there.  Floating point is IEEE
+// (lane 0 alone writes), the lanes cooperate only in the table lookups.  Floating point is IEEE
 // double, one rounded operation at a time (no fused multiply-add), so that the search can be
 // reproduced bit for bit; the exploration factor E of Eq. 3 depends on an integer only and comes
 // from a table the host computes.
 constexpr int MC_MAX_ITER = 160, MC_MAX_K = ADED_DRAFT_MAX_K, MC_MAX_LEN = 8;
 constexpr int MC_MAX_NODES = 1 + MC_MAX_ITER * MC_MAX_K;
-constexpr int MC_CHAIN = 192;          // entries of a context held in shared memory (32 buckets)
 constexpr int MC_CACHE = 64;           // remembered lookups (direct mapped): a search meets the same contexts again and again
 
 struct McParams {
@@ -519,81 +461,34 @@ struct McLookup {                      // top-k list of one context
 };
 
 // All 32 lanes call this with the same (a, b); the result is identical in every lane.
-__device__ __forceinline__ void mc_lookup(const TgView& t, int a, int b, int k, int lane, int32_t* s_tok, uint32_t* s_cnt,
-                                          McLookup& out) {
-    out.n = 0;
-    out.total = 0;
-    int64_t home = -1;
-    if (a >= 0 && b >= 0 && a < t.vocab && b < t.vocab) home = tg_find_home(t, tg_key(a, b), false);
-    if (home < 0) return;
-    // pass 1: the chain into shared memory (six entries per bucket, lanes 0..5 read them)
-    int n_ent = 0;
-    bool overflow = false;
-    int64_t cur = home;
-    for (uint32_t hop = 0; cur >= 0 && hop <= t.n_over; ++hop) {
-        const Bucket* bk = t.buckets + cur;
-        if (n_ent + 6 > MC_CHAIN) { overflow = true; break; }
-        if (lane < 6) { s_tok[n_ent + lane] = bk->e[lane].tok; s_cnt[n_ent + lane] = bk->e[lane].cnt; }
-        n_ent += 6;
-        const uint32_t nxt = bk->next;
-        cur = nxt == 0 ? -1 : (int64_t)nxt;
-    }
-    __syncwarp();
-    unsigned long long prev = ~0ull;
-    if (overflow) {                    // a very long chain: select round by round from global memory
-        for (int round = 0; round < k; ++round) {
-            uint32_t total;
-            const unsigned long long best = tg_select_round(t, home, prev, lane, &total);
-            out.total = total;
-            if (!best) break;
-            out.word[out.n] = (int32_t)(0xFFFFFFFFu - (uint32_t)best);
-            out.count[out.n] = (uint32_t)(best >> 32);
-            ++out.n;
-            prev = best;
-        }
-        return;
-    }
+__device__ __forceinline__ void mc_lookup(const TgView& t, int a, int b, int k, int lane, McLookup& out) {
+    unsigned long long best = 0;
     uint32_t total = 0;
-    for (int i = lane; i < n_ent; i += 32)
-        if (s_tok[i] >= 0) total += s_cnt[i];
-    for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
-    out.total = total;
-    for (int round = 0; round < k; ++round) {
-        unsigned long long best = 0;
-        for (int i = lane; i < n_ent; i += 32) {
-            const int32_t tk = s_tok[i];
-            const uint32_t cn = s_cnt[i];
-            if (tk < 0 || cn == 0 || cn < t.min_count) continue;
-            const unsigned long long key = ((unsigned long long)cn << 32) | (0xFFFFFFFFu - (uint32_t)tk);
-            if (key < prev && key > best) best = key;
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-            const unsigned long long ob = __shfl_xor_sync(0xffffffffu, best, o);
-            if (ob > best) best = ob;
-        }
-        if (!best) break;
-        out.word[out.n] = (int32_t)(0xFFFFFFFFu - (uint32_t)best);
-        out.count[out.n] = (uint32_t)(best >> 32);
-        ++out.n;
-        prev = best;
+    tg_scan(t, tg_open(t, a, b, lane), 0, 1, k, lane, best, total);
+    out.total = __reduce_add_sync(0xffffffffu, total);
+    out.n = __popc(__ballot_sync(0xffffffffu, lane < k && best != 0));
+#pragma unroll
+    for (int r = 0; r < MC_MAX_K; ++r) {
+        const unsigned long long key = __shfl_sync(0xffffffffu, best, r);
+        out.word[r] = tg_packed_tok(key);
+        out.count[r] = tg_packed_cnt(key);
     }
-    __syncwarp();
 }
 
 // mc_lookup through the cache of remembered contexts (the table does not change during a search).
-__device__ __forceinline__ void mc_lookup_cached(const TgView& t, int a, int b, int k, int lane, int32_t* s_tok, uint32_t* s_cnt,
+__device__ __forceinline__ void mc_lookup_cached(const TgView& t, int a, int b, int k, int lane,
                                                  unsigned long long* s_ckey, McLookup* s_cval, McLookup& out) {
     const unsigned long long key = tg_key(a, b);
     const int slot = (int)(tg_hash(key) & (MC_CACHE - 1));
     if (s_ckey[slot] == key) { out = s_cval[slot]; return; }
-    mc_lookup(t, a, b, k, lane, s_tok, s_cnt, out);
+    mc_lookup(t, a, b, k, lane, out);
     __syncwarp();
     if (lane == 0) { s_cval[slot] = out; s_ckey[slot] = key; }
     __syncwarp();
 }
 
 __host__ __device__ constexpr size_t mc_cache_offset() {
-    return (((size_t)MC_MAX_NODES * (2 * 8 + 2 * 4 + 2 * 2 + 2 * 1) + (size_t)MC_CHAIN * 8 + ADED_MAX_NODES * 2) + 15) & ~(size_t)15;
+    return (((size_t)MC_MAX_NODES * (2 * 8 + 2 * 4 + 2 * 2 + 2 * 1) + ADED_MAX_NODES * 2) + 15) & ~(size_t)15;
 }
 
 __host__ __device__ constexpr size_t mc_fill_offset() {
@@ -611,9 +506,7 @@ k_mcts_draft(TgView t, const __grid_constant__ McParams p, const int32_t* __rest
     double* s_prior = s_score + MC_MAX_NODES;                             // Eq. 1 probability of the node's token in its parent's context
     int32_t* s_tok = reinterpret_cast<int32_t*>(s_prior + MC_MAX_NODES);  // token
     int32_t* s_visits = s_tok + MC_MAX_NODES;
-    int32_t* s_ltok = s_visits + MC_MAX_NODES;                            // lookup scratch
-    uint32_t* s_lcnt = reinterpret_cast<uint32_t*>(s_ltok + MC_CHAIN);
-    int16_t* s_par = reinterpret_cast<int16_t*>(s_lcnt + MC_CHAIN);
+    int16_t* s_par = reinterpret_cast<int16_t*>(s_visits + MC_MAX_NODES);
     int16_t* s_first = s_par + MC_MAX_NODES;                              // first child (children are consecutive)
     int16_t* s_queue = s_first + MC_MAX_NODES;                            // [ADED_MAX_NODES] breadth-first order of the result
     uint8_t* s_nkid = reinterpret_cast<uint8_t*>(s_queue + ADED_MAX_NODES);
@@ -668,7 +561,7 @@ k_mcts_draft(TgView t, const __grid_constant__ McParams p, const int32_t* __rest
         // expansion
         if (!(s_flag[node] & 1) && !end) {
             const int a = node == 0 ? prev_token : s_tok[s_par[node]], b = s_tok[node];
-            mc_lookup_cached(t, a, b, p.k, lane, s_ltok, s_lcnt, s_ckey, s_cval, lk);
+            mc_lookup_cached(t, a, b, p.k, lane, s_ckey, s_cval, lk);
             if (lane == 0) {
                 s_flag[node] |= 1;
                 s_first[node] = (int16_t)n_nodes;
@@ -693,7 +586,7 @@ k_mcts_draft(TgView t, const __grid_constant__ McParams p, const int32_t* __rest
         int draws = 0;
         while (len < p.length + 1) {
             const int a = len >= 2 ? state[len - 2] : prev_token, b = state[len - 1];
-            mc_lookup_cached(t, a, b, p.k, lane, s_ltok, s_lcnt, s_ckey, s_cval, lk);
+            mc_lookup_cached(t, a, b, p.k, lane, s_ckey, s_cval, lk);
             if (lk.n == 0) break;
             unsigned long long total = 0;
             for (int j = 0; j < lk.n; ++j) total += lk.count[j];
@@ -820,6 +713,15 @@ static constexpr size_t TG_STAGE = 1 << 16;
 static constexpr int STEP_SPAN = 0, STEP_LEN = ADED_MAX_NODES + 2, STEP_REAL = STEP_LEN + 1, STEP_FILL = STEP_REAL + 1;
 static constexpr int STEP_INTS = STEP_FILL + DRAFT_MAX_FILLER;
 
+// An empty table: home buckets and index.  The pool needs no clearing: an entry is written before anything refers to it.
+static aded_status tg_reset(aded_trigram* t, cudaStream_t st) {
+    k_tg_init<<<2048, 512, 0, st>>>(reinterpret_cast<uint4*>(t->view.buckets), (size_t)t->view.n_home * (sizeof(Bucket) / sizeof(uint4)));
+    ADED_CUDA_TRY(cudaMemsetAsync(t->view.index, 0, (size_t)(t->view.index_mask + 1) * sizeof(TgIndexSlot), st));
+    ADED_CUDA_TRY(cudaMemsetAsync(t->view.used, 0, 2 * sizeof(uint32_t), st));
+    ADED_CUDA_TRY(cudaGetLastError());
+    return ADED_OK;
+}
+
 extern "C" {
 
 aded_status aded_trigram_create(const aded_trigram_config* cfg, aded_trigram** out) {
@@ -836,16 +738,31 @@ aded_status aded_trigram_create(const aded_trigram_config* cfg, aded_trigram** o
     t->stats_dev = nullptr;
     t->step_i = nullptr;
     t->view = TgView();
-    const size_t n_home = (size_t)1 << cfg->log2_buckets, n = n_home + (size_t)cfg->overflow_buckets;
+    const size_t n_home = (size_t)1 << cfg->log2_buckets, n_units = (size_t)tg_pool_units((unsigned long long)cfg->overflow_buckets);
+    if (n_units > 0xFFFFFFF0ull) { delete t; return ADED_ERR_OOM; }      // (units are numbered in 32 bits; more would not fit the device)
+    size_t n_index = 16;                                                 // at most six entries per unit in use: three quarters full
+    while (n_index < 8 * (size_t)cfg->overflow_buckets) n_index *= 2;
     bool ok = cudaGetDevice(&t->device) == cudaSuccess;
     cudaError_t e = cudaSuccess;
-    if (ok) { e = cudaMalloc((void**)&t->view.buckets, n * sizeof(Bucket)); ok = e == cudaSuccess; }
-    if (ok) ok = cudaMalloc((void**)&t->view.over_used, sizeof(uint32_t)) == cudaSuccess;
-    if (ok) ok = cudaMalloc((void**)&t->view.status, sizeof(int32_t)) == cudaSuccess;
-    if (ok) ok = cudaMalloc((void**)&t->stage_i, TG_STAGE * sizeof(int32_t)) == cudaSuccess;
-    if (ok) ok = cudaMalloc((void**)&t->stage_u, TG_STAGE * sizeof(uint32_t)) == cudaSuccess;
-    if (ok) ok = cudaMalloc((void**)&t->stats_dev, 2 * sizeof(unsigned long long)) == cudaSuccess;
-    if (ok) ok = cudaMalloc((void**)&t->step_i, STEP_INTS * sizeof(int32_t)) == cudaSuccess;
+    // one allocation: home buckets, index, pool, then the small arrays (every part a multiple of 64 bytes)
+    const size_t parts[8] = {n_home * sizeof(Bucket), n_index * sizeof(TgIndexSlot), n_units * TG_UNIT * sizeof(TgSlot),
+                             TG_STAGE * sizeof(int32_t), TG_STAGE * sizeof(uint32_t), STEP_INTS * sizeof(int32_t),
+                             2 * sizeof(unsigned long long), 4 * sizeof(uint32_t)};
+    size_t at[9] = {0};
+    for (int i = 0; i < 8; ++i) at[i + 1] = at[i] + (parts[i] + 63) / 64 * 64;
+    char* block = nullptr;
+    if (ok) { e = cudaMalloc((void**)&block, at[8]); ok = e == cudaSuccess; }
+    if (ok) {
+        t->view.buckets = reinterpret_cast<Bucket*>(block + at[0]);
+        t->view.index = reinterpret_cast<TgIndexSlot*>(block + at[1]);
+        t->view.pool = reinterpret_cast<TgSlot*>(block + at[2]);
+        t->stage_i = reinterpret_cast<int32_t*>(block + at[3]);
+        t->stage_u = reinterpret_cast<uint32_t*>(block + at[4]);
+        t->step_i = reinterpret_cast<int32_t*>(block + at[5]);
+        t->stats_dev = reinterpret_cast<unsigned long long*>(block + at[6]);
+        t->view.used = reinterpret_cast<uint32_t*>(block + at[7]);
+        t->view.status = reinterpret_cast<int32_t*>(t->view.used + 2);
+    }
     if (!ok) {
         cudaGetLastError();
         aded_trigram_destroy(t);
@@ -854,11 +771,12 @@ aded_status aded_trigram_create(const aded_trigram_config* cfg, aded_trigram** o
     t->view.n_home = (uint32_t)n_home;
     t->view.n_home_mask = (uint32_t)n_home - 1;
     t->view.n_over = (uint32_t)cfg->overflow_buckets;
+    t->view.n_units = (uint32_t)n_units;
+    t->view.index_mask = n_index - 1;
     t->view.vocab = cfg->vocab;
     t->view.cap = cfg->cap == 0 ? 0x7fffffffu : cfg->cap;
     t->view.min_count = cfg->min_count;
-    k_tg_init<<<1024, 256>>>(t->view.buckets, n);
-    ok = cudaMemset(t->view.over_used, 0, sizeof(uint32_t)) == cudaSuccess &&
+    ok = tg_reset(t, nullptr) == ADED_OK &&
          cudaMemset(t->view.status, 0, sizeof(int32_t)) == cudaSuccess && cudaDeviceSynchronize() == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
@@ -871,13 +789,7 @@ aded_status aded_trigram_create(const aded_trigram_config* cfg, aded_trigram** o
 
 aded_status aded_trigram_destroy(aded_trigram* t) {
     if (!t) return ADED_ERR_INVALID_ARG;
-    if (t->view.buckets) cudaFree(t->view.buckets);
-    if (t->view.over_used) cudaFree(t->view.over_used);
-    if (t->view.status) cudaFree(t->view.status);
-    if (t->stage_i) cudaFree(t->stage_i);
-    if (t->stage_u) cudaFree(t->stage_u);
-    if (t->stats_dev) cudaFree(t->stats_dev);
-    if (t->step_i) cudaFree(t->step_i);
+    if (t->view.buckets) cudaFree(t->view.buckets);     // (the first part of the handle's one allocation)
     delete t;
     return ADED_OK;
 }
@@ -887,7 +799,11 @@ aded_status aded_trigram_update(aded_trigram* t, const int32_t* tokens_dev, int3
     if (n < 3) return ADED_OK;
     const int windows = n - 2;
     note_launch();
-    k_tg_update<<<(windows + 255) / 256, 256, 0, static_cast<cudaStream_t>(stream)>>>(t->view, tokens_dev, n, nullptr);
+    if (windows >= BULK_MIN)
+        k_tg_update_bulk<<<(windows + BULK_WINDOWS - 1) / BULK_WINDOWS, BULK_THREADS, (BULK_WINDOWS + 2 + 2 * BULK_SLOTS) * sizeof(int32_t),
+                           static_cast<cudaStream_t>(stream)>>>(t->view, tokens_dev, windows);
+    else
+        k_tg_update<<<(windows + 255) / 256, 256, 0, static_cast<cudaStream_t>(stream)>>>(t->view, tokens_dev, n, nullptr);
     ADED_CUDA_TRY(cudaGetLastError());
     return ADED_OK;
 }
@@ -913,10 +829,15 @@ aded_status aded_trigram_topk(const aded_trigram* t, const int32_t* ctx_dev, int
     if (!t || q < 0 || k < 1 || k > 32) return ADED_ERR_INVALID_ARG;
     if (q == 0) return ADED_OK;
     if (!ctx_dev || !out_tokens_dev || !out_counts_dev) return ADED_ERR_INVALID_ARG;
-    const int warps_per_block = 4;
+    // As many queries per block as fill the device's block slots once (three blocks per SM).
+    const int wave = ws_grid_limit(t->device) / 2 * 3;
+    int per_block = (q + wave - 1) / wave;
+    per_block = per_block > TOPK_MAX_QUERIES ? TOPK_MAX_QUERIES : per_block;
+    static const cudaError_t prepared = cudaFuncSetAttribute(k_tg_topk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)topk_smem(TOPK_MAX_QUERIES));
+    ADED_CUDA_TRY(prepared);
     note_launch();
-    k_tg_topk<<<(q + warps_per_block - 1) / warps_per_block, warps_per_block * 32, 0, static_cast<cudaStream_t>(stream)>>>(
-        t->view, ctx_dev, q, k, out_tokens_dev, out_counts_dev, out_total_dev);
+    k_tg_topk<<<(q + per_block - 1) / per_block, TOPK_THREADS, topk_smem(per_block), static_cast<cudaStream_t>(stream)>>>(
+        t->view, ctx_dev, q, k, per_block, out_tokens_dev, out_counts_dev, out_total_dev);
     ADED_CUDA_TRY(cudaGetLastError());
     return ADED_OK;
 }
@@ -1092,12 +1013,8 @@ aded_status aded_trigram_import(aded_trigram* t, const int32_t* keys_dev, const 
 
 aded_status aded_trigram_clear(aded_trigram* t, void* stream) {
     if (!t) return ADED_ERR_INVALID_ARG;
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
     note_launch();
-    k_tg_init<<<1024, 256, 0, st>>>(t->view.buckets, (size_t)t->view.n_home + t->view.n_over);
-    ADED_CUDA_TRY(cudaMemsetAsync(t->view.over_used, 0, sizeof(uint32_t), st));
-    ADED_CUDA_TRY(cudaGetLastError());
-    return ADED_OK;
+    return tg_reset(t, static_cast<cudaStream_t>(stream));
 }
 
 // Scratch copy of the entries with count >= min_count; the caller frees *keys / *counts.

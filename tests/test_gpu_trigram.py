@@ -219,3 +219,104 @@ def test_import_of_duplicate_entries_with_large_counts_saturates(cuda_device):
     with pytest.raises(B.AdedError) as err:
         B.aded_trigram_create(100, log2_buckets=8, overflow_buckets=64, cap=2 ** 31)
     assert err.value.status == 1
+
+
+def _star(n, vocab=20000):
+    """A span in which the context (1, 2) has n continuations, first seen in the order of their ids, and a third of them twice."""
+    ids = [3 + i for i in range(n)] + [3 + i for i in range(0, n, 3)]
+    return [t for i in ids for t in (1, 2, i)]
+
+
+@pytest.mark.parametrize("n", [5, 6, 7, 12, 13, 24, 25, 47, 48, 49, 1536, 1537, 2054, 2055, 6150, 6151])
+def test_contexts_at_the_ends_of_extents(cuda_device, n):
+    """Continuations beyond six lie in extents of 6, 12, 24, ... entries: one context just below, at and above their ends (and
+    above the length from which a whole block scans it), asked for many times in one call beside others."""
+    from paper_2407_12021_b200 import binding as B
+    span = _star(n)
+    st = TrigramStore()
+    st.update(span)
+    t = B.aded_trigram_create(20000, log2_buckets=16, overflow_buckets=4096)
+    B.aded_trigram_update(t, torch.tensor(span, dtype=torch.int32, device="cuda"))
+    torch.cuda.synchronize()
+    assert B.aded_trigram_poll_status(t) == 0
+    assert B.aded_trigram_stats(t) == (len(st.entries()), len(st.table) + sum((len(v) - 1) // 6 for v in st.table.values() if len(v) > 6))
+    assert _entries_gpu(B, t) == st.entries()
+    for c in (3, 2 + n, 3 + n, 3 + n // 2):
+        assert B.aded_trigram_get(t, 1, 2, c) == st.count(1, 2, c)
+    contexts = ([(1, 2), (2, 3), (19999, 1), (3, 1)] * 40)[:157]
+    _check_against(B, t, st, contexts, ks=(1, 8, 9, 32))
+    _check_against(B, t, st, contexts[:1], ks=(3,))
+
+
+@pytest.mark.parametrize("n", [7, 12, 13, 18, 19, 43])
+def test_configured_overflow_is_the_limit(cuda_device, n):
+    """Entries beyond six count in units of six against overflow_buckets: exactly enough is enough, one fewer is a full table,
+    which keeps what it holds, goes on counting it and refuses new entries again after the status was read."""
+    from paper_2407_12021_b200 import binding as B
+    need = (n - 6 + 5) // 6
+    rows = [[1, 2, 3 + i] for i in range(n)]
+
+    def update(t, row):
+        B.aded_trigram_update(t, torch.tensor(row, dtype=torch.int32, device="cuda"))
+        torch.cuda.synchronize()
+        return B.aded_trigram_poll_status(t)
+
+    t = B.aded_trigram_create(100, log2_buckets=8, overflow_buckets=need)
+    assert [update(t, r) for r in rows] == [0] * n
+    t = B.aded_trigram_create(100, log2_buckets=8, overflow_buckets=need - 1)
+    fits = 6 * need
+    assert [update(t, r) for r in rows] == [0] * fits + [4] * (n - fits)
+    assert [update(t, r) for r in rows] == [0] * fits + [4] * (n - fits)
+    assert _entries_gpu(B, t) == {tuple(r): 2 for r in rows[:fits]}
+    assert B.aded_trigram_stats(t)[0] == fits
+    # the same at once: whatever is kept is counted right
+    t = B.aded_trigram_create(100, log2_buckets=8, overflow_buckets=need - 1)
+    assert update(t, [x for r in rows for x in r]) == 4
+    kept = _entries_gpu(B, t)
+    assert all(kept[k] == 1 for k in kept) and B.aded_trigram_stats(t)[0] == len(kept)
+    B.aded_trigram_clear(t)
+    assert update(t, rows[0]) == 0 and _entries_gpu(B, t) == {tuple(rows[0]): 1}
+
+
+def test_repeated_and_absent_contexts_in_one_call(cuda_device):
+    """Blocks answer a context once for all queries that ask for it: more queries than one block takes, every context many
+    times, several long ones per block, absent and out-of-range contexts between them."""
+    from paper_2407_12021_b200 import binding as B
+    spans = [1, 2, 3] * 5
+    for a in range(7):                          # seven contexts of 2500 continuations
+        spans += [t for i in range(2500) for t in (a, 10 + a, 100 + (i * 7 + a) % 4000)]
+    st = TrigramStore()
+    st.update(spans)
+    t = B.aded_trigram_create(5000, log2_buckets=16, overflow_buckets=1 << 14)
+    B.aded_trigram_update(t, torch.tensor(spans, dtype=torch.int32, device="cuda"))
+    base = [(a, 10 + a) for a in range(7)] + [(1, 2), (2, 3), (4999, 4999), (-1, 3), (5000, 1), (10, 100)]
+    for q in (len(base), 1000, 40000):
+        contexts = (base * (q // len(base) + 1))[:q]
+        for k in (2, 12):
+            tok, cnt, tot = _topk_gpu(B, t, contexts, k)
+            want = {c: (st.topk(*c, k), st.total(*c)) for c in base}
+            for i, c in enumerate(contexts):
+                assert ((tok[i], cnt[i]), tot[i]) == want[c], (q, k, i, c)
+
+
+@pytest.mark.parametrize("windows", [(1 << 17) - 1, 1 << 17, (1 << 17) + 1, (1 << 17) + 2047])
+def test_long_spans_on_both_sides_of_the_bulk_update(cuda_device, windows):
+    """Spans of 2^17 windows on are added up per block first: the counts at the line, with a ragged last block, with a cap that many
+    blocks reach together, and with a token outside the vocabulary (reported; the windows without it are counted)."""
+    from paper_2407_12021_b200 import binding as B
+    toks = gen.zipf_tokens(windows + 2, 300, 51, 1)
+    for cap in (0, 7):
+        st = TrigramStore(cap=cap) if cap else TrigramStore()
+        t = B.aded_trigram_create(300, log2_buckets=17, overflow_buckets=1 << 16, cap=cap)
+        for _ in range(2):
+            st.update(toks.tolist())
+            B.aded_trigram_update(t, toks.cuda())
+        torch.cuda.synchronize()
+        assert B.aded_trigram_poll_status(t) == 0
+        assert _entries_gpu(B, t) == st.entries()
+    bad = toks.clone()
+    bad[windows // 2] = 300
+    t = B.aded_trigram_create(300, log2_buckets=17, overflow_buckets=1 << 16)
+    B.aded_trigram_update(t, bad.cuda())
+    torch.cuda.synchronize()
+    assert B.aded_trigram_poll_status(t) == 1
