@@ -271,13 +271,17 @@ __global__ void k_argmax_final(const float* __restrict__ pv, const int32_t* __re
     best[r] = bi == 0x7fffffff ? 0 : bi;
 }
 
-__global__ void k_materialize(GemmOut src, float* __restrict__ dst, int n, const int32_t* status) {
+// A projection result as a plain matrix.  Four columns per thread where it lies in partial tiles (n is then a multiple of 128)
+// and the destination's rows start on 16-byte boundaries.
+__global__ void k_materialize(GemmOut src, float* __restrict__ dst, int n, int vec, const int32_t* status) {
     pdl_enter();
     if (first_thread_of_grid()) trace_mark(status, TK_OTHER);
     if (*status != 0) return;
     const int r = blockIdx.y;
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c < n) dst[(size_t)r * n + c] = gemm_out_load(src, r, c);
+    const int c = (blockIdx.x * blockDim.x + threadIdx.x) * (vec ? 4 : 1);
+    if (c >= n) return;
+    if (vec) *reinterpret_cast<float4*>(dst + (size_t)r * n + c) = gemm_out_at4(src, src.tiles[c >> 7], r, c & 127);
+    else dst[(size_t)r * n + c] = gemm_out_load(src, r, c);
 }
 
 // ---- launchers --------------------------------------------------------------------------
@@ -350,8 +354,9 @@ GemmOut launch_gemm(aded_model* m, int w_map, int x_map, const void* x, const vo
 }
 
 void launch_materialize(aded_model* m, const GemmOut& src, float* dst, int rows, cudaStream_t st) {
-    dim3 grid((src.n + 255) / 256, rows);
-    launch_k(k_materialize, grid, 256, 0, st, src, dst, src.n, m->status);
+    const int vec = src.mode == 1 && (reinterpret_cast<uintptr_t>(dst) & 15) == 0, cols = vec ? 1024 : 256;
+    dim3 grid((src.n + cols - 1) / cols, rows);
+    launch_k(k_materialize, grid, 256, 0, st, src, dst, src.n, vec, m->status);
 }
 
 void launch_rope_kv(aded_model* m, aded_kv* kv, const GemmOut& qkv, int layer, int rows, cudaStream_t st) {

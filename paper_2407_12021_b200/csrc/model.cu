@@ -250,13 +250,15 @@ static aded_status enqueue_pass(aded_model* m, aded_kv* kv, const int32_t* offse
             Span sp(m, PROF_OTHER, 3, st);
             if (m->samp_on) {
                 // sampling mode: the logits as a dense matrix, then one drawn token per node in place of the greedy one
-                launch_materialize(m, lg, m->logits, rows, st);
-                ADED_CUDA_TRY(launch_sample_rows(m->logits, rows, c.vocab, c.vocab, m->samp_temp, m->samp_top_p, m->samp_u, m->best,
+                // (straight into the capture buffer when the caller asked for the logits)
+                float* dense = m->dbg_logits ? m->dbg_logits : m->logits;
+                if (lg.mode == 1 || dense != m->logits) launch_materialize(m, lg, dense, rows, st);
+                ADED_CUDA_TRY(launch_sample_rows(dense, rows, c.vocab, c.vocab, m->samp_temp, m->samp_top_p, m->samp_u, m->best,
                                                  m->status, st));
             } else {
                 launch_argmax(m, lg, rows, st);
+                if (m->dbg_logits) launch_materialize(m, lg, m->dbg_logits, rows, st);
             }
-            if (m->dbg_logits) launch_materialize(m, lg, m->dbg_logits, rows, st);
             if (m->dbg_best)
                 ADED_CUDA_TRY(cudaMemcpyAsync(m->dbg_best, m->best, (size_t)rows * sizeof(int32_t),
                                               cudaMemcpyDeviceToDevice, st));

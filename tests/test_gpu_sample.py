@@ -149,3 +149,27 @@ def test_sampled_step_on_the_tensor_core_path(cuda_device):
         assert a == len(want_out) and out[:a].tolist() == want_out
         assert sess.length() == length_before + a
         B.aded_kv_set_len(sess.kv, 0, length_before)
+
+
+@pytest.mark.parametrize("vocab,offset", [(32000, 0), (32000, 1), (31996, 0), (31999, 0), (4096, 0), (4100, 0), (20, 0)])
+def test_peaked_rows_and_unaligned_logits(cuda_device, vocab, offset):
+    """Rows as a model makes them -- one or a few clear maxima over a bulk whose weights all fall into the lowest bins -- plus runs of
+    equal and of alternating weights, from buffers that do and do not allow 16-byte loads."""
+    from paper_2407_12021_b200 import binding as B
+    rows = 9
+    logits = (gen.normal([rows, vocab], 1.3, 91, vocab).numpy() * 1.0).astype(np.float32)
+    for r in range(rows - 3):
+        logits[r, (r * 37) % vocab] = 16.0
+        logits[r, (r * 53 + 7) % vocab] = 16.0 - 0.3 * r
+    logits[rows - 3] = 0.0
+    logits[rows - 2] = np.where(np.arange(vocab) % 2, 0.0, -3.0)
+    logits[rows - 1] = np.where(np.arange(vocab) % 64 < 32, 0.0, -9.0)
+    u = gen.uniform01(rows, 92, vocab).numpy().astype(np.float32)
+    flat = torch.zeros(rows * vocab + offset, dtype=torch.float32, device="cuda")
+    lg = flat[offset:].view(rows, vocab)
+    lg.copy_(torch.from_numpy(logits))
+    out = torch.full((rows,), -5, dtype=torch.int32, device="cuda")
+    for temp, top_p in ((0.7, 0.95), (0.7, 1.0), (1.5, 0.5)):
+        B.aded_sample_tokens(lg, temp, top_p, torch.from_numpy(u).cuda(), out)
+        torch.cuda.synchronize()
+        assert np.array_equal(out.cpu().numpy().astype(np.int64), osmp.sample_rows(logits, temp, top_p, u)), (temp, top_p)
