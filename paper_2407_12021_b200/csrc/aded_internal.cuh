@@ -235,7 +235,8 @@ struct aded_model {
 
     // tensor-core GEMM path (bf16 models): TMA descriptors and split-tile scratch
     bool ws_ready;
-    std::vector<CUtensorMap> ws_maps;   // per layer: wqkv, wo, wgu, wd; then lm_head; then x, attn, act (boxes of 16 rows); then the same three with boxes of 64 rows
+    std::vector<CUtensorMap> ws_maps;   // per layer: wqkv, wo, wgu, wd; then lm_head
+    CUtensorMap ws_x_maps[3][16];       // x, attn, act in boxes of 16, 32, .. 256 rows: the rows of a pass are one request
     std::vector<void*> ws_tiled;        // the weight matrices re-tiled for the tensor-core GEMM (same indices as ws_maps), model-owned
     bool ws_use_tiled;                  // GEMMs read the re-tiled copies (else the caller's matrices through ws_maps)
     float* ws_slots;                    // partial result tiles (see gemm_out.cuh)
@@ -271,7 +272,7 @@ void launch_embed(aded_model* m, int rows, cudaStream_t st);
 void launch_rope_table(aded_model* m, int rows, cudaStream_t st);
 // `y` (may be NULL): projection result added to the residual stream before the norm
 void launch_add_rmsnorm(aded_model* m, const GemmOut* y, const void* gain, int rows, cudaStream_t st);
-// w_map / x_map: indices into m->ws_maps of the operands' TMA descriptors (-1: none, plain kernel).
+// w_map / x_map: index into m->ws_maps / m->ws_x_maps of the operands' TMA descriptors (-1: none, plain kernel).
 // `y` is the fp32 buffer the plain kernel writes; the returned descriptor says where the result is.
 // `epi_mode` (WS_EPI_*): whether the tensor-core kernel's tail also leaves per-tile greedy candidates (LM head).
 GemmOut launch_gemm(aded_model* m, int w_map, int x_map, const void* x, const void* w, float* y, int rows, int n, int k,
@@ -301,10 +302,11 @@ int ws_grid_limit(int device);
 int ws_grid(int device, int n, int k, bool one_per_sm);
 size_t ws_slot_floats(int device, int max_n, int max_rows);
 cudaError_t ws_retile(const void* w, void* out, int n, int k, cudaStream_t st);
-cudaError_t ws_launch(const CUtensorMap& map_w, const void* w_tiled, const CUtensorMap& map_x, const CUtensorMap& map_x64, int rows, int row0, int blk,
+cudaError_t ws_launch(const CUtensorMap& map_w, const void* w_tiled, const CUtensorMap& map_x, int rows, int row0, int blk,
                       int n, int k,
                       float* slots, int32_t* status, const WsEpilogue& epi, int trace_kind, int device, bool one_per_sm, cudaStream_t st);
 enum { WS_MAP_QKV = 0, WS_MAP_O = 1, WS_MAP_GU = 2, WS_MAP_D = 3 };   // per-layer map order
+enum { WS_X = 0, WS_X_ATTN = 1, WS_X_ACT = 2 };
 cudaError_t ws_wait_probe(int which, long long limit_cycles, const uint32_t* never_raised, int32_t* status, cudaStream_t st);
 
 // sample.cu

@@ -47,6 +47,7 @@ constexpr int WS_BM = 128;           // W rows per tile (MMA M)
 constexpr int WS_BK = 64;            // k elements per stage (128 bytes of bf16)
 constexpr int WS_THREADS = 192;
 constexpr long long WS_MEET_CYCLES = 400000000ll;   // about 0.2 s of SM clock: limit of the wait at a counter
+constexpr int WS_MIN_UNITS = 8;      // fewest work units of a CTA (see ws_grid)
 constexpr int WS_GMAX = 16;          // tile groups of a CTA handled per round of its tail
 
 struct WsParams {
@@ -139,8 +140,7 @@ __device__ __forceinline__ void ws_row_argmax(const WsParams& p, const TileRef& 
 
 template <bool TAIL>
 __global__ void __launch_bounds__(WS_THREADS, 2)
-k_gemm_ws(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_x64,
-          const __grid_constant__ WsParams p) {
+k_gemm_ws(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x, const __grid_constant__ WsParams p) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     // carve: stages x (W tile 16 KB | x tile rb*128 B), then barriers
     uint8_t* base = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -184,22 +184,18 @@ k_gemm_ws(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
         if (lane == 0 && live) {
             asm volatile("prefetch.tensormap [%0];" ::"l"(&map_w) : "memory");
             asm volatile("prefetch.tensormap [%0];" ::"l"(&map_x) : "memory");
-            asm volatile("prefetch.tensormap [%0];" ::"l"(&map_x64) : "memory");
             uint64_t pol_stream;
             asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol_stream));
             // Weights do not depend on the previous kernel: fill the pipeline with W tiles first, then
             // wait for the previous kernel (which produces x) and add the x tiles of those stages.
             // This one thread feeds the whole pipeline, so its per-unit work is kept small: (tile, k block) advance
-            // by increments (no 64-bit divisions), x comes in boxes of 64 rows where the pass has that many (one
-            // request instead of four), and W is one bulk copy.
+            // by increments (no 64-bit divisions), the rows of x are one box (there is a tensor map per padded row
+            // count), and W is one bulk copy.  (With boxes of 64 and 16 rows a pass of 97 to 112 rows made four requests for
+            // x per unit: gate/up of the 7B widths 39 us instead of 31 with 128 rows.)
             const int n_units = (int)(u1 - u0);
             const int ahead = n_units < p.stages ? n_units : p.stages;
             const int tile0 = (int)(u0 / p.kb), kb0 = (int)(u0 % p.kb);
-            auto load_x = [&](uint64_t* bar, uint8_t* sb, int kb) {
-                int r = 0;
-                for (; r + 64 <= p.rb; r += 64) tma_load_2d(&map_x64, bar, sb + r * 128, kb * WS_BK, p.row0 + r);
-                for (; r < p.rb; r += 16) tma_load_2d(&map_x, bar, sb + r * 128, kb * WS_BK, p.row0 + r);
-            };
+            auto load_x = [&](uint64_t* bar, uint8_t* sb, int kb) { tma_load_2d(&map_x, bar, sb, kb * WS_BK, p.row0); };
             int tile = tile0, kb = kb0;
             for (int i = 0; i < ahead; ++i) {
                 mbar_expect_tx(&full[i], stage_bytes);
@@ -461,10 +457,15 @@ int ws_grid_limit(int device) {
 // CTAs a launch over n_tiles x kb units uses: two per SM, or one per SM (with twice the stages, so the same bytes
 // in flight).  With one per SM a tile has half as many contributors, so the kernel that gathers the slots reads half
 // as much; used where that kernel is the next thing on the critical path (see ws_one_per_sm in model.cu).
+// A CTA gets at least WS_MIN_UNITS units: a small matrix spread over all SMs leaves every tile in a dozen or more pieces, and the
+// kernel that gathers them takes longer than the GEMM saved.  Measured on a model of width 1024 (45 rows, us per layer): with at
+// least 1, 2, 4, 8 units the four projections take 14.4, 13.6, 15.4, 17.6, the rotary, norm and SwiGLU kernels 29.0, 24.5, 19.3,
+// 15.6 -- the step 468, 426, 400, 385 us.  The 7B and 13B widths have 14 units and more per CTA.
 int ws_grid(int device, int n, int k, bool one_per_sm) {
     const long long units = (long long)(n / WS_BM) * (k / WS_BK);
-    const int g = ws_grid_limit(device) / (one_per_sm ? 2 : 1);
-    return units < g ? (int)units : g;
+    int g = ws_grid_limit(device) / (one_per_sm ? 2 : 1);
+    if (units < (long long)g * WS_MIN_UNITS) g = (int)((units + WS_MIN_UNITS - 1) / WS_MIN_UNITS);
+    return g;
 }
 
 // Floats of slot storage for results of up to max_n columns and max_rows rows.
@@ -475,7 +476,7 @@ size_t ws_slot_floats(int device, int max_n, int max_rows) {
 
 // Raises the kernel's dynamic shared-memory limit; once per process, before any launch or capture.
 bool ws_prepare() {
-    return cudaFuncSetAttribute(k_gemm_ws<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) == cudaSuccess &&
+    return cudaFuncSetAttribute(k_gemm_ws<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024 + 1024 + 256) == cudaSuccess &&
            cudaFuncSetAttribute(k_gemm_ws<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 112 * 1024) == cudaSuccess;
 }
 
@@ -484,7 +485,7 @@ bool ws_supported(int n, int k) { return n % WS_BM == 0 && k % WS_BK == 0 && k >
 
 // One pass: rows [row0, row0 + rows) of x (rows <= blk = 128 or 256) against all of W.  Partial tiles go to the
 // slot region of pass row0 / blk; `epi` says whether the kernel's tail reduces them to greedy candidates.
-cudaError_t ws_launch(const CUtensorMap& map_w, const void* w_tiled, const CUtensorMap& map_x, const CUtensorMap& map_x64, int rows, int row0, int blk,
+cudaError_t ws_launch(const CUtensorMap& map_w, const void* w_tiled, const CUtensorMap& map_x, int rows, int row0, int blk,
                       int n, int k,
                       float* slots, int32_t* status, const WsEpilogue& epi, int trace_kind, int device, bool one_per_sm, cudaStream_t st) {
     WsParams p;
@@ -512,8 +513,8 @@ cudaError_t ws_launch(const CUtensorMap& map_w, const void* w_tiled, const CUten
     p.status = status;
     p.epi = epi;
     const size_t smem = (size_t)p.stages * stage_bytes + 1024 + 256;
-    if (epi.mode == WS_EPI_ARGMAX) return launch_k(k_gemm_ws<true>, dim3(grid), dim3(WS_THREADS), smem, st, map_w, map_x, map_x64, p);
-    return launch_k(k_gemm_ws<false>, dim3(grid), dim3(WS_THREADS), smem, st, map_w, map_x, map_x64, p);
+    if (epi.mode == WS_EPI_ARGMAX) return launch_k(k_gemm_ws<true>, dim3(grid), dim3(WS_THREADS), smem, st, map_w, map_x, p);
+    return launch_k(k_gemm_ws<false>, dim3(grid), dim3(WS_THREADS), smem, st, map_w, map_x, p);
 }
 
 }  // namespace aded

@@ -112,7 +112,7 @@ static aded_status alloc_model(aded_model* m) {
     if (c.dtype == ADED_BF16 && ws_supported(3 * (int)d, (int)d) && ws_supported((int)d, (int)d) && ws_supported(2 * (int)F, (int)d) &&
         ws_supported((int)d, (int)F) && ws_supported((int)V, (int)d)) {
         const int L = c.n_layers;
-        m->ws_maps.resize(4 * L + 7);
+        m->ws_maps.resize(4 * L + 1);
         bool ok = ws_prepare();
         for (int l = 0; l < L && ok; ++l) {
             const aded_layer_weights& w = m->layers[l];
@@ -121,11 +121,11 @@ static aded_status alloc_model(aded_model* m) {
                  ws_make_map(&m->ws_maps[4 * l + WS_MAP_GU], w.wgu, 2 * F, d, 128) &&
                  ws_make_map(&m->ws_maps[4 * l + WS_MAP_D], w.wd, d, F, 128);
         }
-        ok = ok && ws_make_map(&m->ws_maps[4 * L], m->top.lm_head, V, d, 128) &&
-             ws_make_map(&m->ws_maps[4 * L + 1], m->x, R, d, 16) && ws_make_map(&m->ws_maps[4 * L + 2], m->attn, R, d, 16) &&
-             ws_make_map(&m->ws_maps[4 * L + 3], m->act, R, F, 16) &&
-             ws_make_map(&m->ws_maps[4 * L + 4], m->x, R, d, 64) && ws_make_map(&m->ws_maps[4 * L + 5], m->attn, R, d, 64) &&
-             ws_make_map(&m->ws_maps[4 * L + 6], m->act, R, F, 64);
+        ok = ok && ws_make_map(&m->ws_maps[4 * L], m->top.lm_head, V, d, 128);
+        for (uint32_t box = 16; box <= 256 && box <= R; box += 16)
+            ok = ok && ws_make_map(&m->ws_x_maps[WS_X][box / 16 - 1], m->x, R, d, box) &&
+                 ws_make_map(&m->ws_x_maps[WS_X_ATTN][box / 16 - 1], m->attn, R, d, box) &&
+                 ws_make_map(&m->ws_x_maps[WS_X_ACT][box / 16 - 1], m->act, R, F, box);
         if (ok) {
             // Private re-tiled copies of the weight matrices (as many bytes again as the matrices): each GEMM CTA
             // then reads one contiguous run of HBM instead of 128 strided lines per tile.  One allocation; when
@@ -196,7 +196,6 @@ static aded_status enqueue_pass(aded_model* m, aded_kv* kv, const int32_t* offse
                                 int max_tree, int chain_mode, cudaStream_t st) {
     const aded_model_config& c = m->cfg;
     const int d = c.d_model, F = c.d_ffn;
-    const int xm = 4 * c.n_layers + 1;   // TMA descriptor indices of x, attn, act
     const bool ws = m->ws_ready;
     ADED_CUDA_TRY(cudaMemcpyAsync(m->seqs.row_off, offsets_src, (batch + 1) * sizeof(int32_t),
                                   cudaMemcpyHostToDevice, st));
@@ -220,14 +219,14 @@ static aded_status enqueue_pass(aded_model* m, aded_kv* kv, const int32_t* offse
         const void* next_gain = l + 1 < c.n_layers ? m->layers[l + 1].norm1 : m->top.final_norm;
         auto wmap = [&](int which) { return ws ? 4 * l + which : -1; };      // TMA descriptor of a weight matrix (plain GEMM: none)
         GemmOut o;
-        { Span sp(m, PROF_GEMM, passes, st); o = launch_gemm(m, wmap(WS_MAP_QKV), ws ? xm : -1, m->x, w.wqkv, m->y32, rows, 3 * d, d, WS_EPI_SLOTS, TK_GEMM_QKV, st); }
+        { Span sp(m, PROF_GEMM, passes, st); o = launch_gemm(m, wmap(WS_MAP_QKV), ws ? WS_X : -1, m->x, w.wqkv, m->y32, rows, 3 * d, d, WS_EPI_SLOTS, TK_GEMM_QKV, st); }
         { Span sp(m, PROF_OTHER, 1, st); launch_rope_kv(m, kv, o, l, rows, st); }
         { Span sp(m, PROF_ATTN, 1, st); launch_tree_attention(m, kv, l, batch, rows, max_tree, st); }
-        { Span sp(m, PROF_GEMM, passes, st); o = launch_gemm(m, wmap(WS_MAP_O), ws ? xm + 1 : -1, m->attn, w.wo, m->y32, rows, d, d, WS_EPI_SLOTS, TK_GEMM_O, st); }
+        { Span sp(m, PROF_GEMM, passes, st); o = launch_gemm(m, wmap(WS_MAP_O), ws ? WS_X_ATTN : -1, m->attn, w.wo, m->y32, rows, d, d, WS_EPI_SLOTS, TK_GEMM_O, st); }
         { Span sp(m, PROF_OTHER, 1, st); launch_add_rmsnorm(m, &o, w.norm2, rows, st); }
-        { Span sp(m, PROF_GEMM, passes, st); o = launch_gemm(m, wmap(WS_MAP_GU), ws ? xm : -1, m->x, w.wgu, m->y32, rows, 2 * F, d, WS_EPI_SLOTS, TK_GEMM_GU, st); }
+        { Span sp(m, PROF_GEMM, passes, st); o = launch_gemm(m, wmap(WS_MAP_GU), ws ? WS_X : -1, m->x, w.wgu, m->y32, rows, 2 * F, d, WS_EPI_SLOTS, TK_GEMM_GU, st); }
         { Span sp(m, PROF_OTHER, 1, st); launch_swiglu(m, o, rows, st); }
-        { Span sp(m, PROF_GEMM, passes, st); o = launch_gemm(m, wmap(WS_MAP_D), ws ? xm + 2 : -1, m->act, w.wd, m->y32, rows, d, F, WS_EPI_SLOTS, TK_GEMM_DOWN, st); }
+        { Span sp(m, PROF_GEMM, passes, st); o = launch_gemm(m, wmap(WS_MAP_D), ws ? WS_X_ACT : -1, m->act, w.wd, m->y32, rows, d, F, WS_EPI_SLOTS, TK_GEMM_DOWN, st); }
         { Span sp(m, PROF_OTHER, 1, st); launch_add_rmsnorm(m, &o, next_gain, rows, st); }
         if (m->dbg_hidden)
             ADED_CUDA_TRY(cudaMemcpyAsync((char*)m->dbg_hidden + (size_t)(l + 1) * hid_bytes, m->h, hid_bytes,
@@ -239,7 +238,7 @@ static aded_status enqueue_pass(aded_model* m, aded_kv* kv, const int32_t* offse
         const bool dense_logits = !ws || m->samp_on || m->dbg_logits;
         GemmOut lg;
         { Span sp(m, PROF_GEMM, passes, st);
-          lg = launch_gemm(m, ws ? 4 * c.n_layers : -1, ws ? xm : -1, m->x, m->top.lm_head, m->logits, rows, c.vocab, d,
+          lg = launch_gemm(m, ws ? 4 * c.n_layers : -1, ws ? WS_X : -1, m->x, m->top.lm_head, m->logits, rows, c.vocab, d,
                            dense_logits ? WS_EPI_SLOTS : WS_EPI_ARGMAX, TK_GEMM_HEAD, st); }
         if (!dense_logits) {
             Span sp(m, PROF_OTHER, 1, st);
@@ -566,11 +565,11 @@ aded_status aded_debug_gemm(aded_model* m, int32_t layer, int32_t which, const v
     if (which < 4 && (layer < 0 || layer >= m->cfg.n_layers)) return ADED_ERR_INVALID_ARG;
     const aded_model_config& c = m->cfg;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const int d = c.d_model, F = c.d_ffn, xm = 4 * c.n_layers + 1;
+    const int d = c.d_model, F = c.d_ffn;
     const int n = which == 0 ? 3 * d : which == 2 ? 2 * F : which == 4 ? c.vocab : d;
     const int k = which == 3 ? F : d;
     void* xbuf = which == 1 ? m->attn : which == 3 ? m->act : m->x;
-    const int x_map = which == 1 ? xm + 1 : which == 3 ? xm + 2 : xm;
+    const int x_map = which == 1 ? WS_X_ATTN : which == 3 ? WS_X_ACT : WS_X;
     const void* w = which == 4 ? m->top.lm_head
                                : which == 0 ? m->layers[layer].wqkv
                                             : which == 1 ? m->layers[layer].wo

@@ -66,3 +66,19 @@ def test_7b_shape_wide_pass(cuda_device):
     B, w, model = _model(gen.LLAMA7B_1L, cuda_device, 47, max_rows=416)
     for which in (0, 1, 2, 3):
         _check(B, model, w, which, 416, 47)
+
+
+@pytest.mark.parametrize("rows", [33, 48, 65, 80, 97, 112, 113])
+def test_row_counts_between_the_powers_of_two(cuda_device, rows):
+    """The rows of a pass arrive as one box of their padded number; few units per CTA (small shapes)."""
+    B, w, model = _model(SMALL16, cuda_device, 45)
+    for which in range(5):
+        _check(B, model, w, which, rows, 45 + rows)
+
+
+@pytest.mark.parametrize("rows", [177, 192, 193, 208, 256 + 177, 256 + 192])
+def test_wide_passes_of_every_padded_size(cuda_device, rows):
+    """Passes of 129 to 256 rows, those of 177 to 192 among them (five stages of 40 KB: the launch with the most shared memory)."""
+    B, w, model = _model(SMALL16, cuda_device, 46, max_rows=rows)
+    for which in (0, 1, 3):
+        _check(B, model, w, which, rows, 46)
