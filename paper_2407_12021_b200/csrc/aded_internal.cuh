@@ -124,13 +124,14 @@ struct CallPtrs {
 // memory).  A node is approved when its parent is approved and its token equals the model's token at the
 // parent; the deepest approved node (lowest index among equals) ends the accepted path.  Emits the
 // model's token of every path node: the approved drafts' successors, ending with the model's own next
-// token.  A failed pass emits nothing and keeps the committed length.
+// token, and commits the path's length (the compaction that follows works from `moves`).  A failed pass emits nothing and
+// keeps the committed length.
 __device__ __forceinline__ void approval_walk(const int32_t* s_par, const int32_t* s_tok, const int32_t* s_best,
-                                              const int32_t* s_dep, int T, int pass_status, int committed,
-                                              int32_t* out_tokens, int32_t* out_len, int32_t* path, int32_t* new_len) {
+                                              const int32_t* s_dep, int T, int pass_status, int32_t* out_tokens,
+                                              int32_t* out_len, int32_t* path, int32_t* moves, int32_t* len) {
     if (pass_status != 0) {
         *out_len = 0;
-        *new_len = committed;
+        moves[1] = 0;
         return;
     }
     uint64_t ok_lo = 1ull, ok_hi = 0ull;   // approved set; the root always is
@@ -152,14 +153,36 @@ __device__ __forceinline__ void approval_walk(const int32_t* s_par, const int32_
         cur = s_par[cur];
     }
     *out_len = deepest_depth + 1;
-    *new_len = committed + deepest_depth + 1;
+    moves[0] = *len;
+    moves[1] = deepest_depth + 1;
+    *len += deepest_depth + 1;
 }
 
 struct SeqMeta {
     int32_t* row_off;  // [B+1] first row of each sequence
     int32_t* path;     // [B][ADED_MAX_NODES] accepted path (local node indices), root first
-    int32_t* new_len;  // [B] committed length after this call
+    int32_t* moves;    // [B][2] committed length before this call, and how many nodes of the path were kept (compaction)
 };
+
+// The rotary tables of a pass: cos/sin of position * theta^(-2i/hd) for every row, in double, stored as float (the angles reach
+// thousands of radians, where float argument reduction would cost several bf16 ulps).
+struct RopeArgs {
+    const int32_t* pos;      // [R], NULL: nothing to do
+    const double* freq;      // [half]
+    float* cs;               // [R][half]
+    float* sn;
+    int half;
+};
+// Row r's tables, by threads `tid` of `threads`.
+__device__ __forceinline__ void rope_row(const RopeArgs& a, int r, int tid, int threads) {
+    if (!a.pos) return;
+    for (int i = tid; i < a.half; i += threads) {
+        double s, c;
+        sincos((double)a.pos[r] * a.freq[i], &s, &c);
+        a.cs[r * a.half + i] = (float)c;
+        a.sn[r * a.half + i] = (float)s;
+    }
+}
 
 }  // namespace aded
 
@@ -206,6 +229,7 @@ struct aded_model {
     float* logits;  // [R, V] fp32
     float* rope_cos;  // [R, hd/2]
     float* rope_sin;
+    double* rope_freq;  // [hd/2]
     int32_t* best;    // [R] greedy token per row
     int32_t* tokens;  // [R] staging for the _host entry points
     int32_t* parents;
@@ -247,8 +271,6 @@ struct aded_model {
     float* cand_val;                    // [R][vocab / 128] per-tile greedy candidates of the LM head
     int32_t* cand_idx;
 
-    float* norm_ssq;        // [R][32] per-chunk sums of squares of the RMSNorm kernel
-    int32_t* norm_count;    // [R] chunk arrival counters, zero between launches
     float* argmax_val;      // [R][ARGMAX_CHUNKS] best logit of each column chunk
     int32_t* argmax_idx;
 
@@ -261,17 +283,28 @@ struct aded_model {
 
 namespace aded {
 
+inline RopeArgs rope_args(const aded_model* m) {
+    return RopeArgs{m->rows.pos, m->rope_freq, m->rope_cos, m->rope_sin, m->cfg.head_dim / 2};
+}
+
 // ---- launchers (each enqueues on `st`; shapes are validated by the callers) ---------------
 // tree.cu
-void launch_tree_prologue(aded_model* m, aded_kv* kv, int batch, int chain_mode, cudaStream_t st);
+// Calls of up to PROLOGUE_MAX_BATCH sequences pass their record and row offsets to the prologue, which publishes them; larger
+// ones have copied them before.
+enum { PROLOGUE_MAX_BATCH = 64 };
+void launch_tree_prologue(aded_model* m, aded_kv* kv, const CallPtrs& call, const int32_t* offsets_host, int batch, int chain_mode,
+                          cudaStream_t st);
 void launch_accept(aded_model* m, aded_kv* kv, int batch, cudaStream_t st);
-void launch_compact_commit(aded_model* m, aded_kv* kv, int batch, int chain_mode, cudaStream_t st);
+void launch_compact(aded_model* m, aded_kv* kv, int batch, cudaStream_t st);
+void launch_commit_chain(aded_model* m, aded_kv* kv, int batch, cudaStream_t st);
 
 // dense.cu
-void launch_embed(aded_model* m, int rows, cudaStream_t st);
-void launch_rope_table(aded_model* m, int rows, cudaStream_t st);
-// `y` (may be NULL): projection result added to the residual stream before the norm
-void launch_add_rmsnorm(aded_model* m, const GemmOut* y, const void* gain, int rows, cudaStream_t st);
+void launch_rope_freq(double* freq, int half, double theta);
+// embedding lookup, the first RMSNorm and the rotary tables
+void launch_embed_norm(aded_model* m, const void* gain, int rows, cudaStream_t st);
+// projection result added to the residual stream, then the norm
+void launch_add_rmsnorm(aded_model* m, const GemmOut& y, const void* gain, int rows, cudaStream_t st);
+bool gemm_plain_prepare();
 // w_map / x_map: index into m->ws_maps / m->ws_x_maps of the operands' TMA descriptors (-1: none, plain kernel).
 // `y` is the fp32 buffer the plain kernel writes; the returned descriptor says where the result is.
 // `epi_mode` (WS_EPI_*): whether the tensor-core kernel's tail also leaves per-tile greedy candidates (LM head).
@@ -287,11 +320,9 @@ void launch_materialize(aded_model* m, const GemmOut& src, float* dst, int rows,
 void launch_add_rmsnorm_ws(aded_model* m, const GemmOut& y, const void* gain, int rows, cudaStream_t st);
 void launch_swiglu_ws(aded_model* m, const GemmOut& gu, int rows, cudaStream_t st);
 void launch_rope_kv_ws(aded_model* m, aded_kv* kv, const GemmOut& qkv, int layer, int rows, cudaStream_t st);
-bool embed_norm_ws_supported(const aded_model* m);
-// embedding lookup and the first RMSNorm in one kernel
 void launch_embed_norm_ws(aded_model* m, const void* gain, int rows, cudaStream_t st);
-// greedy token per row from the LM head's per-tile candidates, then the approval walk (one launch)
-void launch_pick_accept(aded_model* m, aded_kv* kv, int batch, int n_tiles, cudaStream_t st);
+// greedy token per row from n candidates (value, column) each, then the approval walk (one launch)
+void launch_pick_accept(aded_model* m, aded_kv* kv, int batch, const float* cand_val, const int32_t* cand_idx, int n, cudaStream_t st);
 
 // gemm_ws.cu
 bool ws_make_map(CUtensorMap* map, const void* ptr, uint64_t rows, uint64_t cols, uint32_t box_rows);

@@ -17,147 +17,147 @@ __device__ __forceinline__ float warp_sum(float v) {
     return v;
 }
 
-// Sum over the block; every thread receives the total.  `red` holds 32 floats.
-__device__ __forceinline__ float block_sum(float v, float* red) {
-    v = warp_sum(v);
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
-    __syncthreads();
-    if (l == 0) red[w] = v;
-    __syncthreads();
-    float t = l < nw ? red[l] : 0.f;
-    return warp_sum(t);
+// Frequencies of the rotary embedding, theta^(-2i/hd), in double (once per model; the angles are made per pass, rope_row).
+__global__ void k_rope_freq(double* __restrict__ freq, int half, double theta) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < half) freq[i] = pow(theta, -(double)i / (double)half);
 }
 
+// h = embedding of the token (when `table` is given) or round(h + y);  x = round(h * rsqrt(mean(h^2) + eps) * gain).  One block
+// per row, columns strided over the threads and kept in registers between the sum of squares and the scaling; the sum's
+// order is fixed.  fp32 models; of bf16 models those whose widths the tensor-core GEMM does not take.
+constexpr int NORM_COLS = 8;           // columns per thread: d_model <= 8 x 1024
 template <typename T>
-__global__ void k_embed(const T* __restrict__ table, const CallPtrs* __restrict__ call, T* __restrict__ h,
-                        int d, const int32_t* status) {
-    pdl_enter();
-    if (first_thread_of_grid()) trace_mark(status, TK_OTHER);
-    if (*status != 0) return;
-    const int32_t* __restrict__ tokens = call->tokens;
-    const int r = blockIdx.x;
-    const T* src = table + (size_t)tokens[r] * d;
-    for (int c = threadIdx.x; c < d; c += blockDim.x) h[(size_t)r * d + c] = src[c];
-}
-
-// cos/sin of pos * theta^(-2i/hd) for every row, in double, stored as float: the angles reach
-// thousands of radians, where float argument reduction would cost several bf16 ulps.
-__global__ void k_rope_table(const int32_t* __restrict__ pos, float* __restrict__ cs, float* __restrict__ sn,
-                             int half, double theta, const int32_t* status) {
-    pdl_enter();
-    if (first_thread_of_grid()) trace_mark(status, TK_OTHER);
-    if (*status != 0) return;
-    const int r = blockIdx.x;
-    for (int i = threadIdx.x; i < half; i += blockDim.x) {
-        const double inv = pow(theta, -(double)i / (double)half);
-        double s, c;
-        sincos((double)pos[r] * inv, &s, &c);
-        cs[r * half + i] = (float)c;
-        sn[r * half + i] = (float)s;
-    }
-}
-
-// Residual add + RMSNorm:  h = round(h + y) (when y is given), x = round(h * rsqrt(mean(h^2) + eps) * gain).
-// Grid (column chunks of 256, rows): each thread owns one column of one row, so the partial tiles of
-// y are gathered with full parallelism.  A chunk leaves its sum of squares in `ssq`; the chunk that
-// finishes a row last (per-row counter) adds the row's chunk sums in chunk order and writes x for
-// the whole row.  The order of every sum is fixed, so the result does not depend on timing.
-template <typename T>
-__global__ void __launch_bounds__(256) k_add_rmsnorm(T* __restrict__ h, GemmOut y, int has_y, const T* __restrict__ gain,
-                                                     T* __restrict__ x, int d, float eps, float* __restrict__ ssq,
-                                                     int32_t* __restrict__ row_count, const int32_t* status) {
-    pdl_enter();
-    if (first_thread_of_grid()) trace_mark(status, TK_NORM);
-    if (*status != 0) return;
+__global__ void __launch_bounds__(1024) k_add_rmsnorm(T* __restrict__ h, const float* __restrict__ y, const T* __restrict__ table,
+                                                      const CallPtrs* __restrict__ call, int vocab, const T* __restrict__ gain,
+                                                      T* __restrict__ x, int d, float eps, RopeArgs rope, const int32_t* status) {
+    pdl_launch_dependents();
     __shared__ float red[32];
-    __shared__ int s_last;
-    const int r = blockIdx.y, c = blockIdx.x * 256 + threadIdx.x;
+    const int r = blockIdx.x;
+    float g[NORM_COLS], v[NORM_COLS];
+#pragma unroll
+    for (int i = 0; i < NORM_COLS; ++i) {
+        const int c = threadIdx.x + i * blockDim.x;
+        g[i] = c < d ? to_f32(gain[c]) : 0.f;
+    }
+    pdl_wait();
+    if (first_thread_of_grid()) trace_mark(status, table ? TK_OTHER : TK_NORM);
+    if (*status != 0) return;
+    const T* src = h + (size_t)r * d;
+    if (table) {
+        int tok = call->tokens[r];
+        if (tok < 0 || tok >= vocab) tok = 0;          // a token outside the vocabulary has been reported by the tree check
+        src = table + (size_t)tok * d;
+    }
     float sq = 0.f;
-    if (c < d) {
-        float v = to_f32(h[(size_t)r * d + c]);
-        if (has_y) {
-            const float add = y.mode == 0 ? y.y[(size_t)r * d + c] : gemm_out_at(y, y.tiles[c >> 7], r, c & 127);
-            const T nv = from_f32<T>(v + add);
-            h[(size_t)r * d + c] = nv;
-            v = to_f32(nv);
+#pragma unroll
+    for (int i = 0; i < NORM_COLS; ++i) {
+        const int c = threadIdx.x + i * blockDim.x;
+        v[i] = 0.f;
+        if (c < d) {
+            v[i] = to_f32(src[c]);
+            if (y) v[i] = to_f32(from_f32<T>(v[i] + y[(size_t)r * d + c]));
+            h[(size_t)r * d + c] = from_f32<T>(v[i]);
         }
-        sq = v * v;
+        sq += v[i] * v[i];
     }
-    sq = block_sum(sq, red);
-    if (threadIdx.x == 0) {
-        ssq[r * 32 + blockIdx.x] = sq;
-        __threadfence();
-        const int prev = atomicAdd(&row_count[r], 1);
-        s_last = prev == (int)gridDim.x - 1;
-        if (s_last) row_count[r] = 0;
-    }
+    rope_row(rope, r, threadIdx.x, blockDim.x);
+    sq = warp_sum(sq);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sq;
     __syncthreads();
-    if (!s_last) return;
-    __threadfence();
     float total = 0.f;
-    for (int i = 0; i < (int)gridDim.x; ++i) total += __ldcg(ssq + r * 32 + i);
+    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) total += red[i];
     const float inv = rsqrtf(total / (float)d + eps);
-    if (sizeof(T) == 2) {
-        // two columns per access
-        const uint32_t* hr = reinterpret_cast<const uint32_t*>(h + (size_t)r * d);
-        const uint32_t* gr = reinterpret_cast<const uint32_t*>(gain);
-        uint32_t* xr = reinterpret_cast<uint32_t*>(x + (size_t)r * d);
-        for (int cc = threadIdx.x; cc < d / 2; cc += 256) {
-            const uint32_t hv = __ldcg(hr + cc), gv = gr[cc];
-            const __nv_bfloat162 hb = *reinterpret_cast<const __nv_bfloat162*>(&hv);
-            const __nv_bfloat162 gb = *reinterpret_cast<const __nv_bfloat162*>(&gv);
-            const __nv_bfloat162 o = __floats2bfloat162_rn(__low2float(hb) * inv * __low2float(gb),
-                                                           __high2float(hb) * inv * __high2float(gb));
-            xr[cc] = *reinterpret_cast<const uint32_t*>(&o);
-        }
-    } else {
-        const float* hr = reinterpret_cast<const float*>(h) + (size_t)r * d;
-        for (int cc = threadIdx.x; cc < d; cc += 256)
-            x[(size_t)r * d + cc] = from_f32<T>(__ldcg(hr + cc) * inv * to_f32(gain[cc]));
+#pragma unroll
+    for (int i = 0; i < NORM_COLS; ++i) {
+        const int c = threadIdx.x + i * blockDim.x;
+        if (c < d) x[(size_t)r * d + c] = from_f32<T>(v[i] * inv * g[i]);
     }
 }
 
-// y[r, n] = sum_k x[r, k] * w[n, k]; 64 x 64 output tile per block, 16-wide k slabs in shared
-// memory, 4 x 4 outputs per thread, fp32 accumulation in k order.
-template <typename T>
-__global__ void __launch_bounds__(256) k_gemm_plain(const T* __restrict__ x, const T* __restrict__ w,
-                                                    float* __restrict__ y, int rows, int n, int k,
-                                                    const int32_t* status, int trace_kind) {
-    pdl_enter();
-    if (first_thread_of_grid()) trace_mark(status, trace_kind);
-    if (*status != 0) return;
-    __shared__ float sx[16][64 + 4];
-    __shared__ float sw[16][64 + 4];
-    const int r0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    float acc[4][4] = {};
-    for (int k0 = 0; k0 < k; k0 += 16) {
-        for (int e = threadIdx.x; e < 64 * 16; e += 256) {
-            const int rr = e >> 4, kk = e & 15;
-            const bool kin = k0 + kk < k;
-            sx[kk][rr] = (r0 + rr < rows && kin) ? to_f32(x[(size_t)(r0 + rr) * k + k0 + kk]) : 0.f;
-            sw[kk][rr] = (n0 + rr < n && kin) ? to_f32(w[(size_t)(n0 + rr) * k + k0 + kk]) : 0.f;
+// y[r, n] = sum_k x[r, k] * w[n, k] in fp32.  A block computes BM rows x 32 columns: the operands of a chunk of k are staged in
+// shared memory as they lie (rows padded by four words: the lanes of a warp then read different banks), 4 x 4 outputs per
+// thread, four k per step; the threads beyond one per 4 x 4 split the chunk's k among them, and their sums are added at the end
+// in a fixed order.
+// These are the GEMMs of small models and a handful of rows: bound by latency, not by arithmetic.  So the chunk is all of k where
+// that fits -- one round of loads, of which the weights' are issued before the previous kernel has finished -- and the split of
+// k keeps eight warps busy on 16 rows.  (Blocks of 64 x 64 outputs with 16 k at a time took 23 to 65 us per GEMM of the 256-wide
+// fp32 model at 16 rows, two barriers and one exposed load per 16 k; this: 4.5 to 8.6 us.)
+constexpr int GP_BN = 32, GP_THREADS = 256;
+template <typename T, bool VEC>
+__device__ __forceinline__ float4 gp_load4(const T* p) {
+    if (!VEC) return make_float4(to_f32(p[0]), to_f32(p[1]), to_f32(p[2]), to_f32(p[3]));
+    if (sizeof(T) == 4) return *reinterpret_cast<const float4*>(p);
+    return unpack4_bf16(*reinterpret_cast<const uint2*>(p));
+}
+
+template <typename T, int BM, bool VEC>
+__global__ void __launch_bounds__(GP_THREADS) k_gemm_plain(const T* __restrict__ x, const T* __restrict__ w,
+                                                           float* __restrict__ y, int rows, int n, int k, int chunk,
+                                                           const int32_t* status, int trace_kind) {
+    pdl_launch_dependents();
+    constexpr int RG = BM / 4, SLICES = GP_THREADS / (8 * RG), STEP = 4 * SLICES;
+    extern __shared__ __align__(16) float gp_smem[];
+    const int ld = (chunk + 31) / 32 * 32 + 4;
+    float* sw = gp_smem;                       // [GP_BN][ld]
+    float* sx = gp_smem + GP_BN * ld;          // [BM][ld]
+    const int n0 = blockIdx.x * GP_BN, r0 = blockIdx.y * BM;
+    const int cg = threadIdx.x & 7, rg = (threadIdx.x >> 3) % RG, slice = threadIdx.x / (8 * RG);
+    // rows [from, from + count) of m, columns [k0, k0 + len), zero beyond `limit` rows and beyond k (k % 4 == 0)
+    auto stage = [&](float* dst, const T* m, int from, int count, int limit, int k0, int len) {
+        const int quads = len / 4;
+        for (int i = threadIdx.x; i < count * quads; i += GP_THREADS) {
+            const int rr = i / quads, kk = (i % quads) * 4;
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (from + rr < limit && k0 + kk < k) v = gp_load4<T, VEC>(m + (size_t)(from + rr) * k + k0 + kk);
+            *reinterpret_cast<float4*>(dst + (size_t)rr * ld + kk) = v;
         }
+    };
+    float acc[4][4] = {};
+    for (int k0 = 0; k0 < k; k0 += chunk) {
+        const int here = k - k0 < chunk ? k - k0 : chunk, len = (here + STEP - 1) / STEP * STEP;      // (chunk % STEP == 0 unless it is all of k)
+        if (k0 > 0) __syncthreads();
+        stage(sw, w, n0, GP_BN, n, k0, len);
+        if (k0 == 0) {
+            pdl_wait();
+            if (first_thread_of_grid()) trace_mark(status, trace_kind);
+            if (*status != 0) return;
+        }
+        stage(sx, x, r0, BM, rows, k0, len);
         __syncthreads();
+        const int per = len / SLICES;
+        for (int kk = slice * per; kk < (slice + 1) * per; kk += 4) {
+            float4 a[4], b[4];
 #pragma unroll
-        for (int kk = 0; kk < 16; ++kk) {
-            float a[4], b[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) { a[i] = sx[kk][ty * 4 + i]; b[i] = sw[kk][tx * 4 + i]; }
+            for (int i = 0; i < 4; ++i) {
+                a[i] = *reinterpret_cast<const float4*>(sx + (size_t)(rg + RG * i) * ld + kk);
+                b[i] = *reinterpret_cast<const float4*>(sw + (size_t)(cg + 8 * i) * ld + kk);
+            }
 #pragma unroll
             for (int i = 0; i < 4; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+                for (int j = 0; j < 4; ++j) {
+                    acc[i][j] = fmaf(a[i].x, b[j].x, acc[i][j]);
+                    acc[i][j] = fmaf(a[i].y, b[j].y, acc[i][j]);
+                    acc[i][j] = fmaf(a[i].z, b[j].z, acc[i][j]);
+                    acc[i][j] = fmaf(a[i].w, b[j].w, acc[i][j]);
+                }
         }
-        __syncthreads();
     }
+    __syncthreads();
+    float* part = gp_smem;                     // [SLICES][BM][GP_BN]
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int r = r0 + ty * 4 + i, c = n0 + tx * 4 + j;
-            if (r < rows && c < n) y[(size_t)r * n + c] = acc[i][j];
-        }
+        for (int j = 0; j < 4; ++j) part[(slice * BM + rg + RG * i) * GP_BN + cg + 8 * j] = acc[i][j];
+    __syncthreads();
+    for (int o = threadIdx.x; o < BM * GP_BN; o += GP_THREADS) {
+        float sum = part[o];
+#pragma unroll
+        for (int sl = 1; sl < SLICES; ++sl) sum += part[sl * BM * GP_BN + o];
+        const int r = r0 + o / GP_BN, c = n0 + o % GP_BN;
+        if (r < rows && c < n) y[(size_t)r * n + c] = sum;
+    }
 }
 
 // Rotary embedding of q and k (pairs (i, i + hd/2), angle from the table), then q -> q buffer and
@@ -210,8 +210,8 @@ __global__ void k_swiglu(GemmOut gu, T* __restrict__ act, int F, const int32_t* 
 }
 
 // Greedy choice per row: largest fp32 logit, lowest index among equals.  Stage 1: grid (chunks, rows),
-// every block scans `chunk` columns of one row and leaves (value, index) of its best; stage 2 (one
-// thread per row) takes the best of the chunks in ascending column order.
+// every block scans `chunk` columns of one row and leaves (value, index) of its best, which the approval kernel
+// (k_pick_accept) takes up like the LM head's per-tile candidates.
 __global__ void __launch_bounds__(256) k_argmax_chunks(GemmOut logits, float* __restrict__ pv, int32_t* __restrict__ pi,
                                                        int V, int chunk, const int32_t* status) {
     pdl_enter();
@@ -254,23 +254,6 @@ __global__ void __launch_bounds__(256) k_argmax_chunks(GemmOut logits, float* __
     }
 }
 
-__global__ void k_argmax_final(const float* __restrict__ pv, const int32_t* __restrict__ pi, int32_t* __restrict__ best,
-                               int chunks, int rows, const int32_t* status) {
-    pdl_enter();
-    if (first_thread_of_grid()) trace_mark(status, TK_PICK);
-    if (*status != 0) return;
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= rows) return;
-    float bv = -INFINITY;
-    int bi = 0x7fffffff;
-    for (int i = 0; i < chunks; ++i) {
-        const float v = pv[r * chunks + i];
-        const int idx = pi[r * chunks + i];
-        if (v > bv || (v == bv && idx < bi)) { bv = v; bi = idx; }
-    }
-    best[r] = bi == 0x7fffffff ? 0 : bi;
-}
-
 // A projection result as a plain matrix.  Four columns per thread where it lies in partial tiles (n is then a multiple of 128)
 // and the destination's rows start on 16-byte boundaries.
 __global__ void k_materialize(GemmOut src, float* __restrict__ dst, int n, int vec, const int32_t* status) {
@@ -288,34 +271,59 @@ __global__ void k_materialize(GemmOut src, float* __restrict__ dst, int n, int v
 #define BY_DTYPE(m, CALL_BF16, CALL_F32) \
     do { if ((m)->cfg.dtype == ADED_BF16) { CALL_BF16; } else { CALL_F32; } } while (0)
 
-void launch_embed(aded_model* m, int rows, cudaStream_t st) {
+void launch_rope_freq(double* freq, int half, double theta) { k_rope_freq<<<1, half>>>(freq, half, theta); }
+
+static int norm_threads(int d) { return d >= 1024 ? 1024 : (d + 31) / 32 * 32; }
+
+void launch_embed_norm(aded_model* m, const void* gain, int rows, cudaStream_t st) {
     const int d = m->cfg.d_model;
-    BY_DTYPE(m, (launch_k(k_embed<bf16>, rows, 256, 0, st, (const bf16*)m->top.embed, m->call_dev, (bf16*)m->h, d, m->status)),
-             (launch_k(k_embed<float>, rows, 256, 0, st, (const float*)m->top.embed, m->call_dev, (float*)m->h, d, m->status)));
+    if (m->cfg.dtype == ADED_BF16) { launch_embed_norm_ws(m, gain, rows, st); return; }
+    launch_k(k_add_rmsnorm<float>, rows, norm_threads(d), 0, st, (float*)m->h, nullptr, (const float*)m->top.embed, m->call_dev, m->cfg.vocab,
+             (const float*)gain, (float*)m->x, d, m->cfg.rms_eps, rope_args(m), m->status);
 }
 
-void launch_rope_table(aded_model* m, int rows, cudaStream_t st) {
-    launch_k(k_rope_table, rows, 64, 0, st, m->rows.pos, m->rope_cos, m->rope_sin, m->cfg.head_dim / 2,
-                                      (double)m->cfg.rope_theta, m->status);
-}
-
-void launch_add_rmsnorm(aded_model* m, const GemmOut* y, const void* gain, int rows, cudaStream_t st) {
+void launch_add_rmsnorm(aded_model* m, const GemmOut& y, const void* gain, int rows, cudaStream_t st) {
     const int d = m->cfg.d_model;
-    if (y && y->mode == 1 && m->cfg.dtype == ADED_BF16) { launch_add_rmsnorm_ws(m, *y, gain, rows, st); return; }
-    GemmOut none = {};
-    const GemmOut& yy = y ? *y : none;
-    const int has = y != nullptr;
-    dim3 grid((d + 255) / 256, rows);
-    BY_DTYPE(m, (launch_k(k_add_rmsnorm<bf16>, grid, 256, 0, st, (bf16*)m->h, yy, has, (const bf16*)gain, (bf16*)m->x, d, m->cfg.rms_eps, m->norm_ssq, m->norm_count, m->status)),
-             (launch_k(k_add_rmsnorm<float>, grid, 256, 0, st, (float*)m->h, yy, has, (const float*)gain, (float*)m->x, d, m->cfg.rms_eps, m->norm_ssq, m->norm_count, m->status)));
+    if (y.mode == 1) { launch_add_rmsnorm_ws(m, y, gain, rows, st); return; }
+    const RopeArgs none = {};
+    BY_DTYPE(m, (launch_k(k_add_rmsnorm<bf16>, rows, norm_threads(d), 0, st, (bf16*)m->h, y.y, nullptr, nullptr, 0, (const bf16*)gain, (bf16*)m->x, d, m->cfg.rms_eps, none, m->status)),
+             (launch_k(k_add_rmsnorm<float>, rows, norm_threads(d), 0, st, (float*)m->h, y.y, nullptr, nullptr, 0, (const float*)gain, (float*)m->x, d, m->cfg.rms_eps, none, m->status)));
 }
 
-static void launch_gemm_plain(aded_model* m, const void* x, const void* w, float* y, int rows, int n, int k, int trace_kind,
-                              cudaStream_t st) {
-    dim3 grid((n + 63) / 64, (rows + 63) / 64);
-    BY_DTYPE(m, (launch_k(k_gemm_plain<bf16>, grid, 256, 0, st, (const bf16*)x, (const bf16*)w, y, rows, n, k, m->status, trace_kind)),
-             (launch_k(k_gemm_plain<float>, grid, 256, 0, st, (const float*)x, (const float*)w, y, rows, n, k, m->status, trace_kind)));
+constexpr int GP_SMEM = 160 * 1024, GP_CHUNK = 256;
+
+template <typename T, int BM>
+static void launch_gemm_plain_bm(aded_model* m, const T* x, const T* w, float* y, int rows, int n, int k, int trace_kind, cudaStream_t st) {
+    // all of k at once where it fits (and only few blocks run), else pieces that leave room for more than one block per SM
+    auto bytes = [](int c) { return (size_t)(GP_BN + BM) * ((c + 31) / 32 * 32 + 4) * sizeof(float); };
+    const int chunk = k <= GP_CHUNK || (BM == 16 && bytes(k) <= GP_SMEM) ? k : GP_CHUNK;
+    const size_t sums = (size_t)GP_THREADS * 16 * sizeof(float);       // the partial sums take the operands' place
+    const size_t smem = bytes(chunk) > sums ? bytes(chunk) : sums;
+    const bool vec = k % 4 == 0 && (reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(w)) % (4 * sizeof(T)) == 0;
+    launch_k(vec ? k_gemm_plain<T, BM, true> : k_gemm_plain<T, BM, false>, dim3((n + GP_BN - 1) / GP_BN, (rows + BM - 1) / BM), GP_THREADS, smem, st,
+             x, w, y, rows, n, k, chunk, m->status, trace_kind);
 }
+
+template <typename T>
+static void launch_gemm_plain(aded_model* m, const T* x, const T* w, float* y, int rows, int n, int k, int trace_kind, cudaStream_t st) {
+    // The fewest rows per block that still leave no more than about two waves of blocks: more rows per block read the weights fewer
+    // times from L2, fewer spread a small GEMM over more SMs.
+    const long long cols = (n + GP_BN - 1) / GP_BN, limit = 2ll * ws_grid_limit(m->device);
+    if (cols * ((rows + 15) / 16) <= limit) launch_gemm_plain_bm<T, 16>(m, x, w, y, rows, n, k, trace_kind, st);
+    else if (cols * ((rows + 31) / 32) <= limit) launch_gemm_plain_bm<T, 32>(m, x, w, y, rows, n, k, trace_kind, st);
+    else launch_gemm_plain_bm<T, 64>(m, x, w, y, rows, n, k, trace_kind, st);
+}
+
+template <typename T>
+static bool gemm_plain_prepare_t() {
+    bool ok = true;
+    auto set = [&](auto* f) { ok = ok && cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, GP_SMEM) == cudaSuccess; };
+    set(k_gemm_plain<T, 16, true>); set(k_gemm_plain<T, 16, false>);
+    set(k_gemm_plain<T, 32, true>); set(k_gemm_plain<T, 32, false>);
+    set(k_gemm_plain<T, 64, true>); set(k_gemm_plain<T, 64, false>);
+    return ok;
+}
+bool gemm_plain_prepare() { return gemm_plain_prepare_t<float>() && gemm_plain_prepare_t<bf16>(); }
 
 GemmOut launch_gemm(aded_model* m, int w_map, int x_map, const void* x, const void* w, float* y, int rows, int n, int k,
                     int epi_mode, int trace_kind, cudaStream_t st) {
@@ -347,7 +355,8 @@ GemmOut launch_gemm(aded_model* m, int w_map, int x_map, const void* x, const vo
         out.tiles = m->ws_tiles[table];
         return out;
     }
-    launch_gemm_plain(m, x, w, y, rows, n, k, trace_kind, st);
+    BY_DTYPE(m, (launch_gemm_plain<bf16>(m, (const bf16*)x, (const bf16*)w, y, rows, n, k, trace_kind, st)),
+             (launch_gemm_plain<float>(m, (const float*)x, (const float*)w, y, rows, n, k, trace_kind, st)));
     out.mode = 0;
     out.y = y;
     return out;
@@ -381,7 +390,6 @@ void launch_argmax(aded_model* m, const GemmOut& logits, int rows, cudaStream_t 
     const int chunk = ((V + chunks - 1) / chunks + 127) / 128 * 128;   // whole 128-column tiles per block
     dim3 grid(chunks, rows);
     launch_k(k_argmax_chunks, grid, 256, 0, st, logits, m->argmax_val, m->argmax_idx, V, chunk, m->status);
-    launch_k(k_argmax_final, (rows + 127) / 128, 128, 0, st, m->argmax_val, m->argmax_idx, m->best, chunks, rows, m->status);
 }
 
 }  // namespace aded

@@ -16,11 +16,12 @@ __device__ __forceinline__ float warp_sum_f(float v) {
     return v;
 }
 
-// Embedding lookup + the first layer's RMSNorm in one kernel (bf16): h = embed[token], x = norm(h).
-// One block of 1024 threads per row, four columns per thread and pass, as k_add_rmsnorm_ws.
+// Embedding lookup, the first layer's RMSNorm and the row's rotary tables in one kernel (bf16): h = embed[token], x = norm(h).
+// One block of 1024 threads per row, four columns per thread and pass, as k_add_rmsnorm_ws; the last warps make the tables
+// while the row is on its way (a kernel of their own took 4 us of a pass).
 __global__ void __launch_bounds__(1024) k_embed_norm_ws(const bf16* __restrict__ table, const CallPtrs* __restrict__ call,
                                                         bf16* __restrict__ h, const bf16* __restrict__ gain, bf16* __restrict__ x,
-                                                        int d, int vocab, float eps, const int32_t* status) {
+                                                        int d, int vocab, float eps, RopeArgs rope, const int32_t* status) {
     pdl_launch_dependents();
     __shared__ float red[32];
     const int r = blockIdx.x;
@@ -48,6 +49,7 @@ __global__ void __launch_bounds__(1024) k_embed_norm_ws(const bf16* __restrict__
             sq += v[i].x * v[i].x + v[i].y * v[i].y + v[i].z * v[i].z + v[i].w * v[i].w;
         }
     }
+    if (pass_status == 0) rope_row(rope, r, 1023 - (int)threadIdx.x, 1024);
     sq = warp_sum_f(sq);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sq;
     __syncthreads();
@@ -65,15 +67,15 @@ __global__ void __launch_bounds__(1024) k_embed_norm_ws(const bf16* __restrict__
     }
 }
 
-// Greedy token of every row from the LM head's per-tile candidates (largest value, lowest column among
-// equals -- a tile's candidate already is its lowest best column), then the approval walk of tree.cu.
+// Greedy token of every row from its candidates (the LM head's, one per tile, or k_argmax_chunks', one per chunk; largest value,
+// lowest column among equals -- a candidate already is the lowest best column of its part), then the approval walk.
 // One block of 1024 threads per sequence; a warp per row, every lane's candidates fetched at once.
 constexpr int PICK_THREADS = 1024, PICK_PER_LANE = 8;
 __global__ void __launch_bounds__(PICK_THREADS) k_pick_accept(const CallPtrs* __restrict__ call, const float* __restrict__ cand_val,
                                                               const int32_t* __restrict__ cand_idx, int n_tiles,
                                                               const int32_t* __restrict__ row_off, int32_t* __restrict__ best,
-                                                              const int32_t* __restrict__ depth, const int32_t* __restrict__ len,
-                                                              int32_t* __restrict__ path, int32_t* __restrict__ new_len,
+                                                              const int32_t* __restrict__ depth, int32_t* __restrict__ len,
+                                                              int32_t* __restrict__ path, int32_t* __restrict__ moves,
                                                               const int32_t* status) {
     pdl_enter();
     if (first_thread_of_grid()) trace_mark(status, TK_PICK);
@@ -120,8 +122,8 @@ __global__ void __launch_bounds__(PICK_THREADS) k_pick_accept(const CallPtrs* __
     }
     __syncthreads();
     if (threadIdx.x == 0)
-        approval_walk(s_par, s_tok, s_best, s_dep, T, pass_status, len[b], call->out_tokens + (size_t)b * call->out_stride,
-                      call->out_len + b, path + b * ADED_MAX_NODES, new_len + b);
+        approval_walk(s_par, s_tok, s_best, s_dep, T, pass_status, call->out_tokens + (size_t)b * call->out_stride,
+                      call->out_len + b, path + b * ADED_MAX_NODES, moves + 2 * b, len + b);
 }
 
 // Residual add + RMSNorm (see k_add_rmsnorm): one block of 1024 threads per row, four columns per
@@ -245,19 +247,15 @@ k_rope_kv_ws(GemmOut qkv, const float* __restrict__ cs, const float* __restrict_
 }
 
 // ---- launchers (callers have checked: bf16 model, tensor-core path) ----------------------------
-bool embed_norm_ws_supported(const aded_model* m) {
-    return m->cfg.dtype == ADED_BF16 && m->cfg.d_model % 4 == 0 && m->cfg.d_model <= 8192;
-}
-
 void launch_embed_norm_ws(aded_model* m, const void* gain, int rows, cudaStream_t st) {
     launch_k(k_embed_norm_ws, dim3(rows), dim3(1024), 0, st, (const bf16*)m->top.embed, (const CallPtrs*)m->call_dev, (bf16*)m->h,
-             (const bf16*)gain, (bf16*)m->x, m->cfg.d_model, m->cfg.vocab, m->cfg.rms_eps, (const int32_t*)m->status);
+             (const bf16*)gain, (bf16*)m->x, m->cfg.d_model, m->cfg.vocab, m->cfg.rms_eps, rope_args(m), (const int32_t*)m->status);
 }
 
-void launch_pick_accept(aded_model* m, aded_kv* kv, int batch, int n_tiles, cudaStream_t st) {
-    launch_k(k_pick_accept, dim3(batch), dim3(PICK_THREADS), 0, st, (const CallPtrs*)m->call_dev, (const float*)m->cand_val,
-             (const int32_t*)m->cand_idx, n_tiles, (const int32_t*)m->seqs.row_off, m->best, (const int32_t*)m->rows.depth,
-             (const int32_t*)kv->len_dev, m->seqs.path, m->seqs.new_len, (const int32_t*)m->status);
+void launch_pick_accept(aded_model* m, aded_kv* kv, int batch, const float* cand_val, const int32_t* cand_idx, int n, cudaStream_t st) {
+    launch_k(k_pick_accept, dim3(batch), dim3(PICK_THREADS), 0, st, (const CallPtrs*)m->call_dev, cand_val, cand_idx, n,
+             (const int32_t*)m->seqs.row_off, m->best, (const int32_t*)m->rows.depth, kv->len_dev, m->seqs.path, m->seqs.moves,
+             (const int32_t*)m->status);
 }
 
 void launch_add_rmsnorm_ws(aded_model* m, const GemmOut& y, const void* gain, int rows, cudaStream_t st) {

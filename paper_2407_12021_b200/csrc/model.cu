@@ -88,14 +88,15 @@ static aded_status alloc_model(aded_model* m) {
     TRY(dev_alloc(m, &m->rows.anc, 2 * R));
     TRY(dev_alloc(m, &m->seqs.row_off, B + 1));
     TRY(dev_alloc(m, &m->seqs.path, B * ADED_MAX_NODES));
-    TRY(dev_alloc(m, &m->seqs.new_len, B));
+    TRY(dev_alloc(m, &m->seqs.moves, 2 * B));
     TRY(dev_alloc(m, &m->call_dev, 1));
-    TRY(dev_alloc(m, &m->norm_ssq, R * 32));
-    TRY(dev_alloc(m, &m->norm_count, R));
+    TRY(dev_alloc(m, &m->rope_freq, c.head_dim / 2));
     TRY(dev_alloc(m, &m->argmax_val, R * ARGMAX_CHUNKS));
     TRY(dev_alloc(m, &m->argmax_idx, R * ARGMAX_CHUNKS));
-    ADED_CUDA_TRY(cudaMemset(m->norm_count, 0, R * sizeof(int32_t)));
-    if (d > 32 * 256) return ADED_ERR_UNSUPPORTED;   // the norm kernel keeps at most 32 column chunks per row
+    if (d > 8 * 1024) return ADED_ERR_UNSUPPORTED;   // the norm kernels keep a row in the registers of one block
+    if (!gemm_plain_prepare()) return ADED_ERR_CUDA;
+    launch_rope_freq(m->rope_freq, c.head_dim / 2, (double)c.rope_theta);
+    ADED_CUDA_TRY(cudaGetLastError());
     ADED_CUDA_TRY(cudaMemset(m->status, 0, STATUS_WORDS * sizeof(int32_t)));
     ADED_CUDA_TRY(cudaMemset(m->h, 0, R * d * m->elem));
     ADED_CUDA_TRY(cudaMemset(m->x, 0, R * d * m->elem));
@@ -192,24 +193,19 @@ static aded_status alloc_model(aded_model* m) {
 
 // The launch sequence of one pass over `rows` rows.  chain_mode: the rows form a chain per sequence,
 // every row is accepted and no logits are needed (prefill).
-static aded_status enqueue_pass(aded_model* m, aded_kv* kv, const int32_t* offsets_src, int batch, int rows,
+static aded_status enqueue_pass(aded_model* m, aded_kv* kv, const CallPtrs& call, const int32_t* offsets_src, int batch, int rows,
                                 int max_tree, int chain_mode, cudaStream_t st) {
     const aded_model_config& c = m->cfg;
     const int d = c.d_model, F = c.d_ffn;
     const bool ws = m->ws_ready;
-    ADED_CUDA_TRY(cudaMemcpyAsync(m->seqs.row_off, offsets_src, (batch + 1) * sizeof(int32_t),
-                                  cudaMemcpyHostToDevice, st));
+    if (batch > PROLOGUE_MAX_BATCH) {    // (pageable sources: the runtime stages the bytes before returning)
+        ADED_CUDA_TRY(cudaMemcpyAsync(m->call_dev, &call, sizeof call, cudaMemcpyHostToDevice, st));
+        ADED_CUDA_TRY(cudaMemcpyAsync(m->seqs.row_off, offsets_src, (batch + 1) * sizeof(int32_t), cudaMemcpyHostToDevice, st));
+    }
     {
-        const bool one = embed_norm_ws_supported(m);
-        Span sp(m, PROF_OTHER, one ? 3 : 4, st);
-        launch_tree_prologue(m, kv, batch, chain_mode, st);
-        launch_rope_table(m, rows, st);
-        if (one) {
-            launch_embed_norm_ws(m, m->layers[0].norm1, rows, st);
-        } else {
-            launch_embed(m, rows, st);
-            launch_add_rmsnorm(m, (const GemmOut*)nullptr, m->layers[0].norm1, rows, st);
-        }
+        Span sp(m, PROF_OTHER, 2, st);
+        launch_tree_prologue(m, kv, call, offsets_src, batch, chain_mode, st);
+        launch_embed_norm(m, m->layers[0].norm1, rows, st);
     }
     const size_t hid_bytes = (size_t)rows * d * m->elem;
     if (m->dbg_hidden) ADED_CUDA_TRY(cudaMemcpyAsync(m->dbg_hidden, m->h, hid_bytes, cudaMemcpyDeviceToDevice, st));
@@ -223,11 +219,11 @@ static aded_status enqueue_pass(aded_model* m, aded_kv* kv, const int32_t* offse
         { Span sp(m, PROF_OTHER, 1, st); launch_rope_kv(m, kv, o, l, rows, st); }
         { Span sp(m, PROF_ATTN, 1, st); launch_tree_attention(m, kv, l, batch, rows, max_tree, st); }
         { Span sp(m, PROF_GEMM, passes, st); o = launch_gemm(m, wmap(WS_MAP_O), ws ? WS_X_ATTN : -1, m->attn, w.wo, m->y32, rows, d, d, WS_EPI_SLOTS, TK_GEMM_O, st); }
-        { Span sp(m, PROF_OTHER, 1, st); launch_add_rmsnorm(m, &o, w.norm2, rows, st); }
+        { Span sp(m, PROF_OTHER, 1, st); launch_add_rmsnorm(m, o, w.norm2, rows, st); }
         { Span sp(m, PROF_GEMM, passes, st); o = launch_gemm(m, wmap(WS_MAP_GU), ws ? WS_X : -1, m->x, w.wgu, m->y32, rows, 2 * F, d, WS_EPI_SLOTS, TK_GEMM_GU, st); }
         { Span sp(m, PROF_OTHER, 1, st); launch_swiglu(m, o, rows, st); }
         { Span sp(m, PROF_GEMM, passes, st); o = launch_gemm(m, wmap(WS_MAP_D), ws ? WS_X_ACT : -1, m->act, w.wd, m->y32, rows, d, F, WS_EPI_SLOTS, TK_GEMM_DOWN, st); }
-        { Span sp(m, PROF_OTHER, 1, st); launch_add_rmsnorm(m, &o, next_gain, rows, st); }
+        { Span sp(m, PROF_OTHER, 1, st); launch_add_rmsnorm(m, o, next_gain, rows, st); }
         if (m->dbg_hidden)
             ADED_CUDA_TRY(cudaMemcpyAsync((char*)m->dbg_hidden + (size_t)(l + 1) * hid_bytes, m->h, hid_bytes,
                                           cudaMemcpyDeviceToDevice, st));
@@ -240,33 +236,32 @@ static aded_status enqueue_pass(aded_model* m, aded_kv* kv, const int32_t* offse
         { Span sp(m, PROF_GEMM, passes, st);
           lg = launch_gemm(m, ws ? 4 * c.n_layers : -1, ws ? WS_X : -1, m->x, m->top.lm_head, m->logits, rows, c.vocab, d,
                            dense_logits ? WS_EPI_SLOTS : WS_EPI_ARGMAX, TK_GEMM_HEAD, st); }
-        if (!dense_logits) {
-            Span sp(m, PROF_OTHER, 1, st);
-            launch_pick_accept(m, kv, batch, c.vocab / 128, st);
-            if (m->dbg_best)
-                ADED_CUDA_TRY(cudaMemcpyAsync(m->dbg_best, m->best, (size_t)rows * sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
-        } else {
-            Span sp(m, PROF_OTHER, 3, st);
-            if (m->samp_on) {
-                // sampling mode: the logits as a dense matrix, then one drawn token per node in place of the greedy one
-                // (straight into the capture buffer when the caller asked for the logits)
-                float* dense = m->dbg_logits ? m->dbg_logits : m->logits;
-                if (lg.mode == 1 || dense != m->logits) launch_materialize(m, lg, dense, rows, st);
-                ADED_CUDA_TRY(launch_sample_rows(dense, rows, c.vocab, c.vocab, m->samp_temp, m->samp_top_p, m->samp_u, m->best,
-                                                 m->status, st));
-            } else {
-                launch_argmax(m, lg, rows, st);
-                if (m->dbg_logits) launch_materialize(m, lg, m->dbg_logits, rows, st);
-            }
-            if (m->dbg_best)
-                ADED_CUDA_TRY(cudaMemcpyAsync(m->dbg_best, m->best, (size_t)rows * sizeof(int32_t),
-                                              cudaMemcpyDeviceToDevice, st));
+        if (m->samp_on) {
+            // sampling mode: the logits as a dense matrix (straight into the capture buffer when the caller asked for the logits),
+            // then one drawn token per node in place of the greedy one
+            float* dense = m->dbg_logits ? m->dbg_logits : m->logits;
+            const bool copy = lg.mode == 1 || dense != m->logits;
+            Span sp(m, PROF_OTHER, copy ? 3 : 2, st);
+            if (copy) launch_materialize(m, lg, dense, rows, st);
+            ADED_CUDA_TRY(launch_sample_rows(dense, rows, c.vocab, c.vocab, m->samp_temp, m->samp_top_p, m->samp_u, m->best,
+                                             m->status, st));
             launch_accept(m, kv, batch, st);
+        } else if (dense_logits) {
+            Span sp(m, PROF_OTHER, m->dbg_logits ? 3 : 2, st);
+            if (m->dbg_logits) launch_materialize(m, lg, m->dbg_logits, rows, st);
+            launch_argmax(m, lg, rows, st);
+            launch_pick_accept(m, kv, batch, m->argmax_val, m->argmax_idx, ARGMAX_CHUNKS, st);
+        } else {
+            Span sp(m, PROF_OTHER, 1, st);
+            launch_pick_accept(m, kv, batch, m->cand_val, m->cand_idx, c.vocab / 128, st);
         }
+        if (m->dbg_best)
+            ADED_CUDA_TRY(cudaMemcpyAsync(m->dbg_best, m->best, (size_t)rows * sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
     }
     {
-        Span sp(m, PROF_OTHER, chain_mode ? 1 : 2, st);
-        launch_compact_commit(m, kv, batch, chain_mode, st);
+        Span sp(m, PROF_OTHER, 1, st);
+        if (chain_mode) launch_commit_chain(m, kv, batch, st);
+        else launch_compact(m, kv, batch, st);
     }
     ADED_CUDA_TRY(cudaGetLastError());
     return ADED_OK;
@@ -289,9 +284,7 @@ static aded_status forward(aded_model* m, aded_kv* kv, const int32_t* tokens, co
     cp.out_tokens = out_tokens;
     cp.out_len = out_len;
     cp.out_stride = out_stride;
-    // pageable source: the runtime stages the bytes before returning, so the stack object may go
-    ADED_CUDA_TRY(cudaMemcpyAsync(m->call_dev, &cp, sizeof cp, cudaMemcpyHostToDevice, st));
-    const aded_status s = enqueue_pass(m, kv, offsets_host, batch, rows, max_tree, chain_mode, st);
+    const aded_status s = enqueue_pass(m, kv, cp, offsets_host, batch, rows, max_tree, chain_mode, st);
     m->dbg_logits = nullptr;
     m->dbg_best = nullptr;
     m->dbg_hidden = nullptr;

@@ -8,17 +8,29 @@ namespace aded {
 // other node points at an earlier node, that tokens are in the vocabulary and that the cache has
 // room; then each thread climbs from its node to the root, collecting the ancestor bit set and
 // the depth.  The climb is bounded by the node count (parents decrease strictly).
-__global__ void k_tree_prologue(const CallPtrs* __restrict__ call,
-                                const int32_t* __restrict__ row_off, const int32_t* __restrict__ len,
-                                const int32_t* __restrict__ cap, int vocab, int chain_mode,
+//
+// The call's record and row offsets come as kernel arguments (two small copies ahead of the pass cost it about 10 us) and are
+// published here for the kernels that follow.
+struct PrologueArgs {
+    CallPtrs call;
+    int32_t row_off[PROLOGUE_MAX_BATCH + 1];
+    int batch;
+    int given;             // 0: call and row_off have been copied to their places instead
+};
+__global__ void k_tree_prologue(const __grid_constant__ PrologueArgs pa, CallPtrs* call_dev, int32_t* row_off_dev,
+                                const int32_t* __restrict__ len, const int32_t* __restrict__ cap, int vocab, int chain_mode,
                                 RowMeta rows, int32_t* status) {
     pdl_enter();
     if (first_thread_of_grid()) trace_mark(status, TK_OTHER);
-    const int32_t* __restrict__ tokens = call->tokens;
-    const int32_t* __restrict__ parents = call->parents;
     const int b = blockIdx.x;
-    const int off = row_off[b];
-    const int T = row_off[b + 1] - off;
+    if (pa.given && b == 0) {
+        if (threadIdx.x == 0) *call_dev = pa.call;
+        if ((int)threadIdx.x <= pa.batch) row_off_dev[threadIdx.x] = pa.row_off[threadIdx.x];
+    }
+    const int32_t* __restrict__ tokens = pa.given ? pa.call.tokens : call_dev->tokens;
+    const int32_t* __restrict__ parents = pa.given ? pa.call.parents : call_dev->parents;
+    const int off = pa.given ? pa.row_off[b] : row_off_dev[b];
+    const int T = (pa.given ? pa.row_off[b + 1] : row_off_dev[b + 1]) - off;
     const int i = threadIdx.x;
     __shared__ int s_bad;
     if (i == 0) s_bad = 0;
@@ -63,8 +75,8 @@ __global__ void k_tree_prologue(const CallPtrs* __restrict__ call,
 // every path node: the approved drafts' successors, ending with the model's own next token.
 __global__ void k_accept(const CallPtrs* __restrict__ call,
                          const int32_t* __restrict__ row_off, const int32_t* __restrict__ best,
-                         const int32_t* __restrict__ depth, const int32_t* __restrict__ len,
-                         int32_t* __restrict__ path, int32_t* __restrict__ new_len,
+                         const int32_t* __restrict__ depth, int32_t* __restrict__ len,
+                         int32_t* __restrict__ path, int32_t* __restrict__ moves,
                          const int32_t* status, int batch) {
     pdl_enter();
     if (first_thread_of_grid()) trace_mark(status, TK_PICK);
@@ -88,66 +100,83 @@ __global__ void k_accept(const CallPtrs* __restrict__ call,
     }
     __syncthreads();
     if (threadIdx.x != 0) return;
-    approval_walk(s_par, s_tok, s_best, s_dep, T, pass_status, len[b], out_tokens + (size_t)b * out_stride, out_len + b,
-                  path + b * ADED_MAX_NODES, new_len + b);
+    approval_walk(s_par, s_tok, s_best, s_dep, T, pass_status, out_tokens + (size_t)b * out_stride, out_len + b,
+                  path + b * ADED_MAX_NODES, moves + 2 * b, len + b);
 }
 
 // Compaction: the tree's K/V were written at slots L + node index; the accepted path p_0 = 0 <
 // p_1 < ... moves to slots L + 0, L + 1, ...  Because p_j >= j and the p_j increase, the source of a
-// later move is never the destination of an earlier one, and a thread that owns one element
-// column and walks j upwards reads every slot before it overwrites it.
-template <typename T>
-__global__ void k_compact(char* const* __restrict__ base, const int32_t* __restrict__ cap,
-                          const int32_t* __restrict__ len, const int32_t* __restrict__ new_len,
-                          const int32_t* __restrict__ path, int hd, const int32_t* status) {
+// later move is never the destination of an earlier one, and a thread that owns one 16-byte column of a plane and walks j
+// upwards, COMPACT_BATCH moves at a time, reads every slot before it overwrites it.  Latency-bound: all reads of a batch are in
+// flight together, and a block takes several planes.
+constexpr int COMPACT_THREADS = 128, COMPACT_BATCH = 8;
+__global__ void __launch_bounds__(COMPACT_THREADS)
+k_compact(char* const* __restrict__ base, const int32_t* __restrict__ cap, const int32_t* __restrict__ moves,
+          const int32_t* __restrict__ path, int planes, int chunks, const int32_t* status) {
     pdl_enter();
-    if (first_thread_of_grid()) trace_mark(status, TK_OTHER);
+    if (first_thread_of_grid()) trace_mark(status, TK_STEP_END);
     if (*status != 0) return;
     const int b = blockIdx.y;
-    const int n_acc = new_len[b] - len[b];
+    const int L = moves[2 * b], n_acc = moves[2 * b + 1];
     if (n_acc <= 1) return;
-    const size_t plane = (size_t)blockIdx.x;   // (layer * 2 + k|v) * H + head
-    T* p = reinterpret_cast<T*>(base[b]) + (plane * cap[b] + len[b]) * hd;
-    for (int e = threadIdx.x; e < hd; e += blockDim.x) {
-        for (int j = 1; j < n_acc; ++j) {
-            const int src = path[b * ADED_MAX_NODES + j];
-            if (!ADED_IN_RANGE(src >= j && src < ADED_MAX_NODES && len[b] + src < cap[b], status)) continue;
-            if (src != j) p[(size_t)j * hd + e] = p[(size_t)src * hd + e];
+    const int plane = blockIdx.x * (COMPACT_THREADS / chunks) + (int)threadIdx.x / chunks;      // (layer * 2 + k|v) * H + head
+    if (plane >= planes) return;
+    uint4* p = reinterpret_cast<uint4*>(base[b]) + ((size_t)plane * cap[b] + L) * chunks + threadIdx.x % chunks;
+    for (int j0 = 1; j0 < n_acc; j0 += COMPACT_BATCH) {
+        int src[COMPACT_BATCH];
+        uint4 v[COMPACT_BATCH];
+#pragma unroll
+        for (int i = 0; i < COMPACT_BATCH; ++i) {
+            const int j = j0 + i;
+            src[i] = j < n_acc ? path[b * ADED_MAX_NODES + j] : j;
+            if (!ADED_IN_RANGE(j >= n_acc || (src[i] >= j && src[i] < ADED_MAX_NODES && L + src[i] < cap[b]), status)) src[i] = j;
         }
+#pragma unroll
+        for (int i = 0; i < COMPACT_BATCH; ++i)
+            if (src[i] != j0 + i) v[i] = p[(size_t)src[i] * chunks];
+#pragma unroll
+        for (int i = 0; i < COMPACT_BATCH; ++i)
+            if (src[i] != j0 + i) p[(size_t)(j0 + i) * chunks] = v[i];
     }
 }
 
-__global__ void k_commit(int32_t* len, const int32_t* __restrict__ new_len, const int32_t* __restrict__ row_off,
-                         int chain_mode, const int32_t* status, int batch) {
+// Prefill: every row is kept.
+__global__ void k_commit_chain(int32_t* len, const int32_t* __restrict__ row_off, const int32_t* status, int batch) {
     pdl_enter();
     if (first_thread_of_grid()) trace_mark(status, TK_STEP_END);
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= batch || *status != 0) return;
-    len[b] = chain_mode ? len[b] + (row_off[b + 1] - row_off[b]) : new_len[b];
+    len[b] += row_off[b + 1] - row_off[b];
 }
 
-void launch_tree_prologue(aded_model* m, aded_kv* kv, int batch, int chain_mode, cudaStream_t st) {
-    launch_k(k_tree_prologue, batch, ADED_MAX_NODES, 0, st, m->call_dev, m->seqs.row_off, kv->len_dev, kv->cap_dev,
-                                                      m->cfg.vocab, chain_mode, m->rows, m->status);
+void launch_tree_prologue(aded_model* m, aded_kv* kv, const CallPtrs& call, const int32_t* offsets_host, int batch, int chain_mode,
+                          cudaStream_t st) {
+    static_assert(PROLOGUE_MAX_BATCH < ADED_MAX_NODES, "a thread per row offset");
+    PrologueArgs pa = {};
+    pa.given = batch <= PROLOGUE_MAX_BATCH;
+    pa.batch = batch;
+    if (pa.given) {
+        pa.call = call;
+        for (int b = 0; b <= batch; ++b) pa.row_off[b] = offsets_host[b];
+    }
+    launch_k(k_tree_prologue, batch, ADED_MAX_NODES, 0, st, pa, m->call_dev, m->seqs.row_off, kv->len_dev, kv->cap_dev, m->cfg.vocab, chain_mode,
+             m->rows, m->status);
 }
 
 void launch_accept(aded_model* m, aded_kv* kv, int batch, cudaStream_t st) {
     launch_k(k_accept, batch, 128, 0, st, m->call_dev, m->seqs.row_off, m->best, m->rows.depth,
-                                               kv->len_dev, m->seqs.path, m->seqs.new_len, m->status, batch);
+                                               kv->len_dev, m->seqs.path, m->seqs.moves, m->status, batch);
 }
 
-void launch_compact_commit(aded_model* m, aded_kv* kv, int batch, int chain_mode, cudaStream_t st) {
-    if (!chain_mode) {
-        dim3 grid(m->cfg.n_layers * 2 * m->cfg.n_heads, batch);
-        if (m->cfg.dtype == ADED_BF16)
-            launch_k(k_compact<bf16>, grid, 128, 0, st, kv->base_dev, kv->cap_dev, kv->len_dev, m->seqs.new_len,
-                                                  m->seqs.path, m->cfg.head_dim, m->status);
-        else
-            launch_k(k_compact<float>, grid, 128, 0, st, kv->base_dev, kv->cap_dev, kv->len_dev, m->seqs.new_len,
-                                                   m->seqs.path, m->cfg.head_dim, m->status);
-    }
-    launch_k(k_commit, (batch + 31) / 32, 32, 0, st, kv->len_dev, m->seqs.new_len, m->seqs.row_off, chain_mode,
-                                               m->status, batch);
+void launch_compact(aded_model* m, aded_kv* kv, int batch, cudaStream_t st) {
+    // a row of a plane is head_dim (64 or 128) elements of 2 or 4 bytes: 8, 16 or 32 chunks of 16
+    const int chunks = (int)(m->cfg.head_dim * m->elem / sizeof(uint4)), planes = m->cfg.n_layers * 2 * m->cfg.n_heads, per = COMPACT_THREADS / chunks;
+    launch_k(k_compact, dim3((planes + per - 1) / per, batch), COMPACT_THREADS, 0, st, kv->base_dev, kv->cap_dev, m->seqs.moves, m->seqs.path, planes,
+             chunks, m->status);
+}
+
+void launch_commit_chain(aded_model* m, aded_kv* kv, int batch, cudaStream_t st) {
+    launch_k(k_commit_chain, (batch + 31) / 32, 32, 0, st, kv->len_dev, m->seqs.row_off, m->status, batch);
 }
 
 }  // namespace aded

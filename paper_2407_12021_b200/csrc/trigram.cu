@@ -21,17 +21,17 @@ __global__ void k_tg_init(uint4* b, size_t parts) {
 
 // Algorithm 2, one thread per window.  Duplicate windows inside one call are independent atomic
 // adds, so the result is min(count + multiplicity, cap) whatever the thread order.
-// `n_dev` (may be NULL): the span length lives on the device (at most n).
-__global__ void k_tg_update(TgView t, const int32_t* __restrict__ tok, int n, const int32_t* __restrict__ n_dev) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x + 2;
-    if (n_dev && *n_dev < n) n = *n_dev;
-    if (i >= n || *t.status != 0) return;
-    const int a = tok[i - 2], b = tok[i - 1], c = tok[i];
+__device__ __forceinline__ void tg_add_window(const TgView& t, int a, int b, int c) {
+    if (*t.status != 0) return;
     if (a < 0 || b < 0 || c < 0 || a >= t.vocab || b >= t.vocab || c >= t.vocab) {
-        atomicCAS(t.status, 0, (int)ADED_ERR_INVALID_ARG);
+        tg_report(t, (int)ADED_ERR_INVALID_ARG);
         return;
     }
     tg_add(t, a, b, c, 1u, true);
+}
+__global__ void k_tg_update(TgView t, const int32_t* __restrict__ tok, int n) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x + 2;
+    if (i < n) tg_add_window(t, tok[i - 2], tok[i - 1], tok[i]);
 }
 
 // The same for a long span: a block first adds up equal windows of its BULK_WINDOWS in a hash table in shared memory and then
@@ -294,6 +294,7 @@ k_draft_tree(TgView t, const int32_t* __restrict__ ctx, int n_nodes, int max_dep
     __shared__ unsigned long long s_part[32 * ADED_DRAFT_MAX_K];    // the lists of the warps that share a node
     __shared__ int s_n, s_lo, s_hi, s_fail;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    pdl_enter();
     const int prev_token = ctx[0];
     if (threadIdx.x == 0) {
         s_tok[0] = ctx[1];
@@ -378,25 +379,25 @@ k_draft_tree(TgView t, const int32_t* __restrict__ ctx, int n_nodes, int max_dep
     }
 }
 
-// After a verification step: the span the table learns from (context + emitted tokens) and the
-// context of the next step.  A failed step (accept length < 1) leaves the context and an empty span.
-__global__ void k_decode_advance(const int32_t* __restrict__ out_tok, int32_t* __restrict__ out_len, int32_t* ctx,
-                                 int32_t* __restrict__ span, int32_t* __restrict__ span_len, int max_emit) {
-    __shared__ int32_t s_ctx[2];
+// After a verification step: the table learns the windows of (context, emitted tokens), and the last two tokens become the
+// context of the next step.  A failed step (accept length < 1) leaves context and table as they are.  One thread per window.
+constexpr int FEEDBACK_THREADS = 160;
+static_assert(FEEDBACK_THREADS >= ADED_MAX_NODES + 2, "a thread per token of the longest span");
+__global__ void __launch_bounds__(FEEDBACK_THREADS)
+k_decode_feedback(TgView t, const int32_t* __restrict__ out_tok, int32_t* __restrict__ out_len, int32_t* ctx, int max_emit) {
+    pdl_enter();
+    __shared__ int32_t s_span[FEEDBACK_THREADS];
     int a = *out_len;
     if (a > max_emit) a = max_emit;
-    if (threadIdx.x < 2) s_ctx[threadIdx.x] = ctx[threadIdx.x];
+    const int i = threadIdx.x;
+    if (i < a + 2) s_span[i] = i < 2 ? ctx[i] : out_tok[i - 2];
     __syncthreads();
     if (a < 1) {
-        if (threadIdx.x == 0) { *span_len = 0; *out_len = 0; }
+        if (i == 0) *out_len = 0;
         return;
     }
-    for (int i = threadIdx.x; i < a + 2; i += blockDim.x) span[i] = i < 2 ? s_ctx[i] : out_tok[i - 2];
-    if (threadIdx.x == 0) {
-        *span_len = a + 2;
-        ctx[0] = a >= 2 ? out_tok[a - 2] : s_ctx[1];
-        ctx[1] = out_tok[a - 1];
-    }
+    if (i < 2) ctx[i] = s_span[a + i];
+    if (i < a) tg_add_window(t, s_span[i], s_span[i + 1], s_span[i + 2]);
 }
 
 __global__ void k_tg_get(TgView t, int a, int b, int c, uint32_t* out) {
@@ -514,6 +515,7 @@ k_mcts_draft(TgView t, const __grid_constant__ McParams p, const int32_t* __rest
     unsigned long long* s_ckey = reinterpret_cast<unsigned long long*>(mc_smem + mc_cache_offset());   // [MC_CACHE] context of a remembered lookup
     McLookup* s_cval = reinterpret_cast<McLookup*>(s_ckey + MC_CACHE);
     for (int i = threadIdx.x; i < MC_CACHE; i += 32) s_ckey[i] = TG_EMPTY;
+    pdl_enter();
     float* s_u = reinterpret_cast<float*>(s_cval + MC_CACHE);            // the caller's uniform numbers
     for (int i = threadIdx.x; i < p.iterations * p.length; i += 32) s_u[i] = u[i];
 
@@ -703,14 +705,14 @@ struct aded_trigram {
     uint32_t* stage_u;
     size_t stage_n;
     unsigned long long* stats_dev;
-    int32_t* step_i;     // decoding step: span [ADED_MAX_NODES + 2], span length [1], filler staging
+    int32_t* step_i;     // decoding step: see STEP_SENT
 };
 
 using namespace aded;
 
 static constexpr size_t TG_STAGE = 1 << 16;
-// step_i layout: span, span length, tokens from the table, filler staging
-static constexpr int STEP_SPAN = 0, STEP_LEN = ADED_MAX_NODES + 2, STEP_REAL = STEP_LEN + 1, STEP_FILL = STEP_REAL + 1;
+// step_i layout: sentences of the search, nodes from the table, filler staging
+static constexpr int STEP_SENT = 0, STEP_REAL = 1, STEP_FILL = 2;
 static constexpr int STEP_INTS = STEP_FILL + DRAFT_MAX_FILLER;
 
 // An empty table: home buckets and index.  The pool needs no clearing: an entry is written before anything refers to it.
@@ -803,7 +805,7 @@ aded_status aded_trigram_update(aded_trigram* t, const int32_t* tokens_dev, int3
         k_tg_update_bulk<<<(windows + BULK_WINDOWS - 1) / BULK_WINDOWS, BULK_THREADS, (BULK_WINDOWS + 2 + 2 * BULK_SLOTS) * sizeof(int32_t),
                            static_cast<cudaStream_t>(stream)>>>(t->view, tokens_dev, windows);
     else
-        k_tg_update<<<(windows + 255) / 256, 256, 0, static_cast<cudaStream_t>(stream)>>>(t->view, tokens_dev, n, nullptr);
+        k_tg_update<<<(windows + 255) / 256, 256, 0, static_cast<cudaStream_t>(stream)>>>(t->view, tokens_dev, n);
     ADED_CUDA_TRY(cudaGetLastError());
     return ADED_OK;
 }
@@ -876,10 +878,8 @@ aded_status aded_draft_tree(const aded_trigram* t, const int32_t* context_dev, i
     if (n_nodes < 1 || n_nodes > ADED_MAX_NODES || max_depth < 0 || k < 1 || k > ADED_DRAFT_MAX_K) return ADED_ERR_INVALID_ARG;
     if (n_filler < 0 || n_filler > DRAFT_MAX_FILLER || (n_filler > 0 && !filler_dev)) return ADED_ERR_INVALID_ARG;
     note_launch();
-    k_draft_tree<<<1, 1024, 0, static_cast<cudaStream_t>(stream)>>>(t->view, context_dev, n_nodes, max_depth, k,
-                                                                    n_filler > 0 ? filler_dev : nullptr, n_filler,
-                                                                    tree_tokens_dev, tree_parents_dev, n_from_table_dev);
-    ADED_CUDA_TRY(cudaGetLastError());
+    ADED_CUDA_TRY(launch_k(k_draft_tree, 1, 1024, 0, static_cast<cudaStream_t>(stream), t->view, context_dev, n_nodes, max_depth, k,
+                           n_filler > 0 ? filler_dev : nullptr, n_filler, tree_tokens_dev, tree_parents_dev, n_from_table_dev));
     return ADED_OK;
 }
 
@@ -909,11 +909,9 @@ aded_status aded_mcts_draft(const aded_trigram* t, const int32_t* context_dev, i
     p.k = k;
     for (int n = 0; n <= MC_MAX_ITER; ++n) p.e_table[n] = (double)c1 + std::log(((double)n + (double)c2 + 1.0) / (double)c2);   // Eq. 3
     note_launch();
-    k_mcts_draft<<<1, 32, mc_smem_bytes(), static_cast<cudaStream_t>(stream)>>>(t->view, p, context_dev, u_dev, tree_tokens_dev,
-                                                                               tree_parents_dev, n_nodes_dev, sentence_tokens_dev,
-                                                                               sentence_scores_dev, n_sentences_dev, n_nodes_target,
-                                                                               n_nodes_target > 0 ? filler_dev : nullptr, n_filler);
-    ADED_CUDA_TRY(cudaGetLastError());
+    ADED_CUDA_TRY(launch_k(k_mcts_draft, 1, 32, mc_smem_bytes(), static_cast<cudaStream_t>(stream), t->view, p, context_dev, u_dev, tree_tokens_dev,
+                           tree_parents_dev, n_nodes_dev, sentence_tokens_dev, sentence_scores_dev, n_sentences_dev, n_nodes_target,
+                           n_nodes_target > 0 ? filler_dev : nullptr, n_filler));
     return ADED_OK;
 }
 
@@ -929,12 +927,8 @@ aded_status aded_decode_step(aded_model* m, aded_kv* kv, aded_trigram* t, int32_
     if (s != ADED_OK) return s;
     s = aded_verify(m, kv, m->tokens, m->parents, n_nodes, out_tokens_dev, out_accept_len_dev, stream);
     if (s != ADED_OK) return s;
-    note_launch(2);
-    k_decode_advance<<<1, 160, 0, st>>>(out_tokens_dev, out_accept_len_dev, context_dev, t->step_i + STEP_SPAN,
-                                        t->step_i + STEP_LEN, n_nodes);
-    k_tg_update<<<(ADED_MAX_NODES + 255) / 256, 256, 0, st>>>(t->view, t->step_i + STEP_SPAN, n_nodes + 2,
-                                                              t->step_i + STEP_LEN);
-    ADED_CUDA_TRY(cudaGetLastError());
+    note_launch();
+    ADED_CUDA_TRY(launch_k(k_decode_feedback, 1, FEEDBACK_THREADS, 0, st, t->view, out_tokens_dev, out_accept_len_dev, context_dev, n_nodes));
     return ADED_OK;
 }
 
@@ -952,19 +946,15 @@ aded_status aded_decode_step_mcts(aded_model* m, aded_kv* kv, aded_trigram* t, i
     }
     double* scores = reinterpret_cast<double*>(m->step_mcts);
     int32_t* sent = reinterpret_cast<int32_t*>(scores + ADED_MAX_NODES);
-    int32_t* counts = t->step_i + STEP_REAL;          // found nodes; the sentence count goes to the span-length word, rewritten below
+    int32_t* counts = t->step_i + STEP_REAL;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     aded_status s = aded_mcts_draft(t, context_dev, iterations, length, n_candidates, k, c1, c2, u_dev, m->tokens, m->parents, counts,
-                                    sent, scores, t->step_i + STEP_LEN, n_nodes, filler_dev, n_filler, stream);
+                                    sent, scores, t->step_i + STEP_SENT, n_nodes, filler_dev, n_filler, stream);
     if (s != ADED_OK) return s;
     s = aded_verify(m, kv, m->tokens, m->parents, n_nodes, out_tokens_dev, out_accept_len_dev, stream);
     if (s != ADED_OK) return s;
-    note_launch(2);
-    k_decode_advance<<<1, 160, 0, st>>>(out_tokens_dev, out_accept_len_dev, context_dev, t->step_i + STEP_SPAN,
-                                        t->step_i + STEP_LEN, n_nodes);
-    k_tg_update<<<(ADED_MAX_NODES + 255) / 256, 256, 0, st>>>(t->view, t->step_i + STEP_SPAN, n_nodes + 2,
-                                                              t->step_i + STEP_LEN);
-    ADED_CUDA_TRY(cudaGetLastError());
+    note_launch();
+    ADED_CUDA_TRY(launch_k(k_decode_feedback, 1, FEEDBACK_THREADS, 0, st, t->view, out_tokens_dev, out_accept_len_dev, context_dev, n_nodes));
     return ADED_OK;
 }
 

@@ -82,3 +82,32 @@ def test_wide_passes_of_every_padded_size(cuda_device, rows):
     B, w, model = _model(SMALL16, cuda_device, 46, max_rows=rows)
     for which in (0, 1, 3):
         _check(B, model, w, which, rows, 46)
+
+
+@pytest.mark.parametrize("dtype,rows", [("f32", 1), ("f32", 16), ("f32", 17), ("f32", 128), ("f32", 300), ("bf16", 33), ("bf16", 128)])
+@pytest.mark.parametrize("offset", [0, 1])
+def test_plain_gemm(cuda_device, dtype, rows, offset):
+    """Models the tensor-core GEMM does not take: blocks of 16, 32 and 64 rows, k in one chunk and in several, a ragged number of
+    columns, matrices that do not start on a 16-byte boundary.  Bound: fp32 sums of k products in a fixed order are off by at
+    most k 2^-24 of the sum of their magnitudes, and by far less in the mean; 4e-6 of it is the bound of the tests above."""
+    shape = gen.ModelShape("plain", 1, 1088, 17, 64, 1360, 1000, dtype)
+    from paper_2407_12021_b200 import binding as B
+    w = gen.model_weights(shape, 47, device=cuda_device)
+
+    def moved(m):
+        flat = torch.empty(m.numel() + offset, dtype=m.dtype, device=m.device)
+        flat[offset:].view(m.shape).copy_(m)
+        return flat[offset:].view(m.shape)
+
+    w["lm_head"] = moved(w["lm_head"])
+    w["layers"] = [{k: moved(v) for k, v in p.items()} for p in w["layers"]]
+    model = B.aded_model_create(shape, w, max_rows=rows, max_batch=1)
+    mats = {0: w["layers"][0]["wqkv"], 1: w["layers"][0]["wo"], 2: w["layers"][0]["wgu"], 3: w["layers"][0]["wd"], 4: w["lm_head"]}
+    for which, W in mats.items():
+        x = gen.normal((rows, W.shape[1]), 1.0, 48, 500 + which, device=W.device, dtype=W.dtype)
+        y = B.aded_debug_gemm(model, 0, which, x)
+        torch.cuda.synchronize()
+        assert B.aded_model_poll_status(model) == 0
+        want = x.double() @ W.double().T
+        bound = 4e-6 * (x.double().abs() @ W.double().abs().T) + 1e-12
+        assert bool(((y.double() - want).abs() <= bound).all()), (which, rows)

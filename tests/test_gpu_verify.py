@@ -403,3 +403,72 @@ def test_debug_build_runs_the_small_workloads_without_an_index_complaint(cuda_de
     res = subprocess.run([sys.executable, "-c", code], cwd=root, env=env, capture_output=True, text=True, timeout=900)
     assert res.returncode == 0, res.stdout[-2000:] + res.stderr[-2000:]
     assert "smoke ok" in res.stdout
+
+
+@pytest.mark.parametrize("hd,nodes,depth,ctx", [(64, 128, 8, 508), (64, 37, 6, 512), (128, 65, 5, 1030), (128, 16, 3, 3), (64, 1, 0, 511)])
+def test_fp32_trees_across_key_chunks(cuda_device, hd, nodes, depth, ctx):
+    """fp32 attention takes keys in chunks of 512: contexts that end just before, at and after a chunk, with the tree's own keys in
+    the same or the next one; both head sizes; accepted paths of more than eight nodes move in two batches."""
+    shape = gen.ModelShape("f32-2", 2, 2 * hd, 2, hd, 208, 512, "f32")
+    w = gen.model_weights(shape, 70 + nodes)
+    sess = H.GpuSession(shape, H.weights_to(w, cuda_device), capacity=ctx + 200)
+    arch = ov.arch_from_shape(shape)
+    ow = ov.Weights(w, keep=True)
+    prompt = gen.zipf_tokens(ctx + 1, shape.vocab, 71, 50).tolist()
+    cache = ov.Cache(arch)
+    ov.append(arch, ow, cache, prompt[:-1])
+    sess.append(prompt[:-1])
+    H.compare_cache(shape, sess, cache, 0, ctx, range(shape.n_layers), "prefill")
+    root = prompt[-1]
+    probe = cache.clone()
+    cur, ar = root, []
+    for _ in range(12):
+        cur = ov.verify(arch, ow, probe, [cur], [-1])["out_tokens"][0]
+        ar.append(cur)
+    tokens, parents = gen.make_tree(nodes, depth, 6, shape.vocab, 72, root_token=root)
+    tokens = gen.plant_path(tokens, parents, ar[:min(depth, nodes - 1)])
+    if nodes == 37:                               # a chain: twelve nodes accepted, nothing to move; then one with a stray child first
+        tokens, parents = [root] + ar[:11], [-1] + list(range(11))
+        tokens = tokens[:1] + [(ar[0] + 1) % shape.vocab] + tokens[1:]
+        parents = [-1, 0, 0] + list(range(2, 12))
+    cpu = ov.verify(arch, ow, cache, tokens, parents)
+    gpu = sess.verify(tokens, parents)
+    assert gpu["status"] == 0
+    H.compare_step(shape, gpu, cpu, tokens, parents, f"{hd} {nodes} {ctx}")
+    assert nodes != 37 or cpu["accept_len"] >= 10
+    assert sess.length() == cache.length
+    H.compare_cache(shape, sess, cache, ctx, cache.length - ctx, range(shape.n_layers), "after")
+
+
+def test_batches_beyond_the_inline_offsets(cuda_device):
+    """Calls of up to 64 sequences carry their row offsets as kernel arguments, larger ones copy them: 64 and 65 sequences give
+    every sequence what it gets alone."""
+    from paper_2407_12021_b200 import binding as B
+    shape = gen.ModelShape("f32-1", 1, 64, 1, 64, 96, 128, "f32")
+    w = H.weights_to(gen.model_weights(shape, 81), cuda_device)
+    trees = [gen.make_tree(2 + b % 4, 2, 3, shape.vocab, 82 + b, root_token=b % shape.vocab) for b in range(65)]
+    alone = []
+    model = B.aded_model_create(shape, w, max_rows=16, max_batch=1)
+    for tokens, parents in trees:
+        kv = B.aded_kv_create(model, [32])
+        out, n = torch.zeros(16, dtype=torch.int32, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+        B.aded_append(model, kv, H.i32([5, 6, 7]))
+        B.aded_verify(model, kv, H.i32(tokens), H.i32(parents), out, n)
+        torch.cuda.synchronize()
+        alone.append(out[:int(n[0])].tolist())
+    for batch in (64, 65):
+        rows = sum(len(t[0]) for t in trees[:batch])
+        model = B.aded_model_create(shape, w, max_rows=rows, max_batch=batch)
+        kv = B.aded_kv_create(model, [32] * batch)
+        one = B.aded_model_create(shape, w, max_rows=16, max_batch=1)
+        kv1 = B.aded_kv_create(one, [32])
+        B.aded_append(one, kv1, H.i32([5, 6, 7]))
+        k, v = B.aded_kv_read(kv1, 0, 0, 0, 3)
+        for b in range(batch):
+            B.aded_kv_load(kv, b, 0, k, v)
+        offsets = [sum(len(t[0]) for t in trees[:b]) for b in range(batch + 1)]
+        out, n = torch.zeros((batch, 16), dtype=torch.int32, device="cuda"), torch.zeros(batch, dtype=torch.int32, device="cuda")
+        B.aded_verify_batch(model, kv, offsets, H.i32([x for t in trees[:batch] for x in t[0]]), H.i32([x for t in trees[:batch] for x in t[1]]), out, n)
+        torch.cuda.synchronize()
+        assert B.aded_model_poll_status(model) == 0
+        assert [out[b, :int(n[b])].tolist() for b in range(batch)] == alone[:batch]
