@@ -12,7 +12,8 @@
 //     frequent context -- thousands of continuations -- was a chain of hundreds to thousands of memory round trips.)
 //   * an index over the pool entries: (home bucket, token) -> entry, open addressing, at most three quarters full.
 //     Raising a count is one probe of the home buckets, one of the index and one atomic add, wherever the entry is.
-//     Measured, 10^6 tokens into an empty table: 13.6 ms with chains that every insertion walked from the front.
+//     Measured, 10^6 tokens into an empty table: 0.29 ms (13.6 ms with chains that every insertion walked from the front);
+//     lookups: see k_tg_topk and k_topk_mark; a 64-node draft tree from that table 32 us (490).
 //
 // Entries are never moved or removed.  The configured number of overflow buckets limits units of six entries in use
 // exactly as it limited chain buckets; the pool has room for the unused ends of the extents on top (a context with d units
@@ -126,14 +127,30 @@ __device__ __forceinline__ void tg_raise(const TgView& t, uint32_t* cnt, uint32_
     }
 }
 
+// Publishing a link or an index entry is a release, reading one an acquire.  (With full fences in their places threads spent as
+// long in the fences as in waiting for memory: 35 against 51 of 98 stalled cycles per instruction of the bulk update.)
+__device__ __forceinline__ uint32_t tg_acquire(const uint32_t* p) {
+    uint32_t v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ unsigned long long tg_acquire(const unsigned long long* p) {
+    unsigned long long v;
+    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void tg_release(uint32_t* p, uint32_t v) { asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory"); }
+__device__ __forceinline__ void tg_release(unsigned long long* p, unsigned long long v) {
+    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+
 // Waits (bounded) until another thread has published a link of a directory; 0 when the wait ran out.
 __device__ __forceinline__ uint32_t tg_wait_link(const uint32_t* link) {
-    uint32_t v = *reinterpret_cast<const volatile uint32_t*>(link);
+    uint32_t v = tg_acquire(link);
     for (int spin = 0; v == 0 && spin < TG_MAX_SPIN; ++spin) {
         __nanosleep(32);
-        v = *reinterpret_cast<const volatile uint32_t*>(link);
+        v = tg_acquire(link);
     }
-    __threadfence();
     return v;
 }
 
@@ -167,8 +184,7 @@ __device__ __forceinline__ unsigned long long tg_place(const TgView& t, Bucket* 
                     }
                 }
             }
-            __threadfence();
-            atomicExch(link, base);
+            tg_release(link, base);
         } else if (link) {
             base = tg_wait_link(link);
             if (base == 0) { tg_report(t, (int)ADED_ERR_TIMEOUT); return 0; }
@@ -223,21 +239,19 @@ __device__ __forceinline__ void tg_add(const TgView& t, int a, int b, int c, uin
             k = atomicCAS(&slot->key, 0ull, key);
             if (k == 0) {
                 const unsigned long long at = tg_place(t, bk, c);
-                __threadfence();
-                atomicExch(&slot->at, at ? at : TG_DEAD);
+                tg_release(&slot->at, at ? at : TG_DEAD);
                 if (at) tg_raise(t, &t.pool[at - 1].cnt, inc, windows);
                 return;
             }
         }
         if (k == key) {
-            unsigned long long at = *reinterpret_cast<volatile unsigned long long*>(&slot->at);
+            unsigned long long at = tg_acquire(&slot->at);
             for (int spin = 0; at == 0 && spin < TG_MAX_SPIN; ++spin) {
                 __nanosleep(32);
-                at = *reinterpret_cast<volatile unsigned long long*>(&slot->at);
+                at = tg_acquire(&slot->at);
             }
             if (at == 0) { tg_report(t, (int)ADED_ERR_TIMEOUT); return; }
             if (at == TG_DEAD) { tg_report(t, (int)ADED_ERR_TABLE_FULL); return; }
-            __threadfence();
             tg_raise(t, &t.pool[at - 1].cnt, inc, windows);
             return;
         }
@@ -325,15 +339,39 @@ __device__ __forceinline__ void tg_offer(unsigned long long cand, int k, int lan
     }
 }
 
+// Every lane offers two keys.  Where few beat the k-th best so far they are inserted one by one (about 100 cycles each);
+// where k or more do -- the first entries of a context, the merge of several warps' lists -- the new list is picked in k
+// rounds of warp-wide maxima instead.
+__device__ __forceinline__ void tg_offer2(unsigned long long c0, unsigned long long c1, int k, int lane, unsigned long long& best) {
+    const unsigned long long top = c0 > c1 ? c0 : c1;
+    const unsigned m = __ballot_sync(0xffffffffu, top > __shfl_sync(0xffffffffu, best, k - 1));
+    if (m == 0) return;
+    if (__popc(m) < k) {
+        tg_offer(c0, k, lane, best);
+        tg_offer(c1, k, lane, best);
+        return;
+    }
+    unsigned long long have = lane < k ? best : 0ull, out = 0;
+    for (int r = 0; r < k; ++r) {
+        unsigned long long v = c0 > c1 ? c0 : c1;
+        v = v > have ? v : have;
+        const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(v >> 32));
+        if (hi == 0) break;                     // (counts are at least 1)
+        const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(v >> 32) == hi ? (unsigned)v : 0u);
+        const unsigned long long pick = ((unsigned long long)hi << 32) | lo;
+        if (lane == r) out = pick;
+        if (have == pick) have = 0;
+        if (c0 == pick) c0 = 0;
+        if (c1 == pick) c1 = 0;
+    }
+    best = out;
+}
+
 // Two entries per lane (token -1: none) into the running list and sum.
 __device__ __forceinline__ void tg_take(const TgView& t, uint4 v, int k, int lane, unsigned long long& best, uint32_t& total) {
     if ((int32_t)v.x >= 0) total += v.y;
     if ((int32_t)v.z >= 0) total += v.w;
-    const unsigned long long c0 = tg_pack(t, (int32_t)v.x, v.y), c1 = tg_pack(t, (int32_t)v.z, v.w);
-    if (__any_sync(0xffffffffu, (c0 > c1 ? c0 : c1) > __shfl_sync(0xffffffffu, best, k - 1))) {
-        tg_offer(c0, k, lane, best);
-        tg_offer(c1, k, lane, best);
-    }
+    tg_offer2(tg_pack(t, (int32_t)v.x, v.y), tg_pack(t, (int32_t)v.z, v.w), k, lane, best);
 }
 
 // Part `part` of `parts` of a context's entries (each part by one warp, all lanes): the k <= 32 best of them in `best`, and this

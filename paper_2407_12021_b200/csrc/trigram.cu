@@ -148,7 +148,7 @@ __global__ void k_tg_import(TgView t, const int32_t* __restrict__ keys, const ui
 // the distinct ones of each block): bound by the L2 reads of the entries.
 constexpr int TOPK_THREADS = 512, TOPK_WARPS = TOPK_THREADS / 32, TOPK_MAX_QUERIES = 3072;
 constexpr uint32_t TOPK_LONG = 2048;
-constexpr int TOPK_WIDE = 4;
+constexpr int TOPK_WIDE = 4, TOPK_LEAD_QUERIES = 4096;
 
 // Slots of the block's hash table: a power of two, at most four fifths full.
 static __host__ __device__ int topk_slots(int per_block) {
@@ -157,6 +157,24 @@ static __host__ __device__ int topk_slots(int per_block) {
     return n;
 }
 static size_t topk_smem(int per_block) { return (size_t)topk_slots(per_block) * 8 + (size_t)per_block * 8; }
+
+// One context by all warps of the block; warp 0 hands the list and the sum to `write`.
+template <typename F>
+__device__ __forceinline__ void topk_wide(const TgView& t, int home, int k, int warp, int lane, unsigned long long* s_best, uint32_t* s_total, F write) {
+    unsigned long long best = 0;
+    uint32_t total = 0;
+    tg_scan(t, tg_open(t, (uint32_t)home, lane), warp, TOPK_WARPS, k, lane, best, total);
+    s_best[warp * 32 + lane] = lane < k ? best : 0ull;
+    total = __reduce_add_sync(0xffffffffu, total);
+    if (lane == 0) s_total[warp] = total;
+    __syncthreads();
+    if (warp == 0) {
+        for (int w = 1; w < TOPK_WARPS; w += 2) tg_offer2(s_best[w * 32 + lane], w + 1 < TOPK_WARPS ? s_best[(w + 1) * 32 + lane] : 0ull, k, lane, best);
+        total = __reduce_add_sync(0xffffffffu, lane < TOPK_WARPS ? s_total[lane] : 0u);
+        write(best, total);
+    }
+    __syncthreads();
+}
 
 __global__ void __launch_bounds__(TOPK_THREADS, 3)
 k_tg_topk(TgView t, const int32_t* __restrict__ ctx, int q, int k, int per_block, int32_t* __restrict__ out_tok,
@@ -211,19 +229,7 @@ k_tg_topk(TgView t, const int32_t* __restrict__ ctx, int q, int k, int per_block
     const bool wide = n_long <= TOPK_WIDE;
     for (int j = 0; wide && j < n_long; ++j) {
         const int slot = s_order[per_block - 1 - j];
-        unsigned long long best = 0;
-        uint32_t total = 0;
-        tg_scan(t, tg_open(t, (uint32_t)s_key[slot], lane), warp, TOPK_WARPS, k, lane, best, total);
-        s_best[warp * 32 + lane] = lane < k ? best : 0ull;
-        total = __reduce_add_sync(0xffffffffu, total);
-        if (lane == 0) s_total[warp] = total;
-        __syncthreads();
-        if (warp == 0) {
-            for (int w = 1; w < TOPK_WARPS; ++w) tg_offer(s_best[w * 32 + lane], k, lane, best);
-            total = __reduce_add_sync(0xffffffffu, lane < TOPK_WARPS ? s_total[lane] : 0u);
-            write(slot, best, total);
-        }
-        __syncthreads();
+        topk_wide(t, s_key[slot], k, warp, lane, s_best, s_total, [&](unsigned long long best, uint32_t total) { write(slot, best, total); });
     }
     // the rest, longest first as far as they are sorted
     const int first = wide ? n_long : 0, jobs = n_long - first + n_short;
@@ -238,6 +244,130 @@ k_tg_topk(TgView t, const int32_t* __restrict__ ctx, int q, int k, int per_block
         tg_scan(t, tg_open(t, (uint32_t)s_key[slot], lane), 0, 1, k, lane, best, total);
         write(slot, best, __reduce_add_sync(0xffffffffu, total));
     }
+}
+
+// Many queries: every context of the call is scanned once, by three kernels whose only scratch is the output arrays themselves
+// (lookups of one table may run on several streams, so the table holds none).
+//   1. k_topk_mark: a thread per query finds the home bucket.  Contexts with entries beyond it are grouped: the query's index
+//      goes into a hash table that fills out_cnt (all bits set before), and the first query of a context found there leads the
+//      others.  out_tok[first of the row] says what a row is: MARK_OWN (answer it; its home bucket, or -1, is in the next
+//      word) or the leader's index, encoded below MARK_OWN.
+//   2. k_topk_lead: the leaders' rows, and those of contexts that are all in their home bucket, by the thread that has the row;
+//      the hash table is overwritten with results.
+//   3. k_topk_copy: the followers' rows, from their leaders'.
+// Needs two words per row (k >= 2).  The table has at least q slots and at most half of the queries' words; a query that finds
+// no slot within MARK_PROBES answers itself.
+// Taken from TOPK_BULK queries on.  Measured, 2^20 queries on the table of a 16-million-token text, k = 4: 183 us (54 + 92 + 30 and a
+// memset; the per-block kernel above: 780); 65,536 queries on that of 10^6 tokens, k = 8: 54 us (99).  What bounds it: random
+// access in the first, and in the second the warps' chains of reads, no longer the entries' bytes.
+constexpr int MARK_OWN = -2, MARK_PROBES = 16, TOPK_BULK = 1 << 16;
+__device__ __forceinline__ int mark_leader(int q) { return MARK_OWN - 1 - q; }       // (its own inverse)
+
+__global__ void __launch_bounds__(256) k_topk_mark(TgView t, const int32_t* __restrict__ ctx, int q, int k, int lead_blocks, int per_block, uint32_t mask,
+                                                   int32_t* __restrict__ out_tok, uint32_t* out_cnt) {
+    // neighbouring threads take queries of different blocks of the next kernel: the frequent contexts, which the first threads
+    // meet, then have their leaders spread over all of its blocks
+    const int at = blockIdx.x * 256 + threadIdx.x;
+    const long long row = (long long)(at % lead_blocks) * per_block + at / lead_blocks;
+    if (at / lead_blocks >= per_block || row >= q) return;
+    const int i = (int)row;
+    const int2 c = make_int2(ctx[2 * (size_t)i], ctx[2 * (size_t)i + 1]);
+    int64_t home = -1;
+    if (c.x >= 0 && c.y >= 0 && c.x < t.vocab && c.y < t.vocab) home = tg_find_home(t, tg_key(c.x, c.y), false);
+    int mark = MARK_OWN;
+    if (home >= 0 && t.buckets[home].n_more != 0) {
+        uint32_t probe_at = (uint32_t)home * 0x9E3779B1u;
+        probe_at ^= probe_at >> 15;
+        for (int probe = 0; probe < MARK_PROBES; ++probe, ++probe_at) {
+            uint32_t* slot = out_cnt + (probe_at & mask);
+            uint32_t have = *reinterpret_cast<volatile uint32_t*>(slot);
+            if (have == 0xFFFFFFFFu) have = atomicCAS(slot, 0xFFFFFFFFu, (uint32_t)i);
+            if (have == 0xFFFFFFFFu) break;
+            if (ctx[2 * (size_t)have] == c.x && ctx[2 * (size_t)have + 1] == c.y) { mark = mark_leader((int)have); break; }
+        }
+    }
+    out_tok[(size_t)i * k] = mark;
+    out_tok[(size_t)i * k + 1] = (int32_t)home;
+}
+
+// The k best of a home bucket's six entries, and the sum of their counts, by one thread.
+__device__ __forceinline__ void topk_home(const TgView& t, int home, int k, int32_t* tok, uint32_t* cnt, uint32_t* total_out) {
+    unsigned long long key[6];
+    uint32_t total = 0;
+    const uint4* part = reinterpret_cast<const uint4*>(t.buckets + (home < 0 ? 0 : home));
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        uint4 v = part[i + 1];
+        if (home < 0) v = make_uint4(0xFFFFFFFFu, 0u, 0xFFFFFFFFu, 0u);
+        if ((int32_t)v.x >= 0) total += v.y;
+        if ((int32_t)v.z >= 0) total += v.w;
+        key[2 * i] = tg_pack(t, (int32_t)v.x, v.y);
+        key[2 * i + 1] = tg_pack(t, (int32_t)v.z, v.w);
+    }
+#pragma unroll
+    for (int r = 0; r < 6; ++r) {
+#pragma unroll
+        for (int j = r + 1; j < 6; ++j)
+            if (key[j] > key[r]) { const unsigned long long x = key[r]; key[r] = key[j]; key[j] = x; }
+        if (r < k) { tok[r] = tg_packed_tok(key[r]); cnt[r] = tg_packed_cnt(key[r]); }
+    }
+    for (int r = 6; r < k; ++r) { tok[r] = -1; cnt[r] = 0; }
+    if (total_out) *total_out = total;
+}
+
+__global__ void __launch_bounds__(TOPK_THREADS, 3)
+k_topk_lead(TgView t, int q, int k, int per_block, int32_t* __restrict__ out_tok, uint32_t* __restrict__ out_cnt, uint32_t* __restrict__ out_total) {
+    __shared__ int2 s_job[TOPK_LEAD_QUERIES];      // (row in the block, home bucket); contexts of more than TOPK_LONG entries from the back
+    __shared__ int s_n, s_long, s_cursor;
+    __shared__ unsigned long long s_best[TOPK_WARPS * 32];
+    __shared__ uint32_t s_total[TOPK_WARPS];
+    const int q0 = blockIdx.x * per_block, nq = min(per_block, q - q0);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) { s_n = 0; s_long = 0; s_cursor = 0; }
+    __syncthreads();
+    for (int i = threadIdx.x; i < nq; i += TOPK_THREADS) {
+        const size_t row = (size_t)(q0 + i);
+        if (out_tok[row * k] != MARK_OWN) continue;
+        const int home = out_tok[row * k + 1];
+        const uint32_t n = home < 0 ? 0u : t.buckets[home].n_more & ~TG_CLOSED;
+        if (n == 0) topk_home(t, home, k, out_tok + row * k, out_cnt + row * k, out_total ? out_total + row : nullptr);
+        else if (n > TOPK_LONG) s_job[per_block - 1 - atomicAdd(&s_long, 1)] = make_int2(i, home);
+        else s_job[atomicAdd(&s_n, 1)] = make_int2(i, home);
+    }
+    __syncthreads();
+    auto write = [&](int i, unsigned long long best, uint32_t total) {
+        const size_t row = (size_t)(q0 + i);
+        if (lane < k) {
+            out_tok[row * k + lane] = tg_packed_tok(best);
+            out_cnt[row * k + lane] = tg_packed_cnt(best);
+        }
+        if (lane == 0 && out_total) out_total[row] = total;
+    };
+    const int n_long = s_long, n_short = s_n;
+    const bool wide = n_long <= 4 * TOPK_WIDE;
+    for (int j = 0; wide && j < n_long; ++j) topk_wide(t, s_job[per_block - 1 - j].y, k, warp, lane, s_best, s_total, [&](unsigned long long best, uint32_t total) { write(s_job[per_block - 1 - j].x, best, total); });
+    const int first = wide ? n_long : 0, jobs = n_long - first + n_short;
+    for (;;) {
+        int j = 0;
+        if (lane == 0) j = atomicAdd(&s_cursor, 1);
+        j = __shfl_sync(0xffffffffu, j, 0);
+        if (j >= jobs) break;
+        const int2 job = j < n_long - first ? s_job[per_block - 1 - first - j] : s_job[j - (n_long - first)];
+        unsigned long long best = 0;
+        uint32_t total = 0;
+        tg_scan(t, tg_open(t, (uint32_t)job.y, lane), 0, 1, k, lane, best, total);
+        write(job.x, best, __reduce_add_sync(0xffffffffu, total));
+    }
+}
+
+__global__ void __launch_bounds__(256) k_topk_copy(int q, int k, int32_t* __restrict__ out_tok, uint32_t* __restrict__ out_cnt, uint32_t* __restrict__ out_total) {
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    if (i >= q) return;
+    const int mark = out_tok[(size_t)i * k];
+    if (mark >= MARK_OWN) return;
+    const size_t from = (size_t)mark_leader(mark) * k, to = (size_t)i * k;
+    for (int r = 0; r < k; ++r) { out_tok[to + r] = out_tok[from + r]; out_cnt[to + r] = out_cnt[from + r]; }
+    if (out_total) out_total[i] = out_total[mark_leader(mark)];
 }
 
 // Draft tree of n_nodes nodes for the context (ctx[0], ctx[1]); one block of 32 warps.
@@ -326,9 +456,11 @@ k_draft_tree(TgView t, const int32_t* __restrict__ ctx, int n_nodes, int max_dep
         __syncthreads();
         if (parts > 1 && warp < hi - lo) {
             unsigned long long best = 0;
-            for (int i = 0; i < parts; i += 32 / ADED_DRAFT_MAX_K) {      // four warps' lists at a time
+            constexpr int AT_ONCE = 32 / ADED_DRAFT_MAX_K;                // eight warps' lists at a time, two per lane
+            for (int i = 0; i < parts; i += 2 * AT_ONCE) {
                 const int from = i + lane / ADED_DRAFT_MAX_K, r = lane % ADED_DRAFT_MAX_K;
-                tg_offer(from < parts && r < k ? s_part[(warp * parts + from) * ADED_DRAFT_MAX_K + r] : 0ull, k, lane, best);
+                const unsigned long long* list = s_part + (warp * parts + from) * ADED_DRAFT_MAX_K + r;
+                tg_offer2(from < parts && r < k ? list[0] : 0ull, from + AT_ONCE < parts && r < k ? list[AT_ONCE * ADED_DRAFT_MAX_K] : 0ull, k, lane, best);
             }
             if (lane < k) s_cand[(lo + warp) * ADED_DRAFT_MAX_K + lane] = tg_packed_tok(best);
         }
@@ -440,60 +572,82 @@ __global__ void k_tg_stats(TgView t, unsigned long long* out) {
 
 
 // ---- draft maker: Monte Carlo tree search (Eq. 2-3, Algorithm 1) -----------------------------------
-// One warp runs the search; every lane executes the same scalar logic on the tree in shared memory
-// (lane 0 alone writes), the lanes cooperate only in the table lookups.  Floating point is IEEE
-// double, one rounded operation at a time (no fused multiply-add), so that the search can be
-// reproduced bit for bit; the exploration factor E of Eq. 3 depends on an integer only and comes
-// from a table the host computes.
+// One warp runs the search, in which every iteration reads what the last one left: bound by the latency of its chain of steps.
+// The tree is in shared memory; lanes hold the children of the node that is being left, the nodes of the current path, the
+// continuations of a looked-up context.  Floating point is IEEE double, one rounded operation at a time (no fused multiply-add),
+// so that the search can be reproduced bit for bit; the exploration factor E of Eq. 3 and the square root depend on an integer
+// only and come from tables the host computes; a node's mean score changes only when it is visited, a continuation's
+// probability never during a search, so each is divided out once, not at every look.
 constexpr int MC_MAX_ITER = 160, MC_MAX_K = ADED_DRAFT_MAX_K, MC_MAX_LEN = 8;
 constexpr int MC_MAX_NODES = 1 + MC_MAX_ITER * MC_MAX_K;
-constexpr int MC_CACHE = 64;           // remembered lookups (direct mapped): a search meets the same contexts again and again
+constexpr int MC_CACHE = 512;          // remembered lookups (direct mapped): a search meets the same contexts again and again
 
 struct McParams {
     int iterations, length, n_candidates, k;
     double e_table[MC_MAX_ITER + 1];   // E for sum N = 0 .. iterations
+    double root[MC_MAX_ITER + 1];      // square root of sum N
 };
 
-struct McLookup {                      // top-k list of one context
-    int n;                             // valid entries
+// Top-k list of one context: lane j holds the j-th continuation.
+struct McLookup {
+    int n;                             // continuations (every lane)
+    int32_t word;
+    double prob;                       // Eq. 1: count over the sum of ALL the context's counts
+    unsigned long long upto;           // sum of the counts of continuations 0 .. j
+};
+struct McSlot {                        // the same in shared memory
+    unsigned long long key;
+    unsigned long long upto[MC_MAX_K];
+    double prob[MC_MAX_K];
     int32_t word[MC_MAX_K];
-    uint32_t count[MC_MAX_K];
-    uint32_t total;                    // sum over ALL continuations of the context (Eq. 1's denominator)
+    int32_t n, pad;
 };
 
-// All 32 lanes call this with the same (a, b); the result is identical in every lane.
-__device__ __forceinline__ void mc_lookup(const TgView& t, int a, int b, int k, int lane, McLookup& out) {
+// All 32 lanes call this with the same (a, b).  Remembered contexts come from shared memory (the table does not change during a
+// search); lanes from MC_MAX_K on hold nothing of use.
+__device__ __forceinline__ McLookup mc_lookup(const TgView& t, int a, int b, int k, int lane, McSlot* s_cache) {
+    const unsigned long long key = tg_key(a, b);
+    McSlot& slot = s_cache[tg_hash(key) & (MC_CACHE - 1)];
+    const int j = lane & (MC_MAX_K - 1);
+    McLookup out;
+    if (slot.key == key) {
+        out.n = slot.n;
+        out.word = slot.word[j];
+        out.prob = slot.prob[j];
+        out.upto = slot.upto[j];
+        return out;
+    }
     unsigned long long best = 0;
     uint32_t total = 0;
     tg_scan(t, tg_open(t, a, b, lane), 0, 1, k, lane, best, total);
-    out.total = __reduce_add_sync(0xffffffffu, total);
-    out.n = __popc(__ballot_sync(0xffffffffu, lane < k && best != 0));
-#pragma unroll
-    for (int r = 0; r < MC_MAX_K; ++r) {
-        const unsigned long long key = __shfl_sync(0xffffffffu, best, r);
-        out.word[r] = tg_packed_tok(key);
-        out.count[r] = tg_packed_cnt(key);
+    total = __reduce_add_sync(0xffffffffu, total);
+    if (lane >= k) best = 0;
+    out.n = __popc(__ballot_sync(0xffffffffu, best != 0));
+    out.word = tg_packed_tok(best);
+    out.prob = best ? __ddiv_rn((double)tg_packed_cnt(best), (double)total) : 0.0;
+    out.upto = tg_packed_cnt(best);
+    if (best) {      // one of these is likely the next context: its home bucket comes to L2 meanwhile
+        const Bucket* next = t.buckets + (tg_hash(tg_key(b, out.word)) & t.n_home_mask);
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(next));
     }
-}
-
-// mc_lookup through the cache of remembered contexts (the table does not change during a search).
-__device__ __forceinline__ void mc_lookup_cached(const TgView& t, int a, int b, int k, int lane,
-                                                 unsigned long long* s_ckey, McLookup* s_cval, McLookup& out) {
-    const unsigned long long key = tg_key(a, b);
-    const int slot = (int)(tg_hash(key) & (MC_CACHE - 1));
-    if (s_ckey[slot] == key) { out = s_cval[slot]; return; }
-    mc_lookup(t, a, b, k, lane, out);
+#pragma unroll
+    for (int o = 1; o < MC_MAX_K; o <<= 1) {
+        const unsigned long long other = __shfl_up_sync(0xffffffffu, out.upto, o);
+        if (lane >= o) out.upto += other;
+    }
     __syncwarp();
-    if (lane == 0) { s_cval[slot] = out; s_ckey[slot] = key; }
+    if (lane < MC_MAX_K) { slot.upto[lane] = out.upto; slot.prob[lane] = out.prob; slot.word[lane] = out.word; }
+    if (lane == 0) { slot.n = out.n; slot.key = key; }
     __syncwarp();
+    return out;
 }
 
 __host__ __device__ constexpr size_t mc_cache_offset() {
-    return (((size_t)MC_MAX_NODES * (2 * 8 + 2 * 4 + 2 * 2 + 2 * 1) + ADED_MAX_NODES * 2) + 15) & ~(size_t)15;
+    return (((size_t)MC_MAX_NODES * (3 * 8 + 2 * 4 + 2 * 2 + 2 * 1) + ADED_MAX_NODES * 2) + 15) & ~(size_t)15;
 }
 
 __host__ __device__ constexpr size_t mc_fill_offset() {
-    return (mc_cache_offset() + (size_t)MC_CACHE * (8 + sizeof(McLookup)) + (size_t)MC_MAX_ITER * MC_MAX_LEN * sizeof(float) + 15) & ~(size_t)15;
+    return (mc_cache_offset() + (size_t)MC_CACHE * sizeof(McSlot) + (size_t)MC_MAX_ITER * MC_MAX_LEN * sizeof(float) + 15) & ~(size_t)15;
 }
 
 __global__ void __launch_bounds__(32)
@@ -505,18 +659,18 @@ k_mcts_draft(TgView t, const __grid_constant__ McParams p, const int32_t* __rest
     // 8-byte, then 4-byte, then 2-byte, then 1-byte arrays, so that each starts aligned
     double* s_score = reinterpret_cast<double*>(mc_smem);                 // [MC_MAX_NODES] sum of scores
     double* s_prior = s_score + MC_MAX_NODES;                             // Eq. 1 probability of the node's token in its parent's context
-    int32_t* s_tok = reinterpret_cast<int32_t*>(s_prior + MC_MAX_NODES);  // token
+    double* s_mean = s_prior + MC_MAX_NODES;                              // mean score (0 while not visited)
+    int32_t* s_tok = reinterpret_cast<int32_t*>(s_mean + MC_MAX_NODES);   // token
     int32_t* s_visits = s_tok + MC_MAX_NODES;
     int16_t* s_par = reinterpret_cast<int16_t*>(s_visits + MC_MAX_NODES);
     int16_t* s_first = s_par + MC_MAX_NODES;                              // first child (children are consecutive)
     int16_t* s_queue = s_first + MC_MAX_NODES;                            // [ADED_MAX_NODES] breadth-first order of the result
     uint8_t* s_nkid = reinterpret_cast<uint8_t*>(s_queue + ADED_MAX_NODES);
     uint8_t* s_flag = s_nkid + MC_MAX_NODES;                              // bit 0 expanded, bit 1 chosen, bit 2 kept
-    unsigned long long* s_ckey = reinterpret_cast<unsigned long long*>(mc_smem + mc_cache_offset());   // [MC_CACHE] context of a remembered lookup
-    McLookup* s_cval = reinterpret_cast<McLookup*>(s_ckey + MC_CACHE);
-    for (int i = threadIdx.x; i < MC_CACHE; i += 32) s_ckey[i] = TG_EMPTY;
+    McSlot* s_cache = reinterpret_cast<McSlot*>(mc_smem + mc_cache_offset());   // [MC_CACHE] remembered lookups
+    for (int i = threadIdx.x; i < MC_CACHE; i += 32) s_cache[i].key = TG_EMPTY;
     pdl_enter();
-    float* s_u = reinterpret_cast<float*>(s_cval + MC_CACHE);            // the caller's uniform numbers
+    float* s_u = reinterpret_cast<float*>(s_cache + MC_CACHE);            // the caller's uniform numbers
     for (int i = threadIdx.x; i < p.iterations * p.length; i += 32) s_u[i] = u[i];
 
     const int lane = threadIdx.x;
@@ -524,96 +678,86 @@ k_mcts_draft(TgView t, const __grid_constant__ McParams p, const int32_t* __rest
     int n_nodes = 1;
     if (lane == 0) {
         s_tok[0] = root_token; s_par[0] = -1; s_first[0] = 0; s_nkid[0] = 0; s_flag[0] = 0;
-        s_visits[0] = 0; s_score[0] = 0.0; s_prior[0] = 0.0;
+        s_visits[0] = 0; s_score[0] = 0.0; s_prior[0] = 0.0; s_mean[0] = 0.0;
     }
     __syncwarp();
-    McLookup lk;
     for (int it = 0; it < p.iterations; ++it) {
-        int node = 0, len = 1;
-        int state[MC_MAX_LEN + 1];
-        double sp[MC_MAX_LEN + 1];          // Eq. 1 probability of state[i] given its two predecessors
-        state[0] = root_token;
-        bool end = false;
+        // the sentence so far: its last two tokens, its score (1 + the probabilities in order), and the tree nodes on it --
+        // lane d holds the node at depth d
+        int node = 0, len = 1, on_path = 0, depth = 0;
+        int before = prev_token, last = root_token;
+        double sc = 1.0;
         // selection
-        while ((s_flag[node] & 1) && s_nkid[node] > 0 && !end) {
-            // one lane per child (at most eight): the double divisions run side by side
+        while (s_nkid[node] > 0 && len <= p.length) {       // (a node has children only once it is expanded)
             const int first = s_first[node], nk = s_nkid[node];
             const bool mine = lane < nk;
             const int c = first + (mine ? lane : 0);
             const int nv = mine ? s_visits[c] : 0;
-            int n_sum = nv;
-            for (int o = 16; o > 0; o >>= 1) n_sum += __shfl_xor_sync(0xffffffffu, n_sum, o);
-            const double e = p.e_table[n_sum], root_n = sqrt((double)n_sum);
-            const double q = nv ? __ddiv_rn(s_score[c], (double)nv) : 0.0;
-            const double pr = s_prior[c];
-            double best_s = __dadd_rn(q, __ddiv_rn(__dmul_rn(__dmul_rn(e, pr), root_n), __dadd_rn(1.0, (double)nv)));
-            double best_p = pr;
-            int best = mine ? c : -1;
-            for (int o = 16; o > 0; o >>= 1) {
-                const double os = __shfl_xor_sync(0xffffffffu, best_s, o), op = __shfl_xor_sync(0xffffffffu, best_p, o);
-                const int ob = __shfl_xor_sync(0xffffffffu, best, o);
-                if (ob >= 0 && (best < 0 || os > best_s || (os == best_s && ob < best))) { best = ob; best_s = os; best_p = op; }
-            }
-            node = best;
-            state[len] = s_tok[node];
-            sp[len] = best_p;
+            const double pr = s_prior[c], q = s_mean[c];
+            const int n_sum = (int)__reduce_add_sync(0xffffffffu, (unsigned)nv);
+            const double score = __dadd_rn(q, __ddiv_rn(__dmul_rn(__dmul_rn(p.e_table[n_sum], pr), p.root[n_sum]), __dadd_rn(1.0, (double)nv)));
+            // the largest score, the earliest child among equals: bits of a double in an order that integers have, high half first
+            const unsigned long long bits = (unsigned long long)__double_as_longlong(score);
+            const unsigned long long ord = mine ? bits ^ ((bits >> 63) ? ~0ull : 1ull << 63) : 0ull;
+            const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(ord >> 32));
+            const bool top = mine && (unsigned)(ord >> 32) == hi;
+            const unsigned lo = __reduce_max_sync(0xffffffffu, top ? (unsigned)ord : 0u);
+            const int pick = __ffs((int)__ballot_sync(0xffffffffu, top && (unsigned)ord == lo)) - 1;
+            node = first + pick;
+            ++depth;
+            if (lane == depth) on_path = node;
+            before = last;
+            last = s_tok[node];
+            sc = __dadd_rn(sc, __shfl_sync(0xffffffffu, pr, pick));
             ++len;
-            if (len == p.length + 1) end = true;
         }
         // expansion
-        if (!(s_flag[node] & 1) && !end) {
-            const int a = node == 0 ? prev_token : s_tok[s_par[node]], b = s_tok[node];
-            mc_lookup_cached(t, a, b, p.k, lane, s_ckey, s_cval, lk);
+        if (!(s_flag[node] & 1) && len <= p.length) {
+            const McLookup lk = mc_lookup(t, before, last, p.k, lane, s_cache);
             if (lane == 0) {
                 s_flag[node] |= 1;
                 s_first[node] = (int16_t)n_nodes;
                 s_nkid[node] = (uint8_t)lk.n;
             }
-            if (lane < lk.n) {                            // one lane per child: the divisions run side by side
+            if (lane < lk.n) {
                 const int c = n_nodes + lane;
-                s_tok[c] = lk.word[lane]; s_par[c] = (int16_t)node; s_first[c] = 0; s_nkid[c] = 0; s_flag[c] = 0;
-                s_visits[c] = 0; s_score[c] = 0.0;
-                s_prior[c] = __ddiv_rn((double)lk.count[lane], (double)lk.total);
+                s_tok[c] = lk.word; s_par[c] = (int16_t)node; s_first[c] = 0; s_nkid[c] = 0; s_flag[c] = 0;
+                s_visits[c] = 0; s_score[c] = 0.0; s_mean[c] = 0.0;
+                s_prior[c] = lk.prob;
             }
             __syncwarp();
             if (lk.n > 0) {
                 n_nodes += lk.n;
                 node = n_nodes - 1;                       // the last child created
-                state[len] = s_tok[node];
-                sp[len] = s_prior[node];
+                ++depth;
+                if (lane == depth) on_path = node;
+                before = last;
+                last = __shfl_sync(0xffffffffu, lk.word, lk.n - 1);
+                sc = __dadd_rn(sc, __shfl_sync(0xffffffffu, lk.prob, lk.n - 1));
                 ++len;
             }
         }
         // simulation
-        int draws = 0;
-        while (len < p.length + 1) {
-            const int a = len >= 2 ? state[len - 2] : prev_token, b = state[len - 1];
-            mc_lookup_cached(t, a, b, p.k, lane, s_ckey, s_cval, lk);
+        for (int draws = 0; len <= p.length; ++draws, ++len) {
+            const McLookup lk = mc_lookup(t, before, last, p.k, lane, s_cache);
             if (lk.n == 0) break;
-            unsigned long long total = 0;
-            for (int j = 0; j < lk.n; ++j) total += lk.count[j];
+            const unsigned long long total = __shfl_sync(0xffffffffu, lk.upto, lk.n - 1);
             unsigned long long u24 = __float2uint_rd(__fmul_rn(s_u[it * p.length + draws], 16777216.f));
             if (u24 > 16777215ull) u24 = 16777215ull;
             const unsigned long long target = (total * u24) >> 24;
-            unsigned long long run = 0;
-            int pick = lk.n - 1;
-            for (int j = 0; j < lk.n; ++j) {
-                run += lk.count[j];
-                if (run > target) { pick = j; break; }
-            }
-            state[len] = lk.word[pick];
-            sp[len] = __ddiv_rn((double)lk.count[pick], (double)lk.total);
-            ++len;
-            ++draws;
+            const unsigned past = __ballot_sync(0xffffffffu, lane < lk.n && lk.upto > target);
+            const int pick = past ? __ffs((int)past) - 1 : lk.n - 1;
+            before = last;
+            last = __shfl_sync(0xffffffffu, lk.word, pick);
+            sc = __dadd_rn(sc, __shfl_sync(0xffffffffu, lk.prob, pick));
         }
-        // back propagation
-        double sc = 1.0;
-        for (int i = 1; i < len; ++i) sc = __dadd_rn(sc, sp[i]);
-        if (lane == 0) {
-            for (int cur = node; cur >= 0; cur = s_par[cur]) {
-                s_visits[cur] += 1;
-                s_score[cur] = __dadd_rn(s_score[cur], sc);
-            }
+        // back propagation: a lane per node of the path
+        if (lane <= depth) {
+            const int v = s_visits[on_path] + 1;
+            const double total = __dadd_rn(s_score[on_path], sc);
+            s_visits[on_path] = v;
+            s_score[on_path] = total;
+            s_mean[on_path] = __ddiv_rn(total, (double)v);
         }
         __syncwarp();
     }
@@ -625,7 +769,7 @@ k_mcts_draft(TgView t, const __grid_constant__ McParams p, const int32_t* __rest
         int best_i = -1;
         for (int i = 1 + lane; i < n_nodes; i += 32) {
             if (s_nkid[i] != 0 || (s_flag[i] & 2)) continue;
-            const double m = s_visits[i] ? __ddiv_rn(s_score[i], (double)s_visits[i]) : 0.0;
+            const double m = s_mean[i];
             if (best_i < 0 || m > best_m) { best_m = m; best_i = i; }     // i ascends within a lane: first wins ties
         }
         for (int o = 16; o > 0; o >>= 1) {
@@ -831,14 +975,29 @@ aded_status aded_trigram_topk(const aded_trigram* t, const int32_t* ctx_dev, int
     if (!t || q < 0 || k < 1 || k > 32) return ADED_ERR_INVALID_ARG;
     if (q == 0) return ADED_OK;
     if (!ctx_dev || !out_tokens_dev || !out_counts_dev) return ADED_ERR_INVALID_ARG;
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
     // As many queries per block as fill the device's block slots once (three blocks per SM).
     const int wave = ws_grid_limit(t->device) / 2 * 3;
     int per_block = (q + wave - 1) / wave;
+    if (q >= TOPK_BULK && k >= 2) {
+        uint32_t slots = TOPK_BULK;
+        while ((uint64_t)slots * 2 <= (uint64_t)q * k && slots < (1u << 31)) slots *= 2;
+        per_block = per_block > TOPK_LEAD_QUERIES ? TOPK_LEAD_QUERIES : per_block;
+        ADED_CUDA_TRY(cudaMemsetAsync(out_counts_dev, 0xFF, (size_t)slots * sizeof(uint32_t), st));
+        note_launch(3);
+        const int lead_blocks = (q + per_block - 1) / per_block;
+        k_topk_mark<<<(unsigned)(((long long)lead_blocks * per_block + 255) / 256), 256, 0, st>>>(t->view, ctx_dev, q, k, lead_blocks, per_block, slots - 1,
+                                                                                             out_tokens_dev, out_counts_dev);
+        k_topk_lead<<<lead_blocks, TOPK_THREADS, 0, st>>>(t->view, q, k, per_block, out_tokens_dev, out_counts_dev, out_total_dev);
+        k_topk_copy<<<(q + 255) / 256, 256, 0, st>>>(q, k, out_tokens_dev, out_counts_dev, out_total_dev);
+        ADED_CUDA_TRY(cudaGetLastError());
+        return ADED_OK;
+    }
     per_block = per_block > TOPK_MAX_QUERIES ? TOPK_MAX_QUERIES : per_block;
     static const cudaError_t prepared = cudaFuncSetAttribute(k_tg_topk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)topk_smem(TOPK_MAX_QUERIES));
     ADED_CUDA_TRY(prepared);
     note_launch();
-    k_tg_topk<<<(q + per_block - 1) / per_block, TOPK_THREADS, topk_smem(per_block), static_cast<cudaStream_t>(stream)>>>(
+    k_tg_topk<<<(q + per_block - 1) / per_block, TOPK_THREADS, topk_smem(per_block), st>>>(
         t->view, ctx_dev, q, k, per_block, out_tokens_dev, out_counts_dev, out_total_dev);
     ADED_CUDA_TRY(cudaGetLastError());
     return ADED_OK;
@@ -908,6 +1067,7 @@ aded_status aded_mcts_draft(const aded_trigram* t, const int32_t* context_dev, i
     p.n_candidates = n_candidates;
     p.k = k;
     for (int n = 0; n <= MC_MAX_ITER; ++n) p.e_table[n] = (double)c1 + std::log(((double)n + (double)c2 + 1.0) / (double)c2);   // Eq. 3
+    for (int n = 0; n <= MC_MAX_ITER; ++n) p.root[n] = std::sqrt((double)n);
     note_launch();
     ADED_CUDA_TRY(launch_k(k_mcts_draft, 1, 32, mc_smem_bytes(), static_cast<cudaStream_t>(stream), t->view, p, context_dev, u_dev, tree_tokens_dev,
                            tree_parents_dev, n_nodes_dev, sentence_tokens_dev, sentence_scores_dev, n_sentences_dev, n_nodes_target,

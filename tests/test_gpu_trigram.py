@@ -320,3 +320,33 @@ def test_long_spans_on_both_sides_of_the_bulk_update(cuda_device, windows):
     B.aded_trigram_update(t, bad.cuda())
     torch.cuda.synchronize()
     assert B.aded_trigram_poll_status(t) == 1
+
+
+@pytest.mark.parametrize("q", [(1 << 16) - 1, 1 << 16, (1 << 16) + 1, 150001])
+def test_lookups_on_both_sides_of_the_grouped_path(cuda_device, q):
+    """From 2^16 queries on a context is scanned once per call, with the output arrays as scratch: contexts all in the home bucket,
+    beyond it, long ones, absent ones; each asked for by one and by many queries; with and without the sums."""
+    from paper_2407_12021_b200 import binding as B
+    spans = gen.zipf_tokens(30000, 400, 61, 1).tolist()
+    for a in range(18):                         # more long contexts than a block scans together
+        spans += [t for i in range(2100) for t in (a, 400 + a, 450 + (i * 7 + a) % 3000)]
+    st = TrigramStore()
+    st.update(spans)
+    t = B.aded_trigram_create(5000, log2_buckets=17, overflow_buckets=1 << 15)
+    B.aded_trigram_update(t, torch.tensor(spans, dtype=torch.int32, device="cuda"))
+    keys = list(st.table.keys())
+    rare = keys[::3][:4000]
+    pool = [(a, 400 + a) for a in range(18)] + keys[:50] + [(4999, 4999), (-1, 3), (5000, 1), (7, -2)]
+    contexts = (rare + pool * (q // len(pool) + 1))[:q]
+    for k in (1, 2, 3, 8, 9):
+        tok, cnt, tot = _topk_gpu(B, t, contexts, k)
+        want = {c: (st.topk(*c, k), st.total(*c)) for c in set(contexts)}
+        bad = [(i, c) for i, c in enumerate(contexts) if ((tok[i], cnt[i]), tot[i]) != want[c]]
+        assert not bad, (q, k, bad[:3])
+    c = torch.tensor(contexts, dtype=torch.int32, device="cuda")
+    out_t, out_c = torch.empty((q, 4), dtype=torch.int32, device="cuda"), torch.empty((q, 4), dtype=torch.int32, device="cuda")
+    B.aded_trigram_topk(t, c, 4, out_t, out_c, None)
+    torch.cuda.synchronize()
+    assert B.aded_trigram_poll_status(t) == 0
+    got = list(zip(out_t.tolist(), out_c.tolist()))
+    assert all(got[i] == st.topk(*contexts[i], 4) for i in range(0, q, 97))
