@@ -13,15 +13,16 @@
 //      whose running nucleus sum exceeds target.
 // One block of 1024 threads per row; a thread keeps the weights of its contiguous run of at most 32
 // tokens in registers.  The nucleus comes from a three-pass radix selection on the weights (per-bin
-// integer mass and count in shared memory), ties at the threshold enter in id order; the draw is a
+// integer mass in shared memory), ties at the threshold enter in id order; the draw is a
 // block-wide prefix sum in id order.  All sums are integers, so the result does not depend on the
 // order of the atomic additions.
 //
 // What bounds it: latency -- a row is one block's chain of two passes over its logits (from L2) and some ten block-wide
-// steps.  Nearly all tokens of a peaked distribution have weights far below the largest and share bin 0 of the first radix pass,
-// and a shared 64-bit addition is a loop of compare-and-swaps: adding each token to its bin took 1.9 of the kernel's 2.0 ms
-// (64 rows x 32,000 logits with one clear maximum).  So a thread adds up bin 0, and runs of tokens in one bin, in registers
-// and a warp whose lanes all hold the same bin adds once.  Measured, the eight-layer 7B step in sampling mode: 2.94 -> 1.06 ms.
+// steps.  Many tokens share few bins (of a peaked distribution nearly all have weights far below the largest and lie in the
+// lowest), and a shared 64-bit addition is a loop of compare-and-swaps: adding each token to its bin with one took 1.9 of the
+// kernel's 2.0 ms (64 rows x 32,000 logits of a model).  So a bin's mass is two 32-bit words -- the sums of the masses' low 16
+// bits and of the rest, neither of which can overflow -- and a thread adds up bin 0 and runs of tokens in one bin in
+// registers first.  Measured, the eight-layer 7B step in sampling mode, choice and approval: 160 -> 40 us.
 #include "aded_internal.cuh"
 
 namespace aded {
@@ -56,22 +57,6 @@ __device__ __forceinline__ unsigned long long block_excl_scan_u64(unsigned long 
     return warp_sums[warp] + incl - v;
 }
 
-// Adds (mass, count) to a bin; lanes of the warp may hold the same bin (mass 0: nothing to add).  All lanes.
-__device__ __forceinline__ void bin_add(unsigned long long* s_mass, unsigned int* s_cnt, unsigned int bin, unsigned long long mass, unsigned int cnt) {
-    const unsigned busy = __ballot_sync(0xffffffffu, cnt != 0);
-    if (busy == 0) return;
-    const unsigned int first = __shfl_sync(0xffffffffu, bin, __ffs((int)busy) - 1);
-    if (__all_sync(0xffffffffu, cnt == 0 || bin == first)) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) mass += __shfl_xor_sync(0xffffffffu, mass, o);
-        cnt = __reduce_add_sync(0xffffffffu, cnt);
-        if ((threadIdx.x & 31) == 0) { atomicAdd(&s_mass[first], mass); atomicAdd(&s_cnt[first], cnt); }
-    } else if (cnt != 0) {
-        atomicAdd(&s_mass[bin], mass);
-        atomicAdd(&s_cnt[bin], cnt);
-    }
-}
-
 // VEC: rows start on 16-byte boundaries and a thread's run of tokens is a multiple of four (vocab % 4 == 0, run % 4 == 0).
 template <bool VEC>
 __global__ void __launch_bounds__(SM_THREADS)
@@ -80,8 +65,7 @@ k_sample_rows(const float* __restrict__ logits, int vocab, int ld, float tempera
     pdl_enter();
     if (status && first_thread_of_grid()) trace_mark(status, TK_PICK);
     if (status && *status != 0) return;
-    __shared__ unsigned long long s_mass[2048];
-    __shared__ unsigned int s_cnt[2048];
+    __shared__ unsigned int s_lo[2048], s_hi[2048];    // mass of a bin: low 16 bits summed, the rest summed
     __shared__ unsigned long long s_warp[33];
     __shared__ float s_max[32];
     __shared__ unsigned long long s_sel[3];        // selected bin, mass above it, (unused)
@@ -161,45 +145,41 @@ k_sample_rows(const float* __restrict__ logits, int vocab, int ld, float tempera
     // 4. radix selection of the threshold weight: bits 30..20, 19..10, 9..0
     unsigned int prefix = 0, prefix_mask = 0;
     unsigned long long mass_above = 0;
-    unsigned int cnt_eq = 0;
+    auto add = [&](unsigned int bin, unsigned long long mass) {      // (at most 2^35 per thread: 2^19 x 1024 threads in s_hi)
+        atomicAdd(&s_lo[bin], (unsigned int)mass & 0xFFFFu);
+        atomicAdd(&s_hi[bin], (unsigned int)(mass >> 16));
+    };
+    auto mass_of = [&](int bin) { return ((unsigned long long)s_hi[bin] << 16) + s_lo[bin]; };
     const int shifts[3] = {20, 10, 0};
     const int widths[3] = {11, 10, 10};
 #pragma unroll
     for (int pass = 0; pass < 3; ++pass) {
         const int sh = shifts[pass], bins = 1 << widths[pass];
-        for (int i = tid; i < 2048; i += SM_THREADS) { s_mass[i] = 0; s_cnt[i] = 0; }
+        for (int i = tid; i < 2048; i += SM_THREADS) { s_lo[i] = 0; s_hi[i] = 0; }
         __syncthreads();
         // (bin 0 apart; a run of tokens in one other bin is added when the next bin comes)
         unsigned long long zero_mass = 0, run_mass = 0;
-        unsigned int zero_cnt = 0, run_cnt = 0, run_bin = 0;
+        unsigned int run_bin = 0;
 #pragma unroll
         for (int j = 0; j < SM_PER; ++j) {
             if (q[j] != 0 && (q[j] & prefix_mask) == prefix) {
                 const unsigned int b = (q[j] >> sh) & (bins - 1);
                 if (b == 0) {
                     zero_mass += q[j];
-                    ++zero_cnt;
                 } else {
-                    if (b != run_bin && run_cnt != 0) {
-                        atomicAdd(&s_mass[run_bin], run_mass);
-                        atomicAdd(&s_cnt[run_bin], run_cnt);
-                        run_mass = 0;
-                        run_cnt = 0;
-                    }
+                    if (b != run_bin && run_mass != 0) { add(run_bin, run_mass); run_mass = 0; }
                     run_bin = b;
                     run_mass += q[j];
-                    ++run_cnt;
                 }
             }
         }
-        __syncwarp();
-        bin_add(s_mass, s_cnt, run_bin, run_mass, run_cnt);
-        bin_add(s_mass, s_cnt, 0u, zero_mass, zero_cnt);
+        if (run_mass != 0) add(run_bin, run_mass);
+        if (zero_mass != 0) add(0u, zero_mass);
         __syncthreads();
         // thread t owns bins 2047 - 2t and 2046 - 2t (descending), so that an exclusive scan in thread
         // order gives the mass of all higher bins
         const int b_hi = 2047 - 2 * tid, b_lo = 2046 - 2 * tid;
-        const unsigned long long m_hi = b_hi < bins ? s_mass[b_hi] : 0ull, m_lo = b_lo < bins ? s_mass[b_lo] : 0ull;
+        const unsigned long long m_hi = b_hi < bins ? mass_of(b_hi) : 0ull, m_lo = b_lo < bins ? mass_of(b_lo) : 0ull;
         unsigned long long dummy;
         const unsigned long long above = block_excl_scan_u64(m_hi + m_lo, s_warp, &dummy);
         const unsigned long long rem = need - mass_above;          // still to be found among the candidates
@@ -208,16 +188,14 @@ k_sample_rows(const float* __restrict__ logits, int vocab, int ld, float tempera
         __syncthreads();
         const unsigned int sel = (unsigned int)s_sel[0];
         mass_above += s_sel[1];
-        cnt_eq = s_cnt[sel];
         prefix |= sel << sh;
         prefix_mask |= (unsigned int)(bins - 1) << sh;
         __syncthreads();
     }
     const unsigned int thr = prefix;                               // the smallest weight inside the nucleus
     const unsigned long long rem = need - mass_above;
-    const unsigned long long n_ties = (rem + thr - 1) / thr;       // of the cnt_eq tokens with weight thr, lowest ids first
+    const unsigned long long n_ties = (rem + thr - 1) / thr;       // of the tokens with weight thr, lowest ids first
     const unsigned long long z = mass_above + n_ties * thr;
-    (void)cnt_eq;
 
     // 5. rank the ties in id order, then draw in id order
     unsigned long long my_ties = 0;
