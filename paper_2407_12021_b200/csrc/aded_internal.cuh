@@ -104,8 +104,7 @@ inline cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, siz
 struct RowMeta {
     int32_t* seq;      // [R] sequence of the row
     int32_t* local;    // [R] node index inside its tree
-    int32_t* depth;    // [R] edges from the root
-    int32_t* pos;      // [R] rotary position = committed length + depth
+    int32_t* pos;      // [R] rotary position = committed length + depth in the tree
     uint64_t* anc;     // [R][2] bit j set <=> local node j is an ancestor of the row's node, or itself
 };
 
@@ -120,47 +119,75 @@ struct CallPtrs {
     int32_t out_stride;
 };
 
-// Draft approval of one sequence, by one thread (a tree has at most ADED_MAX_NODES nodes; arrays in shared
-// memory).  A node is approved when its parent is approved and its token equals the model's token at the
-// parent; the deepest approved node (lowest index among equals) ends the accepted path.  Emits the
-// model's token of every path node: the approved drafts' successors, ending with the model's own next
-// token, and commits the path's length (the compaction that follows works from `moves`).  A failed pass emits nothing and
-// keeps the committed length.
-__device__ __forceinline__ void approval_walk(const int32_t* s_par, const int32_t* s_tok, const int32_t* s_best,
-                                              const int32_t* s_dep, int T, int pass_status, int32_t* out_tokens,
-                                              int32_t* out_len, int32_t* path, int32_t* moves, int32_t* len) {
+// Draft approval of one sequence, by one warp (a tree has at most ADED_MAX_NODES nodes; s_* in shared memory).  A node is
+// approved when its parent is approved and its token equals the model's token at the parent -- that is, when all its
+// ancestors but the root match, which its ancestor set (`anc`, two words per node, the node itself included) answers at
+// once; the deepest approved node (lowest index among equals) ends the accepted path, and the nodes of its ancestor set in
+// index order are the path.  Emits the model's token of every path node: the approved drafts' successors, ending with the
+// model's own next token, and commits the path's length (the compaction that follows works from `moves`).  A failed pass
+// emits nothing and keeps the committed length.  (One thread that walked the nodes took about 4 us of a pass.)
+__device__ __forceinline__ void approval_warp(int lane, const int32_t* s_par, const int32_t* s_tok, const int32_t* s_best, const uint64_t* __restrict__ anc,
+                                              int T, int pass_status, int32_t* out_tokens, int32_t* out_len, int32_t* path, int32_t* moves, int32_t* len) {
     if (pass_status != 0) {
-        *out_len = 0;
-        moves[1] = 0;
+        if (lane == 0) { *out_len = 0; moves[1] = 0; }
         return;
     }
-    uint64_t ok_lo = 1ull, ok_hi = 0ull;   // approved set; the root always is
-    int deepest = 0, deepest_depth = 0;
-    for (int i = 1; i < T; ++i) {
-        const int p = s_par[i];
-        const bool p_ok = p < 64 ? (ok_lo >> p) & 1 : (ok_hi >> (p - 64)) & 1;
-        if (p_ok && s_tok[i] == s_best[p]) {
-            if (i < 64) ok_lo |= 1ull << i; else ok_hi |= 1ull << (i - 64);
-            const int d = s_dep[i];
-            if (d > deepest_depth) { deepest_depth = d; deepest = i; }
+    constexpr int PER = ADED_MAX_NODES / 32;
+    static_assert(PER == 4, "two 64-bit words of nodes");
+    uint64_t lo[PER], hi[PER], matched[2] = {0, 0};
+#pragma unroll
+    for (int c = 0; c < PER; ++c) {
+        const int i = c * 32 + lane;
+        lo[c] = i < T ? anc[2 * i] : 0;
+        hi[c] = i < T ? anc[2 * i + 1] : 0;
+        const bool match = i < T && (i == 0 || s_tok[i] == s_best[s_par[i]]);
+        matched[c >> 1] |= (uint64_t)__ballot_sync(0xffffffffu, match) << ((c & 1) * 32);
+    }
+    unsigned key = 0;                       // (depth + 1, lowest index first)
+#pragma unroll
+    for (int c = 0; c < PER; ++c) {
+        const int i = c * 32 + lane;
+        const bool ok = i < T && ((lo[c] & ~matched[0]) | (hi[c] & ~matched[1])) == 0;
+        const unsigned mine = ok ? (unsigned)(__popcll(lo[c]) + __popcll(hi[c])) << 8 | (unsigned)(ADED_MAX_NODES - 1 - i) : 0u;
+        key = max(key, mine);
+    }
+    key = __reduce_max_sync(0xffffffffu, key);
+    const int deepest = ADED_MAX_NODES - 1 - (int)(key & 255u), n = (int)(key >> 8);
+    uint64_t on_lo = 0, on_hi = 0;
+#pragma unroll
+    for (int c = 0; c < PER; ++c) {
+        const uint64_t l = __shfl_sync(0xffffffffu, lo[c], deepest & 31), h = __shfl_sync(0xffffffffu, hi[c], deepest & 31);
+        if (c == deepest >> 5) { on_lo = l; on_hi = h; }
+    }
+#pragma unroll
+    for (int c = 0; c < PER; ++c) {
+        const int i = c * 32 + lane;
+        const uint64_t word = c < 2 ? on_lo : on_hi, below = (1ull << (i & 63)) - 1ull;
+        if ((word >> (i & 63)) & 1) {
+            const int at = __popcll(word & below) + (c < 2 ? 0 : __popcll(on_lo));
+            path[at] = i;
+            out_tokens[at] = s_best[i];
         }
     }
-    // path[j] for j = depth .. 0 by climbing; the node at depth j is path element j
-    int cur = deepest;
-    for (int j = deepest_depth; j >= 0; --j) {
-        path[j] = cur;
-        out_tokens[j] = s_best[cur];
-        cur = s_par[cur];
+    if (lane == 0) {
+        *out_len = n;
+        moves[0] = *len;
+        moves[1] = n;
+        *len += n;
     }
-    *out_len = deepest_depth + 1;
-    moves[0] = *len;
-    moves[1] = deepest_depth + 1;
-    *len += deepest_depth + 1;
+}
+
+// Sequence of the attention kernels' blockIdx.z: z / row_blocks-th in order of work.  (Before the dependency wait the array may
+// hold another call's order: kept in range, and looked at again after the wait.)
+__device__ __forceinline__ int attn_sequence(const int32_t* order, int z, int row_blocks, int batch) {
+    const int place = z / row_blocks;
+    return order ? min(max(__ldcg(order + place), 0), batch - 1) : place;
 }
 
 struct SeqMeta {
     int32_t* row_off;  // [B+1] first row of each sequence
     int32_t* path;     // [B][ADED_MAX_NODES] accepted path (local node indices), root first
+    int32_t* order;    // [B] sequences by falling number of keys (the attention kernel's order of work)
     int32_t* moves;    // [B][2] committed length before this call, and how many nodes of the path were kept (compaction)
 };
 
@@ -265,6 +292,7 @@ struct aded_model {
     bool ws_use_tiled;                  // GEMMs read the re-tiled copies (else the caller's matrices through ws_maps)
     float* ws_slots;                    // partial result tiles (see gemm_out.cuh)
     aded::TileRef* ws_tiles[5];         // contributor tables of the wqkv, wo, wgu, wd and LM-head results
+    int ws_contributors[5];             // most contributors of any of their tiles
     bool ws_one_per_sm[5];              // which of those five GEMMs launch one CTA per SM instead of two
     uint32_t* ws_counters;              // arrival counters of the LM head's tail, one per tile
     uint32_t ws_epoch;                  // LM-head launches with a tail so far (host side of the counters)
@@ -296,6 +324,7 @@ void launch_tree_prologue(aded_model* m, aded_kv* kv, const CallPtrs& call, cons
                           cudaStream_t st);
 void launch_accept(aded_model* m, aded_kv* kv, int batch, cudaStream_t st);
 void launch_compact(aded_model* m, aded_kv* kv, int batch, cudaStream_t st);
+void launch_kv_copy(char* cache_k, char* cache_v, size_t head_bytes, void* user_k, void* user_v, size_t bytes, int heads, bool load, cudaStream_t st);
 void launch_commit_chain(aded_model* m, aded_kv* kv, int batch, cudaStream_t st);
 
 // dense.cu
@@ -304,7 +333,7 @@ void launch_rope_freq(double* freq, int half, double theta);
 void launch_embed_norm(aded_model* m, const void* gain, int rows, cudaStream_t st);
 // projection result added to the residual stream, then the norm
 void launch_add_rmsnorm(aded_model* m, const GemmOut& y, const void* gain, int rows, cudaStream_t st);
-bool gemm_plain_prepare();
+bool gemm_plain_prepare(bool bf16_model);
 // w_map / x_map: index into m->ws_maps / m->ws_x_maps of the operands' TMA descriptors (-1: none, plain kernel).
 // `y` is the fp32 buffer the plain kernel writes; the returned descriptor says where the result is.
 // `epi_mode` (WS_EPI_*): whether the tensor-core kernel's tail also leaves per-tile greedy candidates (LM head).

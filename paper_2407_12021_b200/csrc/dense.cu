@@ -323,7 +323,8 @@ static bool gemm_plain_prepare_t() {
     set(k_gemm_plain<T, 64, true>); set(k_gemm_plain<T, 64, false>);
     return ok;
 }
-bool gemm_plain_prepare() { return gemm_plain_prepare_t<float>() && gemm_plain_prepare_t<bf16>(); }
+// (For the models that use it: the first call on a kernel loads it, which takes the creation of a model milliseconds.)
+bool gemm_plain_prepare(bool bf16_model) { return bf16_model ? gemm_plain_prepare_t<bf16>() : gemm_plain_prepare_t<float>(); }
 
 GemmOut launch_gemm(aded_model* m, int w_map, int x_map, const void* x, const void* w, float* y, int rows, int n, int k,
                     int epi_mode, int trace_kind, cudaStream_t st) {

@@ -74,12 +74,12 @@ constexpr int PICK_THREADS = 1024, PICK_PER_LANE = 8;
 __global__ void __launch_bounds__(PICK_THREADS) k_pick_accept(const CallPtrs* __restrict__ call, const float* __restrict__ cand_val,
                                                               const int32_t* __restrict__ cand_idx, int n_tiles,
                                                               const int32_t* __restrict__ row_off, int32_t* __restrict__ best,
-                                                              const int32_t* __restrict__ depth, int32_t* __restrict__ len,
+                                                              const uint64_t* __restrict__ anc, int32_t* __restrict__ len,
                                                               int32_t* __restrict__ path, int32_t* __restrict__ moves,
                                                               const int32_t* status) {
     pdl_enter();
     if (first_thread_of_grid()) trace_mark(status, TK_PICK);
-    __shared__ int32_t s_par[ADED_MAX_NODES], s_tok[ADED_MAX_NODES], s_best[ADED_MAX_NODES], s_dep[ADED_MAX_NODES];
+    __shared__ int32_t s_par[ADED_MAX_NODES], s_tok[ADED_MAX_NODES], s_best[ADED_MAX_NODES];
     const int b = blockIdx.x;
     const int pass_status = *status;
     const int off = row_off[b];
@@ -118,11 +118,10 @@ __global__ void __launch_bounds__(PICK_THREADS) k_pick_accept(const CallPtrs* __
     for (int i = threadIdx.x; i < T; i += blockDim.x) {
         s_par[i] = call->parents[off + i];
         s_tok[i] = call->tokens[off + i];
-        s_dep[i] = depth[off + i];
     }
     __syncthreads();
-    if (threadIdx.x == 0)
-        approval_walk(s_par, s_tok, s_best, s_dep, T, pass_status, call->out_tokens + (size_t)b * call->out_stride,
+    if (warp == 0)
+        approval_warp(lane, s_par, s_tok, s_best, anc + 2 * (size_t)off, T, pass_status, call->out_tokens + (size_t)b * call->out_stride,
                       call->out_len + b, path + b * ADED_MAX_NODES, moves + 2 * b, len + b);
 }
 
@@ -136,15 +135,18 @@ __global__ void __launch_bounds__(PICK_THREADS) k_pick_accept(const CallPtrs* __
 // running) the step is 1.3 % slower; released after the gather or at exit (its weight prefetch no longer
 // runs under this kernel) 4 % slower.  The SwiGLU and rotary kernels below do the same (for them the top of
 // the kernel measures the same; the difference comes from this kernel, whose blocks each take a whole SM's registers).
-__global__ void __launch_bounds__(1024) k_add_rmsnorm_ws(bf16* __restrict__ h, GemmOut y, const bf16* __restrict__ gain,
+// THREADS x 4 x PASSES columns; BATCH contributors in flight.  Narrow rows (d <= 1024) take 256 threads; their projections have up to
+// 20 contributors per tile (width 1024, 45 rows, us per launch with 8, 12 and 24 in flight: 5.5, 6.0, 5.8; 1024 threads, 12: 6.3).
+template <int THREADS, int PASSES, int BATCH>
+__global__ void __launch_bounds__(THREADS) k_add_rmsnorm_ws(bf16* __restrict__ h, GemmOut y, const bf16* __restrict__ gain,
                                                          bf16* __restrict__ x, int d, float eps, const int32_t* status) {
     __shared__ float red[32];
     const int r = blockIdx.x;
-    TileRef tr[2];
-    float4 gv[2];
+    TileRef tr[PASSES];
+    float4 gv[PASSES];
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const int c = (i * 1024 + threadIdx.x) * 4;
+    for (int i = 0; i < PASSES; ++i) {
+        const int c = (i * THREADS + threadIdx.x) * 4;
         if (c < d) {
             tr[i] = y.tiles[c >> 7];
             gv[i] = unpack4_bf16(*reinterpret_cast<const uint2*>(gain + c));
@@ -154,16 +156,16 @@ __global__ void __launch_bounds__(1024) k_add_rmsnorm_ws(bf16* __restrict__ h, G
     pdl_launch_dependents();
     if (first_thread_of_grid()) trace_mark(status, TK_NORM);
     const int pass_status = *status;     // acted on before the first store; the loads below are valid in any case
-    float4 v[2];
+    float4 v[PASSES];
     float sq = 0.f;
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const int c = (i * 1024 + threadIdx.x) * 4;
+    for (int i = 0; i < PASSES; ++i) {
+        const int c = (i * THREADS + threadIdx.x) * 4;
         if (c < d) {
             uint2* hp = reinterpret_cast<uint2*>(h + (size_t)r * d + c);
             const float4 hv = unpack4_bf16(*hp);
             if (!ADED_IN_RANGE(tr[i].first_slot >= 0 && tr[i].first_slot + tr[i].count <= y.n_tiles + y.g, status)) tr[i].count = 0;
-            const float4 add = gemm_out_at4(y, tr[i], r, c & 127);
+            const float4 add = gemm_out_at4<BATCH>(y, tr[i], r, c & 127);
             const uint2 nv = pack4_bf16(hv.x + add.x, hv.y + add.y, hv.z + add.z, hv.w + add.w);
             if (pass_status == 0) *hp = nv;
             v[i] = unpack4_bf16(nv);
@@ -175,12 +177,12 @@ __global__ void __launch_bounds__(1024) k_add_rmsnorm_ws(bf16* __restrict__ h, G
     __syncthreads();
     float total = 0.f;
 #pragma unroll
-    for (int i = 0; i < 32; ++i) total += red[i];      // same order in every thread
+    for (int i = 0; i < THREADS / 32; ++i) total += red[i];      // same order in every thread
     const float inv = rsqrtf(total / (float)d + eps);
     if (pass_status != 0) return;
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const int c = (i * 1024 + threadIdx.x) * 4;
+    for (int i = 0; i < PASSES; ++i) {
+        const int c = (i * THREADS + threadIdx.x) * 4;
         if (c < d)
             *reinterpret_cast<uint2*>(x + (size_t)r * d + c) =
                 pack4_bf16(v[i].x * inv * gv[i].x, v[i].y * inv * gv[i].y, v[i].z * inv * gv[i].z, v[i].w * inv * gv[i].w);
@@ -188,6 +190,8 @@ __global__ void __launch_bounds__(1024) k_add_rmsnorm_ws(bf16* __restrict__ h, G
 }
 
 // act = round(silu(gate) * up): grid (chunks of 1024 columns, rows), four columns per thread.
+// SB: contributors that a tile may have for all of both gathers to be in flight at once (the launch knows the most there are).
+template <int SB>
 __global__ void __launch_bounds__(256) k_swiglu_ws(GemmOut gu, bf16* __restrict__ act, int F, const int32_t* status) {
     const int r = blockIdx.y, c = (blockIdx.x * 256 + threadIdx.x) * 4;
     TileRef tg = {0, 0}, tu = {0, 0};
@@ -199,7 +203,6 @@ __global__ void __launch_bounds__(256) k_swiglu_ws(GemmOut gu, bf16* __restrict_
     const int pass_status = *status;     // checked before the store, not before the loads
     if (!ADED_IN_RANGE(tg.first_slot + tg.count <= gu.n_tiles + gu.g && tu.first_slot + tu.count <= gu.n_tiles + gu.g, status)) return;
     float4 g, u;
-    constexpr int SB = 4;      // gate/up tiles have two or three contributors at the 7B and 13B widths
     if (tg.count <= SB && tu.count <= SB) {
         float4 fg[SB], fu[SB];
         gemm_out_fetch4<SB>(gu, tg, r, c & 127, fg);
@@ -246,6 +249,46 @@ k_rope_kv_ws(GemmOut qkv, const float* __restrict__ cs, const float* __restrict_
                  pass_status == 0 && in_range);
 }
 
+// The same with a thread per (q, k or v; four pairs) instead of one for all three: for projections whose tiles have so many
+// contributors that a thread cannot hold all three gathers (small widths, where the GEMM's units are spread over all SMs: up to 14 at
+// width 1024: rotary + attention 20.9 us per layer there with k_rope_kv_ws, 17.4 with this and 7 in flight, 18.0 with 14).  At the 7B
+// widths it gains as much as the attention kernel behind it loses.
+template <int B>
+__global__ void __launch_bounds__(ROPE_WS_THREADS)
+k_rope_part_ws(GemmOut qkv, const float* __restrict__ cs, const float* __restrict__ sn,
+               bf16* __restrict__ q, char* const* __restrict__ base, const int32_t* __restrict__ cap,
+               const int32_t* __restrict__ len, const int32_t* __restrict__ row_seq,
+               const int32_t* __restrict__ row_local, int layer, int H, int hd, const int32_t* status) {
+    const int tph = hd >> 3, half = hd >> 1, d = H * hd, r = blockIdx.x;
+    const int item = blockIdx.y * ROPE_WS_THREADS + threadIdx.x;
+    const int part = item / (H * tph), hh = item / tph % H, i = item % tph * 4;
+    const bool mine = part < 3;
+    const int col = (mine ? part : 0) * d + hh * hd + i;
+    const TileRef t = qkv.tiles[col >> 7];                     // constant table (a head's columns lie in one tile)
+    pdl_wait();
+    pdl_launch_dependents();
+    if (first_thread_of_grid()) trace_mark(status, TK_ROPE);
+    if (!mine) return;
+    const int pass_status = *status;     // checked before the stores, not before the loads
+    const int b = row_seq[r];
+    const size_t slot = (size_t)len[b] + row_local[r];
+    const size_t cp = cap[b];
+    const bool in_range = ADED_IN_RANGE(slot < cp && t.first_slot + t.count <= qkv.n_tiles + qkv.g, status);
+    const float4 c = *reinterpret_cast<const float4*>(cs + r * half + i), s = *reinterpret_cast<const float4*>(sn + r * half + i);
+    float4 x0, x1;
+    gemm_out_two4<B>(qkv, t, r, col & 127, (col + half) & 127, x0, x1);
+    if (pass_status != 0 || !in_range) return;
+    bf16* dst = part == 0 ? q + (size_t)r * d + hh * hd + i
+                          : reinterpret_cast<bf16*>(base[b]) + ((((size_t)layer * 2 + part - 1) * H + hh) * cp + slot) * hd + i;
+    if (part < 2) {
+        *reinterpret_cast<uint2*>(dst) = pack4_bf16(x0.x * c.x - x1.x * s.x, x0.y * c.y - x1.y * s.y, x0.z * c.z - x1.z * s.z, x0.w * c.w - x1.w * s.w);
+        *reinterpret_cast<uint2*>(dst + half) = pack4_bf16(x1.x * c.x + x0.x * s.x, x1.y * c.y + x0.y * s.y, x1.z * c.z + x0.z * s.z, x1.w * c.w + x0.w * s.w);
+    } else {
+        *reinterpret_cast<uint2*>(dst) = pack4_bf16(x0.x, x0.y, x0.z, x0.w);
+        *reinterpret_cast<uint2*>(dst + half) = pack4_bf16(x1.x, x1.y, x1.z, x1.w);
+    }
+}
+
 // ---- launchers (callers have checked: bf16 model, tensor-core path) ----------------------------
 void launch_embed_norm_ws(aded_model* m, const void* gain, int rows, cudaStream_t st) {
     launch_k(k_embed_norm_ws, dim3(rows), dim3(1024), 0, st, (const bf16*)m->top.embed, (const CallPtrs*)m->call_dev, (bf16*)m->h,
@@ -254,26 +297,30 @@ void launch_embed_norm_ws(aded_model* m, const void* gain, int rows, cudaStream_
 
 void launch_pick_accept(aded_model* m, aded_kv* kv, int batch, const float* cand_val, const int32_t* cand_idx, int n, cudaStream_t st) {
     launch_k(k_pick_accept, dim3(batch), dim3(PICK_THREADS), 0, st, (const CallPtrs*)m->call_dev, cand_val, cand_idx, n,
-             (const int32_t*)m->seqs.row_off, m->best, (const int32_t*)m->rows.depth, kv->len_dev, m->seqs.path, m->seqs.moves,
+             (const int32_t*)m->seqs.row_off, m->best, (const uint64_t*)m->rows.anc, kv->len_dev, m->seqs.path, m->seqs.moves,
              (const int32_t*)m->status);
 }
 
 void launch_add_rmsnorm_ws(aded_model* m, const GemmOut& y, const void* gain, int rows, cudaStream_t st) {
     const int d = m->cfg.d_model;
-    launch_k(k_add_rmsnorm_ws, dim3(rows), dim3(1024), 0, st, (bf16*)m->h, y, (const bf16*)gain, (bf16*)m->x, d, m->cfg.rms_eps,
-             (const int32_t*)m->status);
+    auto go = [&](auto* kernel, int threads) {
+        launch_k(kernel, dim3(rows), dim3(threads), 0, st, (bf16*)m->h, y, (const bf16*)gain, (bf16*)m->x, d, m->cfg.rms_eps, (const int32_t*)m->status);
+    };
+    if (d <= 1024) go(k_add_rmsnorm_ws<256, 1, 8>, 256);
+    else go(k_add_rmsnorm_ws<1024, 2, 12>, 1024);
 }
 
 void launch_swiglu_ws(aded_model* m, const GemmOut& gu, int rows, cudaStream_t st) {
     const int F = m->cfg.d_ffn;
     dim3 grid((F + 1023) / 1024, rows);
-    launch_k(k_swiglu_ws, grid, dim3(256), 0, st, gu, (bf16*)m->act, F, (const int32_t*)m->status);
+    launch_k(m->ws_contributors[WS_MAP_GU] <= 4 ? k_swiglu_ws<4> : k_swiglu_ws<8>, grid, dim3(256), 0, st, gu, (bf16*)m->act, F, (const int32_t*)m->status);
 }
 
 void launch_rope_kv_ws(aded_model* m, aded_kv* kv, const GemmOut& qkv, int layer, int rows, cudaStream_t st) {
-    const int heads_per_block = ROPE_WS_THREADS / (m->cfg.head_dim / 8);
-    dim3 grid(rows, (m->cfg.n_heads + heads_per_block - 1) / heads_per_block);
-    launch_k(k_rope_kv_ws, grid, dim3(ROPE_WS_THREADS), 0, st, qkv, (const float*)m->rope_cos, (const float*)m->rope_sin, (bf16*)m->q,
+    const int heads_per_block = ROPE_WS_THREADS / (m->cfg.head_dim / 8), items = 3 * m->cfg.n_heads * (m->cfg.head_dim / 8);
+    const bool part = m->ws_contributors[WS_MAP_QKV] > 6;      // more than rope_kv_item holds at once
+    dim3 grid(rows, part ? (items + ROPE_WS_THREADS - 1) / ROPE_WS_THREADS : (m->cfg.n_heads + heads_per_block - 1) / heads_per_block);
+    launch_k(part ? k_rope_part_ws<7> : k_rope_kv_ws, grid, dim3(ROPE_WS_THREADS), 0, st, qkv, (const float*)m->rope_cos, (const float*)m->rope_sin, (bf16*)m->q,
              (char* const*)kv->base_dev, (const int32_t*)kv->cap_dev, (const int32_t*)kv->len_dev,
              (const int32_t*)m->rows.seq, (const int32_t*)m->rows.local, layer, m->cfg.n_heads, m->cfg.head_dim,
              (const int32_t*)m->status);

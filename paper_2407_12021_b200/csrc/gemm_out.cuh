@@ -94,6 +94,7 @@ __device__ __forceinline__ float gemm_out_load(const GemmOut& o, int r, int c) {
 __device__ __forceinline__ float4 f4_add(float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
 
 // Columns col .. col+3 (col % 4 == 0) of tile t, row r: slots added in CTA order.
+template <int GO_BATCH = 12>
 __device__ __forceinline__ float4 gemm_out_at4(const GemmOut& o, const TileRef& t, int r, int col) {
     const int rb = gemm_block_rb(o, r);
     const float* p = gemm_slot_row(o, t, r, rb) + col;
@@ -102,7 +103,6 @@ __device__ __forceinline__ float4 gemm_out_at4(const GemmOut& o, const TileRef& 
     // Up to GO_BATCH contributors are fetched at once (predicated loads, no branch between them) and
     // then added in CTA order: a projection with few tiles (O, down: 32 tiles over 296 CTAs) has about
     // ten contributors per tile, and a loop that fetched them four at a time cost three L2 round trips.
-    constexpr int GO_BATCH = 12;
     for (int i0 = 0; i0 < t.count; i0 += GO_BATCH) {
         float4 v[GO_BATCH];
 #pragma unroll
@@ -136,6 +136,28 @@ __device__ __forceinline__ float4 gemm_out_sum4(const float4 (&v)[B], const Tile
     for (int j = 0; j < B; ++j)
         if (j < t.count) sum = f4_add(sum, v[j]);
     return sum;
+}
+
+// Columns col .. col+3 and col2 .. col2+3 of the same tile and row, up to B contributors of both in flight at once.
+template <int B>
+__device__ __forceinline__ void gemm_out_two4(const GemmOut& o, const TileRef& t, int r, int col, int col2, float4& s0, float4& s1) {
+    const int rb = gemm_block_rb(o, r);
+    const float* p = gemm_slot_row(o, t, r, rb);
+    const size_t stride = (size_t)rb * 128;
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    s0 = zero;
+    s1 = zero;
+    for (int i0 = 0; i0 < t.count; i0 += B) {
+        float4 v0[B], v1[B];
+#pragma unroll
+        for (int j = 0; j < B; ++j) {
+            v0[j] = i0 + j < t.count ? __ldcg(reinterpret_cast<const float4*>(p + (size_t)(i0 + j) * stride + col)) : zero;
+            v1[j] = i0 + j < t.count ? __ldcg(reinterpret_cast<const float4*>(p + (size_t)(i0 + j) * stride + col2)) : zero;
+        }
+#pragma unroll
+        for (int j = 0; j < B; ++j)
+            if (i0 + j < t.count) { s0 = f4_add(s0, v0[j]); s1 = f4_add(s1, v1[j]); }
+    }
 }
 
 __device__ __forceinline__ uint2 pack4_bf16(float a, float b, float c, float d) {

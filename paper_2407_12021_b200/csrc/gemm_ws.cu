@@ -47,7 +47,6 @@ constexpr int WS_BM = 128;           // W rows per tile (MMA M)
 constexpr int WS_BK = 64;            // k elements per stage (128 bytes of bf16)
 constexpr int WS_THREADS = 192;
 constexpr long long WS_MEET_CYCLES = 400000000ll;   // about 0.2 s of SM clock: limit of the wait at a counter
-constexpr int WS_MIN_UNITS = 8;      // fewest work units of a CTA (see ws_grid)
 constexpr int WS_GMAX = 16;          // tile groups of a CTA handled per round of its tail
 
 struct WsParams {
@@ -457,15 +456,10 @@ int ws_grid_limit(int device) {
 // CTAs a launch over n_tiles x kb units uses: two per SM, or one per SM (with twice the stages, so the same bytes
 // in flight).  With one per SM a tile has half as many contributors, so the kernel that gathers the slots reads half
 // as much; used where that kernel is the next thing on the critical path (see ws_one_per_sm in model.cu).
-// A CTA gets at least WS_MIN_UNITS units: a small matrix spread over all SMs leaves every tile in a dozen or more pieces, and the
-// kernel that gathers them takes longer than the GEMM saved.  Measured on a model of width 1024 (45 rows, us per layer): with at
-// least 1, 2, 4, 8 units the four projections take 14.4, 13.6, 15.4, 17.6, the rotary, norm and SwiGLU kernels 29.0, 24.5, 19.3,
-// 15.6 -- the step 468, 426, 400, 385 us.  The 7B and 13B widths have 14 units and more per CTA.
 int ws_grid(int device, int n, int k, bool one_per_sm) {
     const long long units = (long long)(n / WS_BM) * (k / WS_BK);
-    int g = ws_grid_limit(device) / (one_per_sm ? 2 : 1);
-    if (units < (long long)g * WS_MIN_UNITS) g = (int)((units + WS_MIN_UNITS - 1) / WS_MIN_UNITS);
-    return g;
+    const int g = ws_grid_limit(device) / (one_per_sm ? 2 : 1);
+    return units < g ? (int)units : g;
 }
 
 // Floats of slot storage for results of up to max_n columns and max_rows rows.

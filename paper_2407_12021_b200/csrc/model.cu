@@ -83,18 +83,18 @@ static aded_status alloc_model(aded_model* m) {
     TRY(dev_alloc(m, &m->status, (size_t)STATUS_WORDS));
     TRY(dev_alloc(m, &m->rows.seq, R));
     TRY(dev_alloc(m, &m->rows.local, R));
-    TRY(dev_alloc(m, &m->rows.depth, R));
     TRY(dev_alloc(m, &m->rows.pos, R));
     TRY(dev_alloc(m, &m->rows.anc, 2 * R));
     TRY(dev_alloc(m, &m->seqs.row_off, B + 1));
     TRY(dev_alloc(m, &m->seqs.path, B * ADED_MAX_NODES));
     TRY(dev_alloc(m, &m->seqs.moves, 2 * B));
+    TRY(dev_alloc(m, &m->seqs.order, B));
+    ADED_CUDA_TRY(cudaMemset(m->seqs.order, 0, B * sizeof(int32_t)));
     TRY(dev_alloc(m, &m->call_dev, 1));
     TRY(dev_alloc(m, &m->rope_freq, c.head_dim / 2));
     TRY(dev_alloc(m, &m->argmax_val, R * ARGMAX_CHUNKS));
     TRY(dev_alloc(m, &m->argmax_idx, R * ARGMAX_CHUNKS));
     if (d > 8 * 1024) return ADED_ERR_UNSUPPORTED;   // the norm kernels keep a row in the registers of one block
-    if (!gemm_plain_prepare()) return ADED_ERR_CUDA;
     launch_rope_freq(m->rope_freq, c.head_dim / 2, (double)c.rope_theta);
     ADED_CUDA_TRY(cudaGetLastError());
     ADED_CUDA_TRY(cudaMemset(m->status, 0, STATUS_WORDS * sizeof(int32_t)));
@@ -175,7 +175,11 @@ static aded_status alloc_model(aded_model* m) {
                 m->ws_one_per_sm[i] = i == WS_MAP_O || i == WS_MAP_GU || i == WS_MAP_D;
                 const int nt = shapes[i][0] / 128, kb = shapes[i][1] / 64, g = ws_grid(m->device, shapes[i][0], shapes[i][1], m->ws_one_per_sm[i]);
                 std::vector<TileRef> table(nt);
-                for (int t = 0; t < nt; ++t) table[t] = gemm_tile_ref(nt, kb, g, t);
+                m->ws_contributors[i] = 0;
+                for (int t = 0; t < nt; ++t) {
+                    table[t] = gemm_tile_ref(nt, kb, g, t);
+                    if (table[t].count > m->ws_contributors[i]) m->ws_contributors[i] = table[t].count;
+                }
                 TRY(dev_alloc(m, &m->ws_tiles[i], (size_t)nt));
                 ADED_CUDA_TRY(cudaMemcpy(m->ws_tiles[i], table.data(), nt * sizeof(TileRef), cudaMemcpyHostToDevice));
             }
@@ -188,6 +192,7 @@ static aded_status alloc_model(aded_model* m) {
             m->ws_ready = true;
         }
     }
+    if (!m->ws_ready && !gemm_plain_prepare(c.dtype == ADED_BF16)) return ADED_ERR_CUDA;
     return ADED_OK;
 }
 
@@ -437,9 +442,17 @@ static aded_status kv_copy(const aded_kv* kv, int seq, int layer, int pos0, int 
     const aded_model_config& c = kv->model->cfg;
     const size_t row = (size_t)c.head_dim * kv->elem;
     const size_t cap = kv->cap[seq];
+    auto plane_of = [&](int which) { return kv->base[seq] + (((size_t)layer * 2 + which) * c.n_heads * cap + pos0) * row; };
+    if (((reinterpret_cast<uintptr_t>(k) | reinterpret_cast<uintptr_t>(v)) & 15) == 0) {
+        // one kernel for both planes (two strided copies of 16 MB each took 38 us, this 21); rows are multiples of 128 bytes
+        note_launch();
+        launch_kv_copy(plane_of(0), plane_of(1), cap * row, k, v, (size_t)n_pos * row, c.n_heads, into_cache, st);
+        ADED_CUDA_TRY(cudaGetLastError());
+        return ADED_OK;
+    }
     for (int which = 0; which < 2; ++which) {
         char* user = static_cast<char*>(which ? v : k);
-        char* plane = kv->base[seq] + (((size_t)layer * 2 + which) * c.n_heads * cap + pos0) * row;
+        char* plane = plane_of(which);
         // n_heads strided blocks of n_pos rows each
         if (into_cache)
             ADED_CUDA_TRY(cudaMemcpy2DAsync(plane, cap * row, user, (size_t)n_pos * row, (size_t)n_pos * row,

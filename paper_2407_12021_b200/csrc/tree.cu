@@ -17,7 +17,7 @@ struct PrologueArgs {
     int batch;
     int given;             // 0: call and row_off have been copied to their places instead
 };
-__global__ void k_tree_prologue(const __grid_constant__ PrologueArgs pa, CallPtrs* call_dev, int32_t* row_off_dev,
+__global__ void k_tree_prologue(const __grid_constant__ PrologueArgs pa, CallPtrs* call_dev, int32_t* row_off_dev, int32_t* order,
                                 const int32_t* __restrict__ len, const int32_t* __restrict__ cap, int vocab, int chain_mode,
                                 RowMeta rows, int32_t* status) {
     pdl_enter();
@@ -35,6 +35,15 @@ __global__ void k_tree_prologue(const __grid_constant__ PrologueArgs pa, CallPtr
     __shared__ int s_bad;
     if (i == 0) s_bad = 0;
     __syncthreads();
+    if (pa.batch > 1) {        // this sequence's place by falling length
+        const int mine = len[b];
+        int place = 0;
+        for (int o0 = 0; o0 < pa.batch; o0 += ADED_MAX_NODES) {
+            const int o = o0 + i, other = o < pa.batch ? len[o] : -1;
+            place += __syncthreads_count(o < pa.batch && (other > mine || (other == mine && o < b)));
+        }
+        if (i == 0) order[place] = b;
+    }
     if (*status != 0) return;   // an earlier error is still pending: do nothing
     int p = -1;
     if (i < T) {
@@ -62,20 +71,16 @@ __global__ void k_tree_prologue(const __grid_constant__ PrologueArgs pa, CallPtr
         const int r = off + i;
         rows.seq[r] = b;
         rows.local[r] = i;
-        rows.depth[r] = depth;
         rows.pos[r] = len[b] + depth;
         rows.anc[2 * r] = lo;
         rows.anc[2 * r + 1] = hi;
     }
 }
 
-// Draft approval, one thread per sequence (a tree has at most 128 nodes).  A node is approved when
-// its parent is approved and its token equals the model's greedy token at the parent; the deepest
-// approved node (lowest index among equals) ends the accepted path.  Emits the greedy token of
-// every path node: the approved drafts' successors, ending with the model's own next token.
+// Draft approval for tokens that are already chosen (sampling mode); a block per sequence.
 __global__ void k_accept(const CallPtrs* __restrict__ call,
                          const int32_t* __restrict__ row_off, const int32_t* __restrict__ best,
-                         const int32_t* __restrict__ depth, int32_t* __restrict__ len,
+                         const uint64_t* __restrict__ anc, int32_t* __restrict__ len,
                          int32_t* __restrict__ path, int32_t* __restrict__ moves,
                          const int32_t* status, int batch) {
     pdl_enter();
@@ -85,10 +90,9 @@ __global__ void k_accept(const CallPtrs* __restrict__ call,
     int32_t* __restrict__ out_tokens = call->out_tokens;
     int32_t* __restrict__ out_len = call->out_len;
     const int out_stride = call->out_stride;
-    // one block per sequence: the tree's arrays are fetched by all threads at once, then one thread walks
     const int b = blockIdx.x;
     if (b >= batch) return;
-    __shared__ int32_t s_par[ADED_MAX_NODES], s_tok[ADED_MAX_NODES], s_best[ADED_MAX_NODES], s_dep[ADED_MAX_NODES];
+    __shared__ int32_t s_par[ADED_MAX_NODES], s_tok[ADED_MAX_NODES], s_best[ADED_MAX_NODES];
     const int pass_status = *status;
     const int off = row_off[b];
     const int T = min(row_off[b + 1] - off, (int)ADED_MAX_NODES);
@@ -96,11 +100,10 @@ __global__ void k_accept(const CallPtrs* __restrict__ call,
         s_par[i] = parents[off + i];
         s_tok[i] = tokens[off + i];
         s_best[i] = best[off + i];
-        s_dep[i] = depth[off + i];
     }
     __syncthreads();
-    if (threadIdx.x != 0) return;
-    approval_walk(s_par, s_tok, s_best, s_dep, T, pass_status, out_tokens + (size_t)b * out_stride, out_len + b,
+    if (threadIdx.x >= 32) return;
+    approval_warp(threadIdx.x, s_par, s_tok, s_best, anc + 2 * (size_t)off, T, pass_status, out_tokens + (size_t)b * out_stride, out_len + b,
                   path + b * ADED_MAX_NODES, moves + 2 * b, len + b);
 }
 
@@ -149,6 +152,35 @@ __global__ void k_commit_chain(int32_t* len, const int32_t* __restrict__ row_off
     len[b] += row_off[b + 1] - row_off[b];
 }
 
+// Rows [pos0, pos0 + n) of all heads of a layer's K and V planes, to or from the caller's two [head][n] arrays; chunks of 16 bytes.
+// Grid (parts of a head's rows, heads, K and V).
+constexpr int KV_COPY_THREADS = 256, KV_COPY_PER = 4;
+template <bool LOAD>
+__global__ void __launch_bounds__(KV_COPY_THREADS)
+k_kv_copy(uint4* cache_k, uint4* cache_v, size_t head_stride, uint4* user_k, uint4* user_v, size_t n) {
+    uint4* cache = (blockIdx.z ? cache_v : cache_k) + blockIdx.y * head_stride;
+    uint4* user = (blockIdx.z ? user_v : user_k) + blockIdx.y * n;
+    const size_t i0 = (size_t)blockIdx.x * (KV_COPY_THREADS * KV_COPY_PER) + threadIdx.x;
+    uint4 v[KV_COPY_PER];
+#pragma unroll
+    for (int j = 0; j < KV_COPY_PER; ++j)
+        if (i0 + j * KV_COPY_THREADS < n) v[j] = (LOAD ? user : cache)[i0 + j * KV_COPY_THREADS];
+#pragma unroll
+    for (int j = 0; j < KV_COPY_PER; ++j)
+        if (i0 + j * KV_COPY_THREADS < n) (LOAD ? cache : user)[i0 + j * KV_COPY_THREADS] = v[j];
+}
+
+void launch_kv_copy(char* cache_k, char* cache_v, size_t head_bytes, void* user_k, void* user_v, size_t bytes, int heads, bool load, cudaStream_t st) {
+    const size_t n = bytes / sizeof(uint4), per = KV_COPY_THREADS * KV_COPY_PER;
+    const dim3 grid((unsigned)((n + per - 1) / per), heads, 2);
+    auto* ck = reinterpret_cast<uint4*>(cache_k);
+    auto* cv = reinterpret_cast<uint4*>(cache_v);
+    auto* uk = static_cast<uint4*>(user_k);
+    auto* uv = static_cast<uint4*>(user_v);
+    if (load) k_kv_copy<true><<<grid, KV_COPY_THREADS, 0, st>>>(ck, cv, head_bytes / sizeof(uint4), uk, uv, n);
+    else k_kv_copy<false><<<grid, KV_COPY_THREADS, 0, st>>>(ck, cv, head_bytes / sizeof(uint4), uk, uv, n);
+}
+
 void launch_tree_prologue(aded_model* m, aded_kv* kv, const CallPtrs& call, const int32_t* offsets_host, int batch, int chain_mode,
                           cudaStream_t st) {
     static_assert(PROLOGUE_MAX_BATCH < ADED_MAX_NODES, "a thread per row offset");
@@ -159,12 +191,12 @@ void launch_tree_prologue(aded_model* m, aded_kv* kv, const CallPtrs& call, cons
         pa.call = call;
         for (int b = 0; b <= batch; ++b) pa.row_off[b] = offsets_host[b];
     }
-    launch_k(k_tree_prologue, batch, ADED_MAX_NODES, 0, st, pa, m->call_dev, m->seqs.row_off, kv->len_dev, kv->cap_dev, m->cfg.vocab, chain_mode,
+    launch_k(k_tree_prologue, batch, ADED_MAX_NODES, 0, st, pa, m->call_dev, m->seqs.row_off, m->seqs.order, kv->len_dev, kv->cap_dev, m->cfg.vocab, chain_mode,
              m->rows, m->status);
 }
 
 void launch_accept(aded_model* m, aded_kv* kv, int batch, cudaStream_t st) {
-    launch_k(k_accept, batch, 128, 0, st, m->call_dev, m->seqs.row_off, m->best, m->rows.depth,
+    launch_k(k_accept, batch, 128, 0, st, m->call_dev, m->seqs.row_off, m->best, m->rows.anc,
                                                kv->len_dev, m->seqs.path, m->seqs.moves, m->status, batch);
 }
 

@@ -179,6 +179,7 @@ struct AttnArgs {
     const int32_t* cap;
     const int32_t* len;
     const int32_t* row_off;
+    const int32_t* order;          // [batch] sequences by falling length, or NULL (one sequence)
     const uint64_t* anc;
     int layer, H, n_splits, rows_total;
     int row_blocks;                // CTAs (of NW * 16 query rows each) per sequence and key split; grid.z = batch * row_blocks
@@ -200,7 +201,7 @@ __global__ void __launch_bounds__(NW * 32) k_tree_attn_mma(AttnArgs a) {
     // but this kernel does not rely on that: both are read again after the wait and the early blocks
     // are used only if the two reads agree, otherwise they are fetched again.
     // The cache block's address and capacity never change after the cache was created.
-    const int pre_hh = blockIdx.x, pre_b = blockIdx.z / a.row_blocks;
+    const int pre_hh = blockIdx.x, pre_b = attn_sequence(a.order, blockIdx.z, a.row_blocks, gridDim.z / a.row_blocks);
     const size_t pre_cp = a.cap[pre_b];
     const bf16* pre_kg = reinterpret_cast<const bf16*>(a.base[pre_b]) + (((size_t)a.layer * 2 + 0) * a.H + pre_hh) * pre_cp * HD;
     const bf16* pre_vg = reinterpret_cast<const bf16*>(a.base[pre_b]) + (((size_t)a.layer * 2 + 1) * a.H + pre_hh) * pre_cp * HD;
@@ -212,7 +213,7 @@ __global__ void __launch_bounds__(NW * 32) k_tree_attn_mma(AttnArgs a) {
     __syncthreads();
     const int pre_L = s_pre[0], pre_T = s_pre[1];
     int pre_blk0 = 0, n_pre = 0;
-    if (pre_L >= 0 && pre_T >= 1 && pre_T <= ADED_MAX_NODES && (size_t)pre_L + pre_T <= pre_cp) {
+    if (pre_L >= 0 && pre_T > (int)(blockIdx.z % a.row_blocks) * NW * 16 && pre_T <= ADED_MAX_NODES && (size_t)pre_L + pre_T <= pre_cp) {
         const int nb_p = (pre_L + pre_T + TA_BLK - 1) / TA_BLK;
         const int bps_p = (nb_p + a.n_splits - 1) / a.n_splits;
         pre_blk0 = blockIdx.y * bps_p;
@@ -244,7 +245,7 @@ __global__ void __launch_bounds__(NW * 32) k_tree_attn_mma(AttnArgs a) {
     constexpr int KSTEPS = HD / 16;        // k steps of Q K^T
     constexpr int ONT = HD / 8;            // n tiles of the output
 
-    const int hh = blockIdx.x, split = blockIdx.y, b = blockIdx.z / a.row_blocks;
+    const int hh = blockIdx.x, split = blockIdx.y, b = attn_sequence(a.order, blockIdx.z, a.row_blocks, gridDim.z / a.row_blocks);
     const int row_base = (blockIdx.z % a.row_blocks) * NW * 16;    // first query row (node of the tree) of this CTA
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, tig = lane & 3;
     const int off = a.row_off[b];
@@ -255,7 +256,7 @@ __global__ void __launch_bounds__(NW * 32) k_tree_attn_mma(AttnArgs a) {
     const int nb = (n_keys + TA_BLK - 1) / TA_BLK;
     const int bps = (nb + a.n_splits - 1) / a.n_splits;
     const int blk0 = split * bps;
-    const int blk1 = min(nb, blk0 + bps);
+    const int blk1 = row_base < T ? min(nb, blk0 + bps) : blk0;     // (a second block of rows that this tree does not reach: nothing to do)
 
     // this thread's two query rows (local node indices) and their global rows
     const int i0 = row_base + warp * 16 + g, i1 = i0 + 8;
@@ -305,7 +306,7 @@ __global__ void __launch_bounds__(NW * 32) k_tree_attn_mma(AttnArgs a) {
     // exactly one group (an empty one past the end), so "all but the newest TA_STAGES - 2 groups have
     // landed" always means the current block has.  (A split past the last key block has nothing to do
     // but still joins the merge.)
-    if (n_pre > 0 && (L != pre_L || T != pre_T || blk0 != pre_blk0)) {
+    if (n_pre > 0 && (b != pre_b || L != pre_L || T != pre_T || blk0 != pre_blk0 || row_base >= T)) {
         // the early reads were stale: let the early copies land, then fetch the right blocks over them
         cp_async_wait<0>();
         __syncthreads();
@@ -536,6 +537,7 @@ static void launch_mma(aded_model* m, aded_kv* kv, int layer, int batch, int row
     a.cap = kv->cap_dev;
     a.len = kv->len_dev;
     a.row_off = m->seqs.row_off;
+    a.order = batch > 1 ? m->seqs.order : nullptr;     // (see the tcgen05 kernel's launch)
     a.anc = m->rows.anc;
     a.layer = layer;
     a.H = m->cfg.n_heads;

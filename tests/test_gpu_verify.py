@@ -472,3 +472,32 @@ def test_batches_beyond_the_inline_offsets(cuda_device):
         torch.cuda.synchronize()
         assert B.aded_model_poll_status(model) == 0
         assert [out[b, :int(n[b])].tolist() for b in range(batch)] == alone[:batch]
+
+
+@pytest.mark.parametrize("dtype,hd,offset", [("f32", 64, 0), ("bf16", 64, 0), ("bf16", 128, 0), ("bf16", 128, 2), ("f32", 128, 1)])
+def test_kv_load_and_read_are_copies(cuda_device, dtype, hd, offset):
+    """Rows go into the cache and come back bit for bit: whole sequences, one row, ranges that are no multiple of a block's share,
+    from and to arrays that start on a 16-byte boundary and ones that do not; nothing beside the range is touched."""
+    from paper_2407_12021_b200 import binding as B
+    shape = gen.ModelShape("kv", 2, 3 * hd, 3, hd, 96, 64, dtype)
+    model = B.aded_model_create(shape, H.weights_to(gen.model_weights(shape, 90), cuda_device), max_rows=4, max_batch=1)
+    dt = torch.float32 if dtype == "f32" else torch.bfloat16
+    cap = 700
+    for n in (1, 127, 513, 700):
+        kv = B.aded_kv_create(model, [cap])
+
+        def place(x):
+            flat = torch.zeros(x.numel() + offset, dtype=dt, device="cuda")
+            flat[offset:].view(x.shape).copy_(x)
+            return flat[offset:].view(x.shape)
+
+        k, v = (place(torch.randn((3, n, hd), device="cuda").to(dt)) for _ in range(2))
+        B.aded_kv_load(kv, 0, 1, k, v)
+        for pos0, m in ((0, n), (n - 1, 1), (n // 3, n - n // 3)):
+            gk, gv = B.aded_kv_read(kv, 0, 1, pos0, m)
+            assert torch.equal(gk, k[:, pos0:pos0 + m]) and torch.equal(gv, v[:, pos0:pos0 + m])
+        if n < cap:
+            gk, gv = B.aded_kv_read(kv, 0, 1, n, cap - n)
+            assert not gk.any() and not gv.any()
+        gk, gv = B.aded_kv_read(kv, 0, 0, 0, cap)
+        assert not gk.any() and not gv.any()
