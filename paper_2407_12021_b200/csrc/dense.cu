@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(1024) k_add_rmsnorm(T* __restrict__ h, const f
 // These are the GEMMs of small models and a handful of rows: bound by latency, not by arithmetic.  So the chunk is all of k where
 // that fits -- one round of loads, of which the weights' are issued before the previous kernel has finished -- and the split of
 // k keeps eight warps busy on 16 rows.  (Blocks of 64 x 64 outputs with 16 k at a time took 23 to 65 us per GEMM of the 256-wide
-// fp32 model at 16 rows, two barriers and one exposed load per 16 k; this: 4.5 to 8.6 us.)
+// fp32 model at 16 rows, two barriers and one exposed load per 16 k; this: 3.9 to 6.5 us.)
 constexpr int GP_BN = 32, GP_THREADS = 256;
 template <typename T, bool VEC>
 __device__ __forceinline__ float4 gp_load4(const T* p) {
@@ -108,9 +108,14 @@ __global__ void __launch_bounds__(GP_THREADS) k_gemm_plain(const T* __restrict__
         const int quads = len / 4;
         for (int i = threadIdx.x; i < count * quads; i += GP_THREADS) {
             const int rr = i / quads, kk = (i % quads) * 4;
-            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (from + rr < limit && k0 + kk < k) v = gp_load4<T, VEC>(m + (size_t)(from + rr) * k + k0 + kk);
-            *reinterpret_cast<float4*>(dst + (size_t)rr * ld + kk) = v;
+            const bool there = from + rr < limit && k0 + kk < k;
+            const T* src = m + (there ? (size_t)(from + rr) * k + k0 + kk : 0);
+            float* to = dst + (size_t)rr * ld + kk;
+            if (VEC && sizeof(T) == 4) {       // all of a thread's copies in flight, without registers; zeros where there is nothing
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(to)), "l"(src), "r"(there ? 16 : 0) : "memory");
+            } else {
+                *reinterpret_cast<float4*>(to) = there ? gp_load4<T, VEC>(src) : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
         }
     };
     float acc[4][4] = {};
@@ -121,9 +126,13 @@ __global__ void __launch_bounds__(GP_THREADS) k_gemm_plain(const T* __restrict__
         if (k0 == 0) {
             pdl_wait();
             if (first_thread_of_grid()) trace_mark(status, trace_kind);
-            if (*status != 0) return;
+            if (*status != 0) {
+                asm volatile("cp.async.wait_all;" ::: "memory");
+                return;
+            }
         }
         stage(sx, x, r0, BM, rows, k0, len);
+        asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
         const int per = len / SLICES;
         for (int kk = slice * per; kk < (slice + 1) * per; kk += 4) {

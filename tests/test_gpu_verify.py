@@ -501,3 +501,42 @@ def test_kv_load_and_read_are_copies(cuda_device, dtype, hd, offset):
             assert not gk.any() and not gv.any()
         gk, gv = B.aded_kv_read(kv, 0, 0, 0, cap)
         assert not gk.any() and not gv.any()
+
+
+@pytest.mark.parametrize("heads,nodes,ctx", [(40, 64, 700), (48, 33, 1000), (56, 64, 65), (30, 64, 40), (24, 128, 500), (60, 17, 3), (40, 1, 2000), (3, 65, 0)])
+def test_attention_with_every_number_of_splits(cuda_device, heads, nodes, ctx):
+    """The key splits of a head (7, 6, 5, 8, 6, 4, 7 and 8 of them here, some without keys) deal out a row block's rows
+    among themselves for the merge: numbers of splits that do not divide the rows, one and two blocks of rows.  Against attention in float64
+    from the device's own q, K and V; the bound is that of the tests above (2e-2 of the largest output)."""
+    from paper_2407_12021_b200 import binding as B
+    hd, d = 128, 128 * heads
+    shape = gen.ModelShape("splits", 1, d, heads, hd, 128, 256, "bf16")
+    w = gen.model_weights(shape, 95, device=cuda_device)
+    w["layers"][0]["wqkv"] = (w["layers"][0]["wqkv"].float() * 3).to(torch.bfloat16)
+    model = B.aded_model_create(shape, w, max_rows=nodes, max_batch=1)
+    kv = B.aded_kv_create(model, [ctx + nodes])
+    g = torch.Generator(device="cuda").manual_seed(96)
+    if ctx:
+        k, v = (torch.randn((heads, ctx, hd), device="cuda", generator=g).to(torch.bfloat16) for _ in range(2))
+        B.aded_kv_load(kv, 0, 0, k, v)
+    tokens, parents = gen.make_tree(nodes, min(6, nodes - 1), 12, shape.vocab, 97, root_token=1)
+    out, n = torch.zeros(nodes, dtype=torch.int32, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    B.aded_verify(model, kv, H.i32(tokens), H.i32(parents), out, n)
+    torch.cuda.synchronize()
+    assert B.aded_model_poll_status(model) == 0 and int(n[0]) >= 1
+    q = B.aded_debug_read_buffer(model, 2, nodes).double().view(nodes, heads, hd)
+    att = B.aded_debug_read_buffer(model, 3, nodes).double().view(nodes, heads, hd)
+    kk, vv = (x.double() for x in B.aded_kv_read(kv, 0, 0, 0, ctx + nodes))
+    if int(n[0]) > 1:                       # (approved rows moved: their old places no longer hold what was attended to)
+        return
+    mask = torch.zeros((nodes, ctx + nodes), dtype=torch.bool, device="cuda")
+    mask[:, :ctx] = True
+    for i in range(nodes):
+        j = i
+        while j >= 0:
+            mask[i, ctx + j] = True
+            j = parents[j]
+    s = torch.einsum("thd,hld->thl", q, kk) / hd ** 0.5
+    p = torch.softmax(s.masked_fill(~mask[:, None, :], float("-inf")), dim=-1)
+    want = torch.einsum("thl,hld->thd", p, vv)
+    assert float((att - want).abs().max()) <= 2e-2 * float(want.abs().max())
