@@ -332,23 +332,25 @@ void launch_rope_freq(double* freq, int half, double theta);
 // embedding lookup, the first RMSNorm and the rotary tables
 void launch_embed_norm(aded_model* m, const void* gain, int rows, cudaStream_t st);
 // projection result added to the residual stream, then the norm
-void launch_add_rmsnorm(aded_model* m, const GemmOut& y, const void* gain, int rows, cudaStream_t st);
+void launch_add_rmsnorm(aded_model* m, const GemmOut& y, const void* gain, cudaStream_t st);
 bool gemm_plain_prepare(bool bf16_model);
 // w_map / x_map: index into m->ws_maps / m->ws_x_maps of the operands' TMA descriptors (-1: none, plain kernel).
 // `y` is the fp32 buffer the plain kernel writes; the returned descriptor says where the result is.
 // `epi_mode` (WS_EPI_*): whether the tensor-core kernel's tail also leaves per-tile greedy candidates (LM head).
-GemmOut launch_gemm(aded_model* m, int w_map, int x_map, const void* x, const void* w, float* y, int rows, int n, int k,
+// A call is worked in passes of gemm_pass_rows rows: the result of rows [row0, row0 + rows), to be consumed before the next.
+int gemm_pass_rows(const aded_model* m, int rows);
+GemmOut launch_gemm(aded_model* m, int w_map, int x_map, const void* x, const void* w, float* y, int row0, int rows, int n, int k,
                     int epi_mode, int trace_kind, cudaStream_t st);
-void launch_rope_kv(aded_model* m, aded_kv* kv, const GemmOut& qkv, int layer, int rows, cudaStream_t st);
-void launch_swiglu(aded_model* m, const GemmOut& gu, int rows, cudaStream_t st);
-void launch_argmax(aded_model* m, const GemmOut& logits, int rows, cudaStream_t st);
+void launch_rope_kv(aded_model* m, aded_kv* kv, const GemmOut& qkv, int layer, cudaStream_t st);
+void launch_swiglu(aded_model* m, const GemmOut& gu, cudaStream_t st);
+void launch_argmax(aded_model* m, const GemmOut& logits, cudaStream_t st);
 // Writes a projection result as a plain [rows, n] fp32 matrix (debug paths).
-void launch_materialize(aded_model* m, const GemmOut& src, float* dst, int rows, cudaStream_t st);
+void launch_materialize(aded_model* m, const GemmOut& src, float* dst, cudaStream_t st);
 
 // dense_ws.cu: bf16 consumers of slot-resident projection results
-void launch_add_rmsnorm_ws(aded_model* m, const GemmOut& y, const void* gain, int rows, cudaStream_t st);
-void launch_swiglu_ws(aded_model* m, const GemmOut& gu, int rows, cudaStream_t st);
-void launch_rope_kv_ws(aded_model* m, aded_kv* kv, const GemmOut& qkv, int layer, int rows, cudaStream_t st);
+void launch_add_rmsnorm_ws(aded_model* m, const GemmOut& y, const void* gain, cudaStream_t st);
+void launch_swiglu_ws(aded_model* m, const GemmOut& gu, cudaStream_t st);
+void launch_rope_kv_ws(aded_model* m, aded_kv* kv, const GemmOut& qkv, int layer, cudaStream_t st);
 void launch_embed_norm_ws(aded_model* m, const void* gain, int rows, cudaStream_t st);
 // greedy token per row from n candidates (value, column) each, then the approval walk (one launch)
 void launch_pick_accept(aded_model* m, aded_kv* kv, int batch, const float* cand_val, const int32_t* cand_idx, int n, cudaStream_t st);
@@ -362,7 +364,7 @@ int ws_grid_limit(int device);
 int ws_grid(int device, int n, int k, bool one_per_sm);
 size_t ws_slot_floats(int device, int max_n, int max_rows);
 cudaError_t ws_retile(const void* w, void* out, int n, int k, cudaStream_t st);
-cudaError_t ws_launch(const CUtensorMap& map_w, const void* w_tiled, const CUtensorMap& map_x, int rows, int row0, int blk,
+cudaError_t ws_launch(const CUtensorMap& map_w, const void* w_tiled, const CUtensorMap& map_x, int rows, int row0,
                       int n, int k,
                       float* slots, int32_t* status, const WsEpilogue& epi, int trace_kind, int device, bool one_per_sm, cudaStream_t st);
 enum { WS_MAP_QKV = 0, WS_MAP_O = 1, WS_MAP_GU = 2, WS_MAP_D = 3 };   // per-layer map order

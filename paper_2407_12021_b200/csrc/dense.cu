@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(256) k_argmax_chunks(GemmOut logits, float* __
     if (*status != 0) return;
     __shared__ float sv[8];
     __shared__ int si[8];
-    const int r = blockIdx.y;
+    const int r = logits.row0 + blockIdx.y;
     const int c0 = blockIdx.x * chunk, c1 = min(V, c0 + chunk);
     float bv = -INFINITY;
     int bi = 0x7fffffff;
@@ -269,7 +269,7 @@ __global__ void k_materialize(GemmOut src, float* __restrict__ dst, int n, int v
     pdl_enter();
     if (first_thread_of_grid()) trace_mark(status, TK_OTHER);
     if (*status != 0) return;
-    const int r = blockIdx.y;
+    const int r = src.row0 + blockIdx.y;
     const int c = (blockIdx.x * blockDim.x + threadIdx.x) * (vec ? 4 : 1);
     if (c >= n) return;
     if (vec) *reinterpret_cast<float4*>(dst + (size_t)r * n + c) = gemm_out_at4(src, src.tiles[c >> 7], r, c & 127);
@@ -291,12 +291,12 @@ void launch_embed_norm(aded_model* m, const void* gain, int rows, cudaStream_t s
              (const float*)gain, (float*)m->x, d, m->cfg.rms_eps, rope_args(m), m->status);
 }
 
-void launch_add_rmsnorm(aded_model* m, const GemmOut& y, const void* gain, int rows, cudaStream_t st) {
+void launch_add_rmsnorm(aded_model* m, const GemmOut& y, const void* gain, cudaStream_t st) {
     const int d = m->cfg.d_model;
-    if (y.mode == 1) { launch_add_rmsnorm_ws(m, y, gain, rows, st); return; }
+    if (y.mode == 1) { launch_add_rmsnorm_ws(m, y, gain, st); return; }
     const RopeArgs none = {};
-    BY_DTYPE(m, (launch_k(k_add_rmsnorm<bf16>, rows, norm_threads(d), 0, st, (bf16*)m->h, y.y, nullptr, nullptr, 0, (const bf16*)gain, (bf16*)m->x, d, m->cfg.rms_eps, none, m->status)),
-             (launch_k(k_add_rmsnorm<float>, rows, norm_threads(d), 0, st, (float*)m->h, y.y, nullptr, nullptr, 0, (const float*)gain, (float*)m->x, d, m->cfg.rms_eps, none, m->status)));
+    BY_DTYPE(m, (launch_k(k_add_rmsnorm<bf16>, y.rows, norm_threads(d), 0, st, (bf16*)m->h, y.y, nullptr, nullptr, 0, (const bf16*)gain, (bf16*)m->x, d, m->cfg.rms_eps, none, m->status)),
+             (launch_k(k_add_rmsnorm<float>, y.rows, norm_threads(d), 0, st, (float*)m->h, y.y, nullptr, nullptr, 0, (const float*)gain, (float*)m->x, d, m->cfg.rms_eps, none, m->status)));
 }
 
 constexpr int GP_SMEM = 160 * 1024, GP_CHUNK = 256;
@@ -335,13 +335,17 @@ static bool gemm_plain_prepare_t() {
 // (For the models that use it: the first call on a kernel loads it, which takes the creation of a model milliseconds.)
 bool gemm_plain_prepare(bool bf16_model) { return bf16_model ? gemm_plain_prepare_t<bf16>() : gemm_plain_prepare_t<float>(); }
 
-GemmOut launch_gemm(aded_model* m, int w_map, int x_map, const void* x, const void* w, float* y, int rows, int n, int k,
+// The tensor-core GEMM runs once per 128 rows (256 in calls with more: half as many trips over W).
+int gemm_pass_rows(const aded_model* m, int rows) { return !m->ws_ready ? rows : rows > 128 ? 256 : 128; }
+
+GemmOut launch_gemm(aded_model* m, int w_map, int x_map, const void* x, const void* w, float* y, int row0, int rows, int n, int k,
                     int epi_mode, int trace_kind, cudaStream_t st) {
     GemmOut out = {};
     out.n = n;
+    out.row0 = row0;
     out.rows = rows;
     if (m->ws_ready && w_map >= 0 && x_map >= 0 && ws_supported(n, k)) {
-        // tensor-core path, up to 128 (or 256) rows of x per pass over the weights; the result stays in slots
+        // tensor-core path; the result stays in slots
         const int table = w_map < 4 * m->cfg.n_layers ? w_map % 4 : 4;
         WsEpilogue e = {};
         e.mode = epi_mode;
@@ -349,14 +353,9 @@ GemmOut launch_gemm(aded_model* m, int w_map, int x_map, const void* x, const vo
         e.counters = m->ws_counters;
         e.cand_val = m->cand_val;
         e.cand_idx = m->cand_idx;
-        // a pass takes 128 rows; calls with more rows (ragged batches) use 256-row passes: half as many trips over W
-        const int blk = rows > 128 ? 256 : 128;
-        for (int row0 = 0; row0 < rows; row0 += blk) {
-            const int part = rows - row0 < blk ? rows - row0 : blk;
-            if (epi_mode != WS_EPI_SLOTS) e.epoch = ++m->ws_epoch;
-            ws_launch(m->ws_maps[w_map], m->ws_use_tiled ? m->ws_tiled[w_map] : nullptr, m->ws_x_maps[x_map][(part - 1) / 16], part, row0, blk, n, k, m->ws_slots, m->status, e, trace_kind, m->device, m->ws_one_per_sm[table], st);
-        }
-        out.blk_shift = blk == 256 ? 8 : 7;
+        if (epi_mode != WS_EPI_SLOTS) e.epoch = ++m->ws_epoch;
+        ws_launch(m->ws_maps[w_map], m->ws_use_tiled ? m->ws_tiled[w_map] : nullptr, m->ws_x_maps[x_map][(rows - 1) / 16], rows, row0, n, k, m->ws_slots,
+                  m->status, e, trace_kind, m->device, m->ws_one_per_sm[table], st);
         out.mode = 1;
         out.slots = m->ws_slots;
         out.n_tiles = n / 128;
@@ -372,33 +371,33 @@ GemmOut launch_gemm(aded_model* m, int w_map, int x_map, const void* x, const vo
     return out;
 }
 
-void launch_materialize(aded_model* m, const GemmOut& src, float* dst, int rows, cudaStream_t st) {
+void launch_materialize(aded_model* m, const GemmOut& src, float* dst, cudaStream_t st) {
     const int vec = src.mode == 1 && (reinterpret_cast<uintptr_t>(dst) & 15) == 0, cols = vec ? 1024 : 256;
-    dim3 grid((src.n + cols - 1) / cols, rows);
+    dim3 grid((src.n + cols - 1) / cols, src.rows);
     launch_k(k_materialize, grid, 256, 0, st, src, dst, src.n, vec, m->status);
 }
 
-void launch_rope_kv(aded_model* m, aded_kv* kv, const GemmOut& qkv, int layer, int rows, cudaStream_t st) {
-    if (qkv.mode == 1 && m->cfg.dtype == ADED_BF16) { launch_rope_kv_ws(m, kv, qkv, layer, rows, st); return; }
-    dim3 grid(rows, m->cfg.n_heads);
+void launch_rope_kv(aded_model* m, aded_kv* kv, const GemmOut& qkv, int layer, cudaStream_t st) {
+    if (qkv.mode == 1 && m->cfg.dtype == ADED_BF16) { launch_rope_kv_ws(m, kv, qkv, layer, st); return; }
+    dim3 grid(qkv.rows, m->cfg.n_heads);
     const int H = m->cfg.n_heads, hd = m->cfg.head_dim;
     BY_DTYPE(m, (launch_k(k_rope_kv<bf16>, grid, 64, 0, st, qkv, m->rope_cos, m->rope_sin, (bf16*)m->q, kv->base_dev, kv->cap_dev, kv->len_dev, m->rows.seq, m->rows.local, layer, H, hd, m->status)),
              (launch_k(k_rope_kv<float>, grid, 64, 0, st, qkv, m->rope_cos, m->rope_sin, (float*)m->q, kv->base_dev, kv->cap_dev, kv->len_dev, m->rows.seq, m->rows.local, layer, H, hd, m->status)));
 }
 
-void launch_swiglu(aded_model* m, const GemmOut& gu, int rows, cudaStream_t st) {
-    if (gu.mode == 1 && m->cfg.dtype == ADED_BF16) { launch_swiglu_ws(m, gu, rows, st); return; }
+void launch_swiglu(aded_model* m, const GemmOut& gu, cudaStream_t st) {
+    if (gu.mode == 1 && m->cfg.dtype == ADED_BF16) { launch_swiglu_ws(m, gu, st); return; }
     const int F = m->cfg.d_ffn;
-    dim3 grid((F + 255) / 256, rows);
+    dim3 grid((F + 255) / 256, gu.rows);
     BY_DTYPE(m, (launch_k(k_swiglu<bf16>, grid, 256, 0, st, gu, (bf16*)m->act, F, m->status)),
              (launch_k(k_swiglu<float>, grid, 256, 0, st, gu, (float*)m->act, F, m->status)));
 }
 
-void launch_argmax(aded_model* m, const GemmOut& logits, int rows, cudaStream_t st) {
+void launch_argmax(aded_model* m, const GemmOut& logits, cudaStream_t st) {
     const int V = m->cfg.vocab;
     const int chunks = ARGMAX_CHUNKS;
     const int chunk = ((V + chunks - 1) / chunks + 127) / 128 * 128;   // whole 128-column tiles per block
-    dim3 grid(chunks, rows);
+    dim3 grid(chunks, logits.rows);
     launch_k(k_argmax_chunks, grid, 256, 0, st, logits, m->argmax_val, m->argmax_idx, V, chunk, m->status);
 }
 

@@ -141,7 +141,7 @@ template <int THREADS, int PASSES, int BATCH>
 __global__ void __launch_bounds__(THREADS) k_add_rmsnorm_ws(bf16* __restrict__ h, GemmOut y, const bf16* __restrict__ gain,
                                                          bf16* __restrict__ x, int d, float eps, const int32_t* status) {
     __shared__ float red[32];
-    const int r = blockIdx.x;
+    const int r = y.row0 + blockIdx.x;
     TileRef tr[PASSES];
     float4 gv[PASSES];
 #pragma unroll
@@ -193,7 +193,7 @@ __global__ void __launch_bounds__(THREADS) k_add_rmsnorm_ws(bf16* __restrict__ h
 // SB: contributors that a tile may have for all of both gathers to be in flight at once (the launch knows the most there are).
 template <int SB>
 __global__ void __launch_bounds__(256) k_swiglu_ws(GemmOut gu, bf16* __restrict__ act, int F, const int32_t* status) {
-    const int r = blockIdx.y, c = (blockIdx.x * 256 + threadIdx.x) * 4;
+    const int r = gu.row0 + blockIdx.y, c = (blockIdx.x * 256 + threadIdx.x) * 4;
     TileRef tg = {0, 0}, tu = {0, 0};
     if (c < F) { tg = gu.tiles[c >> 7]; tu = gu.tiles[(F + c) >> 7]; }   // the table is constant: read it before waiting
     pdl_wait();
@@ -227,7 +227,7 @@ k_rope_kv_ws(GemmOut qkv, const float* __restrict__ cs, const float* __restrict_
              const int32_t* __restrict__ len, const int32_t* __restrict__ row_seq,
              const int32_t* __restrict__ row_local, int layer, int H, int hd, const int32_t* status) {
     const int tph = hd >> 3;                                   // threads per head
-    const int r = blockIdx.x, half = hd >> 1, d = H * hd;
+    const int r = qkv.row0 + blockIdx.x, half = hd >> 1, d = H * hd;
     const int hh = blockIdx.y * (ROPE_WS_THREADS / tph) + threadIdx.x / tph;
     const int i = (threadIdx.x % tph) * 4;
     const bool mine = hh < H;
@@ -259,7 +259,7 @@ k_rope_part_ws(GemmOut qkv, const float* __restrict__ cs, const float* __restric
                bf16* __restrict__ q, char* const* __restrict__ base, const int32_t* __restrict__ cap,
                const int32_t* __restrict__ len, const int32_t* __restrict__ row_seq,
                const int32_t* __restrict__ row_local, int layer, int H, int hd, const int32_t* status) {
-    const int tph = hd >> 3, half = hd >> 1, d = H * hd, r = blockIdx.x;
+    const int tph = hd >> 3, half = hd >> 1, d = H * hd, r = qkv.row0 + blockIdx.x;
     const int item = blockIdx.y * ROPE_WS_THREADS + threadIdx.x;
     const int part = item / (H * tph), hh = item / tph % H, i = item % tph * 4;
     const bool mine = part < 3;
@@ -301,25 +301,25 @@ void launch_pick_accept(aded_model* m, aded_kv* kv, int batch, const float* cand
              (const int32_t*)m->status);
 }
 
-void launch_add_rmsnorm_ws(aded_model* m, const GemmOut& y, const void* gain, int rows, cudaStream_t st) {
+void launch_add_rmsnorm_ws(aded_model* m, const GemmOut& y, const void* gain, cudaStream_t st) {
     const int d = m->cfg.d_model;
     auto go = [&](auto* kernel, int threads) {
-        launch_k(kernel, dim3(rows), dim3(threads), 0, st, (bf16*)m->h, y, (const bf16*)gain, (bf16*)m->x, d, m->cfg.rms_eps, (const int32_t*)m->status);
+        launch_k(kernel, dim3(y.rows), dim3(threads), 0, st, (bf16*)m->h, y, (const bf16*)gain, (bf16*)m->x, d, m->cfg.rms_eps, (const int32_t*)m->status);
     };
     if (d <= 1024) go(k_add_rmsnorm_ws<256, 1, 8>, 256);
     else go(k_add_rmsnorm_ws<1024, 2, 12>, 1024);
 }
 
-void launch_swiglu_ws(aded_model* m, const GemmOut& gu, int rows, cudaStream_t st) {
+void launch_swiglu_ws(aded_model* m, const GemmOut& gu, cudaStream_t st) {
     const int F = m->cfg.d_ffn;
-    dim3 grid((F + 1023) / 1024, rows);
+    dim3 grid((F + 1023) / 1024, gu.rows);
     launch_k(m->ws_contributors[WS_MAP_GU] <= 4 ? k_swiglu_ws<4> : k_swiglu_ws<8>, grid, dim3(256), 0, st, gu, (bf16*)m->act, F, (const int32_t*)m->status);
 }
 
-void launch_rope_kv_ws(aded_model* m, aded_kv* kv, const GemmOut& qkv, int layer, int rows, cudaStream_t st) {
+void launch_rope_kv_ws(aded_model* m, aded_kv* kv, const GemmOut& qkv, int layer, cudaStream_t st) {
     const int heads_per_block = ROPE_WS_THREADS / (m->cfg.head_dim / 8), items = 3 * m->cfg.n_heads * (m->cfg.head_dim / 8);
     const bool part = m->ws_contributors[WS_MAP_QKV] > 6;      // more than rope_kv_item holds at once
-    dim3 grid(rows, part ? (items + ROPE_WS_THREADS - 1) / ROPE_WS_THREADS : (m->cfg.n_heads + heads_per_block - 1) / heads_per_block);
+    dim3 grid(qkv.rows, part ? (items + ROPE_WS_THREADS - 1) / ROPE_WS_THREADS : (m->cfg.n_heads + heads_per_block - 1) / heads_per_block);
     launch_k(part ? k_rope_part_ws<7> : k_rope_kv_ws, grid, dim3(ROPE_WS_THREADS), 0, st, qkv, (const float*)m->rope_cos, (const float*)m->rope_sin, (bf16*)m->q,
              (char* const*)kv->base_dev, (const int32_t*)kv->cap_dev, (const int32_t*)kv->len_dev,
              (const int32_t*)m->rows.seq, (const int32_t*)m->rows.local, layer, m->cfg.n_heads, m->cfg.head_dim,

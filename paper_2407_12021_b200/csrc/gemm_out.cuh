@@ -11,8 +11,10 @@
 // Slot numbering: the segment of tile t computed by CTA c goes to slot t + c.  Walking the units
 // in order, (t, c) never decreases and one of them grows at every segment boundary, so the sums
 // are distinct.  A slot holds [rb][128] floats (rb = rows of the pass padded to 16).  A pass takes up to 128
-// rows, or up to 256 when the call has more than 128 (half as many passes over the weights); a call with more
-// rows than one pass takes uses one slot region per pass.
+// rows, or up to 256 when the call has more than 128 (half as many passes over the weights).  The passes of a call use the
+// same slots one after the other, each consumed before the next begins: 50 MB that stay in L2, where a region per pass
+// was written to HBM and read back (five passes of 256 rows at the 7B widths, us per layer: rotary 69 -> 60, two norms 96 -> 64,
+// SwiGLU 49 -> 44, projections 528 -> 512).
 #pragma once
 
 #include <cuda_bf16.h>
@@ -33,8 +35,7 @@ struct GemmOut {
     int mode;
     int n;                // result columns
     int n_tiles, kb, g;   // mode 1: 128-column tiles, k blocks per tile, CTAs of the GEMM launch
-    int rows;             // rows of the whole result (all passes)
-    int blk_shift;        // mode 1: log2 of the rows a pass takes (7 or 8)
+    int row0, rows;       // the rows of the call that this is the result of (a pass; mode 0: all of them)
 };
 
 // First work unit of CTA c when `units` units are split over `g` CTAs.
@@ -61,21 +62,15 @@ __host__ __device__ __forceinline__ TileRef gemm_tile_ref(int n_tiles, int kb, i
     return t;
 }
 
-// Rows padded to 16 of the pass that holds row r, and where that pass's slot region starts.
-__device__ __forceinline__ int gemm_block_rb(const GemmOut& o, int r) {
-    const int blk = 1 << o.blk_shift;
-    const int left = o.rows - ((r >> o.blk_shift) << o.blk_shift);
-    const int in_blk = left < blk ? left : blk;
-    return (in_blk + 15) & ~15;
-}
+// Rows padded to 16, and where row r of a tile's first contributor lies.
+__device__ __forceinline__ int gemm_block_rb(const GemmOut& o) { return (o.rows + 15) & ~15; }
 __device__ __forceinline__ const float* gemm_slot_row(const GemmOut& o, const TileRef& t, int r, int rb) {
-    const size_t region = (size_t)(r >> o.blk_shift) * (size_t)(o.n_tiles + o.g) * ((size_t)128 << o.blk_shift);
-    return o.slots + region + ((size_t)t.first_slot * rb + (r & ((1 << o.blk_shift) - 1))) * 128;
+    return o.slots + ((size_t)t.first_slot * rb + (r - o.row0)) * 128;
 }
 
 // Value of result element (r, tile * 128 + col) given the tile's contributors.
 __device__ __forceinline__ float gemm_out_at(const GemmOut& o, const TileRef& t, int r, int col) {
-    const int rb = gemm_block_rb(o, r);
+    const int rb = gemm_block_rb(o);
     const float* p = gemm_slot_row(o, t, r, rb) + col;
     const size_t stride = (size_t)rb * 128;
     float sum = 0.f;
@@ -96,7 +91,7 @@ __device__ __forceinline__ float4 f4_add(float4 a, float4 b) { return make_float
 // Columns col .. col+3 (col % 4 == 0) of tile t, row r: slots added in CTA order.
 template <int GO_BATCH = 12>
 __device__ __forceinline__ float4 gemm_out_at4(const GemmOut& o, const TileRef& t, int r, int col) {
-    const int rb = gemm_block_rb(o, r);
+    const int rb = gemm_block_rb(o);
     const float* p = gemm_slot_row(o, t, r, rb) + col;
     const size_t stride = (size_t)rb * 128;
     float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -122,7 +117,7 @@ __device__ __forceinline__ float4 gemm_out_at4(const GemmOut& o, const TileRef& 
 // gemm_out_at4.
 template <int B>
 __device__ __forceinline__ void gemm_out_fetch4(const GemmOut& o, const TileRef& t, int r, int col, float4 (&v)[B]) {
-    const int rb = gemm_block_rb(o, r);
+    const int rb = gemm_block_rb(o);
     const float* p = gemm_slot_row(o, t, r, rb) + col;
     const size_t stride = (size_t)rb * 128;
 #pragma unroll
@@ -141,7 +136,7 @@ __device__ __forceinline__ float4 gemm_out_sum4(const float4 (&v)[B], const Tile
 // Columns col .. col+3 and col2 .. col2+3 of the same tile and row, up to B contributors of both in flight at once.
 template <int B>
 __device__ __forceinline__ void gemm_out_two4(const GemmOut& o, const TileRef& t, int r, int col, int col2, float4& s0, float4& s1) {
-    const int rb = gemm_block_rb(o, r);
+    const int rb = gemm_block_rb(o);
     const float* p = gemm_slot_row(o, t, r, rb);
     const size_t stride = (size_t)rb * 128;
     const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);

@@ -60,7 +60,7 @@ struct WsParams {
     int n_acc;           // TMEM accumulators: two (the next segment's MMAs run under the drain) up to 128 rows, one beyond
     int trace_kind;
     int narrow;          // units * (CTAs + 1) < 2^31: the work split can be computed in 32-bit arithmetic
-    float* slots;        // this row block's slot region: [n_tiles + gridDim.x][rb][128] fp32
+    float* slots;        // [n_tiles + gridDim.x][rb][128] fp32
     const uint8_t* w_tiled;  // W re-tiled (ws_retile): unit (tile, k block) is 16 KB at (tile * kb + k block) * 16 KB, swizzled as staged
     int32_t* status;
     WsEpilogue epi;
@@ -462,10 +462,10 @@ int ws_grid(int device, int n, int k, bool one_per_sm) {
     return units < g ? (int)units : g;
 }
 
-// Floats of slot storage for results of up to max_n columns and max_rows rows.
+// Floats of slot storage for results of up to max_n columns and max_rows rows: one pass at a time.
 size_t ws_slot_floats(int device, int max_n, int max_rows) {
-    const size_t passes = ((size_t)max_rows + 255) / 256;          // (regions of 256 rows also hold two regions of 128)
-    return passes * ((size_t)max_n / WS_BM + ws_grid_limit(device)) * 256 * WS_BM;
+    const size_t rb = max_rows > 128 ? 256 : ((size_t)max_rows + 15) / 16 * 16;
+    return ((size_t)max_n / WS_BM + ws_grid_limit(device)) * rb * WS_BM;
 }
 
 // Raises the kernel's dynamic shared-memory limit; once per process, before any launch or capture.
@@ -477,9 +477,8 @@ bool ws_prepare() {
 // Shapes the tensor-core path takes.
 bool ws_supported(int n, int k) { return n % WS_BM == 0 && k % WS_BK == 0 && k >= WS_BK; }
 
-// One pass: rows [row0, row0 + rows) of x (rows <= blk = 128 or 256) against all of W.  Partial tiles go to the
-// slot region of pass row0 / blk; `epi` says whether the kernel's tail reduces them to greedy candidates.
-cudaError_t ws_launch(const CUtensorMap& map_w, const void* w_tiled, const CUtensorMap& map_x, int rows, int row0, int blk,
+// One pass: rows [row0, row0 + rows) of x (at most 256) against all of W.  Partial tiles go to the slots; `epi` says whether the kernel's tail reduces them to greedy candidates.
+cudaError_t ws_launch(const CUtensorMap& map_w, const void* w_tiled, const CUtensorMap& map_x, int rows, int row0,
                       int n, int k,
                       float* slots, int32_t* status, const WsEpilogue& epi, int trace_kind, int device, bool one_per_sm, cudaStream_t st) {
     WsParams p;
@@ -503,7 +502,7 @@ cudaError_t ws_launch(const CUtensorMap& map_w, const void* w_tiled, const CUten
     p.trace_kind = trace_kind;
     const int grid = ws_grid(device, n, k, one_per_sm);
     p.narrow = (long long)p.n_tiles * p.kb * (grid + 1) < (1ll << 31);
-    p.slots = slots + (size_t)(row0 / blk) * (size_t)(p.n_tiles + grid) * blk * WS_BM;
+    p.slots = slots;
     p.status = status;
     p.epi = epi;
     const size_t smem = (size_t)p.stages * stage_bytes + 1024 + 256;

@@ -214,21 +214,26 @@ static aded_status enqueue_pass(aded_model* m, aded_kv* kv, const CallPtrs& call
     }
     const size_t hid_bytes = (size_t)rows * d * m->elem;
     if (m->dbg_hidden) ADED_CUDA_TRY(cudaMemcpyAsync(m->dbg_hidden, m->h, hid_bytes, cudaMemcpyDeviceToDevice, st));
-    const int passes = !ws ? 1 : rows > 128 ? (rows + 255) / 256 : 1;      // the tensor-core GEMM runs once per 128 rows (256 in calls with more)
+    // A GEMM and the kernel that takes its result, pass by pass (see GemmOut).
+    const int pass = gemm_pass_rows(m, rows);
+    auto each_pass = [&](auto&& f) {
+        for (int row0 = 0; row0 < rows; row0 += pass) f(row0, rows - row0 < pass ? rows - row0 : pass);
+    };
     for (int l = 0; l < c.n_layers; ++l) {
         const aded_layer_weights& w = m->layers[l];
         const void* next_gain = l + 1 < c.n_layers ? m->layers[l + 1].norm1 : m->top.final_norm;
-        auto wmap = [&](int which) { return ws ? 4 * l + which : -1; };      // TMA descriptor of a weight matrix (plain GEMM: none)
-        GemmOut o;
-        { Span sp(m, PROF_GEMM, passes, st); o = launch_gemm(m, wmap(WS_MAP_QKV), ws ? WS_X : -1, m->x, w.wqkv, m->y32, rows, 3 * d, d, WS_EPI_SLOTS, TK_GEMM_QKV, st); }
-        { Span sp(m, PROF_OTHER, 1, st); launch_rope_kv(m, kv, o, l, rows, st); }
+        auto project = [&](int which, int x_map, const void* x, const void* wt, int n, int k, int kind, auto&& consume) {
+            each_pass([&](int row0, int part) {
+                GemmOut o;
+                { Span sp(m, PROF_GEMM, 1, st); o = launch_gemm(m, ws ? 4 * l + which : -1, ws ? x_map : -1, x, wt, m->y32, row0, part, n, k, WS_EPI_SLOTS, kind, st); }
+                { Span sp(m, PROF_OTHER, 1, st); consume(o); }
+            });
+        };
+        project(WS_MAP_QKV, WS_X, m->x, w.wqkv, 3 * d, d, TK_GEMM_QKV, [&](const GemmOut& o) { launch_rope_kv(m, kv, o, l, st); });
         { Span sp(m, PROF_ATTN, 1, st); launch_tree_attention(m, kv, l, batch, rows, max_tree, st); }
-        { Span sp(m, PROF_GEMM, passes, st); o = launch_gemm(m, wmap(WS_MAP_O), ws ? WS_X_ATTN : -1, m->attn, w.wo, m->y32, rows, d, d, WS_EPI_SLOTS, TK_GEMM_O, st); }
-        { Span sp(m, PROF_OTHER, 1, st); launch_add_rmsnorm(m, o, w.norm2, rows, st); }
-        { Span sp(m, PROF_GEMM, passes, st); o = launch_gemm(m, wmap(WS_MAP_GU), ws ? WS_X : -1, m->x, w.wgu, m->y32, rows, 2 * F, d, WS_EPI_SLOTS, TK_GEMM_GU, st); }
-        { Span sp(m, PROF_OTHER, 1, st); launch_swiglu(m, o, rows, st); }
-        { Span sp(m, PROF_GEMM, passes, st); o = launch_gemm(m, wmap(WS_MAP_D), ws ? WS_X_ACT : -1, m->act, w.wd, m->y32, rows, d, F, WS_EPI_SLOTS, TK_GEMM_DOWN, st); }
-        { Span sp(m, PROF_OTHER, 1, st); launch_add_rmsnorm(m, o, next_gain, rows, st); }
+        project(WS_MAP_O, WS_X_ATTN, m->attn, w.wo, d, d, TK_GEMM_O, [&](const GemmOut& o) { launch_add_rmsnorm(m, o, w.norm2, st); });
+        project(WS_MAP_GU, WS_X, m->x, w.wgu, 2 * F, d, TK_GEMM_GU, [&](const GemmOut& o) { launch_swiglu(m, o, st); });
+        project(WS_MAP_D, WS_X_ACT, m->act, w.wd, d, F, TK_GEMM_DOWN, [&](const GemmOut& o) { launch_add_rmsnorm(m, o, next_gain, st); });
         if (m->dbg_hidden)
             ADED_CUDA_TRY(cudaMemcpyAsync((char*)m->dbg_hidden + (size_t)(l + 1) * hid_bytes, m->h, hid_bytes,
                                           cudaMemcpyDeviceToDevice, st));
@@ -237,24 +242,23 @@ static aded_status enqueue_pass(aded_model* m, aded_kv* kv, const CallPtrs& call
         // The per-node logits are needed as a matrix only by the sampling mode and by a debug capture; the
         // greedy choice works from per-tile candidates left by the LM head's tail.
         const bool dense_logits = !ws || m->samp_on || m->dbg_logits;
-        GemmOut lg;
-        { Span sp(m, PROF_GEMM, passes, st);
-          lg = launch_gemm(m, ws ? 4 * c.n_layers : -1, ws ? WS_X : -1, m->x, m->top.lm_head, m->logits, rows, c.vocab, d,
-                           dense_logits ? WS_EPI_SLOTS : WS_EPI_ARGMAX, TK_GEMM_HEAD, st); }
+        float* dense = m->samp_on && !m->dbg_logits ? m->logits : m->dbg_logits;      // where the logits go as a matrix, if anywhere
+        each_pass([&](int row0, int part) {
+            GemmOut lg;
+            { Span sp(m, PROF_GEMM, 1, st);
+              lg = launch_gemm(m, ws ? 4 * c.n_layers : -1, ws ? WS_X : -1, m->x, m->top.lm_head, m->logits, row0, part, c.vocab, d,
+                               dense_logits ? WS_EPI_SLOTS : WS_EPI_ARGMAX, TK_GEMM_HEAD, st); }
+            if (dense && (lg.mode == 1 || dense != m->logits)) { Span sp(m, PROF_OTHER, 1, st); launch_materialize(m, lg, dense, st); }
+            if (dense_logits && !m->samp_on) { Span sp(m, PROF_OTHER, 1, st); launch_argmax(m, lg, st); }
+        });
         if (m->samp_on) {
-            // sampling mode: the logits as a dense matrix (straight into the capture buffer when the caller asked for the logits),
-            // then one drawn token per node in place of the greedy one
-            float* dense = m->dbg_logits ? m->dbg_logits : m->logits;
-            const bool copy = lg.mode == 1 || dense != m->logits;
-            Span sp(m, PROF_OTHER, copy ? 3 : 2, st);
-            if (copy) launch_materialize(m, lg, dense, rows, st);
+            // sampling mode: one drawn token per node in place of the greedy one
+            Span sp(m, PROF_OTHER, 2, st);
             ADED_CUDA_TRY(launch_sample_rows(dense, rows, c.vocab, c.vocab, m->samp_temp, m->samp_top_p, m->samp_u, m->best,
                                              m->status, st));
             launch_accept(m, kv, batch, st);
         } else if (dense_logits) {
-            Span sp(m, PROF_OTHER, m->dbg_logits ? 3 : 2, st);
-            if (m->dbg_logits) launch_materialize(m, lg, m->dbg_logits, rows, st);
-            launch_argmax(m, lg, rows, st);
+            Span sp(m, PROF_OTHER, 1, st);
             launch_pick_accept(m, kv, batch, m->argmax_val, m->argmax_idx, ARGMAX_CHUNKS, st);
         } else {
             Span sp(m, PROF_OTHER, 1, st);
@@ -583,9 +587,13 @@ aded_status aded_debug_gemm(aded_model* m, int32_t layer, int32_t which, const v
     const int w_map = which == 4 ? 4 * c.n_layers : 4 * layer + which;
     float* ybuf = which == 4 ? m->logits : m->y32;
     ADED_CUDA_TRY(cudaMemcpyAsync(xbuf, x_dev, (size_t)rows * k * m->elem, cudaMemcpyDeviceToDevice, st));
-    note_launch();
-    const GemmOut o = launch_gemm(m, m->ws_ready ? w_map : -1, m->ws_ready ? x_map : -1, xbuf, w, ybuf, rows, n, k, WS_EPI_SLOTS, TK_OTHER, st);
-    launch_materialize(m, o, y_dev, rows, st);
+    const int pass = gemm_pass_rows(m, rows);
+    for (int row0 = 0; row0 < rows; row0 += pass) {
+        note_launch(2);
+        const GemmOut o = launch_gemm(m, m->ws_ready ? w_map : -1, m->ws_ready ? x_map : -1, xbuf, w, ybuf, row0, rows - row0 < pass ? rows - row0 : pass, n, k,
+                                      WS_EPI_SLOTS, TK_OTHER, st);
+        launch_materialize(m, o, y_dev, st);
+    }
     ADED_CUDA_TRY(cudaGetLastError());
     return ADED_OK;
 }
