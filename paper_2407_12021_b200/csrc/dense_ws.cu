@@ -251,8 +251,8 @@ k_rope_kv_ws(GemmOut qkv, const float* __restrict__ cs, const float* __restrict_
 
 // The same with a thread per (q, k or v; four pairs) instead of one for all three: for projections whose tiles have so many
 // contributors that a thread cannot hold all three gathers (small widths, where the GEMM's units are spread over all SMs: up to 14 at
-// width 1024: rotary + attention 20.9 us per layer there with k_rope_kv_ws, 17.4 with this and 7 in flight, 18.0 with 14).  At the 7B
-// widths it gains as much as the attention kernel behind it loses.
+// width 1024: 12.1 us per layer there with k_rope_kv_ws, 4.7 with this; 4.5 with 14 in flight instead of 7).  At the 7B widths it
+// gains as much as the attention kernel behind it loses.
 template <int B>
 __global__ void __launch_bounds__(ROPE_WS_THREADS)
 k_rope_part_ws(GemmOut qkv, const float* __restrict__ cs, const float* __restrict__ sn,

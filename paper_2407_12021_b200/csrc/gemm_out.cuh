@@ -139,15 +139,16 @@ __device__ __forceinline__ void gemm_out_two4(const GemmOut& o, const TileRef& t
     const int rb = gemm_block_rb(o);
     const float* p = gemm_slot_row(o, t, r, rb);
     const size_t stride = (size_t)rb * 128;
-    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-    s0 = zero;
-    s1 = zero;
+    s0 = make_float4(0.f, 0.f, 0.f, 0.f);
+    s1 = s0;
     for (int i0 = 0; i0 < t.count; i0 += B) {
+        // (a slot past the last contributor is the last one's again and not added: loads without predicates stay together)
         float4 v0[B], v1[B];
 #pragma unroll
         for (int j = 0; j < B; ++j) {
-            v0[j] = i0 + j < t.count ? __ldcg(reinterpret_cast<const float4*>(p + (size_t)(i0 + j) * stride + col)) : zero;
-            v1[j] = i0 + j < t.count ? __ldcg(reinterpret_cast<const float4*>(p + (size_t)(i0 + j) * stride + col2)) : zero;
+            const float* from = p + (size_t)(i0 + j < t.count ? i0 + j : t.count - 1) * stride;
+            v0[j] = __ldcg(reinterpret_cast<const float4*>(from + col));
+            v1[j] = __ldcg(reinterpret_cast<const float4*>(from + col2));
         }
 #pragma unroll
         for (int j = 0; j < B; ++j)

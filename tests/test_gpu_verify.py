@@ -540,3 +540,10 @@ def test_attention_with_every_number_of_splits(cuda_device, heads, nodes, ctx):
     p = torch.softmax(s.masked_fill(~mask[:, None, :], float("-inf")), dim=-1)
     want = torch.einsum("thl,hld->thd", p, vv)
     assert float((att - want).abs().max()) <= 2e-2 * float(want.abs().max())
+
+
+@pytest.mark.parametrize("heads,hd,nodes,depth,ctx", [(16, 64, 45, 6, 77), (8, 64, 128, 8, 130), (8, 128, 33, 4, 65)])
+def test_bf16_widths_with_many_contributors(cuda_device, heads, hd, nodes, depth, ctx):
+    """Widths of 512 and 1024: a tile of a projection is spread over 8 to 19 CTAs, and the kernels that gather the parts take them in
+    more than one round (rotary: a thread per q, k or v)."""
+    test_bf16_small_models_tree_shapes(cuda_device, heads, hd, nodes, depth, ctx)
