@@ -180,6 +180,9 @@ k_gemm_ws(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
 
     if (warp == 0) {
         // ---------------- TMA producer ----------------
+        // A CTA with nothing to do (the pass has failed, or the launch has more CTAs than units) still waits for the previous kernel:
+        // the next kernel waits for this one alone, and would otherwise run beside whatever precedes it on the stream.
+        if (lane == 0 && !live) pdl_wait();
         if (lane == 0 && live) {
             asm volatile("prefetch.tensormap [%0];" ::"l"(&map_w) : "memory");
             asm volatile("prefetch.tensormap [%0];" ::"l"(&map_x) : "memory");

@@ -387,6 +387,58 @@ def test_bounded_wait_runs_out_and_the_handle_recovers(cuda_device, which):
     assert again["status"] == 0 and again["out_tokens"] == good["out_tokens"] and sess.length() == 69 + good["accept_len"]
 
 
+@pytest.mark.parametrize("step", ["mcts", "draft"])
+@pytest.mark.parametrize("error", ["append", "wait"])
+def test_decoding_step_submitted_while_an_error_is_pending_changes_nothing(cuda_device, step, error):
+    """A step behind a failed call, without a synchronisation between them: accept length 0, no token, and cache, table and
+    context as they were -- although its search (hundreds of microseconds) runs far longer than the kernels of the failed
+    pass, which do nothing.  One layer: few kernels between the search and the approval.  Afterwards the handles work."""
+    from paper_2407_12021_b200 import binding as B
+    shape = gen.ModelShape("bf16-4x128", 1, 512, 4, 128, 1024, 1024, "bf16")
+    sess = H.GpuSession(shape, H.weights_to(gen.model_weights(shape, 93), cuda_device), capacity=512)
+    corpus = gen.zipf_tokens(20000, shape.vocab, 93, 1)
+    prompt = corpus[:70].tolist()
+    sess.append(prompt[:-1])
+    table = B.aded_trigram_create(shape.vocab, log2_buckets=15, overflow_buckets=1 << 13)
+    B.aded_trigram_update(table, corpus.cuda())
+    nodes, iters, length, candidates, k = 49, 150, 4, 12, 4
+    filler = gen.zipf_tokens(512, shape.vocab, 94, 1).cuda()
+    u = torch.tensor(gen.uniform01(iters * length, 94, 2).numpy().astype(np.float32), device="cuda")
+
+    def run(context):
+        out, n = torch.full((nodes,), -7, dtype=torch.int32, device="cuda"), torch.full((1,), 5, dtype=torch.int32, device="cuda")
+        if step == "mcts":
+            B.aded_decode_step_mcts(sess.model, sess.kv, table, context, nodes, iters, length, candidates, k, u, filler, out, n)
+        else:
+            B.aded_decode_step(sess.model, sess.kv, table, context, nodes, length, k, filler, out, n)
+        return out, n
+
+    def entries():
+        keys, counts = B.aded_trigram_export(table)
+        return sorted(zip(map(tuple, keys.tolist()), counts.tolist()))
+
+    first = H.i32(prompt[-2:])
+    out, n = run(first)                         # (the record of a call that worked is what a mix-up would act on)
+    assert int(n[0]) >= 1 and B.aded_model_poll_status(sess.model) == 0
+    before, length_before, earlier = entries(), sess.length(), (out.tolist(), int(n[0]))
+    context = first.clone()
+    bad = H.i32([shape.vocab, 1, 2])            # a token outside the vocabulary
+    for _ in range(3):
+        if error == "append":
+            B.aded_append(sess.model, sess.kv, bad)
+        else:
+            B.aded_debug_wait_timeout(sess.model, 0, 100_000)
+        out2, n2 = run(context)
+        torch.cuda.synchronize()
+        assert int(n2[0]) == 0 and out2.tolist() == [-7] * nodes
+        assert torch.equal(context, first) and (out.tolist(), int(n[0])) == earlier
+        assert sess.length() == length_before and entries() == before
+        assert B.aded_model_poll_status(sess.model) == (1 if error == "append" else 8)
+        assert B.aded_trigram_poll_status(table) == 0
+    out2, n2 = run(context)
+    assert int(n2[0]) >= 1 and B.aded_model_poll_status(sess.model) == 0 and sess.length() == length_before + int(n2[0])
+
+
 def test_debug_build_runs_the_small_workloads_without_an_index_complaint(cuda_device):
     """The debug build (-DADED_DEBUG_CHECKS: index checks on slot, cache-row and bucket addressing that report
     ADED_ERR_INTERNAL through the status word; the stand-in for a memory checker) runs the fp32 workload, a
