@@ -43,8 +43,10 @@ template <> __device__ __forceinline__ bf16 from_f32<bf16>(float v) { return __f
 // pdl_enter(): it lets the next kernel of the stream start launching at once (its blocks become
 // resident and run their own preamble) and then waits until the previous kernel has finished and
 // its writes are visible.  Nothing may be read from or written to global memory that another kernel
-// of the pass touches before pdl_wait() -- the weight-streaming GEMM alone does work before it: it
-// prefetches weights, which no kernel writes.
+// of the pass touches before pdl_wait().  Done before it: weights, gains and contributor tables, which no kernel
+// writes, and the bf16 attention kernels' first blocks of committed keys and values (attn_sequence says why they may).
+// Every block waits, also one that has nothing to do: a kernel waits for the one before it alone, so that a launch none of
+// whose blocks waited would let the next kernel run beside whatever came earlier on the stream.
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_enter() { pdl_launch_dependents(); pdl_wait(); }
@@ -177,8 +179,15 @@ __device__ __forceinline__ void approval_warp(int lane, const int32_t* s_par, co
     }
 }
 
-// Sequence of the attention kernels' blockIdx.z: z / row_blocks-th in order of work.  (Before the dependency wait the array may
-// hold another call's order: kept in range, and looked at again after the wait.)
+// The bf16 attention kernels read before their dependency wait: this order, a sequence's committed length and tree size, and the first
+// blocks of committed keys and values.  What a failed pass or another call has left there is caught by reading order, length and
+// size again after the wait.  Rows BELOW the length that was read have to be final by then: the approval of a pass
+// publishes the new length before the compaction behind it has moved the rows.  So the kernels that launch right before
+// attention (rotary and K/V write) release it only after their own wait: when a block of attention starts, every earlier
+// kernel on the stream, compaction included, has finished.  (Released at the top of that kernel, a small model whose
+// projections do the same would have the whole chain from approval to attention resident at once.)
+//
+// Sequence of blockIdx.z: z / row_blocks-th in order of work, kept in range.
 __device__ __forceinline__ int attn_sequence(const int32_t* order, int z, int row_blocks, int batch) {
     const int place = z / row_blocks;
     return order ? min(max(__ldcg(order + place), 0), batch - 1) : place;

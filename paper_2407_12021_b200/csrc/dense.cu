@@ -171,12 +171,15 @@ __global__ void __launch_bounds__(GP_THREADS) k_gemm_plain(const T* __restrict__
 
 // Rotary embedding of q and k (pairs (i, i + hd/2), angle from the table), then q -> q buffer and
 // k, v -> the cache at slot committed length + local node index.  Block = (row, head).
+// bf16 models release the next kernel only after this one's wait: see attn_sequence (fp32 attention reads nothing early).
 template <typename T>
 __global__ void k_rope_kv(GemmOut qkv, const float* __restrict__ cs, const float* __restrict__ sn,
                           T* __restrict__ q, char* const* __restrict__ base, const int32_t* __restrict__ cap,
                           const int32_t* __restrict__ len, const int32_t* __restrict__ row_seq,
                           const int32_t* __restrict__ row_local, int layer, int H, int hd, const int32_t* status) {
-    pdl_enter();
+    if (sizeof(T) == 4) pdl_launch_dependents();
+    pdl_wait();
+    if (sizeof(T) != 4) pdl_launch_dependents();
     if (first_thread_of_grid()) trace_mark(status, TK_ROPE);
     if (*status != 0) return;
     const int r = blockIdx.x, hh = blockIdx.y, half = hd >> 1, d = H * hd;

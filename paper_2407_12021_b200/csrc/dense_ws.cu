@@ -220,6 +220,7 @@ __global__ void __launch_bounds__(256) k_swiglu_ws(GemmOut gu, bf16* __restrict_
 // Rotary embedding + K/V write (see k_rope_kv): hd/8 threads per (row, head), each owning four adjacent
 // rotary pairs (i .. i+3, i+half .. i+half+3); a block of ROPE_WS_THREADS threads takes consecutive heads
 // of one row, so its warps are full and a pass is a few hundred blocks instead of rows x heads tiny ones.
+// The attention kernel behind it must not be released before the wait: see attn_sequence.
 constexpr int ROPE_WS_THREADS = 128;
 __global__ void __launch_bounds__(ROPE_WS_THREADS)
 k_rope_kv_ws(GemmOut qkv, const float* __restrict__ cs, const float* __restrict__ sn,
@@ -252,7 +253,7 @@ k_rope_kv_ws(GemmOut qkv, const float* __restrict__ cs, const float* __restrict_
 // The same with a thread per (q, k or v; four pairs) instead of one for all three: for projections whose tiles have so many
 // contributors that a thread cannot hold all three gathers (small widths, where the GEMM's units are spread over all SMs: up to 14 at
 // width 1024: 12.1 us per layer there with k_rope_kv_ws, 4.7 with this; 4.5 with 14 in flight instead of 7).  At the 7B widths it
-// gains as much as the attention kernel behind it loses.
+// gains as much as the attention kernel behind it loses.  (Released after the wait, as k_rope_kv_ws.)
 template <int B>
 __global__ void __launch_bounds__(ROPE_WS_THREADS)
 k_rope_part_ws(GemmOut qkv, const float* __restrict__ cs, const float* __restrict__ sn,

@@ -210,7 +210,7 @@ k_tree_attn_tc(const __grid_constant__ CUtensorMap map_q, AttnTcArgs a) {
     pdl_launch_dependents();
     // While the previous kernel (which writes q and the tree's own K/V rows) is still running, the
     // producer already fetches this CTA's first two key blocks into their stages, if they lie entirely in
-    // the committed part of the cache (which no kernel of the pass writes), and asks L2 for the others.
+    // the committed part of the cache (final by now: attn_sequence), and asks L2 for the others.
     // The committed length and the tree size are read on trust here; both are read again after the wait
     // and the early blocks are used only if the two reads agree, otherwise they are fetched again.
     int n_pre = 0, pre_L = -1, pre_T = -1, pre_b = 0;

@@ -387,6 +387,53 @@ def test_bounded_wait_runs_out_and_the_handle_recovers(cuda_device, which):
     assert again["status"] == 0 and again["out_tokens"] == good["out_tokens"] and sess.length() == 69 + good["accept_len"]
 
 
+@pytest.mark.parametrize("hd,vocab", [(64, 1000), (128, 1000), (64, 1024), (128, 1024)])
+def test_steps_behind_one_another_without_a_synchronisation(cuda_device, hd, vocab):
+    """Steps that accept scattered paths, submitted without waiting (and with nothing else on the stream between them), against the
+    same steps with a synchronisation after each: emitted tokens, lengths and the whole cache of two layers -- the second's keys
+    and values come from the first's attention -- bit for bit.  The attention kernels fetch committed rows before their
+    dependency wait, and the accepted rows of the step before only reach their places after its length is published.
+    Vocabulary 1000: projections without the tensor-core kernel; both attention kernels."""
+    from paper_2407_12021_b200 import binding as B
+    d, steps, depth, ctx = 2 * hd, 40, 7, 70
+    shape = gen.ModelShape("bf16-small", 2, d, 2, hd, 256, vocab, "bf16")
+    w = H.weights_to(gen.model_weights(shape, 98), cuda_device)
+    prompt = gen.zipf_tokens(ctx, vocab, 98, 50).tolist()
+    probe = H.GpuSession(shape, w, capacity=ctx + steps * (depth + 1) + 200)
+    probe.append(prompt[:-1])
+    text = [prompt[-1]]
+    for _ in range(steps * (depth + 1)):
+        text.append(probe.verify([text[-1]], [-1], capture=False)["out_tokens"][0])
+    trees, at = [], 0
+    for _ in range(steps):                      # every path node comes after a stray sibling: the accepted rows 0, 2, 4, .. move
+        tokens, parents, last = [text[at]], [-1], 0
+        for j in range(1, depth + 1):
+            tokens += [(text[at + j] + 1) % vocab, text[at + j]]
+            parents += [last, last]
+            last = len(tokens) - 1
+        trees.append((H.i32(tokens), H.i32(parents)))
+        at += depth + 1
+    n = 2 * depth + 1
+
+    def run(wait):
+        sess = H.GpuSession(shape, w, capacity=ctx + steps * (depth + 1) + 200)
+        sess.append(prompt[:-1])
+        torch.cuda.synchronize()
+        out, acc = (torch.zeros((steps, m), dtype=torch.int32, device="cuda") for m in (n, 1))
+        for i, (tokens, parents) in enumerate(trees):
+            B.aded_verify(sess.model, sess.kv, tokens, parents, out[i], acc[i])
+            if wait:
+                torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        assert B.aded_model_poll_status(sess.model) == 0
+        return [out, acc] + [x for layer in range(2) for x in B.aded_kv_read(sess.kv, 0, layer, 0, sess.length())]
+
+    want = run(True)
+    assert int((want[1] > 2).sum()) > steps // 2, "few steps accept a path"
+    for _ in range(5):
+        assert all(torch.equal(a, b) for a, b in zip(run(False), want))
+
+
 @pytest.mark.parametrize("step", ["mcts", "draft"])
 @pytest.mark.parametrize("error", ["append", "wait"])
 def test_decoding_step_submitted_while_an_error_is_pending_changes_nothing(cuda_device, step, error):
