@@ -6,19 +6,24 @@
 //     context's further entries are;
 //   * a pool of (token, count) entries in units of six (48 bytes).  A context's entries beyond six lie in extents of
 //     1, 2, 4, ... units, each contiguous, handed out by a bump allocator when the extent before is full; the first
-//     extent starts with a directory of the others.  Every entry of a context, however many there are, is therefore two
-//     dependent reads behind its home bucket, and a lookup reads them with coalesced 16-byte loads that are all
-//     independent.  (Chains of single buckets, as before, cost one dependent read per six entries: a lookup of a
-//     frequent context -- thousands of continuations -- was a chain of hundreds to thousands of memory round trips.)
+//     extent starts with a directory: where the others are, and how many units the context has been given.  Every
+//     entry of a context, however many there are, is therefore two dependent reads behind its home bucket, and a lookup
+//     reads them with coalesced 16-byte loads that are all independent.  (Chains of single buckets, as before, cost
+//     one dependent read per six entries: a lookup of a frequent context -- thousands of continuations -- was a chain of
+//     hundreds to thousands of memory round trips.)
 //   * an index over the pool entries: (home bucket, token) -> entry, open addressing, at most three quarters full.
 //     Raising a count is one probe of the home buckets, one of the index and one atomic add, wherever the entry is.
-//     Measured, 10^6 tokens into an empty table: 0.29 ms (13.6 ms with chains that every insertion walked from the front);
+//     Measured, 10^6 tokens into an empty table: 0.30 ms (13.6 ms with chains that every insertion walked from the front);
 //     lookups: see k_tg_topk and k_topk_mark; a 64-node draft tree from that table 32 us (490).
 //
-// Entries are never moved or removed.  The configured number of overflow buckets limits units of six entries in use
-// exactly as it limited chain buckets; the pool has room for the unused ends of the extents on top (a context with d units
-// takes at most 3 d).
+// Entries are never moved or removed.  The configured number of overflow buckets limits the units of six entries in use: as long
+// as one is left any context can grow by it, and a unit that was given out can be filled.  The pool has room for the unused ends
+// of the extents on top: a context opens extent s only once it has been given 2^s units, so that with d units it takes
+// 2 + 1 + 2 + 4 + .. <= 3 d.  (What waiting for that costs: 20,000 tokens into an empty table 32 -> 36 us, 10^6 0.30 -> 0.31 ms, 4 x 10^6 no
+// difference, against extents that were opened on a thread's own unit alone, with which a table at its limit could exceed its pool.)
 #pragma once
+
+#include <cstddef>
 
 #include "aded_internal.cuh"
 
@@ -42,9 +47,11 @@ constexpr int TG_MAX_PROBE = 4096;
 constexpr uint32_t TG_FAILED = 0xFFFFFFFFu, TG_CLOSED = 0x80000000u;
 constexpr int TG_MAX_SPIN = 1 << 20;
 constexpr int TG_UNIT = 6;            // entries of a pool unit
-constexpr int TG_LINKS = 24;          // directory words: extent s (2^s units) is links[s], s >= 1
 constexpr int TG_DIR_UNITS = 2;       // units the directory takes in front of the first extent's entries
-static_assert(TG_LINKS * 4 == TG_DIR_UNITS * TG_UNIT * 8, "the directory fills whole units");
+constexpr int TG_DIR_WORDS = TG_DIR_UNITS * TG_UNIT * 2;
+constexpr int TG_GRANTED = 0;         // directory word: units beyond the first that the limit allowed
+constexpr int TG_REFUSED = TG_DIR_WORDS - 1;   // and those it did not
+constexpr int TG_LINKS = TG_REFUSED;  // words 1 .. TG_LINKS - 1: extent s (2^s units) is word s
 
 struct TgView {
     Bucket* buckets;
@@ -62,8 +69,15 @@ struct TgView {
     uint32_t min_count;
 };
 
-// Pool units for a limit of n_over units in use: a context using d units has extents of 1 + 2 + .. < 2 d units and a directory.
+// Pool units for a limit of n_over units in use (see above).
 __host__ __device__ constexpr unsigned long long tg_pool_units(unsigned long long n_over) { return 3 * n_over; }
+// Index slots: at most three quarters full with every unit filled, and room for the slots of entries that were refused after they had
+// taken one -- threads under way when the limit is reached, of which a device holds some 300,000.
+constexpr unsigned long long tg_index_slots(unsigned long long n_over) {
+    unsigned long long n = 16;
+    while (n < 8 * n_over || n < 6 * n_over + (1ull << 19)) n *= 2;
+    return n;
+}
 
 __device__ __forceinline__ uint32_t tg_hash(unsigned long long k) {
     k ^= k >> 30; k *= 0xBF58476D1CE4E5B9ull;
@@ -154,54 +168,101 @@ __device__ __forceinline__ uint32_t tg_wait_link(const uint32_t* link) {
     return v;
 }
 
+// A new extent: its first unit + 1, or TG_FAILED.  (The pool is sized so that there is room; if not, nothing is written.)
+__device__ __forceinline__ uint32_t tg_new_extent(const TgView& t, uint32_t units) {
+    const uint32_t at = atomicAdd(&t.used[1], units);
+    return (unsigned long long)at + units <= t.n_units ? at + 1 : TG_FAILED;
+}
+
+// Whether unit m >= 1 of a context exists: it does once m units beyond the first have been granted, whichever of the threads that
+// asked for one got it.  It does not when all that have asked are answered and fewer were granted: a refusal means that the
+// limit is reached, so that whoever asks later is refused too.  (Granted, then refused, then asked for are read, none of which
+// falls: granted + refused == asked for says that granted was complete when refused was read.)
+__device__ __forceinline__ bool tg_wait_room(const TgView& t, const Bucket* bk, const uint32_t* dir, uint32_t m) {
+    for (int spin = 0; spin < TG_MAX_SPIN; ++spin) {
+        const uint32_t granted = tg_acquire(dir + TG_GRANTED);
+        if (granted >= m) return true;
+        const uint32_t refused = tg_acquire(dir + TG_REFUSED);
+        if (refused != 0 && granted + refused == ((tg_acquire(&bk->n_more) & ~TG_CLOSED) - 1) / TG_UNIT) return false;
+        __nanosleep(32);
+    }
+    tg_report(t, (int)ADED_ERR_TIMEOUT);
+    return false;
+}
+
 // Takes the next entry of a context beyond its home bucket and writes the token with count 0.  Returns the entry's
-// number in the pool plus one, or 0 (reported) when there is no room.  The thread that takes the first entry of an
-// extent allocates the extent and publishes it; the others of that extent wait for it.  Threads only ever wait for owners
-// of earlier entries, so the waits cannot form a cycle.
-__device__ __forceinline__ unsigned long long tg_place(const TgView& t, Bucket* bk, int c) {
+// number in the pool plus one, or 0 (reported) when there is no room.  The thread that takes the first entry of a unit asks for
+// the unit; all that take one of its entries act on the same answer (tg_wait_room; for the first unit the link in the home bucket).
+// The thread that takes the first entry of an extent allocates the extent and publishes it; the others of that
+// extent wait for it.  `first`: see tg_full.  Threads only ever wait for owners of earlier entries, so the waits cannot form a cycle.
+__device__ __forceinline__ unsigned long long tg_place(const TgView& t, Bucket* bk, uint32_t first, int c) {
     const uint32_t p = atomicAdd(&bk->n_more, 1u) & ~TG_CLOSED;
     const uint32_t m = p / TG_UNIT, e = p % TG_UNIT;
     const int s = tg_extent(m);
     const uint32_t in_extent = m + 1 - (1u << s);             // the unit's place in its extent
-    const bool room = e != 0 || atomicAdd(&t.used[0], 1u) < t.n_over;
+    bool room = true;
     uint32_t base = TG_FAILED;                                // extent's first unit + 1
-    if (s < TG_LINKS) {
-        uint32_t* link = &bk->more;
-        if (s > 0) {
-            const uint32_t first = tg_wait_link(&bk->more);
-            link = first == 0 || first == TG_FAILED ? nullptr : reinterpret_cast<uint32_t*>(t.pool + (size_t)(first - 1) * TG_UNIT) + s;
-            if (first == 0) { tg_report(t, (int)ADED_ERR_TIMEOUT); return 0; }
-        }
-        if (link && e == 0 && in_extent == 0) {
-            if (room) {
-                const uint32_t units = s == 0 ? TG_DIR_UNITS + 1 : 1u << s;
-                const uint32_t at = atomicAdd(&t.used[1], units);
-                if (ADED_IN_RANGE((unsigned long long)at + units <= t.n_units, t.status)) {   // (the pool is sized so that this holds)
-                    base = at + 1;
-                    if (s == 0) {
-                        uint4* dir = reinterpret_cast<uint4*>(t.pool + (size_t)at * TG_UNIT);
-                        for (int i = 0; i < TG_LINKS / 4; ++i) dir[i] = make_uint4(0u, 0u, 0u, 0u);
-                    }
-                }
+    if (m == 0) {
+        if (e == 0) {
+            if (atomicAdd(&t.used[0], 1u) < t.n_over) base = tg_new_extent(t, TG_DIR_UNITS + 1);
+            if (base != TG_FAILED) {
+                uint4* dir = reinterpret_cast<uint4*>(t.pool + (size_t)(base - 1) * TG_UNIT);
+                for (int i = 0; i < TG_DIR_WORDS / 4; ++i) dir[i] = make_uint4(0u, 0u, 0u, 0u);
             }
-            tg_release(link, base);
-        } else if (link) {
-            base = tg_wait_link(link);
+            tg_release(&bk->more, base);
+        } else {
+            base = tg_wait_link(&bk->more);
             if (base == 0) { tg_report(t, (int)ADED_ERR_TIMEOUT); return 0; }
         }
+    } else {
+        if (first == 0) first = tg_wait_link(&bk->more);
+        if (first == 0) { tg_report(t, (int)ADED_ERR_TIMEOUT); return 0; }
+        if (first != TG_FAILED && s < TG_LINKS) {             // (asked only now: what a context is given it can use)
+            uint32_t* dir = reinterpret_cast<uint32_t*>(t.pool + (size_t)(first - 1) * TG_UNIT);
+            // (link and count in one round trip; nothing is read through them)
+            const uint32_t link = *reinterpret_cast<volatile uint32_t*>(dir + s);
+            uint32_t granted = 0;
+            if (e != 0) granted = *reinterpret_cast<volatile uint32_t*>(dir + TG_GRANTED);
+            else if (atomicAdd(&t.used[0], 1u) < t.n_over) granted = atomicAdd(dir + TG_GRANTED, 1u) + 1u;
+            else atomicAdd(dir + TG_REFUSED, 1u);
+            room = granted >= m || tg_wait_room(t, bk, dir, m);
+            if (e == 0 && in_extent == 0) {
+                if (room) base = tg_new_extent(t, 1u << s);
+                tg_release(dir + s, base);
+            } else {
+                base = link != 0 ? link : tg_wait_link(dir + s);
+                if (base == 0) { tg_report(t, (int)ADED_ERR_TIMEOUT); return 0; }
+            }
+        }
     }
-    if (base == TG_FAILED) {
-        atomicOr(&bk->n_more, TG_CLOSED);
-        tg_report(t, (int)ADED_ERR_TABLE_FULL);
-        return 0;
+    unsigned long long at = 0;
+    if (base != TG_FAILED) {
+        at = ((unsigned long long)(base - 1) + (s == 0 ? TG_DIR_UNITS : 0) + in_extent) * TG_UNIT + e;
+        if (!ADED_IN_RANGE(at < (unsigned long long)t.n_units * TG_UNIT, t.status)) return 0;
+        t.pool[at] = TgSlot{room ? c : -1, 0u};               // (an entry without a token is skipped by every reader)
+        if (room) return at + 1;
     }
-    const unsigned long long at = ((unsigned long long)(base - 1) + (s == 0 ? TG_DIR_UNITS : 0) + in_extent) * TG_UNIT + e;
-    if (!ADED_IN_RANGE(at < (unsigned long long)t.n_units * TG_UNIT, t.status)) return 0;
-    t.pool[at] = TgSlot{room ? c : -1, 0u};                   // (an entry without a token is skipped by every reader)
-    if (room) return at + 1;
     atomicOr(&bk->n_more, TG_CLOSED);
     tg_report(t, (int)ADED_ERR_TABLE_FULL);
     return 0;
+}
+
+// Whether a context can take no further entry: it has been refused one, or its next one would open a unit and the limit is reached.
+// (Asked before an index slot is taken: what a full table refuses should leave no trace in the index.)
+// `first`: the context's first extent as seen on the way, 0 if it was not there yet.
+__device__ __forceinline__ bool tg_full(const TgView& t, const Bucket* bk, uint32_t& first) {
+    static_assert(offsetof(Bucket, more) == 8 && offsetof(Bucket, n_more) == 12, "one load for both");
+    const unsigned long long both = tg_acquire(reinterpret_cast<const unsigned long long*>(&bk->more));
+    first = (uint32_t)both;
+    uint32_t n = (uint32_t)(both >> 32);
+    for (;;) {
+        if (n & TG_CLOSED) return true;
+        if (n % TG_UNIT != 0 || tg_acquire(&t.used[0]) < t.n_over) return false;
+        // (still the next entry: whoever takes it asks after the limit was reached; if not, somebody else may have been given the last unit for it)
+        const uint32_t now = tg_acquire(&bk->n_more);
+        if (now == n) return true;
+        n = now;
+    }
 }
 
 // Raises the count of tri-gram (a, b, c) by `inc` (see tg_raise), inserting it if absent; counts
@@ -230,15 +291,15 @@ __device__ __forceinline__ void tg_add(const TgView& t, int a, int b, int c, uin
         TgIndexSlot* slot = t.index + at_index;
         unsigned long long k = *reinterpret_cast<volatile unsigned long long*>(&slot->key);
         if (k == 0) {
-            // A context that could not grow stays as it is (and takes no index slot for what it refuses).
-            const uint32_t n = *reinterpret_cast<volatile uint32_t*>(&bk->n_more);
-            if ((n & TG_CLOSED) || (n % TG_UNIT == 0 && *reinterpret_cast<volatile uint32_t*>(&t.used[0]) >= t.n_over)) {
-                tg_report(t, (int)ADED_ERR_TABLE_FULL);
-                return;
+            uint32_t first;
+            if (tg_full(t, bk, first)) {
+                k = tg_acquire(&slot->key);                   // (unless the last entry has gone to this very token)
+                if (k == 0) { tg_report(t, (int)ADED_ERR_TABLE_FULL); return; }
+            } else {
+                k = atomicCAS(&slot->key, 0ull, key);
             }
-            k = atomicCAS(&slot->key, 0ull, key);
             if (k == 0) {
-                const unsigned long long at = tg_place(t, bk, c);
+                const unsigned long long at = tg_place(t, bk, first, c);
                 tg_release(&slot->at, at ? at : TG_DEAD);
                 if (at) tg_raise(t, &t.pool[at - 1].cnt, inc, windows);
                 return;

@@ -886,8 +886,7 @@ aded_status aded_trigram_create(const aded_trigram_config* cfg, aded_trigram** o
     t->view = TgView();
     const size_t n_home = (size_t)1 << cfg->log2_buckets, n_units = (size_t)tg_pool_units((unsigned long long)cfg->overflow_buckets);
     if (n_units > 0xFFFFFFF0ull) { delete t; return ADED_ERR_OOM; }      // (units are numbered in 32 bits; more would not fit the device)
-    size_t n_index = 16;                                                 // at most six entries per unit in use: three quarters full
-    while (n_index < 8 * (size_t)cfg->overflow_buckets) n_index *= 2;
+    const size_t n_index = (size_t)tg_index_slots((unsigned long long)cfg->overflow_buckets);
     bool ok = cudaGetDevice(&t->device) == cudaSuccess;
     cudaError_t e = cudaSuccess;
     // one allocation: home buckets, index, pool, then the small arrays (every part a multiple of 64 bytes)

@@ -278,6 +278,44 @@ def test_configured_overflow_is_the_limit(cuda_device, n):
     assert update(t, rows[0]) == 0 and _entries_gpu(B, t) == {tuple(rows[0]): 1}
 
 
+@pytest.mark.parametrize("limit", [0, 1, 2, 5, 9, 10, 64, 300])
+def test_many_entries_at_once_fill_the_table_to_its_limit(cuda_device, limit):
+    """Contexts that grow by hundreds of entries in one call when there are fewer units than they ask for: every unit is given out and
+    filled, the rest is refused and reported, what is kept is counted right, nothing else is touched -- the staging of the
+    host entry points lies behind the pool -- and a table at its limit goes on counting what it holds."""
+    from paper_2407_12021_b200 import binding as B
+    vocab, contexts, each = 5000, 6, 400
+    t = B.aded_trigram_create(vocab, log2_buckets=12, overflow_buckets=limit)
+    rows = [[a, 100 + a, 200 + i * 7 % 3001] for i in range(each) for a in range(contexts)]
+    for _ in range(3):
+        B.aded_trigram_clear(t)
+        for part in (rows[:6 * contexts], rows * 2):        # (six of every context are in its home bucket)
+            B.aded_trigram_import(t, torch.tensor(part, dtype=torch.int32, device="cuda"), torch.ones(len(part), dtype=torch.int32, device="cuda"))
+        torch.cuda.synchronize()
+        kept = _entries_gpu(B, t)
+        assert B.aded_trigram_poll_status(t) == 4
+        assert set(kept) <= {tuple(r) for r in rows} and all(1 <= n <= 3 for n in kept.values())
+        beyond = [sum(k[0] == a for k in kept) - 6 for a in range(contexts)]
+        assert all(n >= 0 for n in beyond) and sum((n + 5) // 6 for n in beyond) == limit
+        entries, buckets = B.aded_trigram_stats(t)
+        assert (entries, buckets) == (len(kept), contexts + limit)
+        held = list(kept)[:40]
+        assert all(B.aded_trigram_get(t, *r) == kept[r] for r in held)
+        # what the table holds is counted on; the staging buffers of the host calls are what they say
+        for r in held:
+            B.aded_trigram_update_host(t, torch.tensor(r, dtype=torch.int32))
+        assert B.aded_trigram_poll_status(t) == 0
+        assert all(B.aded_trigram_get(t, *r) == kept[r] + 1 for r in held)
+        after = _entries_gpu(B, t)
+        assert after == {r: n + (r in held) for r, n in kept.items()}
+        st = TrigramStore()
+        st.merge(after)
+        ctx = [(a, 100 + a) for a in range(contexts)] + [(1, 2)]
+        tok, cnt = torch.empty((7, 8), dtype=torch.int32), torch.empty((7, 8), dtype=torch.int32)
+        B.aded_trigram_topk_host(t, torch.tensor(ctx, dtype=torch.int32), 8, tok, cnt)
+        assert [(tok[i].tolist(), cnt[i].tolist()) for i in range(7)] == [st.topk(a, b, 8) for a, b in ctx]
+
+
 def test_repeated_and_absent_contexts_in_one_call(cuda_device):
     """Blocks answer a context once for all queries that ask for it: more queries than one block takes, every context many
     times, several long ones per block, absent and out-of-range contexts between them."""
