@@ -153,17 +153,29 @@ __device__ __forceinline__ unsigned long long tg_acquire(const unsigned long lon
     asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
     return v;
 }
-__device__ __forceinline__ void tg_release(uint32_t* p, uint32_t v) { asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory"); }
 __device__ __forceinline__ void tg_release(unsigned long long* p, unsigned long long v) {
     asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
-// Waits (bounded) until another thread has published a link of a directory; 0 when the wait ran out.
-__device__ __forceinline__ uint32_t tg_wait_link(const uint32_t* link) {
+// Publishes an extent (or TG_FAILED), unless a thread that ran out of patience has given it up.  Returns what the link says now.
+__device__ __forceinline__ uint32_t tg_publish(uint32_t* link, uint32_t base) {
+    uint32_t seen;
+    asm volatile("atom.release.gpu.global.cas.b32 %0, [%1], 0, %2;" : "=r"(seen) : "l"(link), "r"(base) : "memory");
+    return seen == 0 ? base : seen;
+}
+
+// Waits (bounded) until another thread has published an extent.  When the wait runs out the extent is given up for everybody
+// (TG_FAILED, reported): an entry of it that is not written will never be read, whatever its owner does later.
+__device__ __forceinline__ uint32_t tg_wait_link(const TgView& t, uint32_t* link) {
     uint32_t v = tg_acquire(link);
     for (int spin = 0; v == 0 && spin < TG_MAX_SPIN; ++spin) {
         __nanosleep(32);
         v = tg_acquire(link);
+    }
+    if (v == 0) {
+        v = tg_publish(link, TG_FAILED);
+        if (v == TG_FAILED) tg_report(t, (int)ADED_ERR_TIMEOUT);
+        else v = tg_acquire(link);
     }
     return v;
 }
@@ -194,7 +206,9 @@ __device__ __forceinline__ bool tg_wait_room(const TgView& t, const Bucket* bk, 
 // number in the pool plus one, or 0 (reported) when there is no room.  The thread that takes the first entry of a unit asks for
 // the unit; all that take one of its entries act on the same answer (tg_wait_room; for the first unit the link in the home bucket).
 // The thread that takes the first entry of an extent allocates the extent and publishes it; the others of that
-// extent wait for it.  `first`: see tg_full.  Threads only ever wait for owners of earlier entries, so the waits cannot form a cycle.
+// extent wait for it.  `first`: see tg_full.  Threads only ever wait for owners of earlier entries, so the waits cannot form a
+// cycle.  The pool is never cleared: every path leaves the entry written -- with the token, or without one where it was refused or
+// a wait ran out -- or in an extent that no reader will find.
 __device__ __forceinline__ unsigned long long tg_place(const TgView& t, Bucket* bk, uint32_t first, int c) {
     const uint32_t p = atomicAdd(&bk->n_more, 1u) & ~TG_CLOSED;
     const uint32_t m = p / TG_UNIT, e = p % TG_UNIT;
@@ -209,14 +223,12 @@ __device__ __forceinline__ unsigned long long tg_place(const TgView& t, Bucket* 
                 uint4* dir = reinterpret_cast<uint4*>(t.pool + (size_t)(base - 1) * TG_UNIT);
                 for (int i = 0; i < TG_DIR_WORDS / 4; ++i) dir[i] = make_uint4(0u, 0u, 0u, 0u);
             }
-            tg_release(&bk->more, base);
+            base = tg_publish(&bk->more, base);
         } else {
-            base = tg_wait_link(&bk->more);
-            if (base == 0) { tg_report(t, (int)ADED_ERR_TIMEOUT); return 0; }
+            base = tg_wait_link(t, &bk->more);
         }
     } else {
-        if (first == 0) first = tg_wait_link(&bk->more);
-        if (first == 0) { tg_report(t, (int)ADED_ERR_TIMEOUT); return 0; }
+        if (first == 0) first = tg_wait_link(t, &bk->more);
         if (first != TG_FAILED && s < TG_LINKS) {             // (asked only now: what a context is given it can use)
             uint32_t* dir = reinterpret_cast<uint32_t*>(t.pool + (size_t)(first - 1) * TG_UNIT);
             // (link and count in one round trip; nothing is read through them)
@@ -228,10 +240,9 @@ __device__ __forceinline__ unsigned long long tg_place(const TgView& t, Bucket* 
             room = granted >= m || tg_wait_room(t, bk, dir, m);
             if (e == 0 && in_extent == 0) {
                 if (room) base = tg_new_extent(t, 1u << s);
-                tg_release(dir + s, base);
+                base = tg_publish(dir + s, base);
             } else {
-                base = link != 0 ? link : tg_wait_link(dir + s);
-                if (base == 0) { tg_report(t, (int)ADED_ERR_TIMEOUT); return 0; }
+                base = link != 0 ? link : tg_wait_link(t, dir + s);
             }
         }
     }

@@ -859,7 +859,7 @@ static constexpr size_t TG_STAGE = 1 << 16;
 static constexpr int STEP_SENT = 0, STEP_REAL = 1, STEP_FILL = 2;
 static constexpr int STEP_INTS = STEP_FILL + DRAFT_MAX_FILLER;
 
-// An empty table: home buckets and index.  The pool needs no clearing: an entry is written before anything refers to it.
+// An empty table: home buckets and index.  The pool needs no clearing: see tg_place.
 static aded_status tg_reset(aded_trigram* t, cudaStream_t st) {
     k_tg_init<<<2048, 512, 0, st>>>(reinterpret_cast<uint4*>(t->view.buckets), (size_t)t->view.n_home * (sizeof(Bucket) / sizeof(uint4)));
     ADED_CUDA_TRY(cudaMemsetAsync(t->view.index, 0, (size_t)(t->view.index_mask + 1) * sizeof(TgIndexSlot), st));

@@ -17,7 +17,9 @@ def _host_header(spins: int) -> str:
     src, n = re.subn(r'asm volatile\("ld\.acquire[^;]*;[^;]*;', "v = model_load(p);", src)
     assert n == 2
     src, n = re.subn(r'asm volatile\("st\.release[^;]*;[^;]*;', "model_store(p, v);", src)
-    assert n == 2
+    assert n == 1
+    src, n = re.subn(r'asm volatile\("atom\.release[^;]*;[^;]*;', "seen = atomicCAS(link, 0u, base);", src)
+    assert n == 1
     src, n = re.subn(r"\*reinterpret_cast<volatile (unsigned long long|uint32_t)\*>\(([^;]*?)\)(?=[;,) ])", r"model_load((\1*)(\2))", src)
     assert n == 5, n
     src, n = re.subn(r"constexpr int TG_MAX_SPIN = [^;]*;", f"constexpr int TG_MAX_SPIN = {spins};", src)
@@ -43,3 +45,15 @@ def test_random_interleavings_stay_inside_the_pool_and_the_limit(program):
         res = subprocess.run([exe, str(seed), "100", "0"], capture_output=True, text=True, timeout=600)
         assert res.returncode == 0, res.stdout + res.stderr
         assert "0 timed out" in res.stdout
+
+
+def test_waits_that_run_out_leave_nothing_unwritten_in_sight(program):
+    """Threads held back for longer than the others wait for them: reported, and every visible entry is one that was inserted,
+    counted no more often than it was."""
+    exe = program(6)
+    timed_out = 0
+    for seed in range(4):
+        res = subprocess.run([exe, str(seed), "100", "1"], capture_output=True, text=True, timeout=600)
+        assert res.returncode == 0, res.stdout + res.stderr
+        timed_out += int(res.stdout.split()[-3])
+    assert timed_out > 20, "the waits did not run out"
