@@ -92,7 +92,9 @@ typedef struct aded_trigram_config {
     int32_t vocab;            /* token ids are 0 .. vocab-1 */
     int32_t log2_buckets;     /* 2^log2_buckets home buckets (one per two-token context), 4..28 */
     int32_t overflow_buckets; /* extra buckets (six entries each) for contexts with more than 6 continuations;
-                                 they and their index take 272-400 bytes of device memory each */
+                                 they and their index take 272-400 bytes of device memory each (plus 8 MB);
+                                 where the device has no room for that, 64: the same results, but contexts
+                                 with many continuations then take far longer to update and to look up */
     uint32_t cap;             /* counts saturate here (Algorithm 2's maximum); 0 = 2^31 - 1, which is also the largest allowed */
     uint32_t min_count;       /* top-k skips entries below this count; 0 = off */
 } aded_trigram_config;

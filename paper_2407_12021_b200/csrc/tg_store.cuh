@@ -21,6 +21,10 @@
 // of the extents on top: a context opens extent s only once it has been given 2^s units, so that with d units it takes
 // 2 + 1 + 2 + 4 + .. <= 3 d.  (What waiting for that costs: 20,000 tokens into an empty table 32 -> 36 us, 10^6 0.30 -> 0.31 ms, 4 x 10^6 no
 // difference, against extents that were opened on a thread's own unit alone, with which a table at its limit could exceed its pool.)
+//
+// Pool and index take 272-400 bytes per overflow bucket.  Where the device has no room for them the further entries lie in
+// chains of buckets instead (TgView::chain, 64 bytes each): an insertion walks its context's chain from the front and a lookup reads it
+// bucket by bucket -- the same answers, at the speeds named in brackets above, for tables that would otherwise not exist.
 #pragma once
 
 #include <cstddef>
@@ -32,8 +36,8 @@ namespace aded {
 struct TgSlot { int32_t tok; uint32_t cnt; };
 struct __align__(64) Bucket {
     unsigned long long key;   // context
-    uint32_t more;            // first extent: pool unit + 1 (0 none yet, TG_FAILED: there was no room for it)
-    uint32_t n_more;          // entries beyond six; bit 31 (TG_CLOSED): no room for further ones
+    uint32_t more;            // first extent: pool unit + 1 (0 none yet, TG_FAILED: there was no room for it); chained: next bucket + 1
+    uint32_t n_more;          // entries beyond six; bit 31 (TG_CLOSED): no room for further ones; chained: places in the chain
     TgSlot e[6];
 };
 static_assert(sizeof(Bucket) == 64, "bucket must be 64 bytes");
@@ -45,6 +49,7 @@ struct __align__(16) TgIndexSlot {
 constexpr unsigned long long TG_EMPTY = ~0ull, TG_DEAD = ~0ull;
 constexpr int TG_MAX_PROBE = 4096;
 constexpr uint32_t TG_FAILED = 0xFFFFFFFFu, TG_CLOSED = 0x80000000u;
+constexpr uint32_t TG_LOCKED = TG_FAILED;      // chained: the next bucket is being taken
 constexpr int TG_MAX_SPIN = 1 << 20;
 constexpr int TG_UNIT = 6;            // entries of a pool unit
 constexpr int TG_DIR_UNITS = 2;       // units the directory takes in front of the first extent's entries
@@ -57,6 +62,7 @@ struct TgView {
     Bucket* buckets;
     TgSlot* pool;                // [n_units][TG_UNIT]
     TgIndexSlot* index;
+    Bucket* chain;               // [n_over] where the device has no room for pool and index (then unused), else NULL
     uint32_t n_home_mask;
     uint32_t n_home;
     uint32_t n_over;             // configured limit on units of entries in use
@@ -276,13 +282,8 @@ __device__ __forceinline__ bool tg_full(const TgView& t, const Bucket* bk, uint3
     }
 }
 
-// Raises the count of tri-gram (a, b, c) by `inc` (see tg_raise), inserting it if absent; counts
-// saturate at the cap.  Independent atomic adds: the result does not depend on the thread order.
-__device__ __forceinline__ void tg_add(const TgView& t, int a, int b, int c, uint32_t inc, bool windows) {
-    const int64_t home = tg_find_home(t, tg_key(a, b), true);
-    if (home < 0) { tg_report(t, (int)ADED_ERR_TABLE_FULL); return; }
-    if (!ADED_IN_RANGE((uint64_t)home < (uint64_t)t.n_home, t.status)) return;
-    Bucket* bk = t.buckets + home;
+// Count cell of the token in a bucket, claiming the first free entry for it; NULL when others have all six.
+__device__ __forceinline__ uint32_t* tg_entry(Bucket* bk, int c) {
     // the six tokens at once (they are only ever written from -1 to their final value)
     const int4 e01 = __ldcg(reinterpret_cast<const int4*>(bk) + 1), e23 = __ldcg(reinterpret_cast<const int4*>(bk) + 2), e45 = __ldcg(reinterpret_cast<const int4*>(bk) + 3);
     const int32_t seen[6] = {e01.x, e01.z, e23.x, e23.z, e45.x, e45.z};
@@ -293,8 +294,57 @@ __device__ __forceinline__ void tg_add(const TgView& t, int a, int b, int c, uin
             have = atomicCAS(&bk->e[e].tok, -1, c);
             if (have == -1) have = c;
         }
-        if (have == c) { tg_raise(t, &bk->e[e].cnt, inc, windows); return; }
+        if (have == c) return &bk->e[e].cnt;
     }
+    return nullptr;
+}
+
+// The count cell of a token beyond a context's home bucket, in its chain; NULL (reported) when there is none and no room.  The thread
+// that finds no next bucket takes one under a one-word lock, the others wait for it.
+__device__ __forceinline__ uint32_t* tg_chained_entry(const TgView& t, Bucket* home, int c) {
+    Bucket* bk = home;
+    for (uint32_t hop = 0; hop < t.n_over; ++hop) {           // (a chain cannot be longer)
+        uint32_t next = tg_acquire(&bk->more);
+        if (next == 0) {
+            next = atomicCAS(&bk->more, 0u, TG_LOCKED);
+            if (next == 0) {
+                const uint32_t fresh = tg_acquire(&t.used[0]) < t.n_over ? atomicAdd(&t.used[0], 1u) : t.n_over;
+                if (fresh < t.n_over) {
+                    atomicAdd(&home->n_more, (uint32_t)TG_UNIT);
+                    next = fresh + 1;
+                }
+                atomicExch(&bk->more, next);
+            }
+        }
+        for (int spin = 0; next == TG_LOCKED && spin < TG_MAX_SPIN; ++spin) {
+            __nanosleep(64);
+            next = tg_acquire(&bk->more);
+        }
+        if (next == 0 || next == TG_LOCKED) {
+            tg_report(t, next == 0 ? (int)ADED_ERR_TABLE_FULL : (int)ADED_ERR_TIMEOUT);
+            return nullptr;
+        }
+        bk = t.chain + (next - 1);
+        uint32_t* cnt = tg_entry(bk, c);
+        if (cnt) return cnt;
+    }
+    tg_report(t, (int)ADED_ERR_TABLE_FULL);
+    return nullptr;
+}
+
+// Raises the count of tri-gram (a, b, c) by `inc` (see tg_raise), inserting it if absent; counts
+// saturate at the cap.  Independent atomic adds: the result does not depend on the thread order.
+__device__ __forceinline__ void tg_add(const TgView& t, int a, int b, int c, uint32_t inc, bool windows) {
+    const int64_t home = tg_find_home(t, tg_key(a, b), true);
+    if (home < 0) { tg_report(t, (int)ADED_ERR_TABLE_FULL); return; }
+    if (!ADED_IN_RANGE((uint64_t)home < (uint64_t)t.n_home, t.status)) return;
+    Bucket* bk = t.buckets + home;
+    uint32_t* cnt = tg_entry(bk, c);
+    if (!cnt && t.chain) {
+        cnt = tg_chained_entry(t, bk, c);
+        if (!cnt) return;
+    }
+    if (cnt) { tg_raise(t, cnt, inc, windows); return; }
     const unsigned long long key = tg_index_key((uint32_t)home, c);
     unsigned long long at_index = tg_index_start(key) & t.index_mask;
     const int limit = t.index_mask < TG_MAX_PROBE ? (int)t.index_mask + 1 : TG_MAX_PROBE;
@@ -337,6 +387,7 @@ struct TgWalk {
     uint4 part;            // lanes 0..3: the home bucket's 16-byte parts (header, then two entries each); elsewhere no entries
     uint32_t n;            // entries beyond the home bucket
     uint32_t extent;       // lane s: where extent s has its entries (first unit + 1, 0 none)
+    uint32_t chain;        // first bucket of the chain + 1, 0 none
     bool found;            // the context is stored
 };
 
@@ -346,7 +397,9 @@ __device__ __forceinline__ void tg_open_extents(const TgView& t, TgWalk& w, int 
     if (lane == 0 || lane > 3) { w.part.x = 0xFFFFFFFFu; w.part.y = 0u; w.part.z = 0xFFFFFFFFu; w.part.w = 0u; }
     w.n = 0;
     w.extent = 0;
+    w.chain = 0;
     if (more == 0 || more == TG_FAILED) return;
+    if (t.chain) { w.chain = more; return; }
     w.n = n & ~TG_CLOSED;
     if (lane == 0) {
         w.extent = more + TG_DIR_UNITS;
@@ -446,10 +499,25 @@ __device__ __forceinline__ void tg_take(const TgView& t, uint4 v, int k, int lan
     tg_offer2(tg_pack(t, (int32_t)v.x, v.y), tg_pack(t, (int32_t)v.z, v.w), k, lane, best);
 }
 
+// The buckets of a chain, one after the other: `f` gets their 16-byte parts as tg_take takes them.
+template <typename F>
+__device__ __forceinline__ void tg_each_chained(const TgView& t, uint32_t at, int lane, F f) {
+    for (uint32_t hop = 0; at != 0 && at != TG_LOCKED && hop < t.n_over; ++hop) {
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        if (lane < 4 && ADED_IN_RANGE(at <= t.n_over, t.status)) v = reinterpret_cast<const uint4*>(t.chain + (at - 1))[lane];
+        at = __shfl_sync(0xffffffffu, v.z, 0);
+        if (lane == 0 || lane > 3) v = make_uint4(0xFFFFFFFFu, 0u, 0xFFFFFFFFu, 0u);
+        f(v);
+    }
+}
+
 // Part `part` of `parts` of a context's entries (each part by one warp, all lanes): the k <= 32 best of them in `best`, and this
 // lane's share of the sum of the counts in `total` (both are carried on from the caller's values).
 __device__ __forceinline__ void tg_scan(const TgView& t, const TgWalk& w, int part, int parts, int k, int lane, unsigned long long& best, uint32_t& total) {
-    if (part == 0) tg_take(t, w.part, k, lane, best, total);
+    if (part == 0) {
+        tg_take(t, w.part, k, lane, best, total);
+        if (w.chain) tg_each_chained(t, w.chain, lane, [&](uint4 v) { tg_take(t, v, k, lane, best, total); });
+    }
     // The entries beyond, two per lane and load, BATCH loads in flight.  Pair g is the (g % 3)-th of the unit with ordinal g / 3.
     constexpr int BATCH = 4;
     const uint32_t pairs = (w.n + 1) / 2;
@@ -480,6 +548,16 @@ __device__ __forceinline__ const uint32_t* tg_find(const TgView& t, int a, int b
     const Bucket* bk = t.buckets + home;
     for (int e = 0; e < 6; ++e)
         if (bk->e[e].tok == c) return &bk->e[e].cnt;
+    if (t.chain) {
+        uint32_t at = bk->more;
+        for (uint32_t hop = 0; at != 0 && at != TG_LOCKED && hop < t.n_over; ++hop) {
+            bk = t.chain + (at - 1);
+            for (int e = 0; e < 6; ++e)
+                if (bk->e[e].tok == c) return &bk->e[e].cnt;
+            at = bk->more;
+        }
+        return nullptr;
+    }
     const unsigned long long key = tg_index_key((uint32_t)home, c);
     unsigned long long i = tg_index_start(key) & t.index_mask;
     const int limit = t.index_mask < TG_MAX_PROBE ? (int)t.index_mask + 1 : TG_MAX_PROBE;

@@ -112,6 +112,13 @@ __global__ void k_tg_export(TgView t, uint32_t min_count, int32_t* __restrict__ 
             const int src = __ffs((int)more) - 1;
             const TgWalk w = tg_open(t, g * 32 + src, lane);
             const unsigned long long k = __shfl_sync(0xffffffffu, key, src);
+            if (w.chain)
+                tg_each_chained(t, w.chain, lane, [&](uint4 v) {
+                    for (int h = 0; h < 2; ++h) {
+                        const TgSlot s = h ? TgSlot{(int32_t)v.z, v.w} : TgSlot{(int32_t)v.x, v.y};
+                        tg_export_one(k, s.tok, s.cnt, s.tok >= 0 && s.cnt >= min_count && s.cnt != 0, lane, keys, counts, max_entries, n_out);
+                    }
+                });
             for (uint32_t i0 = 0; i0 < w.n; i0 += 32) {
                 const uint32_t m = (i0 + lane) / TG_UNIT;
                 const int x = tg_extent(m);
@@ -548,6 +555,15 @@ __global__ void k_tg_stats(TgView t, unsigned long long* out) {
         ++used;
         for (int e = 0; e < 6; ++e) entries += bk->e[e].tok >= 0;
         if (bk->more == 0 || bk->more == TG_FAILED) continue;
+        if (t.chain) {
+            for (uint32_t at = bk->more, hop = 0; at != 0 && at != TG_LOCKED && hop < t.n_over; ++hop) {
+                const Bucket* next = t.chain + (at - 1);
+                for (int e = 0; e < 6; ++e) entries += next->e[e].tok >= 0;
+                ++used;
+                at = next->more;
+            }
+            continue;
+        }
         const uint32_t n = bk->n_more & ~TG_CLOSED;
         if (!(bk->n_more & TG_CLOSED)) {
             entries += n;
@@ -861,8 +877,9 @@ static constexpr int STEP_INTS = STEP_FILL + DRAFT_MAX_FILLER;
 
 // An empty table: home buckets and index.  The pool needs no clearing: see tg_place.
 static aded_status tg_reset(aded_trigram* t, cudaStream_t st) {
-    k_tg_init<<<2048, 512, 0, st>>>(reinterpret_cast<uint4*>(t->view.buckets), (size_t)t->view.n_home * (sizeof(Bucket) / sizeof(uint4)));
-    ADED_CUDA_TRY(cudaMemsetAsync(t->view.index, 0, (size_t)(t->view.index_mask + 1) * sizeof(TgIndexSlot), st));
+    const size_t buckets = (size_t)t->view.n_home + (t->view.chain ? t->view.n_over : 0);     // (chain buckets follow the home buckets)
+    k_tg_init<<<2048, 512, 0, st>>>(reinterpret_cast<uint4*>(t->view.buckets), buckets * (sizeof(Bucket) / sizeof(uint4)));
+    if (t->view.index) ADED_CUDA_TRY(cudaMemsetAsync(t->view.index, 0, (size_t)(t->view.index_mask + 1) * sizeof(TgIndexSlot), st));
     ADED_CUDA_TRY(cudaMemsetAsync(t->view.used, 0, 2 * sizeof(uint32_t), st));
     ADED_CUDA_TRY(cudaGetLastError());
     return ADED_OK;
@@ -884,23 +901,33 @@ aded_status aded_trigram_create(const aded_trigram_config* cfg, aded_trigram** o
     t->stats_dev = nullptr;
     t->step_i = nullptr;
     t->view = TgView();
-    const size_t n_home = (size_t)1 << cfg->log2_buckets, n_units = (size_t)tg_pool_units((unsigned long long)cfg->overflow_buckets);
-    if (n_units > 0xFFFFFFF0ull) { delete t; return ADED_ERR_OOM; }      // (units are numbered in 32 bits; more would not fit the device)
-    const size_t n_index = (size_t)tg_index_slots((unsigned long long)cfg->overflow_buckets);
+    const size_t n_home = (size_t)1 << cfg->log2_buckets, n_over = (size_t)cfg->overflow_buckets;
     bool ok = cudaGetDevice(&t->device) == cudaSuccess;
     cudaError_t e = cudaSuccess;
-    // one allocation: home buckets, index, pool, then the small arrays (every part a multiple of 64 bytes)
-    const size_t parts[8] = {n_home * sizeof(Bucket), n_index * sizeof(TgIndexSlot), n_units * TG_UNIT * sizeof(TgSlot),
-                             TG_STAGE * sizeof(int32_t), TG_STAGE * sizeof(uint32_t), STEP_INTS * sizeof(int32_t),
-                             2 * sizeof(unsigned long long), 4 * sizeof(uint32_t)};
-    size_t at[9] = {0};
-    for (int i = 0; i < 8; ++i) at[i + 1] = at[i] + (parts[i] + 63) / 64 * 64;
+    // one allocation: home buckets, index and pool (or, where the device has no room for those, or they number more than 32-bit
+    // units, chain buckets), then the small arrays (every part a multiple of 64 bytes)
+    size_t n_units = (size_t)tg_pool_units(n_over), n_index = (size_t)tg_index_slots(n_over), at[9] = {0};
+    bool chained = n_units > 0xFFFFFFF0ull;
     char* block = nullptr;
-    if (ok) { e = cudaMalloc((void**)&block, at[8]); ok = e == cudaSuccess; }
+    for (;; chained = true) {
+        if (chained) n_units = n_index = 0;
+        const size_t parts[8] = {(n_home + (chained ? n_over : 0)) * sizeof(Bucket), n_index * sizeof(TgIndexSlot), n_units * TG_UNIT * sizeof(TgSlot),
+                                 TG_STAGE * sizeof(int32_t), TG_STAGE * sizeof(uint32_t), STEP_INTS * sizeof(int32_t),
+                                 2 * sizeof(unsigned long long), 4 * sizeof(uint32_t)};
+        for (int i = 0; i < 8; ++i) at[i + 1] = at[i] + (parts[i] + 63) / 64 * 64;
+        if (ok) { e = cudaMalloc((void**)&block, at[8]); ok = e == cudaSuccess; }
+        if (ok || chained || e != cudaErrorMemoryAllocation) break;
+        cudaGetLastError();
+        ok = true;
+    }
     if (ok) {
         t->view.buckets = reinterpret_cast<Bucket*>(block + at[0]);
-        t->view.index = reinterpret_cast<TgIndexSlot*>(block + at[1]);
-        t->view.pool = reinterpret_cast<TgSlot*>(block + at[2]);
+        if (chained) {
+            t->view.chain = t->view.buckets + n_home;
+        } else {
+            t->view.index = reinterpret_cast<TgIndexSlot*>(block + at[1]);
+            t->view.pool = reinterpret_cast<TgSlot*>(block + at[2]);
+        }
         t->stage_i = reinterpret_cast<int32_t*>(block + at[3]);
         t->stage_u = reinterpret_cast<uint32_t*>(block + at[4]);
         t->step_i = reinterpret_cast<int32_t*>(block + at[5]);
@@ -917,7 +944,7 @@ aded_status aded_trigram_create(const aded_trigram_config* cfg, aded_trigram** o
     t->view.n_home_mask = (uint32_t)n_home - 1;
     t->view.n_over = (uint32_t)cfg->overflow_buckets;
     t->view.n_units = (uint32_t)n_units;
-    t->view.index_mask = n_index - 1;
+    t->view.index_mask = chained ? 0 : n_index - 1;
     t->view.vocab = cfg->vocab;
     t->view.cap = cfg->cap == 0 ? 0x7fffffffu : cfg->cap;
     t->view.min_count = cfg->min_count;

@@ -388,3 +388,59 @@ def test_lookups_on_both_sides_of_the_grouped_path(cuda_device, q):
     assert B.aded_trigram_poll_status(t) == 0
     got = list(zip(out_t.tolist(), out_c.tolist()))
     assert all(got[i] == st.topk(*contexts[i], 4) for i in range(0, q, 97))
+
+
+def test_table_without_room_for_pool_and_index(cuda_device, tmp_path):
+    """Where the device has no room for the pool and its index (272-400 bytes per overflow bucket) a table is made of chains of buckets
+    (64 bytes): every operation gives what it gives on an ordinary table."""
+    from paper_2407_12021_b200 import binding as B
+    vocab = 5000
+    text = gen.zipf_tokens(200_000, vocab, 71, 1).tolist()
+    text += [t for i in range(2500) for t in (3, 4, 100 + i)] + [t for i in range(0, 2500, 2) for t in (3, 4, 100 + i)]
+    toks = torch.tensor(text, dtype=torch.int32, device="cuda")
+    torch.cuda.empty_cache()
+    full = B.aded_trigram_create(vocab, log2_buckets=18, overflow_buckets=1 << 17)
+    B.aded_trigram_update(full, toks[:3])                  # (kernels are loaded before the room is taken)
+    B.aded_trigram_clear(full)
+    torch.cuda.synchronize()
+    taken = torch.empty(torch.cuda.mem_get_info()[0] - (600 << 20), dtype=torch.uint8, device="cuda")
+    before = torch.cuda.mem_get_info()[0]
+    tight = B.aded_trigram_create(vocab, log2_buckets=18, overflow_buckets=3_000_000)      # 0.2 GB; 1 GB otherwise
+    assert before - torch.cuda.mem_get_info()[0] < 300 << 20
+    del taken
+    torch.cuda.empty_cache()
+    tables, answers = (full, tight), []
+    keys = list(zip(text[0:4000:2], text[1:4000:2]))
+    pool = [(3, 4), (1, 1), (vocab - 1, vocab - 1), (-1, 3)] + keys
+    contexts = (pool * (70_000 // len(pool) + 1))[:70_000]
+    filler = gen.zipf_tokens(512, vocab, 72, 1).cuda()
+    u = torch.tensor(gen.uniform01(600, 73, 1).numpy().astype(np.float32), device="cuda")
+    for t in tables:
+        got = []
+        B.aded_trigram_update(t, toks)                     # a long span, then short ones
+        B.aded_trigram_update(t, toks[:5000])
+        B.aded_trigram_update_host(t, toks[5000:5200].cpu())
+        got.append(sorted(_entries_gpu(B, t).items()))
+        got.append(B.aded_trigram_stats(t))
+        got += [B.aded_trigram_get(t, 3, 4, c) for c in (100, 101, 2599, 2600)]
+        got += [_topk_gpu(B, t, contexts[:q], k) for q, k in ((300, 1), (300, 9), (300, 32), (70_000, 1), (70_000, 4))]
+        for ctx in ((3, 4), keys[5], (vocab - 1, vocab - 1)):
+            tree = [torch.zeros(m, dtype=torch.int32, device="cuda") for m in (64, 64, 1)]
+            B.aded_draft_tree(t, torch.tensor(ctx, dtype=torch.int32, device="cuda"), 64, 6, 8, filler, *tree)
+            got += [x.tolist() for x in tree]
+            got.append(B.aded_mcts_draft(t, torch.tensor(ctx, dtype=torch.int32, device="cuda"), 150, 4, 24, 8, u))
+        B.aded_trigram_save(t, str(tmp_path / "table.bin"))
+        B.aded_trigram_prune(t, 2)
+        got.append(sorted(_entries_gpu(B, t).items()))
+        B.aded_trigram_load(t, str(tmp_path / "table.bin"))
+        got.append(sorted(_entries_gpu(B, t).items()))
+        got.append(B.aded_trigram_stats(t))
+        B.aded_trigram_clear(t)
+        got += [B.aded_trigram_stats(t), B.aded_trigram_poll_status(t)]
+        answers.append(got)
+    assert len(answers[0]) == len(answers[1])
+    assert all(a == b for a, b in zip(*answers)), [i for i, (a, b) in enumerate(zip(*answers)) if a != b]
+    st = TrigramStore()
+    for span in (text, text[:5000], text[5000:5200]):
+        st.update(span)
+    assert dict(answers[1][0]) == st.entries() and answers[1][-1] == 0

@@ -39,21 +39,23 @@ def program(tmp_path_factory):
     return build
 
 
-def test_random_interleavings_stay_inside_the_pool_and_the_limit(program):
+@pytest.mark.parametrize("chained", ["0", "1"])
+def test_random_interleavings_stay_inside_the_pool_and_the_limit(program, chained):
     exe = program(1 << 20)
     for seed in range(4):
-        res = subprocess.run([exe, str(seed), "100", "0"], capture_output=True, text=True, timeout=600)
+        res = subprocess.run([exe, str(seed), "100", "0", chained], capture_output=True, text=True, timeout=600)
         assert res.returncode == 0, res.stdout + res.stderr
         assert "0 timed out" in res.stdout
 
 
-def test_waits_that_run_out_leave_nothing_unwritten_in_sight(program):
+@pytest.mark.parametrize("chained", ["0", "1"])
+def test_waits_that_run_out_leave_nothing_unwritten_in_sight(program, chained):
     """Threads held back for longer than the others wait for them: reported, and every visible entry is one that was inserted,
     counted no more often than it was."""
     exe = program(6)
     timed_out = 0
     for seed in range(4):
-        res = subprocess.run([exe, str(seed), "100", "1"], capture_output=True, text=True, timeout=600)
+        res = subprocess.run([exe, str(seed), "100", "1", chained], capture_output=True, text=True, timeout=600)
         assert res.returncode == 0, res.stdout + res.stderr
         timed_out += int(res.stdout.split()[-3])
     assert timed_out > 20, "the waits did not run out"

@@ -1,7 +1,8 @@
 // The insertion code of the tri-gram store (csrc/tg_store.cuh, turned into a host header by test_tg_store_host.py) under random
 // interleavings of its atomic steps: every simulated thread is a coroutine that gives way at each atomic operation and load, and
 // the next one to run is drawn.  The pool has guard words behind it and is filled with entries that nobody inserted.
-//   tg_store_host <seed> <runs> <late>      late = 1: threads are held back for long stretches, so that bounded waits run out
+//   tg_store_host <seed> <runs> <late> <chained>    late = 1: threads are held back for long stretches, so that bounded waits run out;
+//                                                   chained = 1: the layout without pool and index
 #include <ucontext.h>
 
 #include <cstddef>
@@ -28,6 +29,7 @@ static void give_way();
 template <typename T> static T model_load(const T* p) { give_way(); return *p; }
 template <typename T> static void model_store(T* p, T v) { give_way(); *p = v; }
 template <typename T, typename U> static T atomicAdd(T* p, U v) { give_way(); const T old = *p; *p += (T)v; return old; }
+template <typename T, typename U> static T atomicExch(T* p, U v) { give_way(); const T old = *p; *p = (T)v; return old; }
 template <typename T, typename U> static T atomicOr(T* p, U v) { give_way(); const T old = *p; *p |= (T)v; return old; }
 template <typename T, typename U> static T atomicMin(T* p, U v) { give_way(); const T old = *p; if ((T)v < old) *p = (T)v; return old; }
 template <typename T, typename U, typename V> static T atomicCAS(T* p, U cmp, V v) { give_way(); const T old = *p; if (old == (T)cmp) *p = (T)v; return old; }
@@ -97,6 +99,7 @@ int main(int argc, char** argv) {
     g_rng.seed(strtoull(argv[1], nullptr, 10));
     const int runs = atoi(argv[2]);
     g_late = argc > 3 && atoi(argv[3]) != 0;
+    const bool chained = argc > 4 && atoi(argv[4]) != 0;
     long timeouts = 0, refusals = 0;
     for (int run = 0; run < runs; ++run) {
         static const unsigned limits[] = {0, 1, 2, 3, 4, 5, 8, 9, 10, 17, 40, 64};
@@ -105,10 +108,13 @@ int main(int argc, char** argv) {
         const int contexts = 1 + (int)(g_rng() % 4), threads = 20 + (int)(g_rng() % 240), tokens = 1 + (int)(g_rng() % threads) + threads / 2;
         const size_t n_units = (size_t)tg_pool_units(n_over), guard = 64, n_index = (size_t)tg_index_slots(n_over);
         std::vector<Bucket> home(16);
-        for (Bucket& b : home) {
+        auto clear = [](Bucket& b) {
             b.key = TG_EMPTY; b.more = 0; b.n_more = 0;
             for (TgSlot& e : b.e) e = TgSlot{-1, 0u};
-        }
+        };
+        for (Bucket& b : home) clear(b);
+        std::vector<Bucket> chain(n_over + guard);
+        for (size_t i = 0; i < chain.size(); ++i) { clear(chain[i]); if (i >= n_over) chain[i].more = 77u; }
         std::vector<uint4> pool((n_units + guard) * TG_UNIT / 2 + 2);
         TgSlot* cells = reinterpret_cast<TgSlot*>(pool.data());
         for (size_t i = 0; i < (n_units + guard) * TG_UNIT; ++i) cells[i] = TgSlot{1000000 + (int)i, 777u};
@@ -117,6 +123,7 @@ int main(int argc, char** argv) {
         int32_t status = 0;
         g_view = TgView();
         g_view.buckets = home.data(); g_view.pool = cells; g_view.index = index;
+        if (chained) { g_view.chain = chain.data(); g_view.pool = nullptr; g_view.index = nullptr; }
         g_view.n_home = 16; g_view.n_home_mask = 15; g_view.n_over = n_over; g_view.n_units = (uint32_t)n_units; g_view.index_mask = n_index - 1;
         g_view.used = used; g_view.status = &status; g_view.vocab = 1 << 20; g_view.cap = 0x7fffffffu; g_view.min_count = 0;
         std::map<std::pair<int, int>, uint32_t> added;      // (context, token) -> how often
@@ -131,6 +138,7 @@ int main(int argc, char** argv) {
             run_all();
             for (size_t i = n_units * TG_UNIT; i < (n_units + guard) * TG_UNIT; ++i)
                 CHECK(cells[i].tok == 1000000 + (int)i && cells[i].cnt == 777u, "the pool of %zu units was written %zu entries past its end", n_units, i - n_units * TG_UNIT);
+            for (size_t i = n_over; i < chain.size(); ++i) CHECK(chain[i].more == 77u && chain[i].e[0].tok == -1 && chain[i].n_more == 0, "chain bucket %zu of %u", i, n_over);
             CHECK(status != ADED_ERR_INTERNAL, "an index out of range");
             timeouts += status == ADED_ERR_TIMEOUT;
             refusals += status == ADED_ERR_TABLE_FULL;
@@ -144,7 +152,12 @@ int main(int argc, char** argv) {
                 for (const TgSlot& e : b.e)
                     if (e.tok >= 0) { CHECK(seen.count(e.tok) == 0, "token %d twice", e.tok); seen[e.tok] = e.cnt; }
                 const size_t at_home = seen.size();
-                const uint32_t n = b.more == 0 || b.more == TG_FAILED ? 0u : b.n_more & ~TG_CLOSED;
+                for (uint32_t at = chained ? b.more : 0u; at != 0 && at != TG_LOCKED; at = chain[at - 1].more) {
+                    CHECK(at <= n_over, "chain bucket %u", at - 1);
+                    for (const TgSlot& e : chain[at - 1].e)
+                        if (e.tok >= 0) { CHECK(seen.count(e.tok) == 0, "token %d twice", e.tok); seen[e.tok] = e.cnt; }
+                }
+                const uint32_t n = chained || b.more == 0 || b.more == TG_FAILED ? 0u : b.n_more & ~TG_CLOSED;
                 for (uint32_t p = 0; p < n; ++p) {
                     const uint32_t m = p / TG_UNIT;
                     const int s = tg_extent(m);
