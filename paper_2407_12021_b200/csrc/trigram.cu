@@ -866,6 +866,7 @@ struct aded_trigram {
     size_t stage_n;
     unsigned long long* stats_dev;
     int32_t* step_i;     // decoding step: see STEP_SENT
+    mutable bool search_prepared;   // the tree search's shared-memory limit has been raised on this device
 };
 
 using namespace aded;
@@ -900,6 +901,7 @@ aded_status aded_trigram_create(const aded_trigram_config* cfg, aded_trigram** o
     t->stage_u = nullptr;
     t->stats_dev = nullptr;
     t->step_i = nullptr;
+    t->search_prepared = false;
     t->view = TgView();
     const size_t n_home = (size_t)1 << cfg->log2_buckets, n_over = (size_t)cfg->overflow_buckets;
     bool ok = cudaGetDevice(&t->device) == cudaSuccess;
@@ -1020,8 +1022,9 @@ aded_status aded_trigram_topk(const aded_trigram* t, const int32_t* ctx_dev, int
         return ADED_OK;
     }
     per_block = per_block > TOPK_MAX_QUERIES ? TOPK_MAX_QUERIES : per_block;
-    static const cudaError_t prepared = cudaFuncSetAttribute(k_tg_topk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)topk_smem(TOPK_MAX_QUERIES));
-    ADED_CUDA_TRY(prepared);
+    // (the limit is the device's, not the process's; blocks of so many queries come from k = 1 and some 700,000 of them only)
+    if (topk_smem(per_block) > 40 * 1024)
+        ADED_CUDA_TRY(cudaFuncSetAttribute(k_tg_topk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)topk_smem(TOPK_MAX_QUERIES)));
     note_launch();
     k_tg_topk<<<(q + per_block - 1) / per_block, TOPK_THREADS, topk_smem(per_block), st>>>(
         t->view, ctx_dev, q, k, per_block, out_tokens_dev, out_counts_dev, out_total_dev);
@@ -1082,10 +1085,9 @@ aded_status aded_mcts_draft(const aded_trigram* t, const int32_t* context_dev, i
     if (iterations < 1 || iterations > MC_MAX_ITER || length < 1 || length > MC_MAX_LEN || k < 1 || k > MC_MAX_K ||
         n_candidates < 1 || n_candidates * length + 1 > ADED_MAX_NODES || !(c2 > 0.f))
         return ADED_ERR_INVALID_ARG;
-    static bool prepared = false;
-    if (!prepared) {
+    if (!t->search_prepared) {      // (per handle: the limit is the device's, and a handle belongs to one)
         ADED_CUDA_TRY(cudaFuncSetAttribute(k_mcts_draft, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mc_smem_bytes()));
-        prepared = true;
+        t->search_prepared = true;
     }
     McParams p;
     p.iterations = iterations;

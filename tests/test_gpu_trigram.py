@@ -337,6 +337,26 @@ def test_repeated_and_absent_contexts_in_one_call(cuda_device):
                 assert ((tok[i], cnt[i]), tot[i]) == want[c], (q, k, i, c)
 
 
+def test_more_lookups_than_the_blocks_hold_in_ordinary_shared_memory(cuda_device):
+    """One continuation each for so many contexts that a block's share needs more than 48 KB of shared memory."""
+    from paper_2407_12021_b200 import binding as B
+    toks = gen.zipf_tokens(20000, 300, 81, 1)
+    st = TrigramStore()
+    st.update(toks.tolist())
+    t = B.aded_trigram_create(300, log2_buckets=16, overflow_buckets=1 << 13)
+    B.aded_trigram_update(t, toks.cuda())
+    keys = list(st.table.keys())[:3000] + [(299, 299), (-1, 3)]
+    want = [st.topk(a, b, 1) + (st.total(a, b),) for a, b in keys]
+    q = 1_500_000
+    at = torch.arange(q, device="cuda") % len(keys)
+    ctx = torch.tensor(keys, dtype=torch.int32, device="cuda")[at].contiguous()
+    tok, cnt = torch.empty((q, 1), dtype=torch.int32, device="cuda"), torch.empty((q, 1), dtype=torch.int32, device="cuda")
+    tot = torch.empty(q, dtype=torch.int32, device="cuda")
+    B.aded_trigram_topk(t, ctx, 1, tok, cnt, tot)
+    for got, i in ((tok.view(-1), 0), (cnt.view(-1), 1), (tot, 2)):
+        assert torch.equal(got, torch.tensor([w[i][0] if i < 2 else w[i] for w in want], dtype=torch.int32, device="cuda")[at])
+
+
 @pytest.mark.parametrize("windows", [(1 << 17) - 1, 1 << 17, (1 << 17) + 1, (1 << 17) + 2047])
 def test_long_spans_on_both_sides_of_the_bulk_update(cuda_device, windows):
     """Spans of 2^17 windows on are added up per block first: the counts at the line, with a ragged last block, with a cap that many
