@@ -684,7 +684,8 @@ k_mcts_draft(TgView t, const __grid_constant__ McParams p, const int32_t* __rest
     uint8_t* s_nkid = reinterpret_cast<uint8_t*>(s_queue + ADED_MAX_NODES);
     uint8_t* s_flag = s_nkid + MC_MAX_NODES;                              // bit 0 expanded, bit 1 chosen, bit 2 kept
     McSlot* s_cache = reinterpret_cast<McSlot*>(mc_smem + mc_cache_offset());   // [MC_CACHE] remembered lookups
-    for (int i = threadIdx.x; i < MC_CACHE; i += 32) s_cache[i].key = TG_EMPTY;
+    // (the key of an empty slot is that of the context (-1, -1), which a caller may pass: no continuations, the right answer for it)
+    for (int i = threadIdx.x; i < MC_CACHE; i += 32) { s_cache[i].key = TG_EMPTY; s_cache[i].n = 0; }
     pdl_enter();
     float* s_u = reinterpret_cast<float*>(s_cache + MC_CACHE);            // the caller's uniform numbers
     for (int i = threadIdx.x; i < p.iterations * p.length; i += 32) s_u[i] = u[i];

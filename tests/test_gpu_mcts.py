@@ -65,6 +65,20 @@ def test_hot_context_with_a_long_chain_and_bad_arguments(cuda_device):
             B.aded_mcts_draft(t, H.i32([1, 2]), bad[0], bad[1], bad[2], bad[3], torch.zeros(2000, device="cuda"))
 
 
+@pytest.mark.parametrize("start", [(-1, -1), (-1, 3), (3, -1), (60, 60), (2 ** 31 - 1, -2 ** 31)])
+def test_contexts_outside_the_vocabulary_have_no_continuations(cuda_device, start):
+    """Also right after a search that filled the kernel's shared memory; (-1, -1) is the key of its empty slots."""
+    from paper_2407_12021_b200 import binding as B
+    toks = gen.zipf_tokens(4000, 60, 5, 1)
+    st = TrigramStore()
+    st.update(toks.tolist())
+    t = B.aded_trigram_create(60, log2_buckets=12, overflow_buckets=2048)
+    B.aded_trigram_update(t, toks.cuda())
+    u = gen.uniform01(600, 5, 1).numpy().astype(np.float32)
+    _compare(B, t, st, int(toks[0]), int(toks[1]), 150, 4, 24, 8, u)
+    assert _compare(B, t, st, *start, 150, 4, 24, 8, u) == ([start[1]], [-1], [])
+
+
 def test_drafts_feed_the_verification_step(cuda_device):
     """The merged prefix tree is a valid draft tree: the verification step of workload 1's model takes it
     and emits what the checker emits for the same tree."""
