@@ -274,9 +274,10 @@ __global__ void __launch_bounds__(256) k_topk_mark(TgView t, const int32_t* __re
                                                    int32_t* __restrict__ out_tok, uint32_t* out_cnt) {
     // neighbouring threads take queries of different blocks of the next kernel: the frequent contexts, which the first threads
     // meet, then have their leaders spread over all of its blocks
-    const int at = blockIdx.x * 256 + threadIdx.x;
-    const long long row = (long long)(at % lead_blocks) * per_block + at / lead_blocks;
-    if (at / lead_blocks >= per_block || row >= q) return;
+    // (unsigned: the rounded-up product of blocks and queries per block may pass 2^31 - 1)
+    const uint32_t at = blockIdx.x * 256 + threadIdx.x;
+    const uint32_t row = at % (uint32_t)lead_blocks * per_block + at / (uint32_t)lead_blocks;
+    if (at / (uint32_t)lead_blocks >= (uint32_t)per_block || row >= (uint32_t)q) return;
     const int i = (int)row;
     const int2 c = make_int2(ctx[2 * (size_t)i], ctx[2 * (size_t)i + 1]);
     int64_t home = -1;
@@ -368,8 +369,9 @@ k_topk_lead(TgView t, int q, int k, int per_block, int32_t* __restrict__ out_tok
 }
 
 __global__ void __launch_bounds__(256) k_topk_copy(int q, int k, int32_t* __restrict__ out_tok, uint32_t* __restrict__ out_cnt, uint32_t* __restrict__ out_total) {
-    const int i = blockIdx.x * 256 + threadIdx.x;
-    if (i >= q) return;
+    const uint32_t row = blockIdx.x * 256 + threadIdx.x;
+    if (row >= (uint32_t)q) return;
+    const int i = (int)row;
     const int mark = out_tok[(size_t)i * k];
     if (mark >= MARK_OWN) return;
     const size_t from = (size_t)mark_leader(mark) * k, to = (size_t)i * k;
@@ -975,7 +977,7 @@ aded_status aded_trigram_update(aded_trigram* t, const int32_t* tokens_dev, int3
     const int windows = n - 2;
     note_launch();
     if (windows >= BULK_MIN)
-        k_tg_update_bulk<<<(windows + BULK_WINDOWS - 1) / BULK_WINDOWS, BULK_THREADS, (BULK_WINDOWS + 2 + 2 * BULK_SLOTS) * sizeof(int32_t),
+        k_tg_update_bulk<<<(unsigned)(((int64_t)windows + BULK_WINDOWS - 1) / BULK_WINDOWS), BULK_THREADS, (BULK_WINDOWS + 2 + 2 * BULK_SLOTS) * sizeof(int32_t),
                            static_cast<cudaStream_t>(stream)>>>(t->view, tokens_dev, windows);
     else
         k_tg_update<<<(windows + 255) / 256, 256, 0, static_cast<cudaStream_t>(stream)>>>(t->view, tokens_dev, n);
@@ -1007,18 +1009,18 @@ aded_status aded_trigram_topk(const aded_trigram* t, const int32_t* ctx_dev, int
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     // As many queries per block as fill the device's block slots once (three blocks per SM).
     const int wave = ws_grid_limit(t->device) / 2 * 3;
-    int per_block = (q + wave - 1) / wave;
+    int per_block = (int)(((int64_t)q + wave - 1) / wave);
     if (q >= TOPK_BULK && k >= 2) {
         uint32_t slots = TOPK_BULK;
         while ((uint64_t)slots * 2 <= (uint64_t)q * k && slots < (1u << 31)) slots *= 2;
         per_block = per_block > TOPK_LEAD_QUERIES ? TOPK_LEAD_QUERIES : per_block;
         ADED_CUDA_TRY(cudaMemsetAsync(out_counts_dev, 0xFF, (size_t)slots * sizeof(uint32_t), st));
         note_launch(3);
-        const int lead_blocks = (q + per_block - 1) / per_block;
+        const int lead_blocks = (int)(((int64_t)q + per_block - 1) / per_block);
         k_topk_mark<<<(unsigned)(((long long)lead_blocks * per_block + 255) / 256), 256, 0, st>>>(t->view, ctx_dev, q, k, lead_blocks, per_block, slots - 1,
                                                                                              out_tokens_dev, out_counts_dev);
         k_topk_lead<<<lead_blocks, TOPK_THREADS, 0, st>>>(t->view, q, k, per_block, out_tokens_dev, out_counts_dev, out_total_dev);
-        k_topk_copy<<<(q + 255) / 256, 256, 0, st>>>(q, k, out_tokens_dev, out_counts_dev, out_total_dev);
+        k_topk_copy<<<(unsigned)(((int64_t)q + 255) / 256), 256, 0, st>>>(q, k, out_tokens_dev, out_counts_dev, out_total_dev);
         ADED_CUDA_TRY(cudaGetLastError());
         return ADED_OK;
     }
@@ -1027,7 +1029,7 @@ aded_status aded_trigram_topk(const aded_trigram* t, const int32_t* ctx_dev, int
     if (topk_smem(per_block) > 40 * 1024)
         ADED_CUDA_TRY(cudaFuncSetAttribute(k_tg_topk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)topk_smem(TOPK_MAX_QUERIES)));
     note_launch();
-    k_tg_topk<<<(q + per_block - 1) / per_block, TOPK_THREADS, topk_smem(per_block), st>>>(
+    k_tg_topk<<<(unsigned)(((int64_t)q + per_block - 1) / per_block), TOPK_THREADS, topk_smem(per_block), st>>>(
         t->view, ctx_dev, q, k, per_block, out_tokens_dev, out_counts_dev, out_total_dev);
     ADED_CUDA_TRY(cudaGetLastError());
     return ADED_OK;
