@@ -447,8 +447,10 @@ static aded_status kv_copy(const aded_kv* kv, int seq, int layer, int pos0, int 
     const size_t row = (size_t)c.head_dim * kv->elem;
     const size_t cap = kv->cap[seq];
     auto plane_of = [&](int which) { return kv->base[seq] + (((size_t)layer * 2 + which) * c.n_heads * cap + pos0) * row; };
-    if (((reinterpret_cast<uintptr_t>(k) | reinterpret_cast<uintptr_t>(v)) & 15) == 0) {
-        // one kernel for both planes (two strided copies of 16 MB each took 38 us, this 21); rows are multiples of 128 bytes
+    int current = -1;
+    if (((reinterpret_cast<uintptr_t>(k) | reinterpret_cast<uintptr_t>(v)) & 15) == 0 && cudaGetDevice(&current) == cudaSuccess && current == kv->device) {
+        // one kernel for both planes (two strided copies of 16 MB each took 38 us, this 21); rows are multiples of 128 bytes.  (A kernel
+        // runs on the current device; copies work whichever that is.)
         note_launch();
         launch_kv_copy(plane_of(0), plane_of(1), cap * row, k, v, (size_t)n_pos * row, c.n_heads, into_cache, st);
         ADED_CUDA_TRY(cudaGetLastError());
