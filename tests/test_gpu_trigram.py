@@ -360,7 +360,8 @@ def test_more_lookups_than_the_blocks_hold_in_ordinary_shared_memory(cuda_device
 @pytest.mark.parametrize("windows", [(1 << 17) - 1, 1 << 17, (1 << 17) + 1, (1 << 17) + 2047])
 def test_long_spans_on_both_sides_of_the_bulk_update(cuda_device, windows):
     """Spans of 2^17 windows on are added up per block first: the counts at the line, with a ragged last block, with a cap that many
-    blocks reach together, and with a token outside the vocabulary (reported; the windows without it are counted)."""
+    blocks reach together, and with a token outside the vocabulary (reported; windows with it, and those that come up after the
+    report, are not counted)."""
     from paper_2407_12021_b200 import binding as B
     toks = gen.zipf_tokens(windows + 2, 300, 51, 1)
     for cap in (0, 7):
@@ -378,6 +379,15 @@ def test_long_spans_on_both_sides_of_the_bulk_update(cuda_device, windows):
     B.aded_trigram_update(t, bad.cuda())
     torch.cuda.synchronize()
     assert B.aded_trigram_poll_status(t) == 1
+    st = TrigramStore()
+    st.update(bad.tolist())
+    most = st.entries()
+    assert all(max(k) < 300 and n <= most[k] for k, n in _entries_gpu(B, t).items())
+    B.aded_trigram_clear(t)                                # once it has been read, the table counts again
+    B.aded_trigram_update(t, toks.cuda())
+    st = TrigramStore()
+    st.update(toks.tolist())
+    assert _entries_gpu(B, t) == st.entries() and B.aded_trigram_poll_status(t) == 0
 
 
 @pytest.mark.parametrize("q", [(1 << 16) - 1, 1 << 16, (1 << 16) + 1, 150001])

@@ -620,14 +620,18 @@ def test_attention_with_every_number_of_splits(cuda_device, heads, nodes, ctx):
         B.aded_kv_load(kv, 0, 0, k, v)
     tokens, parents = gen.make_tree(nodes, min(6, nodes - 1), 12, shape.vocab, 97, root_token=1)
     out, n = torch.zeros(nodes, dtype=torch.int32, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    # no draft may be approved (approved rows move, and their old places then no longer hold what was attended to): the root's own
+    # token, which a first call shows, is given to none of its children
+    B.aded_verify(model, kv, H.i32(tokens), H.i32(parents), out, n)
+    first = int(out[0])
+    tokens = [(t + 1) % shape.vocab if p == 0 and t == first else t for t, p in zip(tokens, parents)]
+    B.aded_kv_set_len(kv, 0, ctx)
     B.aded_verify(model, kv, H.i32(tokens), H.i32(parents), out, n)
     torch.cuda.synchronize()
-    assert B.aded_model_poll_status(model) == 0 and int(n[0]) >= 1
+    assert B.aded_model_poll_status(model) == 0 and int(n[0]) == 1 and int(out[0]) == first
     q = B.aded_debug_read_buffer(model, 2, nodes).double().view(nodes, heads, hd)
     att = B.aded_debug_read_buffer(model, 3, nodes).double().view(nodes, heads, hd)
     kk, vv = (x.double() for x in B.aded_kv_read(kv, 0, 0, 0, ctx + nodes))
-    if int(n[0]) > 1:                       # (approved rows moved: their old places no longer hold what was attended to)
-        return
     mask = torch.zeros((nodes, ctx + nodes), dtype=torch.bool, device="cuda")
     mask[:, :ctx] = True
     for i in range(nodes):
@@ -639,6 +643,35 @@ def test_attention_with_every_number_of_splits(cuda_device, heads, nodes, ctx):
     p = torch.softmax(s.masked_fill(~mask[:, None, :], float("-inf")), dim=-1)
     want = torch.einsum("thl,hld->thd", p, vv)
     assert float((att - want).abs().max()) <= 2e-2 * float(want.abs().max())
+
+
+@pytest.mark.parametrize("rows", [129, 177, 184, 192, 193, 256, 256 + 177, 256 + 192])
+def test_greedy_tokens_of_wide_passes(cuda_device, rows):
+    """The LM head's tail (per-tile greedy candidates) in passes of more than 128 rows, 177 to 192 and a second pass of as many among
+    them: every node's token is the first of the largest logits that the same kernel gives as a matrix, bit for bit."""
+    from paper_2407_12021_b200 import binding as B
+    shape = gen.ModelShape("bf16-4x128", 1, 512, 4, 128, 1024, 4096, "bf16")
+    w = H.weights_to(gen.model_weights(shape, 99), cuda_device)
+    batch = (rows + 127) // 128
+    model = B.aded_model_create(shape, w, max_rows=rows, max_batch=batch)
+    sizes = [rows // batch + (b < rows % batch) for b in range(batch)]
+    kv = B.aded_kv_create(model, [200] * batch)
+    trees = [gen.make_tree(n, 6, 6, shape.vocab, 100 + b, root_token=b + 1) for b, n in enumerate(sizes)]
+    best = torch.full((rows,), -1, dtype=torch.int32, device="cuda")
+    out, acc = torch.zeros((batch, 128), dtype=torch.int32, device="cuda"), torch.zeros(batch, dtype=torch.int32, device="cuda")
+    B.aded_debug_capture(model, None, best)
+    B.aded_verify_batch(model, kv, [sum(sizes[:b]) for b in range(batch + 1)], H.i32([t for tr in trees for t in tr[0]]),
+                        H.i32([p for tr in trees for p in tr[1]]), out, acc)
+    torch.cuda.synchronize()
+    assert B.aded_model_poll_status(model) == 0
+    logits = B.aded_debug_gemm(model, 0, 4, B.aded_debug_read_buffer(model, 1, rows))
+    top = logits.max(dim=1, keepdim=True).values
+    assert torch.equal(best.long(), (logits == top).int().argmax(dim=1))
+    at = 0
+    for b, (tokens, parents) in enumerate(trees):
+        want = ov.accept_walk(tokens, parents, best[at:at + sizes[b]].tolist())[1]
+        assert out[b, :int(acc[b])].tolist() == want
+        at += sizes[b]
 
 
 @pytest.mark.parametrize("heads,hd,nodes,depth,ctx", [(16, 64, 45, 6, 77), (8, 64, 128, 8, 130), (8, 128, 33, 4, 65)])
