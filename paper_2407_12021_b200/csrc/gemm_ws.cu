@@ -471,7 +471,7 @@ size_t ws_slot_floats(int device, int max_n, int max_rows) {
     return ((size_t)max_n / WS_BM + ws_grid_limit(device)) * rb * WS_BM;
 }
 
-// Raises the kernel's dynamic shared-memory limit; once per process, before any launch or capture.
+// Raises the kernel's dynamic shared-memory limit on the current device; when a model is created, before any launch or capture.
 bool ws_prepare() {
     return cudaFuncSetAttribute(k_gemm_ws<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024 + 1024 + 256) == cudaSuccess &&
            cudaFuncSetAttribute(k_gemm_ws<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 112 * 1024) == cudaSuccess;

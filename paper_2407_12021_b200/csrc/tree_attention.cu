@@ -554,7 +554,7 @@ static void launch_mma(aded_model* m, aded_kv* kv, int layer, int batch, int row
     launch_mma_nw<HD, 4>(m, a, batch, splits, st);
 }
 
-// Raises the split-KV kernels' dynamic shared-memory limit; once per process, before any launch.
+// Raises the split-KV kernels' dynamic shared-memory limit on the current device; when a model is created, before any launch.
 bool attn_prepare() {
     bool ok = true;
     ok &= cudaFuncSetAttribute(k_tree_attn_mma<128, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)attn_smem<128, 4>()) == cudaSuccess;

@@ -575,7 +575,7 @@ bool attn_tc_make_kv_map(CUtensorMap* map, const void* block, uint64_t capacity,
 
 bool attn_tc_supported(const aded_model_config& c) { return c.dtype == ADED_BF16 && c.head_dim == AT_HD; }
 
-// Raises the kernel's dynamic shared-memory limit; once per process, before any launch.
+// Raises the kernel's dynamic shared-memory limit on the current device; when a model is created, before any launch.
 bool attn_tc_prepare() {
     return cudaFuncSetAttribute(k_tree_attn_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AT_SMEM) == cudaSuccess;
 }

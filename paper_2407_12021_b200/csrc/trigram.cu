@@ -38,11 +38,11 @@ __global__ void k_tg_update(TgView t, const int32_t* __restrict__ tok, int n) {
 // raises every distinct tri-gram once.  In text a few tri-grams are a large share of all windows (one in twenty of the
 // synthetic text's), and a count takes one atomic add at a time.  Sums are the same whatever the order; no count can wrap, as the
 // increments of a launch add up to fewer than 2^31.  `n` windows begin at tok[0].
-// Measured, one thread per window against this (an empty table / one that holds the span already), us: 131,000 tokens 87 / 36
-// against 88 / 39, 262,000 154 / 64 against 117 / 50, 10^6 406 / 255 against 287 / 139, 4 x 10^6 1284 / 1044 against 824 / 499:
-// the line is at BULK_MIN; below, blocks of this size leave the device idle (20,000: 37 / 19 against 68 / 35).  What bounds it
+// Measured, one thread per window against this (an empty table / one that holds the span already), us: 131,000 tokens 103 / 40
+// against 91 / 41, 262,000 183 / 64 against 134 / 54, 10^6 417 / 255 against 309 / 145, 4 x 10^6 1369 / 1106 against 944 / 562:
+// the line is at BULK_MIN; below, blocks of this size leave the device idle (20,000: 37 / 19 against 67 / 33).  What bounds it
 // then is random access to the home buckets and the index (about 7 x 10^9 windows a second), and when filling the hand-overs of
-// new entries.  Blocks of 512 threads and 1024 windows: 291 / 149 at 10^6.
+// new entries.  Blocks of 512 threads and 1024 windows (when these took 287 / 139): 291 / 149 at 10^6.
 constexpr int BULK_THREADS = 1024, BULK_WINDOWS = 2048, BULK_SLOTS = 4096, BULK_MIN = 1 << 17;
 __global__ void __launch_bounds__(BULK_THREADS) k_tg_update_bulk(TgView t, const int32_t* __restrict__ tok, int n) {
     extern __shared__ int32_t bulk_smem[];
@@ -262,11 +262,18 @@ k_tg_topk(TgView t, const int32_t* __restrict__ ctx, int q, int k, int per_block
 //   2. k_topk_lead: the leaders' rows, and those of contexts that are all in their home bucket, by the thread that has the row;
 //      the hash table is overwritten with results.
 //   3. k_topk_copy: the followers' rows, from their leaders'.
-// Needs two words per row (k >= 2).  The table has at least q slots and at most half of the queries' words; a query that finds
-// no slot within MARK_PROBES answers itself.
-// Taken from TOPK_BULK queries on.  Measured, 2^20 queries on the table of a 16-million-token text, k = 4: 183 us (54 + 92 + 30 and a
-// memset; the per-block kernel above: 780); 65,536 queries on that of 10^6 tokens, k = 8: 54 us (99).  What bounds it: random
-// access in the first, and in the second the warps' chains of reads, no longer the entries' bytes.
+// Needs two words per row (k >= 2).  The table takes the largest power of two of the q k count words, so between half and all of
+// them: it has at least q slots, and with k = 2 and many distinct contexts it can fill up; a query that finds no slot within
+// MARK_PROBES answers itself.
+// Measured, 2^20 queries on the table of a 16-million-token text, k = 4: 183 us (54 + 92 + 30 and a memset; the per-block kernel
+// above: 780).  What bounds it: random access in the first, and in the second the warps' chains of reads, no longer the entries' bytes.
+// Taken from TOPK_BULK queries on, from where it is the faster one on every table measured.  k = 4, the per-block kernel against this, us:
+//   queries                    2^12        2^13        2^14        2^15        2^16        2^17
+//   text of 10^5 tokens      25 /  37    28 /  37    30 /  37    38 /  37    48 /  39    72 /  42
+//            10^6            44 /  37    55 /  38    65 /  39    77 /  42    96 /  44   130 /  49
+//            1.6 x 10^7     139 /  47   165 /  48   187 /  49   206 /  56   235 /  62   295 /  74
+// (k = 2 and 8 alike: within 10 us of it on either side.)  Larger tables cross far earlier, but a call does not know how long its
+// contexts are.
 constexpr int MARK_OWN = -2, MARK_PROBES = 16, TOPK_BULK = 1 << 16;
 __device__ __forceinline__ int mark_leader(int q) { return MARK_OWN - 1 - q; }       // (its own inverse)
 
