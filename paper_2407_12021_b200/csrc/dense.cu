@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(1024) k_add_rmsnorm(T* __restrict__ h, const f
     }
 }
 
-// y[r, n] = sum_k x[r, k] * w[n, k] in fp32.  A block computes BM rows x 32 columns: the operands of a chunk of k are staged in
+// y[r, n] = sum_k x[r, k] * w[n, k] in fp32.  A block computes BM rows x BN columns: the operands of a chunk of k are staged in
 // shared memory as they lie (rows padded by four words: the lanes of a warp then read different banks), 4 x 4 outputs per
 // thread, four k per step; the threads beyond one per 4 x 4 split the chunk's k among them, and their sums are added at the end
 // in a fixed order.
@@ -83,7 +83,7 @@ __global__ void __launch_bounds__(1024) k_add_rmsnorm(T* __restrict__ h, const f
 // that fits -- one round of loads, of which the weights' are issued before the previous kernel has finished -- and the split of
 // k keeps eight warps busy on 16 rows.  (Blocks of 64 x 64 outputs with 16 k at a time took 23 to 65 us per GEMM of the 256-wide
 // fp32 model at 16 rows, two barriers and one exposed load per 16 k; this: 3.9 to 6.5 us.)
-constexpr int GP_BN = 32, GP_THREADS = 256;
+constexpr int GP_THREADS = 256;
 template <typename T, bool VEC>
 __device__ __forceinline__ float4 gp_load4(const T* p) {
     if (!VEC) return make_float4(to_f32(p[0]), to_f32(p[1]), to_f32(p[2]), to_f32(p[3]));
@@ -91,18 +91,18 @@ __device__ __forceinline__ float4 gp_load4(const T* p) {
     return unpack4_bf16(*reinterpret_cast<const uint2*>(p));
 }
 
-template <typename T, int BM, bool VEC>
+template <typename T, int BM, int BN, bool VEC>
 __global__ void __launch_bounds__(GP_THREADS) k_gemm_plain(const T* __restrict__ x, const T* __restrict__ w,
                                                            float* __restrict__ y, int rows, int n, int k, int chunk,
                                                            const int32_t* status, int trace_kind) {
     pdl_launch_dependents();
-    constexpr int RG = BM / 4, SLICES = GP_THREADS / (8 * RG), STEP = 4 * SLICES;
+    constexpr int RG = BM / 4, CG = BN / 4, SLICES = GP_THREADS / (CG * RG), STEP = 4 * SLICES;
     extern __shared__ __align__(16) float gp_smem[];
     const int ld = (chunk + 31) / 32 * 32 + 4;
-    float* sw = gp_smem;                       // [GP_BN][ld]
-    float* sx = gp_smem + GP_BN * ld;          // [BM][ld]
-    const int n0 = blockIdx.x * GP_BN, r0 = blockIdx.y * BM;
-    const int cg = threadIdx.x & 7, rg = (threadIdx.x >> 3) % RG, slice = threadIdx.x / (8 * RG);
+    float* sw = gp_smem;                       // [BN][ld]
+    float* sx = gp_smem + BN * ld;             // [BM][ld]
+    const int n0 = blockIdx.x * BN, r0 = blockIdx.y * BM;
+    const int cg = threadIdx.x % CG, rg = threadIdx.x / CG % RG, slice = threadIdx.x / (CG * RG);
     // rows [from, from + count) of m, columns [k0, k0 + len), zero beyond `limit` rows and beyond k (k % 4 == 0)
     auto stage = [&](float* dst, const T* m, int from, int count, int limit, int k0, int len) {
         const int quads = len / 4;
@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(GP_THREADS) k_gemm_plain(const T* __restrict__
     for (int k0 = 0; k0 < k; k0 += chunk) {
         const int here = k - k0 < chunk ? k - k0 : chunk, len = (here + STEP - 1) / STEP * STEP;      // (chunk % STEP == 0 unless it is all of k)
         if (k0 > 0) __syncthreads();
-        stage(sw, w, n0, GP_BN, n, k0, len);
+        stage(sw, w, n0, BN, n, k0, len);
         if (k0 == 0) {
             pdl_wait();
             if (first_thread_of_grid()) trace_mark(status, trace_kind);
@@ -140,7 +140,7 @@ __global__ void __launch_bounds__(GP_THREADS) k_gemm_plain(const T* __restrict__
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 a[i] = *reinterpret_cast<const float4*>(sx + (size_t)(rg + RG * i) * ld + kk);
-                b[i] = *reinterpret_cast<const float4*>(sw + (size_t)(cg + 8 * i) * ld + kk);
+                b[i] = *reinterpret_cast<const float4*>(sw + (size_t)(cg + CG * i) * ld + kk);
             }
 #pragma unroll
             for (int i = 0; i < 4; ++i)
@@ -154,17 +154,17 @@ __global__ void __launch_bounds__(GP_THREADS) k_gemm_plain(const T* __restrict__
         }
     }
     __syncthreads();
-    float* part = gp_smem;                     // [SLICES][BM][GP_BN]
+    float* part = gp_smem;                     // [SLICES][BM][BN]
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) part[(slice * BM + rg + RG * i) * GP_BN + cg + 8 * j] = acc[i][j];
+        for (int j = 0; j < 4; ++j) part[(slice * BM + rg + RG * i) * BN + cg + CG * j] = acc[i][j];
     __syncthreads();
-    for (int o = threadIdx.x; o < BM * GP_BN; o += GP_THREADS) {
+    for (int o = threadIdx.x; o < BM * BN; o += GP_THREADS) {
         float sum = part[o];
 #pragma unroll
-        for (int sl = 1; sl < SLICES; ++sl) sum += part[sl * BM * GP_BN + o];
-        const int r = r0 + o / GP_BN, c = n0 + o % GP_BN;
+        for (int sl = 1; sl < SLICES; ++sl) sum += part[sl * BM * BN + o];
+        const int r = r0 + o / BN, c = n0 + o % BN;
         if (r < rows && c < n) y[(size_t)r * n + c] = sum;
     }
 }
@@ -304,35 +304,39 @@ void launch_add_rmsnorm(aded_model* m, const GemmOut& y, const void* gain, cudaS
 
 constexpr int GP_SMEM = 160 * 1024, GP_CHUNK = 256;
 
-template <typename T, int BM>
+template <typename T, int BM, int BN>
 static void launch_gemm_plain_bm(aded_model* m, const T* x, const T* w, float* y, int rows, int n, int k, int trace_kind, cudaStream_t st) {
     // all of k at once where it fits (and only few blocks run), else pieces that leave room for more than one block per SM
-    auto bytes = [](int c) { return (size_t)(GP_BN + BM) * ((c + 31) / 32 * 32 + 4) * sizeof(float); };
-    const int chunk = k <= GP_CHUNK || (BM == 16 && bytes(k) <= GP_SMEM) ? k : GP_CHUNK;
+    auto bytes = [](int c) { return (size_t)(BN + BM) * ((c + 31) / 32 * 32 + 4) * sizeof(float); };
+    const int piece = BN == 32 ? GP_CHUNK : sizeof(T) == 4 ? GP_CHUNK / 2 : GP_CHUNK / 4;
+    const int chunk = k <= piece || (BM == 16 && bytes(k) <= GP_SMEM) ? k : piece;
     const size_t sums = (size_t)GP_THREADS * 16 * sizeof(float);       // the partial sums take the operands' place
     const size_t smem = bytes(chunk) > sums ? bytes(chunk) : sums;
     const bool vec = k % 4 == 0 && (reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(w)) % (4 * sizeof(T)) == 0;
-    launch_k(vec ? k_gemm_plain<T, BM, true> : k_gemm_plain<T, BM, false>, dim3((n + GP_BN - 1) / GP_BN, (rows + BM - 1) / BM), GP_THREADS, smem, st,
+    launch_k(vec ? k_gemm_plain<T, BM, BN, true> : k_gemm_plain<T, BM, BN, false>, dim3((n + BN - 1) / BN, (rows + BM - 1) / BM), GP_THREADS, smem, st,
              x, w, y, rows, n, k, chunk, m->status, trace_kind);
 }
 
 template <typename T>
 static void launch_gemm_plain(aded_model* m, const T* x, const T* w, float* y, int rows, int n, int k, int trace_kind, cudaStream_t st) {
     // The fewest rows per block that still leave no more than about two waves of blocks: more rows per block read the weights fewer
-    // times from L2, fewer spread a small GEMM over more SMs.
-    const long long cols = (n + GP_BN - 1) / GP_BN, limit = 2ll * ws_grid_limit(m->device);
-    if (cols * ((rows + 15) / 16) <= limit) launch_gemm_plain_bm<T, 16>(m, x, w, y, rows, n, k, trace_kind, st);
-    else if (cols * ((rows + 31) / 32) <= limit) launch_gemm_plain_bm<T, 32>(m, x, w, y, rows, n, k, trace_kind, st);
-    else launch_gemm_plain_bm<T, 64>(m, x, w, y, rows, n, k, trace_kind, st);
+    // times from L2, fewer spread a small GEMM over more SMs.  What is larger than that takes blocks of 64 x 64, which stage each
+    // operand for twice as many outputs as 64 x 32, a thread per 4 x 4 of them over all of k, and pieces of k that let several blocks
+    // share an SM.  Measured, the five projections of a layer and LM head of width 4096, us: bf16, 256 rows 7560 (9830 with 64 x 32
+    // and 256 k at a time; 512 rows 13500 and 19200), fp32 6450 (7300; 12400 and 14000).
+    const long long cols = (n + 31) / 32, limit = 2ll * ws_grid_limit(m->device);
+    if (cols * ((rows + 15) / 16) <= limit) launch_gemm_plain_bm<T, 16, 32>(m, x, w, y, rows, n, k, trace_kind, st);
+    else if (cols * ((rows + 31) / 32) <= limit) launch_gemm_plain_bm<T, 32, 32>(m, x, w, y, rows, n, k, trace_kind, st);
+    else launch_gemm_plain_bm<T, 64, 64>(m, x, w, y, rows, n, k, trace_kind, st);
 }
 
 template <typename T>
 static bool gemm_plain_prepare_t() {
     bool ok = true;
     auto set = [&](auto* f) { ok = ok && cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, GP_SMEM) == cudaSuccess; };
-    set(k_gemm_plain<T, 16, true>); set(k_gemm_plain<T, 16, false>);
-    set(k_gemm_plain<T, 32, true>); set(k_gemm_plain<T, 32, false>);
-    set(k_gemm_plain<T, 64, true>); set(k_gemm_plain<T, 64, false>);
+    set(k_gemm_plain<T, 16, 32, true>); set(k_gemm_plain<T, 16, 32, false>);
+    set(k_gemm_plain<T, 32, 32, true>); set(k_gemm_plain<T, 32, 32, false>);
+    set(k_gemm_plain<T, 64, 64, true>); set(k_gemm_plain<T, 64, 64, false>);
     return ok;
 }
 // (For the models that use it: the first call on a kernel loads it, which takes the creation of a model milliseconds.)

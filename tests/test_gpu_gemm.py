@@ -84,10 +84,10 @@ def test_wide_passes_of_every_padded_size(cuda_device, rows):
         _check(B, model, w, which, rows, 46)
 
 
-@pytest.mark.parametrize("dtype,rows", [("f32", 1), ("f32", 16), ("f32", 17), ("f32", 128), ("f32", 300), ("bf16", 33), ("bf16", 128)])
+@pytest.mark.parametrize("dtype,rows", [("f32", 1), ("f32", 16), ("f32", 17), ("f32", 128), ("f32", 300), ("bf16", 33), ("bf16", 128), ("bf16", 300)])
 @pytest.mark.parametrize("offset", [0, 1])
 def test_plain_gemm(cuda_device, dtype, rows, offset):
-    """Models the tensor-core GEMM does not take: blocks of 16, 32 and 64 rows, k in one chunk and in several, a ragged number of
+    """Models the tensor-core GEMM does not take: blocks of 16, 32 and 64 rows, k in one chunk and in several (pieces of 64, 128 and 256), a ragged number of
     columns, matrices that do not start on a 16-byte boundary.  Bound: fp32 sums of k products in a fixed order are off by at
     most k 2^-24 of the sum of their magnitudes, and by far less in the mean; 4e-6 of it is the bound of the tests above."""
     shape = gen.ModelShape("plain", 1, 1088, 17, 64, 1360, 1000, dtype)
