@@ -80,54 +80,99 @@ __global__ void __launch_bounds__(BULK_THREADS) k_tg_update_bulk(TgView t, const
 
 // Every stored tri-gram with count >= min_count as (a, b, c) and its count, in no particular order;
 // *n_out counts all of them, only the first `max_entries` are written.  A warp takes 32 home buckets at a time, a lane each,
-// and then together the further entries of those that have any.
-__device__ __forceinline__ void tg_export_one(unsigned long long key, int32_t tok, uint32_t cnt, bool take, int lane, int32_t* keys, uint32_t* counts,
-                                              unsigned long long max_entries, unsigned long long* n_out) {
-    const unsigned m = __ballot_sync(0xffffffffu, take);
-    if (m == 0) return;
+// and then together the further entries of those that have any.  The places of N entries per lane are taken with one atomic, and
+// their reads do not depend on one another, and contexts of more than EXPORT_LONG entries are left to all warps of the block: with one atomic
+// per 32 entries and a warp per context the one with the most continuations -- 7254 of them in the text of 10^6 tokens -- was a chain
+// of 227 round trips, and a full export of that table (two passes) 631 us instead of 187.
+constexpr int EXPORT_THREADS = 256, EXPORT_BATCH = 8, EXPORT_MAX_LONG = 64;
+constexpr uint32_t EXPORT_LONG = 512;
+template <int N>
+__device__ __forceinline__ void tg_export_some(unsigned long long key, const TgSlot (&s)[N], uint32_t min_count, int lane, int32_t* keys, uint32_t* counts,
+                                               unsigned long long max_entries, unsigned long long* n_out) {
+    unsigned m[N];
+    int n = 0;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        m[i] = __ballot_sync(0xffffffffu, s[i].tok >= 0 && s[i].cnt >= min_count && s[i].cnt != 0);
+        n += __popc(m[i]);
+    }
+    if (n == 0) return;
     unsigned long long at = 0;
-    if (lane == 0) at = atomicAdd(n_out, (unsigned long long)__popc(m));
-    at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << lane) - 1u));
-    if (take && at < max_entries) {
-        keys[3 * at + 0] = (int32_t)(key >> 32);
-        keys[3 * at + 1] = (int32_t)(key & 0xFFFFFFFFu);
-        keys[3 * at + 2] = tok;
-        counts[at] = cnt;
+    if (lane == 0) at = atomicAdd(n_out, (unsigned long long)n);
+    at = __shfl_sync(0xffffffffu, at, 0);
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        const unsigned long long mine = at + __popc(m[i] & ((1u << lane) - 1u));
+        if ((m[i] >> lane & 1u) && mine < max_entries) {
+            keys[3 * mine + 0] = (int32_t)(key >> 32);
+            keys[3 * mine + 1] = (int32_t)(key & 0xFFFFFFFFu);
+            keys[3 * mine + 2] = s[i].tok;
+            counts[mine] = s[i].cnt;
+        }
+        at += __popc(m[i]);
     }
 }
-__global__ void k_tg_export(TgView t, uint32_t min_count, int32_t* __restrict__ keys, uint32_t* __restrict__ counts,
-                            unsigned long long max_entries, unsigned long long* n_out) {
-    const int lane = threadIdx.x & 31;
+// A context's entries beyond its home bucket, `parts` warps taking turns.
+__device__ __forceinline__ void tg_export_extents(const TgView& t, const TgWalk& w, unsigned long long key, int part, int parts, uint32_t min_count, int lane,
+                                                  int32_t* keys, uint32_t* counts, unsigned long long max_entries, unsigned long long* n_out) {
+    for (uint32_t i0 = (uint32_t)part * 32 * EXPORT_BATCH; i0 < w.n; i0 += (uint32_t)parts * 32 * EXPORT_BATCH) {
+        TgSlot s[EXPORT_BATCH];
+#pragma unroll
+        for (int j = 0; j < EXPORT_BATCH; ++j) {
+            const uint32_t p = i0 + 32 * j + lane, m = p / TG_UNIT;
+            const int x = tg_extent(m);
+            const uint32_t base = __shfl_sync(0xffffffffu, w.extent, x & 31);
+            s[j] = TgSlot{-1, 0u};
+            if (p < w.n && base != 0) s[j] = t.pool[((size_t)(base - 1) + (m + 1 - (1u << x))) * TG_UNIT + p % TG_UNIT];
+        }
+        tg_export_some(key, s, min_count, lane, keys, counts, max_entries, n_out);
+    }
+}
+__global__ void __launch_bounds__(EXPORT_THREADS) k_tg_export(TgView t, uint32_t min_count, int32_t* __restrict__ keys, uint32_t* __restrict__ counts,
+                                                              unsigned long long max_entries, unsigned long long* n_out) {
+    __shared__ uint32_t s_home[EXPORT_MAX_LONG];
+    __shared__ int s_long;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
+    if (threadIdx.x == 0) s_long = 0;
+    __syncthreads();
     for (uint32_t g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; g < (t.n_home + 31) / 32; g += warps) {
         const uint32_t mine = g * 32 + lane;
-        const unsigned long long key = mine < t.n_home ? t.buckets[mine].key : TG_EMPTY;
+        const uint4 head = mine < t.n_home ? *reinterpret_cast<const uint4*>(t.buckets + mine) : make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0u, 0u);
+        const unsigned long long key = (unsigned long long)head.y << 32 | head.x;
         const bool used = key != TG_EMPTY;
         if (!__any_sync(0xffffffffu, used)) continue;
-        for (int e = 0; e < 6; ++e) {
-            const TgSlot s = used ? t.buckets[mine].e[e] : TgSlot{-1, 0u};
-            tg_export_one(key, s.tok, s.cnt, s.tok >= 0 && s.cnt >= min_count && s.cnt != 0, lane, keys, counts, max_entries, n_out);
-        }
-        for (unsigned more = __ballot_sync(0xffffffffu, used && t.buckets[mine].more != 0); more; more &= more - 1) {
+        TgSlot home[6];
+#pragma unroll
+        for (int e = 0; e < 6; ++e) home[e] = used ? t.buckets[mine].e[e] : TgSlot{-1, 0u};
+        tg_export_some(key, home, min_count, lane, keys, counts, max_entries, n_out);
+        for (unsigned more = __ballot_sync(0xffffffffu, used && head.z != 0); more; more &= more - 1) {
             const int src = __ffs((int)more) - 1;
-            const TgWalk w = tg_open(t, g * 32 + src, lane);
+            TgWalk w;
+            w.part = make_uint4(0u, 0u, __shfl_sync(0xffffffffu, head.z, src), __shfl_sync(0xffffffffu, head.w, src));
+            tg_open_extents(t, w, lane);
             const unsigned long long k = __shfl_sync(0xffffffffu, key, src);
             if (w.chain)
                 tg_each_chained(t, w.chain, lane, [&](uint4 v) {
-                    for (int h = 0; h < 2; ++h) {
-                        const TgSlot s = h ? TgSlot{(int32_t)v.z, v.w} : TgSlot{(int32_t)v.x, v.y};
-                        tg_export_one(k, s.tok, s.cnt, s.tok >= 0 && s.cnt >= min_count && s.cnt != 0, lane, keys, counts, max_entries, n_out);
-                    }
+                    const TgSlot two[2] = {TgSlot{(int32_t)v.x, v.y}, TgSlot{(int32_t)v.z, v.w}};
+                    tg_export_some(k, two, min_count, lane, keys, counts, max_entries, n_out);
                 });
-            for (uint32_t i0 = 0; i0 < w.n; i0 += 32) {
-                const uint32_t m = (i0 + lane) / TG_UNIT;
-                const int x = tg_extent(m);
-                const uint32_t base = __shfl_sync(0xffffffffu, w.extent, x & 31);
-                TgSlot s = {-1, 0u};
-                if (i0 + lane < w.n && base != 0) s = t.pool[((size_t)(base - 1) + (m + 1 - (1u << x))) * TG_UNIT + (i0 + lane) % TG_UNIT];
-                tg_export_one(k, s.tok, s.cnt, s.tok >= 0 && s.cnt >= min_count && s.cnt != 0, lane, keys, counts, max_entries, n_out);
+            if (w.n > EXPORT_LONG) {
+                int place = 0;
+                if (lane == 0) place = atomicAdd(&s_long, 1);
+                place = __shfl_sync(0xffffffffu, place, 0);
+                if (place < EXPORT_MAX_LONG) {
+                    if (lane == 0) s_home[place] = g * 32 + src;
+                    continue;
+                }
             }
+            tg_export_extents(t, w, k, 0, 1, min_count, lane, keys, counts, max_entries, n_out);
         }
+    }
+    __syncthreads();
+    for (int i = 0; i < min(s_long, EXPORT_MAX_LONG); ++i) {
+        const unsigned long long key = t.buckets[s_home[i]].key;
+        tg_export_extents(t, tg_open(t, s_home[i], lane), key, warp, EXPORT_THREADS / 32, min_count, lane, keys, counts, max_entries, n_out);
     }
 }
 
@@ -1183,7 +1228,7 @@ aded_status aded_trigram_export(const aded_trigram* t, uint32_t min_count, int32
     unsigned long long n = 0;
     ADED_CUDA_TRY(cudaMemsetAsync(t->stats_dev, 0, sizeof n, st));
     note_launch();
-    k_tg_export<<<1024, 256, 0, st>>>(t->view, min_count, keys_dev, counts_dev, max_entries, t->stats_dev);
+    k_tg_export<<<1024, EXPORT_THREADS, 0, st>>>(t->view, min_count, keys_dev, counts_dev, max_entries, t->stats_dev);
     ADED_CUDA_TRY(cudaMemcpyAsync(&n, t->stats_dev, sizeof n, cudaMemcpyDeviceToHost, st));
     ADED_CUDA_TRY(cudaStreamSynchronize(st));
     *n_out_host = n;

@@ -474,3 +474,26 @@ def test_table_without_room_for_pool_and_index(cuda_device, tmp_path):
     for span in (text, text[:5000], text[5000:5200]):
         st.update(span)
     assert dict(answers[1][0]) == st.entries() and answers[1][-1] == 0
+
+
+@pytest.mark.parametrize("entries", [518, 519, 600, 2600])
+def test_export_with_more_long_contexts_than_a_block_shares(cuda_device, entries):
+    """Contexts of more than 512 entries beyond their home bucket are exported by all warps of a block, up to 64 of them per block; here
+    two blocks hold 200, just below, at and above the line and over several rounds."""
+    from paper_2407_12021_b200 import binding as B
+    a = torch.arange(200, device="cuda").repeat_interleave(entries)
+    c = torch.arange(entries, device="cuda").repeat(200)
+    rows = torch.stack([a, a + 1000, (c * 7 + a) % 4999], dim=1).to(torch.int32).contiguous()
+    counts = (1 + c % 3).to(torch.int32)
+    t = B.aded_trigram_create(5000, log2_buckets=9, overflow_buckets=200 * ((entries + 5) // 6))
+    B.aded_trigram_import(t, rows, counts)
+    torch.cuda.synchronize()
+    assert B.aded_trigram_poll_status(t) == 0
+
+    def packed(r):
+        return ((r[:, 0].long() * 5000 + r[:, 1].long()) * 5000 + r[:, 2].long())
+
+    for least in (0, 2, 4):
+        keys, got = B.aded_trigram_export(t, least)
+        want = packed(rows)[counts >= least] * 4 + counts[counts >= least]
+        assert torch.equal((packed(keys) * 4 + got).sort().values, want.sort().values)
