@@ -13,10 +13,14 @@
 namespace aded {
 
 // Empty home buckets: one 16-byte part per thread and step (header, or two entries), so that a warp's stores are whole lines
-// (a thread per bucket wrote 128 MB in 52 us; with the index, 192 MB: 77 us then, 45 now).
-__global__ void k_tg_init(uint4* b, size_t parts) {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < parts; i += (size_t)gridDim.x * blockDim.x)
+// (a thread per bucket wrote 128 MB in 52 us; with the index, 192 MB: 77 us then, 43 now).  Index and counters are cleared by the same
+// launch: for a small table every further operation on the stream costs as much as its clearing (22 us with two more, 17 now).
+__global__ void k_tg_init(uint4* b, size_t parts, uint4* index, size_t index_parts, uint32_t* used) {
+    const size_t first = blockIdx.x * (size_t)blockDim.x + threadIdx.x, step = (size_t)gridDim.x * blockDim.x;
+    if (first < 2) used[first] = 0;
+    for (size_t i = first; i < parts; i += step)
         b[i] = (i & 3) == 0 ? make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0u, 0u) : make_uint4(0xFFFFFFFFu, 0u, 0xFFFFFFFFu, 0u);
+    for (size_t i = first; i < index_parts; i += step) index[i] = make_uint4(0u, 0u, 0u, 0u);
 }
 
 // Algorithm 2, one thread per window.  Duplicate windows inside one call are independent atomic
@@ -934,9 +938,11 @@ static constexpr int STEP_INTS = STEP_FILL + DRAFT_MAX_FILLER;
 // An empty table: home buckets and index.  The pool needs no clearing: see tg_place.
 static aded_status tg_reset(aded_trigram* t, cudaStream_t st) {
     const size_t buckets = (size_t)t->view.n_home + (t->view.chain ? t->view.n_over : 0);     // (chain buckets follow the home buckets)
-    k_tg_init<<<2048, 512, 0, st>>>(reinterpret_cast<uint4*>(t->view.buckets), buckets * (sizeof(Bucket) / sizeof(uint4)));
-    if (t->view.index) ADED_CUDA_TRY(cudaMemsetAsync(t->view.index, 0, (size_t)(t->view.index_mask + 1) * sizeof(TgIndexSlot), st));
-    ADED_CUDA_TRY(cudaMemsetAsync(t->view.used, 0, 2 * sizeof(uint32_t), st));
+    static_assert(sizeof(TgIndexSlot) == sizeof(uint4), "a slot per store");
+    const size_t parts = buckets * (sizeof(Bucket) / sizeof(uint4)), slots = t->view.index ? (size_t)(t->view.index_mask + 1) : 0;
+    const size_t blocks = ((parts > slots ? parts : slots) + 511) / 512;
+    k_tg_init<<<(unsigned)(blocks < 2048 ? blocks : 2048), 512, 0, st>>>(reinterpret_cast<uint4*>(t->view.buckets), parts, reinterpret_cast<uint4*>(t->view.index),
+                                                                       slots, t->view.used);
     ADED_CUDA_TRY(cudaGetLastError());
     return ADED_OK;
 }
