@@ -234,6 +234,11 @@ aded_status aded_trace_end(aded_model* m, uint64_t* out_ns_host, int32_t* out_ki
  * re-run any single layer from the inputs the device actually had.  Parity checks only. */
 aded_status aded_debug_capture_hidden(aded_model* m, void* hidden_dev);
 
+/* The kernel for calls of many rows divides v by 1 + exp(-v) (SwiGLU) without the division operator's branches.  Compares its
+ * quotient with the operator's for `count` (1 .. 2^32) floats whose bit patterns run from `first` on, as far as they are in the
+ * range it takes, and adds the number of those that differ to *differ_dev.  Asynchronous. */
+aded_status aded_debug_silu_check(uint32_t first, uint64_t count, uint64_t* differ_dev, void* stream);
+
 /* Failure-path check ("every device-side wait is bounded", see Conventions): runs one of the library's two
  * kinds of device-side wait -- which = 0: the mbarrier wait of the tensor-core kernels, 1: the wait at an
  * arrival counter of the LM head's tail -- on something that never happens, with a limit of limit_cycles

@@ -26,7 +26,7 @@ STATUS_NAMES = {0: "ADED_OK", 1: "ADED_ERR_INVALID_ARG", 2: "ADED_ERR_BAD_TREE",
 EXPORTS = [
     "aded_model_create", "aded_model_destroy", "aded_kv_create", "aded_kv_destroy", "aded_kv_len",
     "aded_kv_load", "aded_kv_set_len", "aded_kv_read", "aded_append", "aded_verify", "aded_verify_batch", "aded_verify_host",
-    "aded_debug_capture", "aded_debug_capture_hidden", "aded_debug_gemm", "aded_debug_read_buffer", "aded_greedy_noalloc", "aded_profile_begin", "aded_profile_end", "aded_trace_begin", "aded_trace_end", "aded_debug_attention_kernel", "aded_debug_weight_layout", "aded_debug_wait_timeout", "aded_launch_count", "aded_model_poll_status", "aded_trigram_create", "aded_trigram_destroy",
+    "aded_debug_capture", "aded_debug_capture_hidden", "aded_debug_gemm", "aded_debug_read_buffer", "aded_greedy_noalloc", "aded_profile_begin", "aded_profile_end", "aded_trace_begin", "aded_trace_end", "aded_debug_attention_kernel", "aded_debug_weight_layout", "aded_debug_wait_timeout", "aded_debug_silu_check", "aded_launch_count", "aded_model_poll_status", "aded_trigram_create", "aded_trigram_destroy",
     "aded_trigram_update", "aded_trigram_update_host", "aded_trigram_topk", "aded_trigram_topk_host",
     "aded_trigram_get", "aded_trigram_stats", "aded_trigram_poll_status", "aded_draft_tree", "aded_decode_step",
     "aded_decode_step_host", "aded_verify_sampled", "aded_sample_tokens", "aded_trigram_export",
@@ -325,6 +325,11 @@ def aded_trace_end(model: Model, max_marks: int = 16384):
 
 def aded_debug_wait_timeout(model: Model, which: int, limit_cycles: int) -> None:
     _check(_lib.aded_debug_wait_timeout(model.handle, c_int32(which), c_uint64(limit_cycles), _stream()), "aded_debug_wait_timeout")
+
+
+def aded_debug_silu_check(first: int, count: int, differ) -> None:
+    """differ: one int64 on the device, to which the number of quotients that differ is added."""
+    _check(_lib.aded_debug_silu_check(c_uint32(first), c_uint64(count), c_void_p(differ.data_ptr()), _stream()), "aded_debug_silu_check")
 
 
 def aded_debug_attention_kernel(model: Model, which: int) -> None:

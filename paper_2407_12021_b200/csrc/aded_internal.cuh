@@ -87,19 +87,28 @@ __device__ __forceinline__ bool first_thread_of_grid() {
     return threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0;
 }
 
+// (`cluster`: blocks of a cluster along x)
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
+inline cudaError_t launch_clusters(int cluster, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+}
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
+    return launch_clusters(1, kernel, grid, block, smem, st, args...);
 }
 
 // ---- per-call row bookkeeping (device arrays sized for max_rows / max_batch) --------------
@@ -233,6 +242,28 @@ struct WsEpilogue {
     uint32_t epoch;              //   n x epoch arrivals (modulo 2^32)
     float* cand_val; int32_t* cand_idx;   // best logit and its column per (row, tile): [R][n_tiles]
 };
+
+// What the GEMM for calls of many rows (gemm_many.cu) does with its complete results.
+enum { MANY_PLAIN = 0, MANY_ROPE = 1, MANY_RESIDUAL = 2, MANY_SWIGLU = 3, MANY_ARGMAX = 4 };
+struct ManyEpilogue {
+    int kind;
+    float* out;              // PLAIN: [tile][rb][128] fp32
+    int rb;
+    bf16* h;                 // RESIDUAL: h += y
+    bf16* act;               // SWIGLU
+    float* cand_val;         // ARGMAX: best logit of 32 columns and its column, [R][vocab / 32]
+    int32_t* cand_idx;
+    // ROPE: rotated q, and k and v to the cache (as k_rope_kv_ws)
+    const float* cs;
+    const float* sn;
+    bf16* q;
+    char* const* base;
+    const int32_t* cap;
+    const int32_t* len;
+    const int32_t* row_seq;
+    const int32_t* row_local;
+    int layer, heads, hd, d;
+};
 }  // namespace aded
 
 struct aded_kv {
@@ -298,7 +329,12 @@ struct aded_model {
     std::vector<CUtensorMap> ws_maps;   // per layer: wqkv, wo, wgu, wd; then lm_head
     CUtensorMap ws_x_maps[3][16];       // x, attn, act in boxes of 16, 32, .. 256 rows: the rows of a pass are one request
     std::vector<void*> ws_tiled;        // the weight matrices re-tiled for the tensor-core GEMM (same indices as ws_maps), model-owned
+    std::vector<CUtensorMap> ws_tiled_maps, ws_half_maps;   // calls of many rows: descriptors of the re-tiled copies, and of the caller's matrices, half a tile per box
     bool ws_use_tiled;                  // GEMMs read the re-tiled copies (else the caller's matrices through ws_maps)
+    bool many_ok;                       // the kernel for calls of many rows can be used
+    aded::TileRef* many_tiles;          // "tile t is slot t, complete" (aded_debug_gemm)
+    uint32_t* many_flags;               // their hand-over flags (MANY_FLAGS)
+    uint32_t many_epoch;                // launches so far
     float* ws_slots;                    // partial result tiles (see gemm_out.cuh)
     aded::TileRef* ws_tiles[5];         // contributor tables of the wqkv, wo, wgu, wd and LM-head results
     int ws_contributors[5];             // most contributors of any of their tiles
@@ -348,6 +384,11 @@ bool gemm_plain_prepare(bool bf16_model);
 // `epi_mode` (WS_EPI_*): whether the tensor-core kernel's tail also leaves per-tile greedy candidates (LM head).
 // A call is worked in passes of gemm_pass_rows rows: the result of rows [row0, row0 + rows), to be consumed before the next.
 int gemm_pass_rows(const aded_model* m, int rows);
+// The same for all rows of a call of many rows, result and all, where gemm_is_many.
+bool gemm_is_many(const aded_model* m, int rows, int n, int k);
+void launch_gemm_many(aded_model* m, int w_map, int x_map, int rows, int n, int k, const ManyEpilogue& epi, int trace_kind, cudaStream_t st);
+// The norm alone (h is complete).
+void launch_rmsnorm(aded_model* m, int rows, const void* gain, cudaStream_t st);
 GemmOut launch_gemm(aded_model* m, int w_map, int x_map, const void* x, const void* w, float* y, int row0, int rows, int n, int k,
                     int epi_mode, int trace_kind, cudaStream_t st);
 void launch_rope_kv(aded_model* m, aded_kv* kv, const GemmOut& qkv, int layer, cudaStream_t st);
@@ -366,6 +407,7 @@ void launch_pick_accept(aded_model* m, aded_kv* kv, int batch, const float* cand
 
 // gemm_ws.cu
 bool ws_make_map(CUtensorMap* map, const void* ptr, uint64_t rows, uint64_t cols, uint32_t box_rows);
+bool ws_make_tiled_map(CUtensorMap* map, const void* ptr, uint64_t units);
 bool ws_supported(int n, int k);
 bool ws_prepare();
 bool attn_prepare();
@@ -376,6 +418,12 @@ cudaError_t ws_retile(const void* w, void* out, int n, int k, cudaStream_t st);
 cudaError_t ws_launch(const CUtensorMap& map_w, const void* w_tiled, const CUtensorMap& map_x, int rows, int row0,
                       int n, int k,
                       float* slots, int32_t* status, const WsEpilogue& epi, int trace_kind, int device, bool one_per_sm, cudaStream_t st);
+// gemm_many.cu: calls of many rows
+bool many_prepare();
+int many_block_rows(int device, int rows, int n, int k);      // 0: not a call for it
+cudaError_t many_silu_check(uint32_t first, uint64_t count, uint64_t* differ, cudaStream_t st);
+cudaError_t many_launch(const CUtensorMap& map_w, bool tiled, const CUtensorMap* x_maps, int rows, int block_rows, int n, int k, int ws_ctas,
+                        float* partial, uint32_t* flags, uint32_t epoch, int32_t* status, const ManyEpilogue& epi, int trace_kind, int device, cudaStream_t st);
 enum { WS_MAP_QKV = 0, WS_MAP_O = 1, WS_MAP_GU = 2, WS_MAP_D = 3 };   // per-layer map order
 enum { WS_X = 0, WS_X_ATTN = 1, WS_X_ACT = 2 };
 cudaError_t ws_wait_probe(int which, long long limit_cycles, const uint32_t* never_raised, int32_t* status, cudaStream_t st);

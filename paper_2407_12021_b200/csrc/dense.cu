@@ -345,6 +345,21 @@ bool gemm_plain_prepare(bool bf16_model) { return bf16_model ? gemm_plain_prepar
 // The tensor-core GEMM runs once per 128 rows (256 in calls with more: half as many trips over W).
 int gemm_pass_rows(const aded_model* m, int rows) { return !m->ws_ready ? rows : rows > 128 ? 256 : 128; }
 
+bool gemm_is_many(const aded_model* m, int rows, int n, int k) { return m->many_ok && many_block_rows(m->device, rows, n, k) > 0; }
+
+void launch_gemm_many(aded_model* m, int w_map, int x_map, int rows, int n, int k, const ManyEpilogue& epi, int trace_kind, cudaStream_t st) {
+    const int block = many_block_rows(m->device, rows, n, k);
+    const int table = w_map < 4 * m->cfg.n_layers ? w_map % 4 : 4;
+    many_launch(m->ws_use_tiled ? m->ws_tiled_maps[w_map] : m->ws_half_maps[w_map], m->ws_use_tiled, m->ws_x_maps[x_map], rows, block, n, k,
+                ws_grid(m->device, n, k, m->ws_one_per_sm[table]), m->ws_slots, m->many_flags, ++m->many_epoch, m->status, epi, trace_kind, m->device, st);
+}
+
+void launch_rmsnorm(aded_model* m, int rows, const void* gain, cudaStream_t st) {
+    GemmOut none = {};
+    none.rows = rows;
+    launch_add_rmsnorm_ws(m, none, gain, st);
+}
+
 GemmOut launch_gemm(aded_model* m, int w_map, int x_map, const void* x, const void* w, float* y, int row0, int rows, int n, int k,
                     int epi_mode, int trace_kind, cudaStream_t st) {
     GemmOut out = {};

@@ -135,7 +135,8 @@ __global__ void __launch_bounds__(PICK_THREADS) k_pick_accept(const CallPtrs* __
 // running) the step is 1.3 % slower; released after the gather or at exit (its weight prefetch no longer
 // runs under this kernel) 4 % slower.  The SwiGLU and rotary kernels below do the same (for them the top of
 // the kernel measures the same; the difference comes from this kernel, whose blocks each take a whole SM's registers).
-// THREADS x 4 x PASSES columns; BATCH contributors in flight.  Narrow rows (d <= 1024) take 256 threads; their projections have up to
+// THREADS x 4 x PASSES columns; BATCH contributors in flight (0: the norm alone, of a row that is complete).  Narrow rows (d <= 1024)
+// take 256 threads; their projections have up to
 // 20 contributors per tile (width 1024, 45 rows, us per launch with 8, 12 and 24 in flight: 5.5, 6.0, 5.8; 1024 threads, 12: 6.3).
 template <int THREADS, int PASSES, int BATCH>
 __global__ void __launch_bounds__(THREADS) k_add_rmsnorm_ws(bf16* __restrict__ h, GemmOut y, const bf16* __restrict__ gain,
@@ -148,7 +149,7 @@ __global__ void __launch_bounds__(THREADS) k_add_rmsnorm_ws(bf16* __restrict__ h
     for (int i = 0; i < PASSES; ++i) {
         const int c = (i * THREADS + threadIdx.x) * 4;
         if (c < d) {
-            tr[i] = y.tiles[c >> 7];
+            if (BATCH > 0) tr[i] = y.tiles[c >> 7];
             gv[i] = unpack4_bf16(*reinterpret_cast<const uint2*>(gain + c));
         }
     }
@@ -164,11 +165,14 @@ __global__ void __launch_bounds__(THREADS) k_add_rmsnorm_ws(bf16* __restrict__ h
         if (c < d) {
             uint2* hp = reinterpret_cast<uint2*>(h + (size_t)r * d + c);
             const float4 hv = unpack4_bf16(*hp);
-            if (!ADED_IN_RANGE(tr[i].first_slot >= 0 && tr[i].first_slot + tr[i].count <= y.n_tiles + y.g, status)) tr[i].count = 0;
-            const float4 add = gemm_out_at4<BATCH>(y, tr[i], r, c & 127);
-            const uint2 nv = pack4_bf16(hv.x + add.x, hv.y + add.y, hv.z + add.z, hv.w + add.w);
-            if (pass_status == 0) *hp = nv;
-            v[i] = unpack4_bf16(nv);
+            v[i] = hv;
+            if constexpr (BATCH > 0) {
+                if (!ADED_IN_RANGE(tr[i].first_slot >= 0 && tr[i].first_slot + tr[i].count <= y.n_tiles + y.g, status)) tr[i].count = 0;
+                const float4 add = gemm_out_at4<BATCH>(y, tr[i], r, c & 127);
+                const uint2 nv = pack4_bf16(hv.x + add.x, hv.y + add.y, hv.z + add.z, hv.w + add.w);
+                if (pass_status == 0) *hp = nv;
+                v[i] = unpack4_bf16(nv);
+            }
             sq += v[i].x * v[i].x + v[i].y * v[i].y + v[i].z * v[i].z + v[i].w * v[i].w;
         }
     }
@@ -282,8 +286,8 @@ k_rope_part_ws(GemmOut qkv, const float* __restrict__ cs, const float* __restric
     bf16* dst = part == 0 ? q + (size_t)r * d + hh * hd + i
                           : reinterpret_cast<bf16*>(base[b]) + ((((size_t)layer * 2 + part - 1) * H + hh) * cp + slot) * hd + i;
     if (part < 2) {
-        *reinterpret_cast<uint2*>(dst) = pack4_bf16(x0.x * c.x - x1.x * s.x, x0.y * c.y - x1.y * s.y, x0.z * c.z - x1.z * s.z, x0.w * c.w - x1.w * s.w);
-        *reinterpret_cast<uint2*>(dst + half) = pack4_bf16(x1.x * c.x + x0.x * s.x, x1.y * c.y + x0.y * s.y, x1.z * c.z + x0.z * s.z, x1.w * c.w + x0.w * s.w);
+        *reinterpret_cast<uint2*>(dst) = rope_first4(x0, x1, c, s);
+        *reinterpret_cast<uint2*>(dst + half) = rope_second4(x0, x1, c, s);
     } else {
         *reinterpret_cast<uint2*>(dst) = pack4_bf16(x0.x, x0.y, x0.z, x0.w);
         *reinterpret_cast<uint2*>(dst + half) = pack4_bf16(x1.x, x1.y, x1.z, x1.w);
@@ -307,7 +311,8 @@ void launch_add_rmsnorm_ws(aded_model* m, const GemmOut& y, const void* gain, cu
     auto go = [&](auto* kernel, int threads) {
         launch_k(kernel, dim3(y.rows), dim3(threads), 0, st, (bf16*)m->h, y, (const bf16*)gain, (bf16*)m->x, d, m->cfg.rms_eps, (const int32_t*)m->status);
     };
-    if (d <= 1024) go(k_add_rmsnorm_ws<256, 1, 8>, 256);
+    if (!y.tiles) d <= 1024 ? go(k_add_rmsnorm_ws<256, 1, 0>, 256) : go(k_add_rmsnorm_ws<1024, 2, 0>, 1024);
+    else if (d <= 1024) go(k_add_rmsnorm_ws<256, 1, 8>, 256);
     else go(k_add_rmsnorm_ws<1024, 2, 12>, 1024);
 }
 

@@ -175,6 +175,16 @@ __device__ __forceinline__ uint2 swiglu4(float4 g, float4 u) {
                       g.z / (1.f + expf(-g.z)) * u.z, g.w / (1.f + expf(-g.w)) * u.w);
 }
 
+// A rotated pair.  The roundings are spelled out: a row's q and k are the same bits whichever kernel rotates them.
+__device__ __forceinline__ float rope_first(float x0, float x1, float c, float s) { return fmaf(x0, c, -__fmul_rn(x1, s)); }
+__device__ __forceinline__ float rope_second(float x0, float x1, float c, float s) { return fmaf(x0, s, __fmul_rn(x1, c)); }
+__device__ __forceinline__ uint2 rope_first4(float4 a, float4 b, float4 c, float4 s) {
+    return pack4_bf16(rope_first(a.x, b.x, c.x, s.x), rope_first(a.y, b.y, c.y, s.y), rope_first(a.z, b.z, c.z, s.z), rope_first(a.w, b.w, c.w, s.w));
+}
+__device__ __forceinline__ uint2 rope_second4(float4 a, float4 b, float4 c, float4 s) {
+    return pack4_bf16(rope_second(a.x, b.x, c.x, s.x), rope_second(a.y, b.y, c.y, s.y), rope_second(a.z, b.z, c.z, s.z), rope_second(a.w, b.w, c.w, s.w));
+}
+
 // Rotary embedding of four adjacent pairs (i .. i+3 with i+half .. i+half+3) of one head's q and k of
 // row r, and the copy of v: gathers the QKV projection's partial tiles, rotates with the row's
 // cos/sin, rounds to bf16 and (when `store`) writes q to qd and K/V to the cache rows kdst / vdst.
@@ -202,10 +212,10 @@ __device__ __forceinline__ void rope_kv_item(const GemmOut& qkv, const TileRef& 
     }
     const float4 c = *reinterpret_cast<const float4*>(cs_row + i), s = *reinterpret_cast<const float4*>(sn_row + i);
     if (!store) return;
-    *reinterpret_cast<uint2*>(qd + i) = pack4_bf16(q0.x * c.x - q1.x * s.x, q0.y * c.y - q1.y * s.y, q0.z * c.z - q1.z * s.z, q0.w * c.w - q1.w * s.w);
-    *reinterpret_cast<uint2*>(qd + i + half) = pack4_bf16(q1.x * c.x + q0.x * s.x, q1.y * c.y + q0.y * s.y, q1.z * c.z + q0.z * s.z, q1.w * c.w + q0.w * s.w);
-    *reinterpret_cast<uint2*>(kdst + i) = pack4_bf16(k0.x * c.x - k1.x * s.x, k0.y * c.y - k1.y * s.y, k0.z * c.z - k1.z * s.z, k0.w * c.w - k1.w * s.w);
-    *reinterpret_cast<uint2*>(kdst + i + half) = pack4_bf16(k1.x * c.x + k0.x * s.x, k1.y * c.y + k0.y * s.y, k1.z * c.z + k0.z * s.z, k1.w * c.w + k0.w * s.w);
+    *reinterpret_cast<uint2*>(qd + i) = rope_first4(q0, q1, c, s);
+    *reinterpret_cast<uint2*>(qd + i + half) = rope_second4(q0, q1, c, s);
+    *reinterpret_cast<uint2*>(kdst + i) = rope_first4(k0, k1, c, s);
+    *reinterpret_cast<uint2*>(kdst + i + half) = rope_second4(k0, k1, c, s);
     *reinterpret_cast<uint2*>(vdst + i) = pack4_bf16(v0.x, v0.y, v0.z, v0.w);
     *reinterpret_cast<uint2*>(vdst + i + half) = pack4_bf16(v1.x, v1.y, v1.z, v1.w);
 }

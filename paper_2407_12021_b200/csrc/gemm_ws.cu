@@ -445,6 +445,20 @@ bool ws_make_map(CUtensorMap* map, const void* ptr, uint64_t rows, uint64_t cols
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// The re-tiled copy of a matrix (ws_retile) as a tensor of 128-byte lines, boxes of 64 lines, half a unit: the lines are stored as
+// they are staged, so the copy does not swizzle.  (For gemm_many.cu: only tensor copies complete on another CTA's barrier.)
+bool ws_make_tiled_map(CUtensorMap* map, const void* ptr, uint64_t units) {
+    EncodeTiledFn fn = encode_fn();
+    if (!fn) return false;
+    const cuuint64_t dims[2] = {WS_BK, units * WS_BM};
+    const cuuint64_t strides[1] = {WS_BK * 2};
+    const cuuint32_t box[2] = {WS_BK, WS_BM / 2};
+    const cuuint32_t elem[2] = {1, 1};
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims, strides, box, elem,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 int ws_grid_limit(int device) {
     static int cached_dev = -1, cached = 0;
     if (cached_dev != device) {

@@ -183,17 +183,56 @@ static aded_status alloc_model(aded_model* m) {
                 TRY(dev_alloc(m, &m->ws_tiles[i], (size_t)nt));
                 ADED_CUDA_TRY(cudaMemcpy(m->ws_tiles[i], table.data(), nt * sizeof(TileRef), cudaMemcpyHostToDevice));
             }
+            // calls of many rows: every tile complete, in the order of the tiles
+            m->many_ok = R > 256;
+            for (int i = 0; i < 5; ++i) m->many_ok = m->many_ok && ws_grid(m->device, shapes[i][0], shapes[i][1], m->ws_one_per_sm[i]) % 2 == 0;
+            if (m->many_ok) {
+                if (!many_prepare()) return ADED_ERR_CUDA;
+                m->ws_half_maps.resize(4 * L + 1);
+                m->ws_tiled_maps.resize(4 * L + 1);
+                for (int i = 0; i < 4 * L + 1; ++i) {
+                    const void* src; size_t nn, kk;
+                    matrix(i, &src, &nn, &kk);
+                    if (!ws_make_map(&m->ws_half_maps[i], src, nn, kk, 64)) return ADED_ERR_CUDA;
+                    if (m->ws_use_tiled && !ws_make_tiled_map(&m->ws_tiled_maps[i], m->ws_tiled[i], nn / 128 * (kk / 64))) return ADED_ERR_CUDA;
+                }
+                std::vector<TileRef> identity(widest / 128);
+                for (int t = 0; t < (int)identity.size(); ++t) identity[t] = TileRef{t, 1};
+                TRY(dev_alloc(m, &m->many_tiles, identity.size()));
+                ADED_CUDA_TRY(cudaMemcpy(m->many_tiles, identity.data(), identity.size() * sizeof(TileRef), cudaMemcpyHostToDevice));
+                TRY(dev_alloc(m, &m->many_flags, (size_t)ws_grid_limit(m->device) / 2 * 8));
+                ADED_CUDA_TRY(cudaMemset(m->many_flags, 0, (size_t)ws_grid_limit(m->device) / 2 * 8 * sizeof(uint32_t)));
+                m->many_epoch = 0;
+            }
             // the LM head's tail: one arrival counter per tile, per-tile greedy candidates of every row
             TRY(dev_alloc(m, &m->ws_counters, V / 128));
             ADED_CUDA_TRY(cudaMemset(m->ws_counters, 0, (V / 128) * sizeof(uint32_t)));
             m->ws_epoch = 0;
-            TRY(dev_alloc(m, &m->cand_val, R * (V / 128)));
-            TRY(dev_alloc(m, &m->cand_idx, R * (V / 128)));
+            TRY(dev_alloc(m, &m->cand_val, R * (V / (m->many_ok ? 32 : 128))));
+            TRY(dev_alloc(m, &m->cand_idx, R * (V / (m->many_ok ? 32 : 128))));
             m->ws_ready = true;
         }
     }
     if (!m->ws_ready && !gemm_plain_prepare(c.dtype == ADED_BF16)) return ADED_ERR_CUDA;
     return ADED_OK;
+}
+
+static ManyEpilogue many_rope(const aded_model* m, const aded_kv* kv, int layer) {
+    ManyEpilogue e = {};
+    e.kind = MANY_ROPE;
+    e.cs = m->rope_cos;
+    e.sn = m->rope_sin;
+    e.q = (bf16*)m->q;
+    e.base = kv->base_dev;
+    e.cap = kv->cap_dev;
+    e.len = kv->len_dev;
+    e.row_seq = m->rows.seq;
+    e.row_local = m->rows.local;
+    e.layer = layer;
+    e.heads = m->cfg.n_heads;
+    e.hd = m->cfg.head_dim;
+    e.d = m->cfg.d_model;
+    return e;
 }
 
 // The launch sequence of one pass over `rows` rows.  chain_mode: the rows form a chain per sequence,
@@ -219,6 +258,13 @@ static aded_status enqueue_pass(aded_model* m, aded_kv* kv, const CallPtrs& call
     auto each_pass = [&](auto&& f) {
         for (int row0 = 0; row0 < rows; row0 += pass) f(row0, rows - row0 < pass ? rows - row0 : pass);
     };
+    // The same for all rows at once, result and all, where the call has enough of them.
+    auto many = [&](int w_map, int x_map, int n, int k, const ManyEpilogue& e, int kind) {
+        if (!gemm_is_many(m, rows, n, k)) return false;
+        Span sp(m, PROF_GEMM, 1, st);
+        launch_gemm_many(m, w_map, x_map, rows, n, k, e, kind, st);
+        return true;
+    };
     for (int l = 0; l < c.n_layers; ++l) {
         const aded_layer_weights& w = m->layers[l];
         const void* next_gain = l + 1 < c.n_layers ? m->layers[l + 1].norm1 : m->top.final_norm;
@@ -229,11 +275,23 @@ static aded_status enqueue_pass(aded_model* m, aded_kv* kv, const CallPtrs& call
                 { Span sp(m, PROF_OTHER, 1, st); consume(o); }
             });
         };
-        project(WS_MAP_QKV, WS_X, m->x, w.wqkv, 3 * d, d, TK_GEMM_QKV, [&](const GemmOut& o) { launch_rope_kv(m, kv, o, l, st); });
+        auto residual = [&](int which, int x_map, const void* x, const void* wt, int k, int kind, const void* gain) {
+            ManyEpilogue e = {};
+            e.kind = MANY_RESIDUAL;
+            e.h = (bf16*)m->h;
+            if (many(4 * l + which, x_map, d, k, e, kind)) { Span sp(m, PROF_OTHER, 1, st); launch_rmsnorm(m, rows, gain, st); }
+            else project(which, x_map, x, wt, d, k, kind, [&](const GemmOut& o) { launch_add_rmsnorm(m, o, gain, st); });
+        };
+        if (!many(4 * l + WS_MAP_QKV, WS_X, 3 * d, d, many_rope(m, kv, l), TK_GEMM_QKV))
+            project(WS_MAP_QKV, WS_X, m->x, w.wqkv, 3 * d, d, TK_GEMM_QKV, [&](const GemmOut& o) { launch_rope_kv(m, kv, o, l, st); });
         { Span sp(m, PROF_ATTN, 1, st); launch_tree_attention(m, kv, l, batch, rows, max_tree, st); }
-        project(WS_MAP_O, WS_X_ATTN, m->attn, w.wo, d, d, TK_GEMM_O, [&](const GemmOut& o) { launch_add_rmsnorm(m, o, w.norm2, st); });
-        project(WS_MAP_GU, WS_X, m->x, w.wgu, 2 * F, d, TK_GEMM_GU, [&](const GemmOut& o) { launch_swiglu(m, o, st); });
-        project(WS_MAP_D, WS_X_ACT, m->act, w.wd, d, F, TK_GEMM_DOWN, [&](const GemmOut& o) { launch_add_rmsnorm(m, o, next_gain, st); });
+        residual(WS_MAP_O, WS_X_ATTN, m->attn, w.wo, d, TK_GEMM_O, w.norm2);
+        ManyEpilogue e = {};
+        e.kind = MANY_SWIGLU;
+        e.act = (bf16*)m->act;
+        if (!many(4 * l + WS_MAP_GU, WS_X, 2 * F, d, e, TK_GEMM_GU))
+            project(WS_MAP_GU, WS_X, m->x, w.wgu, 2 * F, d, TK_GEMM_GU, [&](const GemmOut& o) { launch_swiglu(m, o, st); });
+        residual(WS_MAP_D, WS_X_ACT, m->act, w.wd, F, TK_GEMM_DOWN, next_gain);
         if (m->dbg_hidden)
             ADED_CUDA_TRY(cudaMemcpyAsync((char*)m->dbg_hidden + (size_t)(l + 1) * hid_bytes, m->h, hid_bytes,
                                           cudaMemcpyDeviceToDevice, st));
@@ -243,7 +301,14 @@ static aded_status enqueue_pass(aded_model* m, aded_kv* kv, const CallPtrs& call
         // greedy choice works from per-tile candidates left by the LM head's tail.
         const bool dense_logits = !ws || m->samp_on || m->dbg_logits;
         float* dense = m->samp_on && !m->dbg_logits ? m->logits : m->dbg_logits;      // where the logits go as a matrix, if anywhere
-        each_pass([&](int row0, int part) {
+        int candidates = c.vocab / 128;                   // per row
+        ManyEpilogue e = {};
+        e.kind = MANY_ARGMAX;
+        e.cand_val = m->cand_val;
+        e.cand_idx = m->cand_idx;
+        const bool many_head = !dense_logits && many(4 * c.n_layers, WS_X, c.vocab, d, e, TK_GEMM_HEAD);
+        if (many_head) candidates = c.vocab / 32;
+        else each_pass([&](int row0, int part) {
             GemmOut lg;
             { Span sp(m, PROF_GEMM, 1, st);
               lg = launch_gemm(m, ws ? 4 * c.n_layers : -1, ws ? WS_X : -1, m->x, m->top.lm_head, m->logits, row0, part, c.vocab, d,
@@ -262,7 +327,7 @@ static aded_status enqueue_pass(aded_model* m, aded_kv* kv, const CallPtrs& call
             launch_pick_accept(m, kv, batch, m->argmax_val, m->argmax_idx, ARGMAX_CHUNKS, st);
         } else {
             Span sp(m, PROF_OTHER, 1, st);
-            launch_pick_accept(m, kv, batch, m->cand_val, m->cand_idx, c.vocab / 128, st);
+            launch_pick_accept(m, kv, batch, m->cand_val, m->cand_idx, candidates, st);
         }
         if (m->dbg_best)
             ADED_CUDA_TRY(cudaMemcpyAsync(m->dbg_best, m->best, (size_t)rows * sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
@@ -341,6 +406,7 @@ aded_status aded_model_create(const aded_model_config* cfg, const aded_weights* 
     m->prof_on = false;
     m->call_dev = nullptr;
     m->ws_ready = false;
+    m->many_ok = false;
     m->ws_slots = nullptr;
     if (cudaGetDevice(&m->device) != cudaSuccess) {
         delete m;
@@ -589,6 +655,23 @@ aded_status aded_debug_gemm(aded_model* m, int32_t layer, int32_t which, const v
     const int w_map = which == 4 ? 4 * c.n_layers : 4 * layer + which;
     float* ybuf = which == 4 ? m->logits : m->y32;
     ADED_CUDA_TRY(cudaMemcpyAsync(xbuf, x_dev, (size_t)rows * k * m->elem, cudaMemcpyDeviceToDevice, st));
+    if (gemm_is_many(m, rows, n, k)) {
+        ManyEpilogue e = {};
+        e.kind = MANY_PLAIN;
+        e.out = ybuf;
+        e.rb = (rows + 15) / 16 * 16;
+        GemmOut o = {};
+        o.mode = 1;
+        o.n = n;
+        o.rows = rows;
+        o.slots = ybuf;
+        o.tiles = m->many_tiles;
+        note_launch(2);
+        launch_gemm_many(m, w_map, x_map, rows, n, k, e, TK_OTHER, st);
+        launch_materialize(m, o, y_dev, st);
+        ADED_CUDA_TRY(cudaGetLastError());
+        return ADED_OK;
+    }
     const int pass = gemm_pass_rows(m, rows);
     for (int row0 = 0; row0 < rows; row0 += pass) {
         note_launch(2);
@@ -597,6 +680,13 @@ aded_status aded_debug_gemm(aded_model* m, int32_t layer, int32_t which, const v
         launch_materialize(m, o, y_dev, st);
     }
     ADED_CUDA_TRY(cudaGetLastError());
+    return ADED_OK;
+}
+
+aded_status aded_debug_silu_check(uint32_t first, uint64_t count, uint64_t* differ_dev, void* stream) {
+    if (!differ_dev || count < 1 || count > (1ull << 32)) return ADED_ERR_INVALID_ARG;
+    note_launch(1);
+    ADED_CUDA_TRY(many_silu_check(first, count, differ_dev, static_cast<cudaStream_t>(stream)));
     return ADED_OK;
 }
 

@@ -1,0 +1,104 @@
+"""Calls of more than 256 rows: the GEMM on pairs of SMs adds the same products in the same order as the weight-streaming kernel, and
+its epilogues (rotary + K/V write, residual add, SwiGLU, greedy candidates) round as the kernels that they stand for.  So almost
+everything here is compared bit for bit."""
+import pytest
+import torch
+
+from paper_2407_12021_b200 import inputs as gen
+from tests import helpers as H
+
+pytestmark = pytest.mark.gpu
+
+HD64 = gen.ModelShape("many-16x64", 1, 1024, 16, 64, 2816, 32000, "bf16")
+SHAPES = {"7b": gen.LLAMA7B_1L, "hd64": HD64}
+
+
+def _matrices(w):
+    p = w["layers"][0]
+    return [p["wqkv"], p["wo"], p["wgu"], p["wd"], w["lm_head"]]
+
+
+@pytest.mark.parametrize("shape,rows", [("7b", (257, 320, 513, 640, 641, 1228)), ("hd64", (385, 1228, 2400))])
+@pytest.mark.parametrize("layout", [0, 1])
+def test_sums_are_those_of_a_small_call(cuda_device, shape, rows, layout):
+    """Row counts around the edges of row blocks: two blocks of 160, ragged last blocks, items that are divided between two pairs
+    and none; both layouts of the weights.  The first and the last rows of the call must be what a call of 200 rows gives."""
+    from paper_2407_12021_b200 import binding as B
+    shape = SHAPES[shape]
+    w = gen.model_weights(shape, 61, device=cuda_device)
+    model = B.aded_model_create(shape, w, max_rows=max(rows), max_batch=16)
+    B.aded_debug_weight_layout(model, layout)
+    for which, m in enumerate(_matrices(w)):
+        x = gen.normal((max(rows), m.shape[1]), 1.0, 62, 500 + which, device=cuda_device, dtype=torch.bfloat16)
+        for n in rows:
+            y = B.aded_debug_gemm(model, 0, which, x[:n].contiguous())
+            head, tail = B.aded_debug_gemm(model, 0, which, x[:200].contiguous()), B.aded_debug_gemm(model, 0, which, x[n - 200:n].contiguous())
+            torch.cuda.synchronize()
+            assert B.aded_model_poll_status(model) == 0
+            assert torch.equal(y[:200], head) and torch.equal(y[n - 200:], tail), (which, n)
+
+
+@pytest.mark.parametrize("shape", ["7b", "hd64"])
+@pytest.mark.parametrize("batch,nodes", [(5, 61), (11, 128)])
+def test_a_batch_layer_by_parts(cuda_device, shape, batch, nodes):
+    """One layer + LM head of a ragged batch.  Rotated queries and cache rows equal those of each sequence's own call; the residual adds
+    and the greedy tokens equal what the projections alone (aded_debug_gemm) give for the same inputs; the SwiGLU product lies
+    within bf16 rounding of the formula: its factors' inputs are normalised here in another order of sums, which moves a bf16
+    input by one place at most, 2^-8 of a term, and a sum of thousands of such terms by far less than 2e-2 of the largest."""
+    from paper_2407_12021_b200 import binding as B
+    shape = SHAPES[shape]
+    w = gen.model_weights(shape, 63, device=cuda_device)
+    layer = w["layers"][0]
+    lens, sizes = [40 + 7 * b for b in range(batch)], [max(1, nodes - 3 * b) for b in range(batch)]
+    rows, d, hd = sum(sizes), shape.d_model, shape.head_dim
+    model = B.aded_model_create(shape, w, max_rows=rows, max_batch=batch)
+    trees = [gen.make_tree(n, min(5, n - 1), 8, shape.vocab, 64 + b) for b, n in enumerate(sizes)]
+    caches = [[gen.normal((shape.n_heads, lens[b], hd), 1.0, 65, 2 * b + e, device=cuda_device, dtype=torch.bfloat16) for e in range(2)] for b in range(batch)]
+    offsets = [sum(sizes[:b]) for b in range(batch + 1)]
+    tok, par = H.i32([t for tr in trees for t in tr[0]]), H.i32([p for tr in trees for p in tr[1]])
+
+    def cache(which):
+        kv = B.aded_kv_create(model, [lens[b] + sizes[b] for b in which])
+        for i, b in enumerate(which):
+            B.aded_kv_load(kv, i, 0, *caches[b])
+        return kv
+
+    kv, best = cache(range(batch)), torch.zeros(rows, dtype=torch.int32, device=cuda_device)
+    out, n_out = torch.zeros((batch, 128), dtype=torch.int32, device=cuda_device), torch.zeros(batch, dtype=torch.int32, device=cuda_device)
+    B.aded_debug_capture(model, None, best)
+    B.aded_verify_batch(model, kv, offsets, tok, par, out, n_out)
+    q, attn, act, h, x = (B.aded_debug_read_buffer(model, i, rows).clone() for i in (2, 3, 4, 0, 1))
+    torch.cuda.synchronize()
+    assert B.aded_model_poll_status(model) == 0
+    assert bool((n_out >= 1).all())
+
+    gemm = lambda which, a: B.aded_debug_gemm(model, 0, which, a.contiguous())
+    mid = (w["embed"][tok.long()].float() + gemm(1, attn)).bfloat16()
+    assert torch.equal(h, (mid.float() + gemm(3, act)).bfloat16())
+    logits = gemm(4, x)
+    assert torch.equal(best.long(), (logits == logits.amax(1, keepdim=True)).int().argmax(1))
+    normed = (mid.double() * torch.rsqrt(mid.double().pow(2).mean(1, keepdim=True) + shape.rms_eps) * layer["norm2"].double()).bfloat16()
+    gate, up = (normed.float() @ layer["wgu"].float().T).chunk(2, dim=1)
+    want = torch.nn.functional.silu(gate) * up
+    assert float((act.float() - want).abs().max()) <= 2e-2 * float(want.abs().max())
+
+    accepted = n_out.tolist()
+    for b in range(batch):
+        own = cache([b])
+        a, e = offsets[b], offsets[b + 1]
+        one, n_one = torch.zeros(128, dtype=torch.int32, device=cuda_device), torch.zeros(1, dtype=torch.int32, device=cuda_device)
+        B.aded_verify(model, own, tok[a:e].contiguous(), par[a:e].contiguous(), one, n_one)
+        assert torch.equal(B.aded_debug_read_buffer(model, 2, e - a), q[a:e]), b
+        if int(n_one[0]) == accepted[b]:
+            n = lens[b] + accepted[b]          # committed rows, the accepted nodes' among them
+            for got, ref in zip(B.aded_kv_read(kv, b, 0, 0, n), B.aded_kv_read(own, 0, 0, 0, n)):
+                assert torch.equal(got, ref), b
+    assert B.aded_model_poll_status(model) == 0
+
+
+def test_quotient_of_the_swiglu_epilogue(cuda_device):
+    """Every float of the range in which the epilogue divides without the operator: the same quotient, bit for bit."""
+    from paper_2407_12021_b200 import binding as B
+    differ = torch.zeros(1, dtype=torch.int64, device=cuda_device)
+    B.aded_debug_silu_check(0, 1 << 32, differ)
+    assert int(differ[0]) == 0
