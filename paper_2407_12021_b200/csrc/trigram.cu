@@ -204,7 +204,7 @@ __global__ void k_tg_import(TgView t, const int32_t* __restrict__ keys, const ui
 // the distinct ones of each block): bound by the L2 reads of the entries.
 constexpr int TOPK_THREADS = 512, TOPK_WARPS = TOPK_THREADS / 32, TOPK_MAX_QUERIES = 3072;
 constexpr uint32_t TOPK_LONG = 2048;
-constexpr int TOPK_WIDE = 4, TOPK_LEAD_QUERIES = 4096;
+constexpr int TOPK_WIDE = 4, TOPK_LEAD_QUERIES = 2432;
 
 // Slots of the block's hash table: a power of two, at most four fifths full.
 static __host__ __device__ int topk_slots(int per_block) {
@@ -305,134 +305,308 @@ k_tg_topk(TgView t, const int32_t* __restrict__ ctx, int q, int k, int per_block
 // Many queries: every context of the call is scanned once, by three kernels whose only scratch is the output arrays themselves
 // (lookups of one table may run on several streams, so the table holds none).
 //   1. k_topk_mark: a thread per query finds the home bucket.  Contexts with entries beyond it are grouped: the query's index
-//      goes into a hash table that fills out_cnt (all bits set before), and the first query of a context found there leads the
+//      goes into a hash table that lies in out_cnt (all bits set before), and the first query of a context found there leads the
 //      others.  out_tok[first of the row] says what a row is: MARK_OWN (answer it; its home bucket, or -1, is in the next
-//      word) or the leader's index, encoded below MARK_OWN.
-//   2. k_topk_lead: the leaders' rows, and those of contexts that are all in their home bucket, by the thread that has the row;
-//      the hash table is overwritten with results.
+//      word) or the leader's index, encoded below MARK_OWN.  Contexts that are all in their home bucket are answered there and then.
+//   2. k_topk_lead: the leaders' rows, and those whose counts the hash table took; it is overwritten with results.
 //   3. k_topk_copy: the followers' rows, from their leaders'.
-// Needs two words per row (k >= 2).  The table takes the largest power of two of the q k count words, so between half and all of
-// them: it has at least q slots, and with k = 2 and many distinct contexts it can fill up; a query that finds no slot within
-// MARK_PROBES answers itself.
-// Measured, 2^20 queries on the table of a 16-million-token text, k = 4: 183 us (54 + 92 + 30 and a memset; the per-block kernel
-// above: 780).  What bounds it: random access in the first, and in the second the warps' chains of reads, no longer the entries' bytes.
-// Taken from TOPK_BULK queries on, from where it is the faster one on every table measured.  k = 4, the per-block kernel against this, us:
-//   queries                    2^12        2^13        2^14        2^15        2^16        2^17
-//   text of 10^5 tokens      25 /  37    28 /  37    30 /  37    38 /  37    48 /  39    72 /  42
-//            10^6            44 /  37    55 /  38    65 /  39    77 /  42    96 /  44   130 /  49
-//            1.6 x 10^7     139 /  47   165 /  48   187 /  49   206 /  56   235 /  62   295 /  74
-// (k = 2 and 8 alike: within 10 us of it on either side.)  Larger tables cross far earlier, but a call does not know how long its
-// contexts are.
-constexpr int MARK_OWN = -2, MARK_PROBES = 16, TOPK_BULK = 1 << 16;
+// Needs two words per row (k >= 2).  The table takes the smallest power of two that is at least half the queries; a query that
+// finds no slot within MARK_PROBES answers itself.
+// What bounds it: dependent reads of a table far larger than L2 (home bucket, directory, entries), in each kernel; the stores of the
+// short rows, one word at a time, took as long as the reads, and a warp for every context with seven continuations twice as long as
+// now.  Measured, 2^20 queries on the table of a 16-million-token text, us: k = 2, 4, 8: 151, 188, 253 before; 92, 100, 124 now
+// (mark 46, lead 48, copy 14 under ncu, 57 + 93 + 32 before).
+// Taken from the number of queries on from where it is the faster one, which depends on how long contexts are and so on how
+// much text the table holds, of which its size is what a call knows (topk_bulk_min).  k = 4, the per-block kernel against this, us:
+//   home buckets                      2^11        2^12        2^13        2^14        2^15        2^16 queries
+//   2^18 (text of 10^5 tokens)      13 /  22    14 /  20    16 /  21    19 /  21    27 /  22    28 /  23
+//   2^19          2 x 10^5          15 /  24    17 /  24    20 /  23    24 /  23    32 /  24
+//   2^20          4 x 10^5          23 /  25    26 /  26    31 /  25    37 /  24    45 /  26
+//   2^21          8 x 10^5          27 /  28    31 /  28    42 /  30    48 /  28    60 /  28
+//   2^25        1.6 x 10^7         117 /  43   120 /  42   149 /  43   170 /  42   193 /  44
+constexpr int MARK_OWN = -2, MARK_PROBES = 16;
+static int topk_bulk_min(uint32_t n_home) { return n_home >= 1u << 21 ? 1 << 12 : n_home >= 1u << 20 ? 1 << 13 : n_home >= 1u << 19 ? 1 << 15 : 1 << 16; }
 __device__ __forceinline__ int mark_leader(int q) { return MARK_OWN - 1 - q; }       // (its own inverse)
 
-__global__ void __launch_bounds__(256) k_topk_mark(TgView t, const int32_t* __restrict__ ctx, int q, int k, int lead_blocks, int per_block, uint32_t mask,
-                                                   int32_t* __restrict__ out_tok, uint32_t* out_cnt) {
-    // neighbouring threads take queries of different blocks of the next kernel: the frequent contexts, which the first threads
-    // meet, then have their leaders spread over all of its blocks
-    // (unsigned: the rounded-up product of blocks and queries per block may pass 2^31 - 1)
-    const uint32_t at = blockIdx.x * 256 + threadIdx.x;
-    const uint32_t row = at % (uint32_t)lead_blocks * per_block + at / (uint32_t)lead_blocks;
-    if (at / (uint32_t)lead_blocks >= (uint32_t)per_block || row >= (uint32_t)q) return;
-    const int i = (int)row;
-    const int2 c = make_int2(ctx[2 * (size_t)i], ctx[2 * (size_t)i + 1]);
-    int64_t home = -1;
-    if (c.x >= 0 && c.y >= 0 && c.x < t.vocab && c.y < t.vocab) home = tg_find_home(t, tg_key(c.x, c.y), false);
-    int mark = MARK_OWN;
-    if (home >= 0 && t.buckets[home].n_more != 0) {
-        uint32_t probe_at = (uint32_t)home * 0x9E3779B1u;
-        probe_at ^= probe_at >> 15;
-        for (int probe = 0; probe < MARK_PROBES; ++probe, ++probe_at) {
-            uint32_t* slot = out_cnt + (probe_at & mask);
-            uint32_t have = *reinterpret_cast<volatile uint32_t*>(slot);
-            if (have == 0xFFFFFFFFu) have = atomicCAS(slot, 0xFFFFFFFFu, (uint32_t)i);
-            if (have == 0xFFFFFFFFu) break;
-            if (ctx[2 * (size_t)have] == c.x && ctx[2 * (size_t)have + 1] == c.y) { mark = mark_leader((int)have); break; }
+// One thread's list: the first k of `key` (in order; eight of them, none beyond) as a row.  `vec`: the words of a row that one store takes.
+__device__ __forceinline__ void topk_store(const unsigned long long (&key)[8], int k, int vec, int32_t* tok, uint32_t* cnt) {
+#pragma unroll
+    for (int r = 0; r < 8; r += 4) {
+        if (r >= k) break;
+        const int4 a = make_int4(tg_packed_tok(key[r]), tg_packed_tok(key[r + 1]), tg_packed_tok(key[r + 2]), tg_packed_tok(key[r + 3]));
+        const uint4 c = make_uint4(tg_packed_cnt(key[r]), tg_packed_cnt(key[r + 1]), tg_packed_cnt(key[r + 2]), tg_packed_cnt(key[r + 3]));
+        if (vec == 4) {
+            *reinterpret_cast<int4*>(tok + r) = a;
+            *reinterpret_cast<uint4*>(cnt + r) = c;
+        } else if (vec == 2) {
+            *reinterpret_cast<int2*>(tok + r) = make_int2(a.x, a.y);
+            *reinterpret_cast<uint2*>(cnt + r) = make_uint2(c.x, c.y);
+            if (r + 2 < k) {
+                *reinterpret_cast<int2*>(tok + r + 2) = make_int2(a.z, a.w);
+                *reinterpret_cast<uint2*>(cnt + r + 2) = make_uint2(c.z, c.w);
+            }
+        } else {
+            tok[r] = a.x; cnt[r] = c.x;
+            if (r + 1 < k) { tok[r + 1] = a.y; cnt[r + 1] = c.y; }
+            if (r + 2 < k) { tok[r + 2] = a.z; cnt[r + 2] = c.z; }
+            if (r + 3 < k) { tok[r + 3] = a.w; cnt[r + 3] = c.w; }
         }
     }
-    out_tok[(size_t)i * k] = mark;
-    out_tok[(size_t)i * k + 1] = (int32_t)home;
+    for (int r = 8; r < k; ++r) { tok[r] = -1; cnt[r] = 0; }
 }
 
-// The k best of a home bucket's six entries, and the sum of their counts, by one thread.
-__device__ __forceinline__ void topk_home(const TgView& t, int home, int k, int32_t* tok, uint32_t* cnt, uint32_t* total_out) {
-    unsigned long long key[6];
+// The six entries of a home bucket, best first, by one thread; the sum of their counts.
+__device__ __forceinline__ uint32_t topk_bucket(const TgView& t, int home, unsigned long long (&key)[8]) {
     uint32_t total = 0;
     const uint4* part = reinterpret_cast<const uint4*>(t.buckets + (home < 0 ? 0 : home));
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-        uint4 v = part[i + 1];
-        if (home < 0) v = make_uint4(0xFFFFFFFFu, 0u, 0xFFFFFFFFu, 0u);
+        uint4 v = make_uint4(0xFFFFFFFFu, 0u, 0xFFFFFFFFu, 0u);
+        if (home >= 0) v = part[i + 1];
         if ((int32_t)v.x >= 0) total += v.y;
         if ((int32_t)v.z >= 0) total += v.w;
         key[2 * i] = tg_pack(t, (int32_t)v.x, v.y);
         key[2 * i + 1] = tg_pack(t, (int32_t)v.z, v.w);
     }
+    key[6] = key[7] = 0;
 #pragma unroll
-    for (int r = 0; r < 6; ++r) {
+    for (int r = 0; r < 6; ++r)
 #pragma unroll
         for (int j = r + 1; j < 6; ++j)
             if (key[j] > key[r]) { const unsigned long long x = key[r]; key[r] = key[j]; key[j] = x; }
-        if (r < k) { tok[r] = tg_packed_tok(key[r]); cnt[r] = tg_packed_cnt(key[r]); }
+    return total;
+}
+// A context that is all in its home bucket (or not stored: home < 0).
+__device__ __forceinline__ void topk_home(const TgView& t, int home, int k, int vec, int32_t* tok, uint32_t* cnt, uint32_t* total_out) {
+    unsigned long long key[8];
+    const uint32_t total = topk_bucket(t, home, key);
+    topk_store(key, k, vec, tok, cnt);
+    if (total_out) *total_out = total;
+}
+
+// A block first finds equal contexts among its own queries (a hash table in shared memory, as k_tg_topk), and only the first of each
+// goes to the table: one in twelve of the synthetic text's queries asks for the same context.  A context that is all in its home
+// bucket is answered at once, where its row's counts are not part of the hash table (row >= deferred).
+constexpr int MARK_THREADS = 512, MARK_SLOTS = 2 * MARK_THREADS;
+__global__ void __launch_bounds__(MARK_THREADS, 4)
+k_topk_mark(TgView t, const int32_t* __restrict__ ctx, int q, int k, int vec, uint32_t mask, int deferred, int32_t* __restrict__ out_tok,
+            uint32_t* out_cnt, uint32_t* __restrict__ out_total) {
+    __shared__ int2 s_ctx[MARK_THREADS];
+    __shared__ int s_slot[MARK_SLOTS], s_mark[MARK_THREADS];
+    pdl_enter();
+    const int me = threadIdx.x;
+    const long long at_row = (long long)blockIdx.x * MARK_THREADS + me;
+    const bool mine = at_row < q;
+    const int row = mine ? (int)at_row : 0;
+    int2 c = make_int2(-1, -1);
+    if (mine) c = make_int2(ctx[2 * (size_t)row], ctx[2 * (size_t)row + 1]);
+    s_ctx[me] = c;
+    s_slot[me] = -1;
+    s_slot[MARK_THREADS + me] = -1;
+    __syncthreads();
+    const uint32_t hash = tg_hash(tg_key(c.x, c.y));
+    int first = me;                                            // first of the block's queries with this context
+    if (mine) {
+        for (uint32_t at = hash & (MARK_SLOTS - 1);; at = (at + 1) & (MARK_SLOTS - 1)) {      // (twice as many slots as queries: ends)
+            const int have = atomicCAS(&s_slot[at], -1, me);
+            if (have == -1) break;
+            if (s_ctx[have].x == c.x && s_ctx[have].y == c.y) { first = have; break; }
+        }
     }
-    for (int r = 6; r < k; ++r) { tok[r] = -1; cnt[r] = 0; }
+    int mark = MARK_OWN, home = -1;
+    if (mine && first == me) {
+        bool further = false;                                  // entries beyond the home bucket: the context is grouped
+        if (c.x >= 0 && c.y >= 0 && c.x < t.vocab && c.y < t.vocab) {
+            const int limit = t.n_home < (uint32_t)TG_MAX_PROBE ? (int)t.n_home : TG_MAX_PROBE;
+            for (int probe = 0; probe < limit; ++probe) {
+                const uint32_t at = (hash + probe) & t.n_home_mask;
+                uint4 head;                                    // (all of the bucket comes from memory at once: its entries may be wanted next)
+                asm volatile("ld.global.L2::64B.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(head.x), "=r"(head.y), "=r"(head.z), "=r"(head.w) : "l"(t.buckets + at));
+                if (head.y == (uint32_t)c.x && head.x == (uint32_t)c.y) {
+                    home = (int)at;
+                    further = head.w != 0;
+                    break;
+                }
+                if ((head.x & head.y) == 0xFFFFFFFFu) break;   // TG_EMPTY
+            }
+        }
+        if (further) {
+            uint32_t probe_at = (uint32_t)home * 0x9E3779B1u;
+            probe_at ^= probe_at >> 15;
+            for (int probe = 0; probe < MARK_PROBES; ++probe, ++probe_at) {
+                uint32_t* slot = out_cnt + (probe_at & mask);
+                uint32_t have = *reinterpret_cast<volatile uint32_t*>(slot);
+                if (have == 0xFFFFFFFFu) have = atomicCAS(slot, 0xFFFFFFFFu, (uint32_t)row);
+                if (have == 0xFFFFFFFFu) break;
+                if (ctx[2 * (size_t)have] == c.x && ctx[2 * (size_t)have + 1] == c.y) { mark = mark_leader((int)have); break; }
+            }
+        }
+        s_mark[me] = mark;
+        if (!further && row >= deferred) {
+            topk_home(t, home, k, vec, out_tok + (size_t)row * k, out_cnt + (size_t)row * k, out_total ? out_total + row : nullptr);
+            mark = 0;                                          // (answered)
+        }
+    }
+    __syncthreads();
+    if (!mine || mark == 0) return;
+    if (first != me) mark = s_mark[first] == MARK_OWN ? mark_leader(row - me + first) : s_mark[first];
+    if (vec > 1) {
+        *reinterpret_cast<int2*>(out_tok + (size_t)row * k) = make_int2(mark, home);
+    } else {
+        out_tok[(size_t)row * k] = mark;
+        out_tok[(size_t)row * k + 1] = home;
+    }
+}
+
+// A context to look up: its row, its home bucket, and what the bucket's header says (first extent, entries beyond the bucket).
+struct TopkJob { int row, home; uint32_t more, n; };
+
+// Contexts of up to LEAD_SMALL further entries, a thread each (k <= 8): most contexts have few, and a warp for one spends its
+// instructions on lists of four that 32 lanes hold together (eight lanes each, four contexts per warp: 1000 instructions per four
+// contexts, 20 us of 80 on the table of a 16-million-token text).
+constexpr uint32_t LEAD_SMALL = 48;                // (units 0 .. 7, extents 0 .. 3: the directory's first four words say where)
+__device__ __forceinline__ void topk_thread(const TgView& t, const TopkJob& job, int k, int vec, int32_t* tok, uint32_t* cnt, uint32_t* total_out) {
+    unsigned long long key[8];
+    const uint4 dir = *reinterpret_cast<const uint4*>(t.pool + (size_t)(job.more - 1) * TG_UNIT);
+    uint32_t total = topk_bucket(t, job.home, key);
+    const uint32_t pairs = (job.n + 1) / 2;
+    constexpr int BATCH = 3;                       // a unit's entries at a time
+    unsigned long long floor_key = key[0];         // the k-th best so far
+#pragma unroll
+    for (int r = 1; r < 8; ++r)
+        if (r < k) floor_key = key[r];
+    for (uint32_t m = 0; m * BATCH < pairs; ++m) {
+        const int s = tg_extent(m);
+        const uint32_t base = s == 0 ? job.more + TG_DIR_UNITS : s == 1 ? dir.y : s == 2 ? dir.z : dir.w;
+        if (base == 0 || base == TG_FAILED) continue;
+        const size_t unit = (size_t)(base - 1) + (m + 1 - (1u << s));
+        if (!ADED_IN_RANGE(unit < t.n_units, t.status)) continue;
+        const uint4* from = reinterpret_cast<const uint4*>(t.pool + unit * TG_UNIT);
+        uint4 v[BATCH];
+#pragma unroll
+        for (int i = 0; i < BATCH; ++i) {
+            v[i] = make_uint4(0xFFFFFFFFu, 0u, 0xFFFFFFFFu, 0u);
+            if (m * BATCH + i < pairs) v[i] = from[i];
+            if (2 * (m * BATCH + i) + 1 >= job.n) { v[i].z = 0xFFFFFFFFu; v[i].w = 0u; }
+        }
+#pragma unroll
+        for (int e = 0; e < 2 * BATCH; ++e) {
+            const int32_t token = (int32_t)(e & 1 ? v[e / 2].z : v[e / 2].x);
+            const uint32_t count = e & 1 ? v[e / 2].w : v[e / 2].y;
+            if (token >= 0) total += count;
+            unsigned long long x = tg_pack(t, token, count);
+            if (x <= floor_key) continue;
+#pragma unroll
+            for (int r = 0; r < 8; ++r)
+                if (x > key[r]) { const unsigned long long y = key[r]; key[r] = x; x = y; }
+            floor_key = key[0];
+#pragma unroll
+            for (int r = 1; r < 8; ++r)
+                if (r < k) floor_key = key[r];
+        }
+    }
+    topk_store(key, k, vec, tok, cnt);
     if (total_out) *total_out = total;
 }
 
 __global__ void __launch_bounds__(TOPK_THREADS, 3)
-k_topk_lead(TgView t, int q, int k, int per_block, int32_t* __restrict__ out_tok, uint32_t* __restrict__ out_cnt, uint32_t* __restrict__ out_total) {
-    __shared__ int2 s_job[TOPK_LEAD_QUERIES];      // (row in the block, home bucket); contexts of more than TOPK_LONG entries from the back
-    __shared__ int s_n, s_long, s_cursor;
+k_topk_lead(TgView t, int q, int k, int vec, int per_block, int32_t* __restrict__ out_tok, uint32_t* __restrict__ out_cnt, uint32_t* __restrict__ out_total) {
+    __shared__ TopkJob s_job[TOPK_LEAD_QUERIES];   // few entries from the front, more from the back
+    __shared__ int s_rows, s_n, s_big, s_long, s_cursor;
+    __shared__ int2 s_long_job[4 * TOPK_WIDE];
     __shared__ unsigned long long s_best[TOPK_WARPS * 32];
     __shared__ uint32_t s_total[TOPK_WARPS];
-    const int q0 = blockIdx.x * per_block, nq = min(per_block, q - q0);
+    __shared__ uint16_t s_row[TOPK_LEAD_QUERIES];  // the block's rows that have to be answered
+    pdl_enter();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (threadIdx.x == 0) { s_n = 0; s_long = 0; s_cursor = 0; }
+    if (threadIdx.x == 0) { s_rows = 0; s_n = 0; s_big = 0; s_long = 0; s_cursor = 0; }
     __syncthreads();
-    for (int i = threadIdx.x; i < nq; i += TOPK_THREADS) {
-        const size_t row = (size_t)(q0 + i);
-        if (out_tok[row * k] != MARK_OWN) continue;
-        const int home = out_tok[row * k + 1];
-        const uint32_t n = home < 0 ? 0u : t.buckets[home].n_more & ~TG_CLOSED;
-        if (n == 0) topk_home(t, home, k, out_tok + row * k, out_cnt + row * k, out_total ? out_total + row : nullptr);
-        else if (n > TOPK_LONG) s_job[per_block - 1 - atomicAdd(&s_long, 1)] = make_int2(i, home);
-        else s_job[atomicAdd(&s_n, 1)] = make_int2(i, home);
+    const bool by_thread = k <= 8 && t.chain == nullptr;
+    // A block takes every gridDim.x-th row: the frequent contexts' leaders are among the rows that were marked first.
+#pragma unroll 4
+    for (int i = threadIdx.x; i < per_block; i += TOPK_THREADS) {
+        const long long row = (long long)i * gridDim.x + blockIdx.x;
+        if (row < q && out_tok[row * k] == MARK_OWN) s_row[atomicAdd(&s_rows, 1)] = (uint16_t)i;
     }
     __syncthreads();
-    auto write = [&](int i, unsigned long long best, uint32_t total) {
-        const size_t row = (size_t)(q0 + i);
+    for (int i = threadIdx.x; i < s_rows; i += TOPK_THREADS) {
+        TopkJob job;
+        job.row = (int)((long long)s_row[i] * gridDim.x + blockIdx.x);
+        job.home = out_tok[(size_t)job.row * k + 1];
+        uint4 head = make_uint4(0u, 0u, 0u, 0u);
+        if (job.home >= 0) head = *reinterpret_cast<const uint4*>(t.buckets + job.home);
+        job.more = head.z;
+        job.n = head.w & ~TG_CLOSED;
+        if (job.n == 0) {
+            topk_home(t, job.home, k, vec, out_tok + (size_t)job.row * k, out_cnt + (size_t)job.row * k, out_total ? out_total + job.row : nullptr);
+            continue;
+        }
+        if (by_thread && job.n <= LEAD_SMALL && job.more != TG_FAILED && job.more != 0) {
+            // (directory and first unit are on their way to L2 while the others are sorted)
+            const char* dir = reinterpret_cast<const char*>(t.pool + (size_t)(job.more - 1) * TG_UNIT);
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(dir));
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(dir + (TG_DIR_UNITS + 1) * TG_UNIT * sizeof(TgSlot) - 1));
+            s_job[atomicAdd(&s_n, 1)] = job;
+            continue;
+        }
+        int place = 4 * TOPK_WIDE;
+        if (job.n > TOPK_LONG) place = atomicAdd(&s_long, 1);
+        if (place < 4 * TOPK_WIDE) s_long_job[place] = make_int2(job.row, job.home);
+        else s_job[TOPK_LEAD_QUERIES - 1 - atomicAdd(&s_big, 1)] = job;
+    }
+    __syncthreads();
+    auto write = [&](int row, unsigned long long best, uint32_t total) {
         if (lane < k) {
-            out_tok[row * k + lane] = tg_packed_tok(best);
-            out_cnt[row * k + lane] = tg_packed_cnt(best);
+            out_tok[(size_t)row * k + lane] = tg_packed_tok(best);
+            out_cnt[(size_t)row * k + lane] = tg_packed_cnt(best);
         }
         if (lane == 0 && out_total) out_total[row] = total;
     };
-    const int n_long = s_long, n_short = s_n;
-    const bool wide = n_long <= 4 * TOPK_WIDE;
-    for (int j = 0; wide && j < n_long; ++j) topk_wide(t, s_job[per_block - 1 - j].y, k, warp, lane, s_best, s_total, [&](unsigned long long best, uint32_t total) { write(s_job[per_block - 1 - j].x, best, total); });
-    const int first = wide ? n_long : 0, jobs = n_long - first + n_short;
+    // the longest by the whole block (as many as there is room for); then, as warps come free, 32 small ones at a time and the others one by one
+    const int n_long = min(s_long, 4 * TOPK_WIDE), n_small = s_n, small_steps = (n_small + 31) / 32, steps = small_steps + s_big;
+    for (int j = 0; j < n_long; ++j)
+        topk_wide(t, s_long_job[j].y, k, warp, lane, s_best, s_total, [&](unsigned long long best, uint32_t total) { write(s_long_job[j].x, best, total); });
     for (;;) {
         int j = 0;
         if (lane == 0) j = atomicAdd(&s_cursor, 1);
         j = __shfl_sync(0xffffffffu, j, 0);
-        if (j >= jobs) break;
-        const int2 job = j < n_long - first ? s_job[per_block - 1 - first - j] : s_job[j - (n_long - first)];
-        unsigned long long best = 0;
-        uint32_t total = 0;
-        tg_scan(t, tg_open(t, (uint32_t)job.y, lane), 0, 1, k, lane, best, total);
-        write(job.x, best, __reduce_add_sync(0xffffffffu, total));
+        if (j >= steps) break;
+        if (j < small_steps) {
+            const int i = j * 32 + lane;
+            if (i < n_small) {
+                const TopkJob job = s_job[i];
+                topk_thread(t, job, k, vec, out_tok + (size_t)job.row * k, out_cnt + (size_t)job.row * k, out_total ? out_total + job.row : nullptr);
+            }
+            __syncwarp();
+        } else {
+            const TopkJob job = s_job[TOPK_LEAD_QUERIES - 1 - (j - small_steps)];
+            unsigned long long best = 0;
+            uint32_t total = 0;
+            tg_scan(t, tg_open(t, (uint32_t)job.home, lane), 0, 1, k, lane, best, total);
+            write(job.row, best, __reduce_add_sync(0xffffffffu, total));
+        }
     }
 }
 
-__global__ void __launch_bounds__(256) k_topk_copy(int q, int k, int32_t* __restrict__ out_tok, uint32_t* __restrict__ out_cnt, uint32_t* __restrict__ out_total) {
+// V: the words of a row that one load takes (1, 2, 4: k is a multiple of it and the arrays are aligned to it).
+template <typename V>
+__global__ void __launch_bounds__(256) k_topk_copy(int q, int k, V* __restrict__ out_tok, V* __restrict__ out_cnt, uint32_t* __restrict__ out_total) {
+    pdl_enter();
     const uint32_t row = blockIdx.x * 256 + threadIdx.x;
     if (row >= (uint32_t)q) return;
-    const int i = (int)row;
-    const int mark = out_tok[(size_t)i * k];
+    const int words = k / (int)(sizeof(V) / sizeof(int32_t));
+    const int mark = reinterpret_cast<const int32_t*>(out_tok)[(size_t)row * k];
     if (mark >= MARK_OWN) return;
-    const size_t from = (size_t)mark_leader(mark) * k, to = (size_t)i * k;
-    for (int r = 0; r < k; ++r) { out_tok[to + r] = out_tok[from + r]; out_cnt[to + r] = out_cnt[from + r]; }
-    if (out_total) out_total[i] = out_total[mark_leader(mark)];
+    const uint32_t lead = (uint32_t)mark_leader(mark);
+    const size_t from = (size_t)lead * words, to = (size_t)row * words;
+    uint32_t total = 0;
+    if (out_total) total = out_total[lead];
+    for (int r = 0; r < words; ++r) {
+        const V a = out_tok[from + r], b = out_cnt[from + r];
+        out_tok[to + r] = a;
+        out_cnt[to + r] = b;
+    }
+    if (out_total) out_total[row] = total;
 }
 
 // Draft tree of n_nodes nodes for the context (ctx[0], ctx[1]); one block of 32 warps.
@@ -1068,17 +1242,26 @@ aded_status aded_trigram_topk(const aded_trigram* t, const int32_t* ctx_dev, int
     // As many queries per block as fill the device's block slots once (three blocks per SM).
     const int wave = ws_grid_limit(t->device) / 2 * 3;
     int per_block = (int)(((int64_t)q + wave - 1) / wave);
-    if (q >= TOPK_BULK && k >= 2) {
-        uint32_t slots = TOPK_BULK;
-        while ((uint64_t)slots * 2 <= (uint64_t)q * k && slots < (1u << 31)) slots *= 2;
+    if (q >= topk_bulk_min(t->view.n_home) && k >= 2) {
+        uint32_t slots = 1;
+        while ((uint64_t)slots * 2 < (uint64_t)q) slots *= 2;
+        const int deferred = (int)((slots + k - 1) / k);             // rows whose counts the hash table lies in
         per_block = per_block > TOPK_LEAD_QUERIES ? TOPK_LEAD_QUERIES : per_block;
         ADED_CUDA_TRY(cudaMemsetAsync(out_counts_dev, 0xFF, (size_t)slots * sizeof(uint32_t), st));
         note_launch(3);
         const int lead_blocks = (int)(((int64_t)q + per_block - 1) / per_block);
-        k_topk_mark<<<(unsigned)(((long long)lead_blocks * per_block + 255) / 256), 256, 0, st>>>(t->view, ctx_dev, q, k, lead_blocks, per_block, slots - 1,
-                                                                                             out_tokens_dev, out_counts_dev);
-        k_topk_lead<<<lead_blocks, TOPK_THREADS, 0, st>>>(t->view, q, k, per_block, out_tokens_dev, out_counts_dev, out_total_dev);
-        k_topk_copy<<<(unsigned)(((int64_t)q + 255) / 256), 256, 0, st>>>(q, k, out_tokens_dev, out_counts_dev, out_total_dev);
+        const uintptr_t low = reinterpret_cast<uintptr_t>(out_tokens_dev) | reinterpret_cast<uintptr_t>(out_counts_dev);
+        const int vec = k % 4 == 0 && low % 16 == 0 ? 4 : k % 2 == 0 && low % 8 == 0 ? 2 : 1;      // words of a row that one load or store takes
+        launch_k(k_topk_mark, dim3((unsigned)(((int64_t)q + MARK_THREADS - 1) / MARK_THREADS)), dim3(MARK_THREADS), 0, st, t->view, ctx_dev, q, k, vec, slots - 1,
+                 deferred, out_tokens_dev, out_counts_dev, out_total_dev);
+        launch_k(k_topk_lead, dim3(lead_blocks), dim3(TOPK_THREADS), 0, st, t->view, q, k, vec, per_block, out_tokens_dev, out_counts_dev, out_total_dev);
+        const dim3 grid((unsigned)(((int64_t)q + 255) / 256));
+        if (vec == 4)
+            launch_k(k_topk_copy<int4>, grid, dim3(256), 0, st, q, k, reinterpret_cast<int4*>(out_tokens_dev), reinterpret_cast<int4*>(out_counts_dev), out_total_dev);
+        else if (vec == 2)
+            launch_k(k_topk_copy<int2>, grid, dim3(256), 0, st, q, k, reinterpret_cast<int2*>(out_tokens_dev), reinterpret_cast<int2*>(out_counts_dev), out_total_dev);
+        else
+            launch_k(k_topk_copy<int32_t>, grid, dim3(256), 0, st, q, k, out_tokens_dev, reinterpret_cast<int32_t*>(out_counts_dev), out_total_dev);
         ADED_CUDA_TRY(cudaGetLastError());
         return ADED_OK;
     }

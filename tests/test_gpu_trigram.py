@@ -497,3 +497,41 @@ def test_export_with_more_long_contexts_than_a_block_shares(cuda_device, entries
         keys, got = B.aded_trigram_export(t, least)
         want = packed(rows)[counts >= least] * 4 + counts[counts >= least]
         assert torch.equal((packed(keys) * 4 + got).sort().values, want.sort().values)
+
+
+@pytest.mark.parametrize("k,offset", [(2, 0), (2, 1), (3, 0), (4, 0), (4, 1), (4, 2), (6, 0), (8, 0), (12, 0), (32, 0)])
+def test_grouped_lookups_of_a_large_table(cuda_device, k, offset):
+    """Tables of many home buckets group from 4096 queries on.  Rows that are answered in the first kernel and rows whose counts its hash
+    table takes, contexts of every size on both sides of what a thread, a warp and a block look up, repeated within and across the first
+    kernel's blocks, absent and invalid ones, rows of one, two and four words per store: all as the same lookups in small calls."""
+    from paper_2407_12021_b200 import binding as B
+    vocab = 3000
+    t = B.aded_trigram_create(vocab, log2_buckets=21, overflow_buckets=1 << 16)
+    sizes = [1, 5, 6, 7, 8, 12, 13, 18, 19, 30, 31, 53, 54, 55, 60, 200, 2053, 2054, 2055, 2600]
+    for i, n in enumerate(sizes):                          # context (2900 + i, i): n continuations, some of them twice
+        span = [tok for c in range(n) for tok in (2900 + i, i, (c * 7 + i) % vocab)] + [tok for c in range(0, n, 3) for tok in (2900 + i, i, (c * 7 + i) % vocab)]
+        B.aded_trigram_update(t, torch.tensor(span, dtype=torch.int32, device="cuda"))
+    B.aded_trigram_update(t, gen.zipf_tokens(20000, 300, 71, 1).cuda())
+    g = torch.Generator().manual_seed(72)
+    for q in (4096, 5001):
+        ctx = torch.stack([gen.zipf_tokens(q, 300, 73, 1), gen.zipf_tokens(q, 300, 74, 1)], dim=1)
+        pick = torch.randint(0, 4 * len(sizes), (q,), generator=g)
+        for i in range(len(sizes)):
+            ctx[pick == i] = torch.tensor([2900 + i, i], dtype=ctx.dtype)
+        ctx[::97] = torch.tensor([-1, 5], dtype=ctx.dtype)
+        ctx[5::89] = torch.tensor([7, vocab], dtype=ctx.dtype)
+        ctx = ctx.to(torch.int32).cuda().contiguous()
+
+        def rows(n):
+            flat = [torch.full((n * k + offset,), -5, dtype=torch.int32, device="cuda") for _ in range(2)]
+            return [f[offset:].view(n, k) for f in flat] + [torch.full((n,), -5, dtype=torch.int32, device="cuda")]
+
+        tok, cnt, total = rows(q)
+        B.aded_trigram_topk(t, ctx, k, tok, cnt, total)
+        for a in range(0, q, 1000):
+            part = ctx[a:a + 1000].contiguous()
+            want = rows(part.shape[0])
+            B.aded_trigram_topk(t, part, k, *want)
+            for got, ref in zip((tok, cnt, total), want):
+                assert torch.equal(got[a:a + 1000], ref), (q, a)
+    assert B.aded_trigram_poll_status(t) == 0
