@@ -613,44 +613,73 @@ __global__ void __launch_bounds__(256) k_topk_copy(int q, int k, V* __restrict__
 // Level by level: every node of the current level gets its top-k list -- the block's warps are shared out evenly, so that
 // the first levels' few nodes, whose contexts may have thousands of continuations, are scanned by several warps each --
 // then one warp appends the lists in node order, rank order: the same tree as visiting the nodes in index order.
-// Latency-bound: a level is the chain home bucket -> directory -> entries -> merge.  The filler pass (one thread; child lists kept in shared memory) hangs caller-
+// Latency-bound: a level is the chain home bucket -> directory -> entries -> merge.  The filler pass (draft_fill) hangs caller-
 // supplied tokens under nodes with room, round-robin, until the tree is full.
 constexpr int DRAFT_MAX_FILLER = 4 * ADED_MAX_NODES;
 
-// Filler pass of one thread over a tree held in shared memory (tok, par, dep; kid[p][0 .. nkid[p]) the
-// child tokens of node p): nodes are visited round-robin, a visited node with depth < max_depth and
-// fewer than k children gets the next filler token none of its children holds.  Returns the new node
-// count; *fail when the filler runs out, holds a token outside the vocabulary, or no node has room.
+// Filler pass over a tree held in shared memory (tok, par, dep; kid[p][0 .. nkid[p]) the child tokens of node p), by one warp:
+// nodes are visited round-robin, a visited node with depth < max_depth and fewer than k children gets the next filler token
+// none of its children holds.  Returns the new node count (every lane); *fail when the filler runs out, holds a token outside the
+// vocabulary, or no node has room.  The steps depend on one another, so each is kept short: the nodes with room wait in two lists
+// (`turn`, [2][ADED_MAX_NODES]: of this round, to which new nodes are added, and of the next), and the lanes compare a token with all
+// children at once.  (A thread that visited every node took 28 us for 50 of 97 nodes.)
 __device__ __forceinline__ int draft_fill(int32_t* tok, int32_t* par, int32_t* dep, int32_t* nkid, int32_t* kid, int n, int n_nodes,
-                                          int max_depth, int k, const int32_t* fill, int n_filler, int vocab, bool* fail) {
-    int pos = 0, p = 0, idle = 0;
+                                          int max_depth, int k, const int32_t* fill, int n_filler, int vocab, int lane, int16_t* turn, bool* fail) {
+    int16_t *now = turn, *then = turn + ADED_MAX_NODES;
+    int n_now = 0, n_then = 0, at = 0;
+    for (int i0 = 0; i0 < n; i0 += 32) {
+        const int i = i0 + lane;
+        const bool room = i < n && dep[i] < max_depth && nkid[i] < k;
+        const unsigned m = __ballot_sync(0xffffffffu, room);
+        if (room) now[n_now + __popc(m & ((1u << lane) - 1u))] = (int16_t)i;
+        n_now += __popc(m);
+    }
+    __syncwarp();
+    int pos = 0;
     while (n < n_nodes) {
-        const int nk = nkid[p];
-        if (dep[p] < max_depth && nk < k) {
-            int32_t f = -1;
-            for (; pos < n_filler; ++pos) {
-                f = fill[pos];
-                bool clash = false;
-                for (int j = 0; j < nk; ++j) clash |= kid[p * ADED_DRAFT_MAX_K + j] == f;
-                if (!clash) break;
-            }
-            if (pos >= n_filler || f < 0 || f >= vocab) { *fail = true; break; }
-            ++pos;
+        if (at == n_now) {
+            int16_t* const x = now;
+            now = then;
+            then = x;
+            n_now = n_then;
+            n_then = at = 0;
+            if (n_now == 0) { *fail = true; break; }
+        }
+        const int p = now[at++];
+        const int nk = nkid[p], depth = dep[p] + 1, child = lane < ADED_DRAFT_MAX_K ? kid[p * ADED_DRAFT_MAX_K + lane] : 0;
+        int32_t f = -1;
+        for (; pos < n_filler; ++pos) {
+            f = fill[pos];
+            if (!__any_sync(0xffffffffu, lane < nk && child == f)) break;
+        }
+        if (pos >= n_filler || f < 0 || f >= vocab) { *fail = true; break; }
+        ++pos;
+        if (lane == 0) {
             kid[p * ADED_DRAFT_MAX_K + nk] = f;
             nkid[p] = nk + 1;
             tok[n] = f;
             par[n] = p;
-            dep[n] = dep[p] + 1;
+            dep[n] = depth;
             nkid[n] = 0;
-            ++n;
-            idle = 0;
-        } else if (++idle > n) {
-            *fail = true;
-            break;
+            if (depth < max_depth) now[n_now] = (int16_t)n;
+            if (nk + 1 < k) then[n_then] = (int16_t)p;
         }
-        if (++p >= n) p = 0;
+        n_now += depth < max_depth;
+        n_then += nk + 1 < k;
+        ++n;
+        __syncwarp();
     }
     return n;
+}
+
+// The k best of the lists of `parts` warps, [parts][ADED_DRAFT_MAX_K] in shared memory, of which the first k of each are used.
+__device__ __forceinline__ void draft_merge(const unsigned long long* lists, int parts, int k, int lane, unsigned long long& best) {
+    constexpr int AT_ONCE = 32 / ADED_DRAFT_MAX_K;                // eight warps' lists at a time, two per lane
+    for (int i = 0; i < parts; i += 2 * AT_ONCE) {
+        const int from = i + lane / ADED_DRAFT_MAX_K, r = lane % ADED_DRAFT_MAX_K;
+        const unsigned long long* list = lists + from * ADED_DRAFT_MAX_K + r;
+        tg_offer2(from < parts && r < k ? list[0] : 0ull, from + AT_ONCE < parts && r < k ? list[AT_ONCE * ADED_DRAFT_MAX_K] : 0ull, k, lane, best);
+    }
 }
 
 __global__ void __launch_bounds__(1024)
@@ -661,6 +690,7 @@ k_draft_tree(TgView t, const int32_t* __restrict__ ctx, int n_nodes, int max_dep
     __shared__ int32_t s_cand[ADED_MAX_NODES * ADED_DRAFT_MAX_K];   // top-k lists, later the child tokens of every node
     __shared__ int32_t s_fill[DRAFT_MAX_FILLER];
     __shared__ unsigned long long s_part[32 * ADED_DRAFT_MAX_K];    // the lists of the warps that share a node
+    __shared__ int16_t s_turn[2 * ADED_MAX_NODES];
     __shared__ int s_n, s_lo, s_hi, s_fail;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     pdl_enter();
@@ -695,12 +725,7 @@ k_draft_tree(TgView t, const int32_t* __restrict__ ctx, int n_nodes, int max_dep
         __syncthreads();
         if (parts > 1 && warp < hi - lo) {
             unsigned long long best = 0;
-            constexpr int AT_ONCE = 32 / ADED_DRAFT_MAX_K;                // eight warps' lists at a time, two per lane
-            for (int i = 0; i < parts; i += 2 * AT_ONCE) {
-                const int from = i + lane / ADED_DRAFT_MAX_K, r = lane % ADED_DRAFT_MAX_K;
-                const unsigned long long* list = s_part + (warp * parts + from) * ADED_DRAFT_MAX_K + r;
-                tg_offer2(from < parts && r < k ? list[0] : 0ull, from + AT_ONCE < parts && r < k ? list[AT_ONCE * ADED_DRAFT_MAX_K] : 0ull, k, lane, best);
-            }
+            draft_merge(s_part + warp * parts * ADED_DRAFT_MAX_K, parts, k, lane, best);
             if (lane < k) s_cand[(lo + warp) * ADED_DRAFT_MAX_K + lane] = tg_packed_tok(best);
         }
         __syncthreads();
@@ -708,9 +733,12 @@ k_draft_tree(TgView t, const int32_t* __restrict__ ctx, int n_nodes, int max_dep
             int n = s_n;
             for (int node0 = lo; node0 < hi && n < n_nodes; node0 += 32) {
                 const int node = node0 + lane;
+                int32_t tok[ADED_DRAFT_MAX_K];
                 int mine = 0;                               // this node's children (valid entries come first)
-                if (node < hi)
-                    while (mine < k && s_cand[node * ADED_DRAFT_MAX_K + mine] >= 0) ++mine;
+#pragma unroll
+                for (int j = 0; j < ADED_DRAFT_MAX_K; ++j) tok[j] = node < hi && j < k ? s_cand[node * ADED_DRAFT_MAX_K + j] : -1;
+#pragma unroll
+                for (int j = 0; j < ADED_DRAFT_MAX_K; ++j) mine += tok[j] >= 0;
                 int upto = mine;
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
@@ -719,11 +747,13 @@ k_draft_tree(TgView t, const int32_t* __restrict__ ctx, int n_nodes, int max_dep
                 }
                 const int at = n + upto - mine;
                 const int kept = max(0, min(mine, n_nodes - at));
-                for (int j = 0; j < kept; ++j) {
-                    s_tok[at + j] = s_cand[node * ADED_DRAFT_MAX_K + j];
-                    s_par[at + j] = node;
-                    s_dep[at + j] = d + 1;
-                }
+#pragma unroll
+                for (int j = 0; j < ADED_DRAFT_MAX_K; ++j)
+                    if (j < kept) {
+                        s_tok[at + j] = tok[j];
+                        s_par[at + j] = node;
+                        s_dep[at + j] = d + 1;
+                    }
                 if (kept > 0) s_nkid[node] = kept;          // s_cand[node][0 .. kept) are this node's child tokens
                 n = min(n_nodes, n + __shfl_sync(0xffffffffu, upto, 31));
             }
@@ -731,16 +761,16 @@ k_draft_tree(TgView t, const int32_t* __restrict__ ctx, int n_nodes, int max_dep
         }
         __syncthreads();
     }
-    if (threadIdx.x == 0) {
+    if (warp == 0) {
         int n = s_n;
-        if (out_real) *out_real = n;
-        if (filler && n < n_nodes) {
-            bool fail = false;
-            n = draft_fill(s_tok, s_par, s_dep, s_nkid, s_cand, n, n_nodes, max_depth, k, s_fill, n_filler, t.vocab, &fail);
-            if (fail) s_fail = 1;
+        bool fail = false;
+        if (lane == 0 && out_real) *out_real = n;
+        if (filler && n < n_nodes) n = draft_fill(s_tok, s_par, s_dep, s_nkid, s_cand, n, n_nodes, max_depth, k, s_fill, n_filler, t.vocab, lane, s_turn, &fail);
+        __syncwarp();
+        if (lane == 0) {
             s_n = n;
+            if (fail) { s_fail = 1; atomicCAS(t.status, 0, (int)ADED_ERR_INVALID_ARG); }
         }
-        if (s_fail) atomicCAS(t.status, 0, (int)ADED_ERR_INVALID_ARG);
     }
     __syncthreads();
     const int n = s_n;
@@ -822,54 +852,62 @@ __global__ void k_tg_stats(TgView t, unsigned long long* out) {
 // ---- draft maker: Monte Carlo tree search (Eq. 2-3, Algorithm 1) -----------------------------------
 // One warp runs the search, in which every iteration reads what the last one left: bound by the latency of its chain of steps.
 // The tree is in shared memory; lanes hold the children of the node that is being left, the nodes of the current path, the
-// continuations of a looked-up context.  Floating point is IEEE double, one rounded operation at a time (no fused multiply-add),
-// so that the search can be reproduced bit for bit; the exploration factor E of Eq. 3 and the square root depend on an integer
-// only and come from tables the host computes; a node's mean score changes only when it is visited, a continuation's
-// probability never during a search, so each is divided out once, not at every look.
+// continuations of a looked-up context.  Floating point is IEEE double, one rounded operation at a time (no fused multiply-add
+// where the formulas have none), so that the search can be reproduced bit for bit; the exploration factor E of Eq. 3 and the
+// square root depend on an integer only and come from tables the host computes; a node's mean score changes only when it is
+// visited, a continuation's probability never during a search, so each is divided out once, not at every look.
+// A lookup in the table is three dependent reads of memory and took most of an iteration.  The contexts a search can meet are the
+// k-ary tree of continuations below the root's, which is small near the root: all warps of the block look up its first MC_AHEAD
+// contexts, level by level, before the search begins (85 contexts are all there are for sentences of 4 and k = 4).  Ranking the
+// sentences and laying out the result are the block's work too.
+// Measured, 150 iterations, sentences of 4, 24 of them, k = 4, table of 200,000 tokens, with the pass between two steps around it
+// (compaction, table update): 385 us with a warp for everything, 188 with this (search 125, looking up ahead 25, and what the kernel's own code costs to fetch).
 constexpr int MC_MAX_ITER = 160, MC_MAX_K = ADED_DRAFT_MAX_K, MC_MAX_LEN = 8;
 constexpr int MC_MAX_NODES = 1 + MC_MAX_ITER * MC_MAX_K;
-constexpr int MC_CACHE = 512;          // remembered lookups (direct mapped): a search meets the same contexts again and again
+constexpr int MC_WARPS = 16, MC_THREADS = MC_WARPS * 32;
+constexpr int MC_AHEAD = 352;          // contexts looked up ahead (all of k = 8 and two words, of k = 4 and four)
+constexpr int MC_CACHE_BYTES = 96 * 1024;
 
 struct McParams {
     int iterations, length, n_candidates, k;
+    int slots;                         // of the remembered lookups: a power of two
     double e_table[MC_MAX_ITER + 1];   // E for sum N = 0 .. iterations
     double root[MC_MAX_ITER + 1];      // square root of sum N
 };
+static int mc_slots(int k) {
+    int n = 64;
+    while (2 * n * (12 + 20 * k) <= MC_CACHE_BYTES) n *= 2;
+    return n;
+}
 
-// Top-k list of one context: lane j holds the j-th continuation.
+// A node of the search tree: visits, token, link, and visits of its children together | the child that is to be visited next << 16.
+// link: first child (children are consecutive), number of children << 16, flags.
+constexpr int MC_EXPANDED = 1 << 24, MC_CHOSEN = 1 << 25, MC_KEPT = 1 << 26;
+__device__ __forceinline__ int mc_first(int link) { return link & 0xFFFF; }
+__device__ __forceinline__ int mc_kids(int link) { return link >> 16 & 0xFF; }
+
+// Remembered lookups, each in one of two neighbouring slots.  (The key of an empty slot is that of the context (-1, -1), which a caller
+// may pass: no continuations, the right answer for it.)
+struct McCache {
+    unsigned long long* key;           // [slots]
+    unsigned long long* upto;          // [slots][k] sum of the counts of continuations 0 .. j
+    double* prob;                      // [slots][k]
+    int32_t* word;                     // [slots][k]
+    int32_t* n;                        // [slots]
+    uint32_t mask;
+    int k;
+};
+// Top-k list of one context: lane j < k holds the j-th continuation, the others nothing of use.
 struct McLookup {
     int n;                             // continuations (every lane)
     int32_t word;
     double prob;                       // Eq. 1: count over the sum of ALL the context's counts
     unsigned long long upto;           // sum of the counts of continuations 0 .. j
 };
-struct McSlot {                        // the same in shared memory
-    unsigned long long key;
-    unsigned long long upto[MC_MAX_K];
-    double prob[MC_MAX_K];
-    int32_t word[MC_MAX_K];
-    int32_t n, pad;
-};
-
-// All 32 lanes call this with the same (a, b).  Remembered contexts come from shared memory (the table does not change during a
-// search); lanes from MC_MAX_K on hold nothing of use.
-__device__ __forceinline__ McLookup mc_lookup(const TgView& t, int a, int b, int k, int lane, McSlot* s_cache) {
-    const unsigned long long key = tg_key(a, b);
-    McSlot& slot = s_cache[tg_hash(key) & (MC_CACHE - 1)];
-    const int j = lane & (MC_MAX_K - 1);
+// The k best of a context whose second token is b, and the sum of its counts, as a lookup, into slot `slot` (all 32 lanes).
+__device__ __forceinline__ McLookup mc_keep(const TgView& t, int b, unsigned long long best, uint32_t total, int lane, const McCache& c, uint32_t slot) {
+    if (lane >= c.k) best = 0;
     McLookup out;
-    if (slot.key == key) {
-        out.n = slot.n;
-        out.word = slot.word[j];
-        out.prob = slot.prob[j];
-        out.upto = slot.upto[j];
-        return out;
-    }
-    unsigned long long best = 0;
-    uint32_t total = 0;
-    tg_scan(t, tg_open(t, a, b, lane), 0, 1, k, lane, best, total);
-    total = __reduce_add_sync(0xffffffffu, total);
-    if (lane >= k) best = 0;
     out.n = __popc(__ballot_sync(0xffffffffu, best != 0));
     out.word = tg_packed_tok(best);
     out.prob = best ? __ddiv_rn((double)tg_packed_cnt(best), (double)total) : 0.0;
@@ -883,209 +921,425 @@ __device__ __forceinline__ McLookup mc_lookup(const TgView& t, int a, int b, int
         const unsigned long long other = __shfl_up_sync(0xffffffffu, out.upto, o);
         if (lane >= o) out.upto += other;
     }
+    if (lane < c.k) {
+        c.upto[slot * c.k + lane] = out.upto;
+        c.prob[slot * c.k + lane] = out.prob;
+        c.word[slot * c.k + lane] = out.word;
+    }
+    if (lane == 0) c.n[slot] = out.n;
+    return out;
+}
+__device__ __forceinline__ McLookup mc_read(const TgView& t, int a, int b, int lane, const McCache& c, uint32_t slot) {
+    unsigned long long best = 0;
+    uint32_t total = 0;
+    tg_scan(t, tg_open(t, a, b, lane), 0, 1, c.k, lane, best, total);
+    return mc_keep(t, b, best, __reduce_add_sync(0xffffffffu, total), lane, c, slot);
+}
+// A slot for a context: -1 when somebody has it already, or both its slots are taken.
+__device__ __forceinline__ int mc_claim(const McCache& c, int2 context) {
+    const unsigned long long key = tg_key(context.x, context.y);
+    const uint32_t h = tg_hash(key) & c.mask;
+    for (uint32_t way = 0; way < 2; ++way) {
+        const unsigned long long have = atomicCAS(&c.key[h ^ way], TG_EMPTY, key);
+        if (have == TG_EMPTY) return (int)(h ^ way);
+        if (have == key) return -1;
+    }
+    return -1;
+}
+// The searching warp's lookup (all 32 lanes the same context; the table does not change during a search).
+__device__ __forceinline__ McLookup mc_lookup(const TgView& t, int a, int b, int lane, const McCache& c) {
+    const unsigned long long key = tg_key(a, b);
+    const uint32_t h = tg_hash(key) & c.mask;
+    const unsigned long long k0 = c.key[h], k1 = c.key[h ^ 1];
+    if (k0 == key || k1 == key) {
+        const uint32_t slot = k0 == key ? h : h ^ 1, at = slot * c.k + min(lane, c.k - 1);
+        McLookup out;
+        out.n = c.n[slot];
+        out.word = c.word[at];
+        out.prob = c.prob[at];
+        out.upto = c.upto[at];
+        return out;
+    }
+    const uint32_t slot = k0 == TG_EMPTY || k1 != TG_EMPTY ? h : h ^ 1;
+    const McLookup out = mc_read(t, a, b, lane, c, slot);
     __syncwarp();
-    if (lane < MC_MAX_K) { slot.upto[lane] = out.upto; slot.prob[lane] = out.prob; slot.word[lane] = out.word; }
-    if (lane == 0) { slot.n = out.n; slot.key = key; }
+    if (lane == 0) c.key[slot] = key;
     __syncwarp();
     return out;
 }
 
-__host__ __device__ constexpr size_t mc_cache_offset() {
-    return (((size_t)MC_MAX_NODES * (3 * 8 + 2 * 4 + 2 * 2 + 2 * 1) + ADED_MAX_NODES * 2) + 15) & ~(size_t)15;
+// a / n for n = 1 .. MC_MAX_ITER + 1, correctly rounded, given the correctly rounded 1 / n: the quotient within one place of the exact
+// one, then Markstein's last step ("Computation of elementary functions on the IBM RISC System/6000 processor", 1990).  What could
+// overflow or lose bits on the way takes the operator.
+__device__ __forceinline__ double mc_div(double a, int n, double rcp) {
+    const unsigned hi = (unsigned)__double2hiint(a) & 0x7FFFFFFFu;
+    if (hi - 0x06000000u >= 0x78000000u) return a == 0.0 ? a : __ddiv_rn(a, (double)n);      // (zero, |a| < 2^-927, > 2^992, infinite, NaN)
+    const double d = -(double)n;
+    double q = __dmul_rn(a, rcp);
+    q = __fma_rn(__fma_rn(d, q, a), rcp, q);
+    return __fma_rn(__fma_rn(d, q, a), rcp, q);
 }
 
-__host__ __device__ constexpr size_t mc_fill_offset() {
-    return (mc_cache_offset() + (size_t)MC_CACHE * sizeof(McSlot) + (size_t)MC_MAX_ITER * MC_MAX_LEN * sizeof(float) + 15) & ~(size_t)15;
+struct McLayout {          // byte offsets in shared memory
+    size_t score, prior, mean, er, rcp, list, node, par, queue, key, upto, prob, word, n, u, tok, fpar, dep, nkid, kid, fill, end;
+};
+__host__ __device__ constexpr McLayout mc_layout(int slots, int k) {
+    McLayout l = {};
+    size_t at = 0;
+    auto take = [&](size_t bytes) { const size_t here = at; at += (bytes + 15) / 16 * 16; return here; };
+    l.score = take((size_t)MC_MAX_NODES * 8);                  // sum of scores
+    l.prior = take((size_t)MC_MAX_NODES * 8);                  // Eq. 1 probability of the node's token in its parent's context
+    l.mean = take((size_t)MC_MAX_NODES * 8);                   // mean score (0 while not visited)
+    l.er = take((size_t)(MC_MAX_ITER + 1) * 16);               // E and square root
+    l.rcp = take((size_t)(MC_MAX_ITER + 2) * 8);               // 1 / n
+    l.list = take((size_t)MC_AHEAD * 8);                       // contexts looked up ahead
+    l.node = take((size_t)MC_MAX_NODES * 16);
+    l.par = take((size_t)MC_MAX_NODES * 2);
+    l.queue = take((size_t)ADED_MAX_NODES * 2);                // breadth-first order of the result
+    l.key = take((size_t)slots * 8);
+    l.upto = take((size_t)slots * k * 8);
+    l.prob = take((size_t)slots * k * 8);
+    l.word = take((size_t)slots * k * 4);
+    l.n = take((size_t)slots * 4);
+    l.u = take((size_t)MC_MAX_ITER * MC_MAX_LEN * 4);          // the caller's uniform numbers
+    l.tok = take((size_t)ADED_MAX_NODES * 4);                  // the result (see draft_fill)
+    l.fpar = take((size_t)ADED_MAX_NODES * 4);
+    l.dep = take((size_t)ADED_MAX_NODES * 4);
+    l.nkid = take((size_t)ADED_MAX_NODES * 4);
+    l.kid = take((size_t)ADED_MAX_NODES * ADED_DRAFT_MAX_K * 4);
+    l.fill = take((size_t)DRAFT_MAX_FILLER * 4);
+    l.end = at;
+    return l;
 }
 
-__global__ void __launch_bounds__(32)
+__global__ void __launch_bounds__(MC_THREADS, 1)
 k_mcts_draft(TgView t, const __grid_constant__ McParams p, const int32_t* __restrict__ ctx, const float* __restrict__ u,
              int32_t* __restrict__ out_tok, int32_t* __restrict__ out_par, int32_t* __restrict__ out_n,
              int32_t* __restrict__ sent_tok, double* __restrict__ sent_score, int32_t* __restrict__ out_n_sent,
              int n_target, const int32_t* __restrict__ filler, int n_filler) {
     extern __shared__ __align__(16) uint8_t mc_smem[];
-    // 8-byte, then 4-byte, then 2-byte, then 1-byte arrays, so that each starts aligned
-    double* s_score = reinterpret_cast<double*>(mc_smem);                 // [MC_MAX_NODES] sum of scores
-    double* s_prior = s_score + MC_MAX_NODES;                             // Eq. 1 probability of the node's token in its parent's context
-    double* s_mean = s_prior + MC_MAX_NODES;                              // mean score (0 while not visited)
-    int32_t* s_tok = reinterpret_cast<int32_t*>(s_mean + MC_MAX_NODES);   // token
-    int32_t* s_visits = s_tok + MC_MAX_NODES;
-    int16_t* s_par = reinterpret_cast<int16_t*>(s_visits + MC_MAX_NODES);
-    int16_t* s_first = s_par + MC_MAX_NODES;                              // first child (children are consecutive)
-    int16_t* s_queue = s_first + MC_MAX_NODES;                            // [ADED_MAX_NODES] breadth-first order of the result
-    uint8_t* s_nkid = reinterpret_cast<uint8_t*>(s_queue + ADED_MAX_NODES);
-    uint8_t* s_flag = s_nkid + MC_MAX_NODES;                              // bit 0 expanded, bit 1 chosen, bit 2 kept
-    McSlot* s_cache = reinterpret_cast<McSlot*>(mc_smem + mc_cache_offset());   // [MC_CACHE] remembered lookups
-    // (the key of an empty slot is that of the context (-1, -1), which a caller may pass: no continuations, the right answer for it)
-    for (int i = threadIdx.x; i < MC_CACHE; i += 32) { s_cache[i].key = TG_EMPTY; s_cache[i].n = 0; }
-    pdl_enter();
-    float* s_u = reinterpret_cast<float*>(s_cache + MC_CACHE);            // the caller's uniform numbers
-    for (int i = threadIdx.x; i < p.iterations * p.length; i += 32) s_u[i] = u[i];
-
-    const int lane = threadIdx.x;
-    const int prev_token = ctx[0], root_token = ctx[1];
-    int n_nodes = 1;
-    if (lane == 0) {
-        s_tok[0] = root_token; s_par[0] = -1; s_first[0] = 0; s_nkid[0] = 0; s_flag[0] = 0;
-        s_visits[0] = 0; s_score[0] = 0.0; s_prior[0] = 0.0; s_mean[0] = 0.0;
+    __shared__ int s_count, s_next, s_nodes;
+    __shared__ unsigned long long s_part[MC_WARPS * MC_MAX_K];
+    __shared__ uint32_t s_total[MC_WARPS];
+    __shared__ int s_slot[MC_WARPS], s_sent[ADED_MAX_NODES];
+    __shared__ uint3 s_top[MC_WARPS];
+    const McLayout lay = mc_layout(p.slots, p.k);
+    double* s_score = reinterpret_cast<double*>(mc_smem + lay.score);
+    double* s_prior = reinterpret_cast<double*>(mc_smem + lay.prior);
+    double* s_mean = reinterpret_cast<double*>(mc_smem + lay.mean);
+    double2* s_er = reinterpret_cast<double2*>(mc_smem + lay.er);
+    double* s_rcp = reinterpret_cast<double*>(mc_smem + lay.rcp);
+    int2* s_list = reinterpret_cast<int2*>(mc_smem + lay.list);
+    int4* s_node = reinterpret_cast<int4*>(mc_smem + lay.node);
+    int16_t* s_par = reinterpret_cast<int16_t*>(mc_smem + lay.par);
+    int16_t* s_queue = reinterpret_cast<int16_t*>(mc_smem + lay.queue);
+    float* s_u = reinterpret_cast<float*>(mc_smem + lay.u);
+    int32_t* f_fill = reinterpret_cast<int32_t*>(mc_smem + lay.fill);
+    McCache cache;
+    cache.key = reinterpret_cast<unsigned long long*>(mc_smem + lay.key);
+    cache.upto = reinterpret_cast<unsigned long long*>(mc_smem + lay.upto);
+    cache.prob = reinterpret_cast<double*>(mc_smem + lay.prob);
+    cache.word = reinterpret_cast<int32_t*>(mc_smem + lay.word);
+    cache.n = reinterpret_cast<int32_t*>(mc_smem + lay.n);
+    cache.mask = (uint32_t)p.slots - 1;
+    cache.k = p.k;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    for (int i = tid; i < p.slots; i += MC_THREADS) { cache.key[i] = TG_EMPTY; cache.n[i] = 0; }
+    for (int i = tid; i <= MC_MAX_ITER; i += MC_THREADS) {
+        s_er[i] = make_double2(p.e_table[i], p.root[i]);
+        s_rcp[i + 1] = __ddiv_rn(1.0, (double)(i + 1));
     }
-    __syncwarp();
-    for (int it = 0; it < p.iterations; ++it) {
-        // the sentence so far: its last two tokens, its score (1 + the probabilities in order), and the tree nodes on it --
-        // lane d holds the node at depth d
-        int node = 0, len = 1, on_path = 0, depth = 0;
-        int before = prev_token, last = root_token;
-        double sc = 1.0;
-        // selection
-        while (s_nkid[node] > 0 && len <= p.length) {       // (a node has children only once it is expanded)
-            const int first = s_first[node], nk = s_nkid[node];
-            const bool mine = lane < nk;
-            const int c = first + (mine ? lane : 0);
-            const int nv = mine ? s_visits[c] : 0;
-            const double pr = s_prior[c], q = s_mean[c];
-            const int n_sum = (int)__reduce_add_sync(0xffffffffu, (unsigned)nv);
-            const double score = __dadd_rn(q, __ddiv_rn(__dmul_rn(__dmul_rn(p.e_table[n_sum], pr), p.root[n_sum]), __dadd_rn(1.0, (double)nv)));
-            // the largest score, the earliest child among equals: bits of a double in an order that integers have, high half first
-            const unsigned long long bits = (unsigned long long)__double_as_longlong(score);
-            const unsigned long long ord = mine ? bits ^ ((bits >> 63) ? ~0ull : 1ull << 63) : 0ull;
-            const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(ord >> 32));
-            const bool top = mine && (unsigned)(ord >> 32) == hi;
-            const unsigned lo = __reduce_max_sync(0xffffffffu, top ? (unsigned)ord : 0u);
-            const int pick = __ffs((int)__ballot_sync(0xffffffffu, top && (unsigned)ord == lo)) - 1;
-            node = first + pick;
-            ++depth;
-            if (lane == depth) on_path = node;
-            before = last;
-            last = s_tok[node];
-            sc = __dadd_rn(sc, __shfl_sync(0xffffffffu, pr, pick));
-            ++len;
+    pdl_enter();
+    for (int i = tid; i < p.iterations * p.length; i += MC_THREADS) s_u[i] = u[i];
+    if (n_target > 0 && filler)
+        for (int i = tid; i < n_filler; i += MC_THREADS) f_fill[i] = filler[i];
+    const int prev_token = ctx[0], root_token = ctx[1];
+    if (tid == 0) {
+        s_node[0] = make_int4(0, root_token, 0, 0);
+        s_par[0] = -1;
+        s_score[0] = 0.0;
+        s_prior[0] = 0.0;
+        s_mean[0] = 0.0;
+        s_list[0] = make_int2(prev_token, root_token);
+        s_count = 1;
+        s_next = 1;
+    }
+    __syncthreads();
+
+    // look up ahead: a level's contexts, by several warps each while they are few (the first may have thousands of continuations)
+    for (int lo = 0, level = 0; level < p.length; ++level) {
+        const int hi = s_count, n_ctx = hi - lo;
+        if (n_ctx <= 0) break;
+        const bool deeper = level + 1 < p.length && hi + n_ctx * p.k <= MC_AHEAD;
+        auto append = [&](int b, const McLookup& lk) {
+            if (!deeper || lk.n == 0) return;
+            int at = 0;
+            if (lane == 0) at = atomicAdd(&s_next, lk.n);
+            at = __shfl_sync(0xffffffffu, at, 0) + lane;
+            if (lane < lk.n) s_list[at] = make_int2(b, lk.word);      // (never more than MC_AHEAD: `deeper`)
+        };
+        int parts = 1;
+        while (parts * 2 * n_ctx <= MC_WARPS) parts *= 2;
+        if (parts > 1) {
+            const int g = warp / parts, part = warp % parts;
+            const int2 c = s_list[lo + min(g, n_ctx - 1)];
+            if (tid < n_ctx) s_slot[tid] = mc_claim(cache, s_list[lo + tid]);
+            unsigned long long best = 0;
+            uint32_t total = 0;
+            if (g < n_ctx) tg_scan(t, tg_open(t, c.x, c.y, lane), part, parts, p.k, lane, best, total);
+            total = __reduce_add_sync(0xffffffffu, total);
+            if (lane < MC_MAX_K) s_part[warp * MC_MAX_K + lane] = lane < p.k ? best : 0ull;
+            if (lane == 0) s_total[warp] = total;
+            __syncthreads();
+            if (g < n_ctx && part == 0 && s_slot[g] >= 0) {
+                best = 0;
+                draft_merge(s_part + warp * MC_MAX_K, parts, p.k, lane, best);
+                total = __reduce_add_sync(0xffffffffu, lane < parts ? s_total[warp + lane] : 0u);
+                append(c.y, mc_keep(t, c.y, best, total, lane, cache, (uint32_t)s_slot[g]));
+            }
+        } else {
+            for (int i = lo + warp; i < hi; i += MC_WARPS) {
+                const int2 c = s_list[i];
+                int slot = -1;
+                if (lane == 0) slot = mc_claim(cache, c);
+                slot = __shfl_sync(0xffffffffu, slot, 0);
+                if (slot >= 0) append(c.y, mc_read(t, c.x, c.y, lane, cache, (uint32_t)slot));
+            }
         }
-        // expansion
-        if (!(s_flag[node] & 1) && len <= p.length) {
-            const McLookup lk = mc_lookup(t, before, last, p.k, lane, s_cache);
-            if (lane == 0) {
-                s_flag[node] |= 1;
-                s_first[node] = (int16_t)n_nodes;
-                s_nkid[node] = (uint8_t)lk.n;
-            }
-            if (lane < lk.n) {
-                const int c = n_nodes + lane;
-                s_tok[c] = lk.word; s_par[c] = (int16_t)node; s_first[c] = 0; s_nkid[c] = 0; s_flag[c] = 0;
-                s_visits[c] = 0; s_score[c] = 0.0; s_mean[c] = 0.0;
-                s_prior[c] = lk.prob;
-            }
-            __syncwarp();
-            if (lk.n > 0) {
-                n_nodes += lk.n;
-                node = n_nodes - 1;                       // the last child created
+        __syncthreads();
+        if (tid == 0) s_count = s_next;
+        lo = hi;
+        __syncthreads();
+    }
+
+    if (warp == 0) {
+        const int kid_bits = p.k <= 4 ? 2 : 3;              // lanes per node of the path
+        int n_nodes = 1;
+        for (int it = 0; it < p.iterations; ++it) {
+            // the sentence so far: its last two tokens, its score (1 + the probabilities in order), and the tree nodes on it --
+            // lane d holds the node at depth d
+            int node = 0, len = 1, on_path = 0, depth = 0;
+            int before = prev_token, last = root_token;
+            double sc = 1.0;
+            int4 nd = s_node[0];
+            // selection: every node knows which child is next (see below)
+            while (mc_kids(nd.z) > 0 && len <= p.length) {      // (a node has children only once it is expanded)
+                node = nd.w >> 16;
+                nd = s_node[node];
+                sc = __dadd_rn(sc, s_prior[node]);
                 ++depth;
                 if (lane == depth) on_path = node;
                 before = last;
-                last = __shfl_sync(0xffffffffu, lk.word, lk.n - 1);
-                sc = __dadd_rn(sc, __shfl_sync(0xffffffffu, lk.prob, lk.n - 1));
+                last = nd.y;
                 ++len;
             }
+            const int link = nd.z;
+            // expansion
+            if (!(link & MC_EXPANDED) && len <= p.length) {
+                const McLookup lk = mc_lookup(t, before, last, lane, cache);
+                if (lane == 0) s_node[node].z = n_nodes | lk.n << 16 | MC_EXPANDED;
+                if (lane < lk.n) {
+                    const int c = n_nodes + lane;
+                    s_node[c] = make_int4(0, lk.word, 0, 0);
+                    s_par[c] = (int16_t)node;
+                    s_score[c] = 0.0;
+                    s_mean[c] = 0.0;
+                    s_prior[c] = lk.prob;
+                }
+                __syncwarp();
+                if (lk.n > 0) {
+                    n_nodes += lk.n;
+                    node = n_nodes - 1;                       // the last child created
+                    ++depth;
+                    if (lane == depth) on_path = node;
+                    before = last;
+                    last = __shfl_sync(0xffffffffu, lk.word, lk.n - 1);
+                    sc = __dadd_rn(sc, __shfl_sync(0xffffffffu, lk.prob, lk.n - 1));
+                    ++len;
+                }
+            }
+            // simulation
+            for (int draws = 0; len <= p.length; ++draws, ++len) {
+                const McLookup lk = mc_lookup(t, before, last, lane, cache);
+                if (lk.n == 0) break;
+                const unsigned long long total = __shfl_sync(0xffffffffu, lk.upto, lk.n - 1);
+                unsigned long long u24 = __float2uint_rd(__fmul_rn(s_u[it * p.length + draws], 16777216.f));
+                if (u24 > 16777215ull) u24 = 16777215ull;
+                const unsigned long long target = (total * u24) >> 24;
+                const unsigned past = __ballot_sync(0xffffffffu, lane < lk.n && lk.upto > target);
+                const int pick = past ? __ffs((int)past) - 1 : lk.n - 1;
+                before = last;
+                last = __shfl_sync(0xffffffffu, lk.word, pick);
+                sc = __dadd_rn(sc, __shfl_sync(0xffffffffu, lk.prob, pick));
+            }
+            // Back propagation, and every path node's next choice.  A choice depends on the node's children and their visits alone, which
+            // change only when the node is on the path: it is made now, for all nodes of the path side by side (a lane per child), not one
+            // after the other when they are met again (450 cycles a level, nearly all of them the chain of double-precision operations).
+            for (int d0 = 0; d0 < depth; d0 += 32 >> kid_bits) {
+                const int d = d0 + (lane >> kid_bits), j = lane & ((1 << kid_bits) - 1);
+                const int parent = __shfl_sync(0xffffffffu, on_path, d & 31), visited = __shfl_sync(0xffffffffu, on_path, (d + 1) & 31);
+                const int4 up = s_node[parent];
+                const int first = mc_first(up.z), below = (up.w & 0xFFFF) + 1;
+                const bool mine = d < depth && j < mc_kids(up.z);
+                const int c = mine ? first + j : 0;
+                const double2 er = s_er[min(below, MC_MAX_ITER)];
+                double mean = s_mean[c];
+                int visits = s_node[c].x;
+                const double explore = __dmul_rn(__dmul_rn(er.x, s_prior[c]), er.y);
+                if (mine && c == visited) {
+                    const double total = __dadd_rn(s_score[c], sc);
+                    ++visits;
+                    mean = mc_div(total, visits, s_rcp[visits]);
+                    s_node[c].x = visits;
+                    s_score[c] = total;
+                    s_mean[c] = mean;
+                }
+                const double score = __dadd_rn(mean, mc_div(explore, visits + 1, s_rcp[visits + 1]));
+                // the largest score, the earliest child among equals: bits of a double in an order that integers have
+                const unsigned long long bits = (unsigned long long)__double_as_longlong(score);
+                unsigned long long best = mine ? bits ^ ((bits >> 63) ? ~0ull : 1ull << 63) : 0ull;
+                int pick = j;
+                for (int o = 1 << kid_bits >> 1; o > 0; o >>= 1) {
+                    const unsigned long long other = __shfl_xor_sync(0xffffffffu, best, o);
+                    const int who = __shfl_xor_sync(0xffffffffu, pick, o);
+                    if (other > best || (other == best && who < pick)) { best = other; pick = who; }
+                }
+                if (j == 0 && d < depth) s_node[parent].w = below | (first + pick) << 16;
+            }
+            __syncwarp();
         }
-        // simulation
-        for (int draws = 0; len <= p.length; ++draws, ++len) {
-            const McLookup lk = mc_lookup(t, before, last, p.k, lane, s_cache);
-            if (lk.n == 0) break;
-            const unsigned long long total = __shfl_sync(0xffffffffu, lk.upto, lk.n - 1);
-            unsigned long long u24 = __float2uint_rd(__fmul_rn(s_u[it * p.length + draws], 16777216.f));
-            if (u24 > 16777215ull) u24 = 16777215ull;
-            const unsigned long long target = (total * u24) >> 24;
-            const unsigned past = __ballot_sync(0xffffffffu, lane < lk.n && lk.upto > target);
-            const int pick = past ? __ffs((int)past) - 1 : lk.n - 1;
-            before = last;
-            last = __shfl_sync(0xffffffffu, lk.word, pick);
-            sc = __dadd_rn(sc, __shfl_sync(0xffffffffu, lk.prob, pick));
-        }
-        // back propagation: a lane per node of the path
-        if (lane <= depth) {
-            const int v = s_visits[on_path] + 1;
-            const double total = __dadd_rn(s_score[on_path], sc);
-            s_visits[on_path] = v;
-            s_score[on_path] = total;
-            s_mean[on_path] = __ddiv_rn(total, (double)v);
-        }
-        __syncwarp();
+        if (lane == 0) s_nodes = n_nodes;
     }
+    __syncthreads();
+    const int n_nodes = s_nodes;
 
     // ranking: leaves of the search tree by mean score (descending), earlier nodes first on ties
     int n_sent = 0;
-    for (int r = 0; r < p.n_candidates; ++r) {
-        double best_m = -1.0;
-        int best_i = -1;
-        for (int i = 1 + lane; i < n_nodes; i += 32) {
-            if (s_nkid[i] != 0 || (s_flag[i] & 2)) continue;
-            const double m = s_mean[i];
-            if (best_i < 0 || m > best_m) { best_m = m; best_i = i; }     // i ascends within a lane: first wins ties
+    auto order = [&](int i) {                        // bits of a leaf's mean in an order that integers have; 0 for other nodes
+        const unsigned long long bits = (unsigned long long)__double_as_longlong(s_mean[i] + 0.0);
+        return mc_kids(s_node[i].z) != 0 ? 0ull : bits ^ ((bits >> 63) ? ~0ull : 1ull << 63);
+    };
+    if (n_nodes <= MC_THREADS) {                     // a thread per node counts the leaves in front of it (a round per sentence, below, takes about 0.5 us)
+        unsigned long long* s_order = reinterpret_cast<unsigned long long*>(s_score);     // (the sums are not needed any more)
+        const unsigned long long mine = tid >= 1 && tid < n_nodes ? order(tid) : 0ull;
+        __syncthreads();
+        s_order[tid] = mine;
+        const int leaves = __syncthreads_count(mine != 0);
+        n_sent = min(leaves, p.n_candidates);
+        if (mine != 0) {
+            int before = 0;
+            for (int i = 1; i < n_nodes; ++i) before += s_order[i] > mine || (s_order[i] == mine && i < tid);
+            if (before < n_sent) s_sent[before] = tid;
         }
-        for (int o = 16; o > 0; o >>= 1) {
-            const double om = __shfl_xor_sync(0xffffffffu, best_m, o);
-            const int oi = __shfl_xor_sync(0xffffffffu, best_i, o);
-            if (oi >= 0 && (best_i < 0 || om > best_m || (om == best_m && oi < best_i))) { best_m = om; best_i = oi; }
+        __syncthreads();
+    } else
+    for (; n_sent < p.n_candidates; ++n_sent) {
+        unsigned long long best = 0;                 // (bits of the mean in an order that integers have: 0 is none)
+        int best_i = MC_MAX_NODES;
+        for (int i = 1 + tid; i < n_nodes; i += MC_THREADS) {
+            const unsigned long long ord = s_node[i].z & MC_CHOSEN ? 0ull : order(i);
+            if (ord > best) { best = ord; best_i = i; }     // i ascends within a thread: first wins ties
         }
-        if (best_i < 0) break;
-        if (lane == 0) {
-            s_flag[best_i] |= 2;
-            int path[MC_MAX_LEN], d = 0;
-            for (int j = best_i; j > 0; j = s_par[j]) { s_flag[j] |= 4; path[d++] = s_tok[j]; }
-            for (int j = 0; j < p.length; ++j) sent_tok[r * p.length + j] = j < d ? path[d - 1 - j] : -1;
-            sent_score[r] = best_m;
+        auto top = [&]() {                           // over the warp, in every lane
+            const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(best >> 32));
+            const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(best >> 32) == hi ? (unsigned)best : 0u);
+            const unsigned long long all = (unsigned long long)hi << 32 | lo;
+            best_i = (int)__reduce_min_sync(0xffffffffu, best == all ? (unsigned)best_i : (unsigned)MC_MAX_NODES);
+            best = all;
+        };
+        top();
+        if (lane == 0) s_top[warp] = make_uint3((unsigned)(best >> 32), (unsigned)best, (unsigned)best_i);
+        __syncthreads();
+        const uint3 other = s_top[lane & (MC_WARPS - 1)];
+        best = (unsigned long long)other.x << 32 | other.y;
+        best_i = (int)other.z;
+        top();
+        if (best == 0) break;                        // (every thread has the same answer)
+        if (tid == 0) {
+            s_node[best_i].z |= MC_CHOSEN;
+            s_sent[n_sent] = best_i;
         }
-        __syncwarp();
-        ++n_sent;
+        __syncthreads();
     }
-    if (n_target > 0 && filler) {
-        int32_t* f_fill = reinterpret_cast<int32_t*>(mc_smem + mc_fill_offset()) + ADED_MAX_NODES * (4 + ADED_DRAFT_MAX_K);
-        for (int i = lane; i < n_filler; i += 32) f_fill[i] = filler[i];
-        __syncwarp();
+    for (int r = tid; r < n_sent; r += MC_THREADS) {
+        int d = 0;
+        for (int j = s_sent[r]; j > 0; j = s_par[j]) { atomicOr(&s_node[j].z, MC_KEPT); ++d; }
+        for (int e = d; e < p.length; ++e) sent_tok[r * p.length + e] = -1;
+        for (int j = s_sent[r]; j > 0; j = s_par[j]) sent_tok[r * p.length + --d] = s_node[j].y;
+        sent_score[r] = s_mean[s_sent[r]];
     }
-    // prefix tree of the chosen sentences, breadth first, children in creation order
+    __syncthreads();
+    if (warp != 0) return;
+    // prefix tree of the chosen sentences, breadth first, children in creation order: 32 nodes' children at a time
+    int32_t* f_tok = reinterpret_cast<int32_t*>(mc_smem + lay.tok);          // [ADED_MAX_NODES] each
+    int32_t* f_par = reinterpret_cast<int32_t*>(mc_smem + lay.fpar);
+    int32_t* f_dep = reinterpret_cast<int32_t*>(mc_smem + lay.dep);
+    int32_t* f_nkid = reinterpret_cast<int32_t*>(mc_smem + lay.nkid);
+    int32_t* f_kid = reinterpret_cast<int32_t*>(mc_smem + lay.kid);          // [ADED_MAX_NODES][ADED_DRAFT_MAX_K]
     if (lane == 0) {
-        int count = 1;
         s_queue[0] = 0;
-        out_tok[0] = root_token;
-        out_par[0] = -1;
-        for (int head = 0; head < count; ++head) {
-            const int nd = s_queue[head];
-            for (int c = s_first[nd]; c < s_first[nd] + s_nkid[nd]; ++c) {
-                if (!(s_flag[c] & 4) || count >= ADED_MAX_NODES) continue;
-                s_queue[count] = (int16_t)c;
-                out_tok[count] = s_tok[c];
-                out_par[count] = head;
-                ++count;
-            }
+        f_tok[0] = root_token;
+        f_par[0] = -1;
+        f_dep[0] = 0;
+    }
+    __syncwarp();
+    int count = 1;
+    for (int head0 = 0; head0 < count; ) {
+        const int head = head0 + lane, heads = min(32, count - head0);
+        int first = 0, nk = 0, mine = 0;
+        if (lane < heads) {
+            const int link = s_node[s_queue[head]].z;
+            first = mc_first(link);
+            nk = mc_kids(link);
+            for (int c = 0; c < nk; ++c) mine += (s_node[first + c].z & MC_KEPT) != 0;
         }
-        if (n_target > count && filler) {
-            // complete the prefix tree to a fixed number of nodes, by the rule of the draft-tree kernel
-            int32_t* f_tok = reinterpret_cast<int32_t*>(mc_smem + mc_fill_offset());       // [ADED_MAX_NODES] each
-            int32_t* f_par = f_tok + ADED_MAX_NODES;
-            int32_t* f_dep = f_par + ADED_MAX_NODES;
-            int32_t* f_nkid = f_dep + ADED_MAX_NODES;
-            int32_t* f_kid = f_nkid + ADED_MAX_NODES;                                      // [ADED_MAX_NODES][ADED_DRAFT_MAX_K]
-            int32_t* f_fill = f_kid + ADED_MAX_NODES * ADED_DRAFT_MAX_K;                   // [DRAFT_MAX_FILLER], staged above by the whole warp
-            for (int i = 0; i < count; ++i) { f_nkid[i] = 0; }
-            for (int i = 0; i < count; ++i) {
-                f_tok[i] = out_tok[i];
-                f_par[i] = out_par[i];
-                f_dep[i] = i == 0 ? 0 : f_dep[f_par[i]] + 1;
-                if (i > 0) { const int pp = f_par[i]; f_kid[pp * ADED_DRAFT_MAX_K + f_nkid[pp]] = f_tok[i]; f_nkid[pp] += 1; }
-            }
-            bool fail = false;
-            const int n2 = draft_fill(f_tok, f_par, f_dep, f_nkid, f_kid, count, n_target, p.length, p.k, f_fill, n_filler, t.vocab, &fail);
-            for (int i = count; i < n2; ++i) { out_tok[i] = f_tok[i]; out_par[i] = f_par[i]; }
-            count = n2;
-            if (fail) { atomicCAS(t.status, 0, (int)ADED_ERR_INVALID_ARG); out_tok[0] = -1; }
+        int upto = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int other = __shfl_up_sync(0xffffffffu, upto, o);
+            if (lane >= o) upto += other;
         }
+        int at = count + upto - mine, kept = 0;
+        if (lane < heads) {
+            for (int c = 0; c < nk; ++c) {
+                const int4 nd = s_node[first + c];
+                if (!(nd.z & MC_KEPT) || at >= ADED_MAX_NODES) continue;
+                s_queue[at] = (int16_t)(first + c);
+                f_tok[at] = nd.y;
+                f_par[at] = head;
+                f_dep[at] = f_dep[head] + 1;
+                f_kid[head * ADED_DRAFT_MAX_K + kept++] = nd.y;
+                ++at;
+            }
+            f_nkid[head] = kept;
+        }
+        count = min(ADED_MAX_NODES, count + __shfl_sync(0xffffffffu, upto, 31));
+        head0 += heads;
+        __syncwarp();
+    }
+    bool fail = false;
+    if (n_target > count && filler) {
+        // complete the prefix tree to a fixed number of nodes, by the rule of the draft-tree kernel
+        count = draft_fill(f_tok, f_par, f_dep, f_nkid, f_kid, count, n_target, p.length, p.k, f_fill, n_filler, t.vocab, lane, reinterpret_cast<int16_t*>(s_list), &fail);
+        __syncwarp();
+        if (fail && lane == 0) { atomicCAS(t.status, 0, (int)ADED_ERR_INVALID_ARG); f_tok[0] = -1; }
+        __syncwarp();
+    }
+    for (int i = lane; i < count; i += 32) {
+        out_tok[i] = f_tok[i];
+        out_par[i] = f_par[i];
+    }
+    if (lane == 0) {
         *out_n = count;
         *out_n_sent = n_sent;
     }
 }
 
-static size_t mc_smem_bytes() {
-    return mc_fill_offset() + (size_t)ADED_MAX_NODES * 4 * (4 + ADED_DRAFT_MAX_K) + (size_t)DRAFT_MAX_FILLER * 4 + 64;
+static int mc_smem_bytes(int slots, int k) { return (int)mc_layout(slots, k).end; }
+static int mc_smem_most() {
+    int most = 0;
+    for (int k = 1; k <= MC_MAX_K; ++k) most = mc_smem_bytes(mc_slots(k), k) > most ? mc_smem_bytes(mc_slots(k), k) : most;
+    return most;
 }
 
 }  // namespace aded
@@ -1330,7 +1584,7 @@ aded_status aded_mcts_draft(const aded_trigram* t, const int32_t* context_dev, i
         n_candidates < 1 || n_candidates * length + 1 > ADED_MAX_NODES || !(c2 > 0.f))
         return ADED_ERR_INVALID_ARG;
     if (!t->search_prepared) {      // (per handle: the limit is the device's, and a handle belongs to one)
-        ADED_CUDA_TRY(cudaFuncSetAttribute(k_mcts_draft, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mc_smem_bytes()));
+        ADED_CUDA_TRY(cudaFuncSetAttribute(k_mcts_draft, cudaFuncAttributeMaxDynamicSharedMemorySize, mc_smem_most()));
         t->search_prepared = true;
     }
     McParams p;
@@ -1338,10 +1592,11 @@ aded_status aded_mcts_draft(const aded_trigram* t, const int32_t* context_dev, i
     p.length = length;
     p.n_candidates = n_candidates;
     p.k = k;
+    p.slots = mc_slots(k);
     for (int n = 0; n <= MC_MAX_ITER; ++n) p.e_table[n] = (double)c1 + std::log(((double)n + (double)c2 + 1.0) / (double)c2);   // Eq. 3
     for (int n = 0; n <= MC_MAX_ITER; ++n) p.root[n] = std::sqrt((double)n);
     note_launch();
-    ADED_CUDA_TRY(launch_k(k_mcts_draft, 1, 32, mc_smem_bytes(), static_cast<cudaStream_t>(stream), t->view, p, context_dev, u_dev, tree_tokens_dev,
+    ADED_CUDA_TRY(launch_k(k_mcts_draft, 1, MC_THREADS, mc_smem_bytes(p.slots, k), static_cast<cudaStream_t>(stream), t->view, p, context_dev, u_dev, tree_tokens_dev,
                            tree_parents_dev, n_nodes_dev, sentence_tokens_dev, sentence_scores_dev, n_sentences_dev, n_nodes_target,
                            n_nodes_target > 0 ? filler_dev : nullptr, n_filler));
     return ADED_OK;
