@@ -344,6 +344,7 @@ struct aded_model {
     float* cand_val;                    // [R][vocab / 128] per-tile greedy candidates of the LM head
     int32_t* cand_idx;
 
+    bool f32_ok;            // fp32 model that dense_f32.cu takes, for calls of few rows (f32_fused)
     float* argmax_val;      // [R][ARGMAX_CHUNKS] best logit of each column chunk
     int32_t* argmax_idx;
 
@@ -396,6 +397,15 @@ void launch_swiglu(aded_model* m, const GemmOut& gu, cudaStream_t st);
 void launch_argmax(aded_model* m, const GemmOut& logits, cudaStream_t st);
 // Writes a projection result as a plain [rows, n] fp32 matrix (debug paths).
 void launch_materialize(aded_model* m, const GemmOut& src, float* dst, cudaStream_t st);
+
+// dense_f32.cu: fp32 models of small widths, calls of few rows
+bool f32_prepare(const aded_model* m);
+bool f32_fused(const aded_model* m, int rows);
+int f32_candidates(const aded_model* m);        // per row, of the LM head's result
+void launch_f32_qkv(aded_model* m, int layer, int rows, cudaStream_t st);
+void launch_f32_attention(aded_model* m, aded_kv* kv, int layer, int rows, cudaStream_t st);
+void launch_f32_rest(aded_model* m, int layer, int rows, cudaStream_t st);
+void launch_f32_head(aded_model* m, float* logits, int rows, cudaStream_t st);
 
 // dense_ws.cu: bf16 consumers of slot-resident projection results
 void launch_add_rmsnorm_ws(aded_model* m, const GemmOut& y, const void* gain, cudaStream_t st);

@@ -357,7 +357,8 @@ void launch_gemm_many(aded_model* m, int w_map, int x_map, int rows, int n, int 
 void launch_rmsnorm(aded_model* m, int rows, const void* gain, cudaStream_t st) {
     GemmOut none = {};
     none.rows = rows;
-    launch_add_rmsnorm_ws(m, none, gain, st);
+    if (m->ws_ready) launch_add_rmsnorm_ws(m, none, gain, st);
+    else launch_add_rmsnorm(m, none, gain, st);
 }
 
 GemmOut launch_gemm(aded_model* m, int w_map, int x_map, const void* x, const void* w, float* y, int row0, int rows, int n, int k,

@@ -214,6 +214,11 @@ static aded_status alloc_model(aded_model* m) {
         }
     }
     if (!m->ws_ready && !gemm_plain_prepare(c.dtype == ADED_BF16)) return ADED_ERR_CUDA;
+    m->f32_ok = f32_prepare(m);
+    if (m->f32_ok) {
+        TRY(dev_alloc(m, &m->cand_val, R * f32_candidates(m)));
+        TRY(dev_alloc(m, &m->cand_idx, R * f32_candidates(m)));
+    }
     return ADED_OK;
 }
 
@@ -265,7 +270,20 @@ static aded_status enqueue_pass(aded_model* m, aded_kv* kv, const CallPtrs& call
         launch_gemm_many(m, w_map, x_map, rows, n, k, e, kind, st);
         return true;
     };
+    const bool fused = f32_fused(m, rows);
+    auto capture_hidden = [&](int l) -> aded_status {
+        if (m->dbg_hidden)
+            ADED_CUDA_TRY(cudaMemcpyAsync((char*)m->dbg_hidden + (size_t)(l + 1) * hid_bytes, m->h, hid_bytes, cudaMemcpyDeviceToDevice, st));
+        return ADED_OK;
+    };
     for (int l = 0; l < c.n_layers; ++l) {
+        if (fused) {
+            { Span sp(m, PROF_GEMM, 1, st); launch_f32_qkv(m, l, rows, st); }
+            { Span sp(m, PROF_ATTN, 1, st); launch_f32_attention(m, kv, l, rows, st); }
+            { Span sp(m, PROF_GEMM, 3, st); launch_f32_rest(m, l, rows, st); }
+            TRY(capture_hidden(l));
+            continue;
+        }
         const aded_layer_weights& w = m->layers[l];
         const void* next_gain = l + 1 < c.n_layers ? m->layers[l + 1].norm1 : m->top.final_norm;
         auto project = [&](int which, int x_map, const void* x, const void* wt, int n, int k, int kind, auto&& consume) {
@@ -292,10 +310,9 @@ static aded_status enqueue_pass(aded_model* m, aded_kv* kv, const CallPtrs& call
         if (!many(4 * l + WS_MAP_GU, WS_X, 2 * F, d, e, TK_GEMM_GU))
             project(WS_MAP_GU, WS_X, m->x, w.wgu, 2 * F, d, TK_GEMM_GU, [&](const GemmOut& o) { launch_swiglu(m, o, st); });
         residual(WS_MAP_D, WS_X_ACT, m->act, w.wd, F, TK_GEMM_DOWN, next_gain);
-        if (m->dbg_hidden)
-            ADED_CUDA_TRY(cudaMemcpyAsync((char*)m->dbg_hidden + (size_t)(l + 1) * hid_bytes, m->h, hid_bytes,
-                                          cudaMemcpyDeviceToDevice, st));
+        TRY(capture_hidden(l));
     }
+    if (fused && chain_mode) { Span sp(m, PROF_OTHER, 1, st); launch_rmsnorm(m, rows, m->top.final_norm, st); }     // (nobody else makes m->x then)
     if (!chain_mode) {
         // The per-node logits are needed as a matrix only by the sampling mode and by a debug capture; the
         // greedy choice works from per-tile candidates left by the LM head's tail.
@@ -308,6 +325,7 @@ static aded_status enqueue_pass(aded_model* m, aded_kv* kv, const CallPtrs& call
         e.cand_idx = m->cand_idx;
         const bool many_head = !dense_logits && many(4 * c.n_layers, WS_X, c.vocab, d, e, TK_GEMM_HEAD);
         if (many_head) candidates = c.vocab / 32;
+        else if (fused) { Span sp(m, PROF_GEMM, 1, st); launch_f32_head(m, dense ? dense : m->logits, rows, st); }
         else each_pass([&](int row0, int part) {
             GemmOut lg;
             { Span sp(m, PROF_GEMM, 1, st);
@@ -316,7 +334,10 @@ static aded_status enqueue_pass(aded_model* m, aded_kv* kv, const CallPtrs& call
             if (dense && (lg.mode == 1 || dense != m->logits)) { Span sp(m, PROF_OTHER, 1, st); launch_materialize(m, lg, dense, st); }
             if (dense_logits && !m->samp_on) { Span sp(m, PROF_OTHER, 1, st); launch_argmax(m, lg, st); }
         });
-        if (m->samp_on) {
+        if (fused && !m->samp_on) {
+            Span sp(m, PROF_OTHER, 1, st);
+            launch_pick_accept(m, kv, batch, m->cand_val, m->cand_idx, f32_candidates(m), st);
+        } else if (m->samp_on) {
             // sampling mode: one drawn token per node in place of the greedy one
             Span sp(m, PROF_OTHER, 2, st);
             ADED_CUDA_TRY(launch_sample_rows(dense, rows, c.vocab, c.vocab, m->samp_temp, m->samp_top_p, m->samp_u, m->best,
@@ -407,6 +428,7 @@ aded_status aded_model_create(const aded_model_config* cfg, const aded_weights* 
     m->call_dev = nullptr;
     m->ws_ready = false;
     m->many_ok = false;
+    m->f32_ok = false;
     m->ws_slots = nullptr;
     if (cudaGetDevice(&m->device) != cudaSuccess) {
         delete m;
