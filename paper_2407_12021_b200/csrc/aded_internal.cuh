@@ -212,23 +212,11 @@ struct SeqMeta {
 // The rotary tables of a pass: cos/sin of position * theta^(-2i/hd) for every row, in double, stored as float (the angles reach
 // thousands of radians, where float argument reduction would cost several bf16 ulps).
 struct RopeArgs {
-    const int32_t* pos;      // [R], NULL: nothing to do
     const double* freq;      // [half]
     float* cs;               // [R][half]
     float* sn;
     int half;
 };
-// Row r's tables, by threads `tid` of `threads`.
-__device__ __forceinline__ void rope_row(const RopeArgs& a, int r, int tid, int threads) {
-    if (!a.pos) return;
-    for (int i = tid; i < a.half; i += threads) {
-        double s, c;
-        sincos((double)a.pos[r] * a.freq[i], &s, &c);
-        a.cs[r * a.half + i] = (float)c;
-        a.sn[r * a.half + i] = (float)s;
-    }
-}
-
 }  // namespace aded
 
 namespace aded {
@@ -358,7 +346,7 @@ struct aded_model {
 namespace aded {
 
 inline RopeArgs rope_args(const aded_model* m) {
-    return RopeArgs{m->rows.pos, m->rope_freq, m->rope_cos, m->rope_sin, m->cfg.head_dim / 2};
+    return RopeArgs{m->rope_freq, m->rope_cos, m->rope_sin, m->cfg.head_dim / 2};
 }
 
 // ---- launchers (each enqueues on `st`; shapes are validated by the callers) ---------------
@@ -366,8 +354,8 @@ inline RopeArgs rope_args(const aded_model* m) {
 // Calls of up to PROLOGUE_MAX_BATCH sequences pass their record and row offsets to the prologue, which publishes them; larger
 // ones have copied them before.
 enum { PROLOGUE_MAX_BATCH = 64 };
-void launch_tree_prologue(aded_model* m, aded_kv* kv, const CallPtrs& call, const int32_t* offsets_host, int batch, int chain_mode,
-                          cudaStream_t st);
+// checks, row bookkeeping, embedding lookup, the first RMSNorm and the rotary tables
+void launch_pass_begin(aded_model* m, aded_kv* kv, const CallPtrs& call, const int32_t* offsets_host, int batch, int rows, int chain_mode, cudaStream_t st);
 void launch_accept(aded_model* m, aded_kv* kv, int batch, cudaStream_t st);
 void launch_compact(aded_model* m, aded_kv* kv, int batch, cudaStream_t st);
 void launch_kv_copy(char* cache_k, char* cache_v, size_t head_bytes, void* user_k, void* user_v, size_t bytes, int heads, bool load, cudaStream_t st);
@@ -375,8 +363,6 @@ void launch_commit_chain(aded_model* m, aded_kv* kv, int batch, cudaStream_t st)
 
 // dense.cu
 void launch_rope_freq(double* freq, int half, double theta);
-// embedding lookup, the first RMSNorm and the rotary tables
-void launch_embed_norm(aded_model* m, const void* gain, int rows, cudaStream_t st);
 // projection result added to the residual stream, then the norm
 void launch_add_rmsnorm(aded_model* m, const GemmOut& y, const void* gain, cudaStream_t st);
 bool gemm_plain_prepare(bool bf16_model);
@@ -411,7 +397,6 @@ void launch_f32_head(aded_model* m, float* logits, int rows, cudaStream_t st);
 void launch_add_rmsnorm_ws(aded_model* m, const GemmOut& y, const void* gain, cudaStream_t st);
 void launch_swiglu_ws(aded_model* m, const GemmOut& gu, cudaStream_t st);
 void launch_rope_kv_ws(aded_model* m, aded_kv* kv, const GemmOut& qkv, int layer, cudaStream_t st);
-void launch_embed_norm_ws(aded_model* m, const void* gain, int rows, cudaStream_t st);
 // greedy token per row from n candidates (value, column) each, then the approval walk (one launch)
 void launch_pick_accept(aded_model* m, aded_kv* kv, int batch, const float* cand_val, const int32_t* cand_idx, int n, cudaStream_t st);
 

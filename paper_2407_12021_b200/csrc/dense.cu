@@ -23,14 +23,13 @@ __global__ void k_rope_freq(double* __restrict__ freq, int half, double theta) {
     if (i < half) freq[i] = pow(theta, -(double)i / (double)half);
 }
 
-// h = embedding of the token (when `table` is given) or round(h + y);  x = round(h * rsqrt(mean(h^2) + eps) * gain).  One block
+// h = round(h + y) (y may be absent);  x = round(h * rsqrt(mean(h^2) + eps) * gain).  One block
 // per row, columns strided over the threads and kept in registers between the sum of squares and the scaling; the sum's
 // order is fixed.  fp32 models; of bf16 models those whose widths the tensor-core GEMM does not take.
 constexpr int NORM_COLS = 8;           // columns per thread: d_model <= 8 x 1024
 template <typename T>
-__global__ void __launch_bounds__(1024) k_add_rmsnorm(T* __restrict__ h, const float* __restrict__ y, const T* __restrict__ table,
-                                                      const CallPtrs* __restrict__ call, int vocab, const T* __restrict__ gain,
-                                                      T* __restrict__ x, int d, float eps, RopeArgs rope, const int32_t* status) {
+__global__ void __launch_bounds__(1024) k_add_rmsnorm(T* __restrict__ h, const float* __restrict__ y, const T* __restrict__ gain, T* __restrict__ x, int d,
+                                                      float eps, const int32_t* status) {
     pdl_launch_dependents();
     __shared__ float red[32];
     const int r = blockIdx.x;
@@ -41,27 +40,20 @@ __global__ void __launch_bounds__(1024) k_add_rmsnorm(T* __restrict__ h, const f
         g[i] = c < d ? to_f32(gain[c]) : 0.f;
     }
     pdl_wait();
-    if (first_thread_of_grid()) trace_mark(status, table ? TK_OTHER : TK_NORM);
+    if (first_thread_of_grid()) trace_mark(status, TK_NORM);
     if (*status != 0) return;
-    const T* src = h + (size_t)r * d;
-    if (table) {
-        int tok = call->tokens[r];
-        if (tok < 0 || tok >= vocab) tok = 0;          // a token outside the vocabulary has been reported by the tree check
-        src = table + (size_t)tok * d;
-    }
     float sq = 0.f;
 #pragma unroll
     for (int i = 0; i < NORM_COLS; ++i) {
         const int c = threadIdx.x + i * blockDim.x;
         v[i] = 0.f;
         if (c < d) {
-            v[i] = to_f32(src[c]);
+            v[i] = to_f32(h[(size_t)r * d + c]);
             if (y) v[i] = to_f32(from_f32<T>(v[i] + y[(size_t)r * d + c]));
             h[(size_t)r * d + c] = from_f32<T>(v[i]);
         }
         sq += v[i] * v[i];
     }
-    rope_row(rope, r, threadIdx.x, blockDim.x);
     sq = warp_sum(sq);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sq;
     __syncthreads();
@@ -287,19 +279,11 @@ void launch_rope_freq(double* freq, int half, double theta) { k_rope_freq<<<1, h
 
 static int norm_threads(int d) { return d >= 1024 ? 1024 : (d + 31) / 32 * 32; }
 
-void launch_embed_norm(aded_model* m, const void* gain, int rows, cudaStream_t st) {
-    const int d = m->cfg.d_model;
-    if (m->cfg.dtype == ADED_BF16) { launch_embed_norm_ws(m, gain, rows, st); return; }
-    launch_k(k_add_rmsnorm<float>, rows, norm_threads(d), 0, st, (float*)m->h, nullptr, (const float*)m->top.embed, m->call_dev, m->cfg.vocab,
-             (const float*)gain, (float*)m->x, d, m->cfg.rms_eps, rope_args(m), m->status);
-}
-
 void launch_add_rmsnorm(aded_model* m, const GemmOut& y, const void* gain, cudaStream_t st) {
     const int d = m->cfg.d_model;
     if (y.mode == 1) { launch_add_rmsnorm_ws(m, y, gain, st); return; }
-    const RopeArgs none = {};
-    BY_DTYPE(m, (launch_k(k_add_rmsnorm<bf16>, y.rows, norm_threads(d), 0, st, (bf16*)m->h, y.y, nullptr, nullptr, 0, (const bf16*)gain, (bf16*)m->x, d, m->cfg.rms_eps, none, m->status)),
-             (launch_k(k_add_rmsnorm<float>, y.rows, norm_threads(d), 0, st, (float*)m->h, y.y, nullptr, nullptr, 0, (const float*)gain, (float*)m->x, d, m->cfg.rms_eps, none, m->status)));
+    BY_DTYPE(m, (launch_k(k_add_rmsnorm<bf16>, y.rows, norm_threads(d), 0, st, (bf16*)m->h, y.y, (const bf16*)gain, (bf16*)m->x, d, m->cfg.rms_eps, m->status)),
+             (launch_k(k_add_rmsnorm<float>, y.rows, norm_threads(d), 0, st, (float*)m->h, y.y, (const float*)gain, (float*)m->x, d, m->cfg.rms_eps, m->status)));
 }
 
 constexpr int GP_SMEM = 160 * 1024, GP_CHUNK = 256;

@@ -4,8 +4,7 @@
 // SwiGLU), specialised for the case that matters for speed: the projection result lives in slots
 // (gemm_out.cuh) and the model is bf16.  Each thread gathers four adjacent columns of every
 // contributing slot with 16-byte loads that are all in flight at once, so a kernel is one or two
-// memory round trips deep instead of one per contributor.  Also here: embedding lookup + first
-// RMSNorm, and the greedy choice + approval walk that follows the LM head's per-tile candidates.
+// memory round trips deep instead of one per contributor.  Also here: the greedy choice + approval walk that follows the LM head's per-tile candidates.
 #include "aded_internal.cuh"
 
 namespace aded {
@@ -16,64 +15,13 @@ __device__ __forceinline__ float warp_sum_f(float v) {
     return v;
 }
 
-// Embedding lookup, the first layer's RMSNorm and the row's rotary tables in one kernel (bf16): h = embed[token], x = norm(h).
-// One block of 1024 threads per row, four columns per thread and pass, as k_add_rmsnorm_ws; the last warps make the tables
-// while the row is on its way (a kernel of their own took 4 us of a pass).
-__global__ void __launch_bounds__(1024) k_embed_norm_ws(const bf16* __restrict__ table, const CallPtrs* __restrict__ call,
-                                                        bf16* __restrict__ h, const bf16* __restrict__ gain, bf16* __restrict__ x,
-                                                        int d, int vocab, float eps, RopeArgs rope, const int32_t* status) {
-    pdl_launch_dependents();
-    __shared__ float red[32];
-    const int r = blockIdx.x;
-    float4 gv[2];
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const int c = (i * 1024 + threadIdx.x) * 4;
-        if (c < d) gv[i] = unpack4_bf16(*reinterpret_cast<const uint2*>(gain + c));
-    }
-    pdl_wait();
-    if (first_thread_of_grid()) trace_mark(status, TK_OTHER);
-    const int pass_status = *status;
-    int tok = call->tokens[r];
-    if (tok < 0 || tok >= vocab) tok = 0;          // a token outside the vocabulary has been reported by the tree check
-    const bf16* src = table + (size_t)tok * d;
-    float4 v[2];
-    float sq = 0.f;
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const int c = (i * 1024 + threadIdx.x) * 4;
-        if (c < d) {
-            const uint2 raw = *reinterpret_cast<const uint2*>(src + c);
-            if (pass_status == 0) *reinterpret_cast<uint2*>(h + (size_t)r * d + c) = raw;
-            v[i] = unpack4_bf16(raw);
-            sq += v[i].x * v[i].x + v[i].y * v[i].y + v[i].z * v[i].z + v[i].w * v[i].w;
-        }
-    }
-    if (pass_status == 0) rope_row(rope, r, 1023 - (int)threadIdx.x, 1024);
-    sq = warp_sum_f(sq);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sq;
-    __syncthreads();
-    float total = 0.f;
-#pragma unroll
-    for (int i = 0; i < 32; ++i) total += red[i];
-    const float inv = rsqrtf(total / (float)d + eps);
-    if (pass_status != 0) return;
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const int c = (i * 1024 + threadIdx.x) * 4;
-        if (c < d)
-            *reinterpret_cast<uint2*>(x + (size_t)r * d + c) =
-                pack4_bf16(v[i].x * inv * gv[i].x, v[i].y * inv * gv[i].y, v[i].z * inv * gv[i].z, v[i].w * inv * gv[i].w);
-    }
-}
-
 // Greedy token of every row from its candidates (the LM head's, one per tile, or k_argmax_chunks', one per chunk; largest value,
 // lowest column among equals -- a candidate already is the lowest best column of its part), then the approval walk.
 // One block of 1024 threads per sequence; a warp per row, every lane's candidates fetched at once.
 constexpr int PICK_THREADS = 1024, PICK_PER_LANE = 8;
 __global__ void __launch_bounds__(PICK_THREADS) k_pick_accept(const CallPtrs* __restrict__ call, const float* __restrict__ cand_val,
                                                               const int32_t* __restrict__ cand_idx, int n_tiles,
-                                                              const int32_t* __restrict__ row_off, int32_t* __restrict__ best,
+                                                              const int32_t* __restrict__ row_off, int32_t* __restrict__ best, int32_t* __restrict__ best_copy,
                                                               const uint64_t* __restrict__ anc, int32_t* __restrict__ len,
                                                               int32_t* __restrict__ path, int32_t* __restrict__ moves,
                                                               const int32_t* status) {
@@ -112,7 +60,10 @@ __global__ void __launch_bounds__(PICK_THREADS) k_pick_accept(const CallPtrs* __
         if (lane == 0) {
             const int pick = bi == 0x7fffffff ? 0 : bi;
             s_best[i] = pick;
-            if (pass_status == 0) best[off + i] = pick;
+            if (pass_status == 0) {
+                best[off + i] = pick;
+                if (best_copy) best_copy[off + i] = pick;      // (the caller's: a copy behind the kernel would cost the pass 2 us)
+            }
         }
     }
     for (int i = threadIdx.x; i < T; i += blockDim.x) {
@@ -295,14 +246,9 @@ k_rope_part_ws(GemmOut qkv, const float* __restrict__ cs, const float* __restric
 }
 
 // ---- launchers (callers have checked: bf16 model, tensor-core path) ----------------------------
-void launch_embed_norm_ws(aded_model* m, const void* gain, int rows, cudaStream_t st) {
-    launch_k(k_embed_norm_ws, dim3(rows), dim3(1024), 0, st, (const bf16*)m->top.embed, (const CallPtrs*)m->call_dev, (bf16*)m->h,
-             (const bf16*)gain, (bf16*)m->x, m->cfg.d_model, m->cfg.vocab, m->cfg.rms_eps, rope_args(m), (const int32_t*)m->status);
-}
-
 void launch_pick_accept(aded_model* m, aded_kv* kv, int batch, const float* cand_val, const int32_t* cand_idx, int n, cudaStream_t st) {
     launch_k(k_pick_accept, dim3(batch), dim3(PICK_THREADS), 0, st, (const CallPtrs*)m->call_dev, cand_val, cand_idx, n,
-             (const int32_t*)m->seqs.row_off, m->best, (const uint64_t*)m->rows.anc, kv->len_dev, m->seqs.path, m->seqs.moves,
+             (const int32_t*)m->seqs.row_off, m->best, m->dbg_best, (const uint64_t*)m->rows.anc, kv->len_dev, m->seqs.path, m->seqs.moves,
              (const int32_t*)m->status);
 }
 

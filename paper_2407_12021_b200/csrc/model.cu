@@ -252,9 +252,8 @@ static aded_status enqueue_pass(aded_model* m, aded_kv* kv, const CallPtrs& call
         ADED_CUDA_TRY(cudaMemcpyAsync(m->seqs.row_off, offsets_src, (batch + 1) * sizeof(int32_t), cudaMemcpyHostToDevice, st));
     }
     {
-        Span sp(m, PROF_OTHER, 2, st);
-        launch_tree_prologue(m, kv, call, offsets_src, batch, chain_mode, st);
-        launch_embed_norm(m, m->layers[0].norm1, rows, st);
+        Span sp(m, PROF_OTHER, 1, st);
+        launch_pass_begin(m, kv, call, offsets_src, batch, rows, chain_mode, st);
     }
     const size_t hid_bytes = (size_t)rows * d * m->elem;
     if (m->dbg_hidden) ADED_CUDA_TRY(cudaMemcpyAsync(m->dbg_hidden, m->h, hid_bytes, cudaMemcpyDeviceToDevice, st));
@@ -350,7 +349,7 @@ static aded_status enqueue_pass(aded_model* m, aded_kv* kv, const CallPtrs& call
             Span sp(m, PROF_OTHER, 1, st);
             launch_pick_accept(m, kv, batch, m->cand_val, m->cand_idx, candidates, st);
         }
-        if (m->dbg_best)
+        if (m->dbg_best && m->samp_on)         // (the greedy choice has written them)
             ADED_CUDA_TRY(cudaMemcpyAsync(m->dbg_best, m->best, (size_t)rows * sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
     }
     {

@@ -1,13 +1,15 @@
 // Draft-tree bookkeeping around the forward pass ("Draft Construction and Verification"):
 // validation + depths + ancestor masks before it, draft approval and cache compaction after it.
+#include <type_traits>
+
 #include "aded_internal.cuh"
 
 namespace aded {
 
-// One block per sequence, one thread per node.  Checks that node 0 is the only root and every
-// other node points at an earlier node, that tokens are in the vocabulary and that the cache has
-// room; then each thread climbs from its node to the root, collecting the ancestor bit set and
-// the depth.  The climb is bounded by the node count (parents decrease strictly).
+// The start of a pass: a block per row.  Every block checks its sequence's tree, a thread per node: node 0 is the only root and every
+// other node points at an earlier node, tokens are in the vocabulary, the cache has room.  Then its row's ancestor bit set and depth
+// (a climb to the root, bounded as parents decrease strictly), embedding, first RMSNorm and rotary tables (made by the last warps
+// while the row is on its way).  One kernel: as two, a check per sequence and then the rows, a pass took 3.5 us more.
 //
 // The call's record and row offsets come as kernel arguments (two small copies ahead of the pass cost it about 10 us) and are
 // published here for the kernels that follow.
@@ -17,63 +19,130 @@ struct PrologueArgs {
     int batch;
     int given;             // 0: call and row_off have been copied to their places instead
 };
-__global__ void k_tree_prologue(const __grid_constant__ PrologueArgs pa, CallPtrs* call_dev, int32_t* row_off_dev, int32_t* order,
-                                const int32_t* __restrict__ len, const int32_t* __restrict__ cap, int vocab, int chain_mode,
-                                RowMeta rows, int32_t* status) {
-    pdl_enter();
-    if (first_thread_of_grid()) trace_mark(status, TK_OTHER);
-    const int b = blockIdx.x;
-    if (pa.given && b == 0) {
-        if (threadIdx.x == 0) *call_dev = pa.call;
-        if ((int)threadIdx.x <= pa.batch) row_off_dev[threadIdx.x] = pa.row_off[threadIdx.x];
+__device__ __forceinline__ float4 begin_load4(const float* p, int vec) { return vec ? *reinterpret_cast<const float4*>(p) : make_float4(p[0], p[1], p[2], p[3]); }
+__device__ __forceinline__ float4 begin_load4(const bf16* p, int) { return unpack4_bf16(*reinterpret_cast<const uint2*>(p)); }
+__device__ __forceinline__ void begin_store4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
+__device__ __forceinline__ void begin_store4(bf16* p, float4 v) { *reinterpret_cast<uint2*>(p) = pack4_bf16(v.x, v.y, v.z, v.w); }
+
+// Four columns per thread and pass, two passes: d <= 8 x the block's threads.  vec: table and gain of an fp32 model lie on 16-byte boundaries.
+template <typename T>
+__global__ void __launch_bounds__(1024) k_pass_begin(const __grid_constant__ PrologueArgs pa, CallPtrs* call_dev, int32_t* row_off_dev, int32_t* order,
+                                                     const int32_t* __restrict__ len, const int32_t* __restrict__ cap, int vocab, int chain_mode, RowMeta rows,
+                                                     const T* __restrict__ table, const T* __restrict__ gain, T* __restrict__ h, T* __restrict__ x, int d,
+                                                     float eps, RopeArgs rope, int vec, int32_t* status) {
+    pdl_launch_dependents();
+    __shared__ float red[32];
+    __shared__ int s_bad, s_pending, s_par[ADED_MAX_NODES];
+    const int r = blockIdx.x, tid = threadIdx.x, threads = blockDim.x;
+    float4 gv[2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        const int c = (e * threads + tid) * 4;
+        if (c < d) gv[e] = begin_load4(gain + c, vec);
     }
+    pdl_wait();
+    if (tid == 0) {                                // (read once: another block may be reporting)
+        s_bad = 0;
+        s_pending = *status;
+    }
+    if (first_thread_of_grid()) trace_mark(status, TK_OTHER);
+    const int32_t* __restrict__ offsets = pa.given ? pa.row_off : row_off_dev;
     const int32_t* __restrict__ tokens = pa.given ? pa.call.tokens : call_dev->tokens;
     const int32_t* __restrict__ parents = pa.given ? pa.call.parents : call_dev->parents;
-    const int off = pa.given ? pa.row_off[b] : row_off_dev[b];
-    const int T = (pa.given ? pa.row_off[b + 1] : row_off_dev[b + 1]) - off;
-    const int i = threadIdx.x;
-    __shared__ int s_bad;
-    if (i == 0) s_bad = 0;
+    int b = 0;                                     // the row's sequence: the last that begins at or before it
+    for (int hi = pa.batch; hi - b > 1; ) {
+        const int mid = (b + hi) >> 1;
+        if (offsets[mid] <= r) b = mid;
+        else hi = mid;
+    }
+    const int off = offsets[b], T_nodes = offsets[b + 1] - off, i = r - off, L = len[b];
+    int tok = tokens[r];
+    if (pa.given && r == 0) {
+        if (tid == 0) *call_dev = pa.call;
+        if (tid <= pa.batch) row_off_dev[tid] = pa.row_off[tid];
+    }
+    if (tok < 0 || tok >= vocab) tok = 0;          // (reported below)
+    const T* src = table + (size_t)tok * d;
+    float4 v[2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        const int c = (e * threads + tid) * 4;
+        if (c < d) v[e] = begin_load4(src + c, vec);
+    }
     __syncthreads();
-    if (pa.batch > 1) {        // this sequence's place by falling length
-        const int mine = len[b];
+    if (pa.batch > 1 && i == 0) {                  // this sequence's place by falling length
         int place = 0;
-        for (int o0 = 0; o0 < pa.batch; o0 += ADED_MAX_NODES) {
-            const int o = o0 + i, other = o < pa.batch ? len[o] : -1;
-            place += __syncthreads_count(o < pa.batch && (other > mine || (other == mine && o < b)));
+        for (int o0 = 0; o0 < pa.batch; o0 += threads) {
+            const int o = o0 + tid, other = o < pa.batch ? len[o] : -1;
+            place += __syncthreads_count(o < pa.batch && (other > L || (other == L && o < b)));
         }
-        if (i == 0) order[place] = b;
+        if (tid == 0) order[place] = b;
     }
-    if (*status != 0) return;   // an earlier error is still pending: do nothing
-    int p = -1;
-    if (i < T) {
-        p = chain_mode ? i - 1 : parents[off + i];
-        const int t = tokens[off + i];
+    if (s_pending != 0) return;                    // an earlier error is still pending: do nothing
+    if (tid < T_nodes) {
+        const int p = chain_mode ? tid - 1 : parents[off + tid], t = tokens[off + tid];
+        s_par[tid] = p;
         if (t < 0 || t >= vocab) atomicMax(&s_bad, (int)ADED_ERR_INVALID_ARG);
-        if (i == 0 ? (p != -1) : (p < 0 || p >= i)) atomicMax(&s_bad, (int)ADED_ERR_BAD_TREE);
+        if (tid == 0 ? (p != -1) : (p < 0 || p >= tid)) atomicMax(&s_bad, (int)ADED_ERR_BAD_TREE);
+        if (tid == 0 && L + T_nodes > cap[b]) atomicMax(&s_bad, (int)ADED_ERR_KV_CAPACITY);
     }
-    if (i == 0 && len[b] + T > cap[b]) atomicMax(&s_bad, (int)ADED_ERR_KV_CAPACITY);
     __syncthreads();
     if (s_bad != 0) {
-        if (i == 0) atomicCAS(status, 0, s_bad);
+        if (tid == 0) atomicCAS(status, 0, s_bad);
         return;
     }
-    if (i < T) {
-        uint64_t lo = 0, hi = 0;
-        int depth = 0, cur = i;
-        for (int step = 0; step < T; ++step) {
-            if (cur < 64) lo |= 1ull << cur; else hi |= 1ull << (cur - 64);
-            const int up = chain_mode ? cur - 1 : parents[off + cur];
-            if (up < 0) break;
-            cur = up;
-            ++depth;
+    float sq = 0.f;
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        const int c = (e * threads + tid) * 4;
+        if (c < d) {
+            begin_store4(h + (size_t)r * d + c, v[e]);
+            sq += v[e].x * v[e].x + v[e].y * v[e].y + v[e].z * v[e].z + v[e].w * v[e].w;
         }
-        const int r = off + i;
-        rows.seq[r] = b;
-        rows.local[r] = i;
-        rows.pos[r] = len[b] + depth;
-        rows.anc[2 * r] = lo;
-        rows.anc[2 * r + 1] = hi;
+    }
+    const int last = threads - 1 - tid;
+    if (last < max(rope.half, 1)) {                // each of these threads climbs
+        uint64_t lo, hi;
+        int depth;
+        if (chain_mode) {
+            depth = i;
+            lo = i < 63 ? (2ull << i) - 1ull : ~0ull;
+            hi = i < 64 ? 0ull : i < 127 ? (2ull << (i - 64)) - 1ull : ~0ull;
+        } else {
+            lo = hi = 0;
+            depth = -1;
+            for (int cur = i; cur >= 0; cur = s_par[cur]) {
+                if (cur < 64) lo |= 1ull << cur;
+                else hi |= 1ull << (cur - 64);
+                ++depth;
+            }
+        }
+        if (last == 0) {
+            rows.seq[r] = b;
+            rows.local[r] = i;
+            rows.pos[r] = L + depth;
+            rows.anc[2 * r] = lo;
+            rows.anc[2 * r + 1] = hi;
+        }
+        for (int e = last; e < rope.half; e += threads) {
+            double s, c;
+            sincos((double)(L + depth) * rope.freq[e], &s, &c);
+            rope.cs[r * rope.half + e] = (float)c;
+            rope.sn[r * rope.half + e] = (float)s;
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+    if ((tid & 31) == 0) red[tid >> 5] = sq;
+    __syncthreads();
+    float total = 0.f;
+    for (int e = 0; e < threads / 32; ++e) total += red[e];
+    const float inv = rsqrtf(total / (float)d + eps);
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        const int c = (e * threads + tid) * 4;
+        if (c < d)
+            begin_store4(x + (size_t)r * d + c, make_float4(v[e].x * inv * gv[e].x, v[e].y * inv * gv[e].y, v[e].z * inv * gv[e].z, v[e].w * inv * gv[e].w));
     }
 }
 
@@ -181,9 +250,7 @@ void launch_kv_copy(char* cache_k, char* cache_v, size_t head_bytes, void* user_
     else k_kv_copy<false><<<grid, KV_COPY_THREADS, 0, st>>>(ck, cv, head_bytes / sizeof(uint4), uk, uv, n);
 }
 
-void launch_tree_prologue(aded_model* m, aded_kv* kv, const CallPtrs& call, const int32_t* offsets_host, int batch, int chain_mode,
-                          cudaStream_t st) {
-    static_assert(PROLOGUE_MAX_BATCH < ADED_MAX_NODES, "a thread per row offset");
+void launch_pass_begin(aded_model* m, aded_kv* kv, const CallPtrs& call, const int32_t* offsets_host, int batch, int rows, int chain_mode, cudaStream_t st) {
     PrologueArgs pa = {};
     pa.given = batch <= PROLOGUE_MAX_BATCH;
     pa.batch = batch;
@@ -191,8 +258,16 @@ void launch_tree_prologue(aded_model* m, aded_kv* kv, const CallPtrs& call, cons
         pa.call = call;
         for (int b = 0; b <= batch; ++b) pa.row_off[b] = offsets_host[b];
     }
-    launch_k(k_tree_prologue, batch, ADED_MAX_NODES, 0, st, pa, m->call_dev, m->seqs.row_off, m->seqs.order, kv->len_dev, kv->cap_dev, m->cfg.vocab, chain_mode,
-             m->rows, m->status);
+    const aded_model_config& c = m->cfg;
+    const void* gain = m->layers[0].norm1;
+    static_assert(PROLOGUE_MAX_BATCH < 256 && ADED_MAX_NODES <= 256, "a thread per row offset and per node");
+    auto go = [&](auto* kernel, auto* type, int threads, int vec) {
+        using T = std::remove_pointer_t<decltype(type)>;
+        launch_k(kernel, dim3(rows), dim3(threads), 0, st, pa, m->call_dev, m->seqs.row_off, m->seqs.order, kv->len_dev, kv->cap_dev, c.vocab, chain_mode, m->rows,
+                 (const T*)m->top.embed, (const T*)gain, (T*)m->h, (T*)m->x, c.d_model, c.rms_eps, rope_args(m), vec, m->status);
+    };
+    if (c.dtype == ADED_BF16) go(k_pass_begin<bf16>, (bf16*)nullptr, 1024, 1);
+    else go(k_pass_begin<float>, (float*)nullptr, c.d_model <= 1024 ? 256 : 1024, (reinterpret_cast<uintptr_t>(m->top.embed) | reinterpret_cast<uintptr_t>(gain)) % 16 == 0);
 }
 
 void launch_accept(aded_model* m, aded_kv* kv, int batch, cudaStream_t st) {
