@@ -17,7 +17,7 @@ __device__ __forceinline__ float warp_sum(float v) {
     return v;
 }
 
-// Frequencies of the rotary embedding, theta^(-2i/hd), in double (once per model; the angles are made per pass, rope_row).
+// Frequencies of the rotary embedding, theta^(-2i/hd), in double (once per model; the angles are made per pass, k_pass_begin).
 __global__ void k_rope_freq(double* __restrict__ freq, int half, double theta) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < half) freq[i] = pow(theta, -(double)i / (double)half);

@@ -9,7 +9,8 @@
 //   * the attention kernel rotates its row's query and its ancestors' keys as it reads them from the QKV result, and writes its row's key
 //     and value to the cache (for the calls to come; this one's tree is never read from it).
 // Sums are fp32 as in dense.cu; those of a norm are taken in another order and its factors applied in another place.
-// Measured, 2 layers of width 256, 16 nodes, 64 positions: 24 launches, 102 us, before; 15 and 78 with this.
+// Measured, 2 layers of width 256, 16 nodes, 64 positions: 24 launches, 102 us, before; 15 and 78 with
+// this, 14 and 72 since a pass begins with one kernel (tree.cu).
 #include "aded_internal.cuh"
 
 namespace aded {
