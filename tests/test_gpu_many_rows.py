@@ -102,3 +102,59 @@ def test_quotient_of_the_swiglu_epilogue(cuda_device):
     differ = torch.zeros(1, dtype=torch.int64, device=cuda_device)
     B.aded_debug_silu_check(0, 1 << 32, differ)
     assert int(differ[0]) == 0
+
+
+@pytest.mark.parametrize("shape", ["7b", "hd64"])
+@pytest.mark.parametrize("fault,code", [("parent", 2), ("token", 1), ("room", 3)])
+def test_a_refused_batch_leaves_the_cache_as_it_is(cuda_device, shape, fault, code):
+    """The last sequence of a call is malformed, or has no room: found out by the blocks of the last rows, when the first projection's
+    are already running.  No row of any head changes, also none beyond the committed length; the call ends as quickly as a good one; and the
+    next good call gives what it gives on a new cache.  Before it, a good call of more sequences leaves its bookkeeping behind."""
+    from paper_2407_12021_b200 import binding as B
+    shape = SHAPES[shape]
+    w = gen.model_weights(shape, 66, device=cuda_device)
+    sizes, short = [60] * 5 + [20], 10
+    model = B.aded_model_create(shape, w, max_rows=480, max_batch=12)
+    lens = [25 + 9 * b for b in range(12)]
+    caches = [[gen.normal((shape.n_heads, lens[b], shape.head_dim), 1.0, 67, 2 * b + e, device=cuda_device, dtype=torch.bfloat16) for e in range(2)] for b in range(12)]
+    trees = [gen.make_tree(n, 5, 8, shape.vocab, 68 + b) for b, n in enumerate(sizes[:5] + [short])]
+    bad = gen.make_tree(sizes[5], 5, 8, shape.vocab, 68)
+
+    def cache(room):
+        kv = B.aded_kv_create(model, [n + r for n, r in zip(lens, room)])
+        for b in range(len(room)):
+            B.aded_kv_load(kv, b, 0, *caches[b])
+        return kv
+
+    def call(kv, trees):
+        offsets = [sum(len(t[0]) for t in trees[:b]) for b in range(len(trees) + 1)]
+        out, n_out = torch.full((len(trees), 128), -7, dtype=torch.int32, device=cuda_device), torch.full((len(trees),), -7, dtype=torch.int32, device=cuda_device)
+        tok, par = H.i32([t for tr in trees for t in tr[0]]), H.i32([p for tr in trees for p in tr[1]])
+        start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        start.record()
+        B.aded_verify_batch(model, kv, offsets, tok, par, out, n_out)
+        end.record()
+        end.synchronize()
+        return out, n_out, start.elapsed_time(end)
+
+    everything = lambda kv, room: [x for b, r in enumerate(room) for x in B.aded_kv_read(kv, b, 0, 0, lens[b] + r)]
+    assert bool((call(cache([40] * 12), [gen.make_tree(40, 5, 8, shape.vocab, 69 + b) for b in range(12)])[1] >= 1).all())
+    room = [60] * 5 + [short if fault == "room" else sizes[5]]
+    want = call(cache(room), trees)
+    assert B.aded_model_poll_status(model) == 0
+    if fault == "parent":
+        bad[1][-1] = sizes[5]
+    elif fault == "token":
+        bad[0][-1] = shape.vocab
+    for _ in range(3):
+        kv = cache(room)
+        before = everything(kv, room)
+        out, n_out, ms = call(kv, trees[:5] + [bad])
+        assert bool((n_out == 0).all()) and bool((out == -7).all())
+        assert B.aded_model_poll_status(model) == code
+        assert ms < 50, "a wait ran out"                   # (a good call takes about one; the kernels' limit is 200)
+        assert [B.aded_kv_len(kv, b) for b in range(6)] == lens[:6]
+        assert all(torch.equal(a, b) for a, b in zip(before, everything(kv, room)))
+        got = call(kv, trees)
+        assert B.aded_model_poll_status(model) == 0
+        assert torch.equal(got[1], want[1]) and torch.equal(got[0], want[0])
