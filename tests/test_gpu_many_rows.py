@@ -96,6 +96,40 @@ def test_a_batch_layer_by_parts(cuda_device, shape, batch, nodes):
     assert B.aded_model_poll_status(model) == 0
 
 
+@pytest.mark.parametrize("shape", ["7b", "hd64"])
+@pytest.mark.parametrize("batch,nodes", [(10, 30), (12, 35), (16, 40), (31, 40)])
+def test_a_layer_is_that_of_each_sequences_own_call(cuda_device, shape, batch, nodes):
+    """Blocks of 160, 224, 224 and 256 rows for gate and up of the 7B widths: the first three are an odd number of 16-row groups per warp.  Trees and caches
+    that fit one block of keys, so that the attention adds alike whatever the batch: everything the layer leaves, the SwiGLU product among
+    it, is what the weight-streaming kernel and the kernels behind it give a sequence alone, bit for bit."""
+    from paper_2407_12021_b200 import binding as B
+    shape, context = SHAPES[shape], 20
+    w = gen.model_weights(shape, 71, device=cuda_device)
+    rows = batch * nodes
+    model = B.aded_model_create(shape, w, max_rows=rows, max_batch=batch)
+    trees = [gen.make_tree(nodes, 5, 8, shape.vocab, 72 + b) for b in range(batch)]
+    caches = [[gen.normal((shape.n_heads, context, shape.head_dim), 1.0, 73, 2 * b + e, device=cuda_device, dtype=torch.bfloat16) for e in range(2)] for b in range(batch)]
+    tok, par = H.i32([t for tr in trees for t in tr[0]]), H.i32([p for tr in trees for p in tr[1]])
+
+    def call(which):
+        kv = B.aded_kv_create(model, [context + nodes] * len(which))
+        for i, b in enumerate(which):
+            B.aded_kv_load(kv, i, 0, *caches[b])
+        a, e = which[0] * nodes, (which[-1] + 1) * nodes
+        best = torch.zeros(e - a, dtype=torch.int32, device=cuda_device)
+        out, n_out = torch.zeros((len(which), 128), dtype=torch.int32, device=cuda_device), torch.zeros(len(which), dtype=torch.int32, device=cuda_device)
+        B.aded_debug_capture(model, None, best)
+        B.aded_verify_batch(model, kv, [nodes * i for i in range(len(which) + 1)], tok[a:e].contiguous(), par[a:e].contiguous(), out, n_out)
+        left = [B.aded_debug_read_buffer(model, i, e - a).clone() for i in (2, 3, 4, 0, 1)] + [best]
+        assert B.aded_model_poll_status(model) == 0
+        return left
+
+    together = call(range(batch))
+    for b in range(batch):
+        for name, got, own in zip(("q", "attention", "SwiGLU", "residual", "norm", "greedy"), together, call([b])):
+            assert torch.equal(got[b * nodes:(b + 1) * nodes], own), (name, b)
+
+
 def test_quotient_of_the_swiglu_epilogue(cuda_device):
     """Every float of the range in which the epilogue divides without the operator: the same quotient, bit for bit."""
     from paper_2407_12021_b200 import binding as B
