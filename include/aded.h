@@ -239,9 +239,11 @@ aded_status aded_debug_capture_hidden(aded_model* m, void* hidden_dev);
  * range it takes, and adds the number of those that differ to *differ_dev.  Asynchronous. */
 aded_status aded_debug_silu_check(uint32_t first, uint64_t count, uint64_t* differ_dev, void* stream);
 
-/* Failure-path check ("every device-side wait is bounded", see Conventions): runs one of the library's two
+/* Failure-path check ("every device-side wait is bounded", see Conventions): runs one of the library's three
  * kinds of device-side wait -- which = 0: the mbarrier wait of the tensor-core kernels, 1: the wait at an
- * arrival counter of the LM head's tail -- on something that never happens, with a limit of limit_cycles
+ * arrival counter of the LM head's tail, 2: the wait for a neighbour's running sums in the GEMM for calls of
+ * many rows, which here come after all once the wait has run out (ADED_ERR_UNSUPPORTED for a model that never makes
+ * such calls) -- on something that never happens, with a limit of limit_cycles
  * SM clock cycles (1 .. 2^32; about 2 x 10^6 per millisecond).  The wait runs out, the kernel returns, and
  * the model's status word becomes ADED_ERR_TIMEOUT exactly as after a real time-out: later calls do nothing
  * until aded_model_poll_status has read and cleared it.  Nothing faults or hangs.  Asynchronous. */

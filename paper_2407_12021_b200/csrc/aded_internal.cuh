@@ -321,8 +321,7 @@ struct aded_model {
     bool ws_use_tiled;                  // GEMMs read the re-tiled copies (else the caller's matrices through ws_maps)
     bool many_ok;                       // the kernel for calls of many rows can be used
     aded::TileRef* many_tiles;          // "tile t is slot t, complete" (aded_debug_gemm)
-    uint32_t* many_flags;               // their hand-over flags (MANY_FLAGS)
-    uint32_t many_epoch;                // launches so far
+    uint32_t* many_flags;               // its hand-over flags, [many_flag_count]
     float* ws_slots;                    // partial result tiles (see gemm_out.cuh)
     aded::TileRef* ws_tiles[5];         // contributor tables of the wqkv, wo, wgu, wd and LM-head results
     int ws_contributors[5];             // most contributors of any of their tiles
@@ -416,9 +415,11 @@ cudaError_t ws_launch(const CUtensorMap& map_w, const void* w_tiled, const CUten
 // gemm_many.cu: calls of many rows
 bool many_prepare();
 int many_block_rows(int device, int rows, int n, int k);      // 0: not a call for it
+size_t many_flag_count(int device);
+cudaError_t many_wait_probe(uint32_t* flag, long long limit, int32_t* status, cudaStream_t st);
 cudaError_t many_silu_check(uint32_t first, uint64_t count, uint64_t* differ, cudaStream_t st);
 cudaError_t many_launch(const CUtensorMap& map_w, bool tiled, const CUtensorMap* x_maps, int rows, int block_rows, int n, int k, int ws_ctas,
-                        float* partial, uint32_t* flags, uint32_t epoch, int32_t* status, const ManyEpilogue& epi, int trace_kind, int device, cudaStream_t st);
+                        float* partial, uint32_t* flags, int32_t* status, const ManyEpilogue& epi, int trace_kind, int device, cudaStream_t st);
 enum { WS_MAP_QKV = 0, WS_MAP_O = 1, WS_MAP_GU = 2, WS_MAP_D = 3 };   // per-layer map order
 enum { WS_X = 0, WS_X_ATTN = 1, WS_X_ACT = 2 };
 cudaError_t ws_wait_probe(int which, long long limit_cycles, const uint32_t* never_raised, int32_t* status, cudaStream_t st);

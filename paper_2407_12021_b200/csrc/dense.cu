@@ -335,7 +335,7 @@ void launch_gemm_many(aded_model* m, int w_map, int x_map, int rows, int n, int 
     const int block = many_block_rows(m->device, rows, n, k);
     const int table = w_map < 4 * m->cfg.n_layers ? w_map % 4 : 4;
     many_launch(m->ws_use_tiled ? m->ws_tiled_maps[w_map] : m->ws_half_maps[w_map], m->ws_use_tiled, m->ws_x_maps[x_map], rows, block, n, k,
-                ws_grid(m->device, n, k, m->ws_one_per_sm[table]), m->ws_slots, m->many_flags, ++m->many_epoch, m->status, epi, trace_kind, m->device, st);
+                ws_grid(m->device, n, k, m->ws_one_per_sm[table]), m->ws_slots, m->many_flags, m->status, epi, trace_kind, m->device, st);
 }
 
 void launch_rmsnorm(aded_model* m, int rows, const void* gain, cudaStream_t st) {

@@ -200,9 +200,8 @@ static aded_status alloc_model(aded_model* m) {
                 for (int t = 0; t < (int)identity.size(); ++t) identity[t] = TileRef{t, 1};
                 TRY(dev_alloc(m, &m->many_tiles, identity.size()));
                 ADED_CUDA_TRY(cudaMemcpy(m->many_tiles, identity.data(), identity.size() * sizeof(TileRef), cudaMemcpyHostToDevice));
-                TRY(dev_alloc(m, &m->many_flags, (size_t)ws_grid_limit(m->device) / 2 * 8));
-                ADED_CUDA_TRY(cudaMemset(m->many_flags, 0, (size_t)ws_grid_limit(m->device) / 2 * 8 * sizeof(uint32_t)));
-                m->many_epoch = 0;
+                TRY(dev_alloc(m, &m->many_flags, many_flag_count(m->device)));
+                ADED_CUDA_TRY(cudaMemset(m->many_flags, 0, many_flag_count(m->device) * sizeof(uint32_t)));
             }
             // the LM head's tail: one arrival counter per tile, per-tile greedy candidates of every row
             TRY(dev_alloc(m, &m->ws_counters, V / 128));
@@ -796,7 +795,13 @@ aded_status aded_trace_end(aded_model* m, uint64_t* out_ns_host, int32_t* out_ki
 }
 
 aded_status aded_debug_wait_timeout(aded_model* m, int32_t which, uint64_t limit_cycles, void* stream) {
-    if (!m || which < 0 || which > 1 || limit_cycles < 1 || limit_cycles > (1ull << 32)) return ADED_ERR_INVALID_ARG;
+    if (!m || which < 0 || which > 2 || limit_cycles < 1 || limit_cycles > (1ull << 32)) return ADED_ERR_INVALID_ARG;
+    if (which == 2) {
+        if (!m->many_ok) return ADED_ERR_UNSUPPORTED;
+        note_launch();
+        ADED_CUDA_TRY(many_wait_probe(m->many_flags, (long long)limit_cycles, m->status, static_cast<cudaStream_t>(stream)));
+        return ADED_OK;
+    }
     // the counter the probe polls: a word of the trace area that only ever holds a small count
     const uint32_t* quiet = reinterpret_cast<const uint32_t*>(m->status + 3);
     note_launch();
@@ -839,6 +844,8 @@ aded_status aded_model_poll_status(aded_model* m, aded_status* out_host, void* s
             ADED_CUDA_TRY(cudaMemsetAsync(m->ws_counters, 0, (size_t)(m->cfg.vocab / 128) * sizeof(uint32_t), st));
             m->ws_epoch = 0;
         }
+        // ... or running sums handed over that nobody took
+        if (m->many_ok) ADED_CUDA_TRY(cudaMemsetAsync(m->many_flags, 0, many_flag_count(m->device) * sizeof(uint32_t), st));
         ADED_CUDA_TRY(cudaStreamSynchronize(st));
     }
     *out_host = static_cast<aded_status>(v);

@@ -130,6 +130,26 @@ def test_a_layer_is_that_of_each_sequences_own_call(cuda_device, shape, batch, n
             assert torch.equal(got[b * nodes:(b + 1) * nodes], own), (name, b)
 
 
+def test_the_wait_for_a_neighbours_sums_runs_out_and_the_handle_recovers(cuda_device):
+    """The sums that come after the wait has run out must not be there for the next launch: reading the status lowers their flag, so a
+    second wait runs out too, and calls of many rows give afterwards what they gave before.  A model without such calls has no such wait."""
+    from paper_2407_12021_b200 import binding as B
+    w = gen.model_weights(HD64, 76, device=cuda_device)
+    model = B.aded_model_create(HD64, w, max_rows=1228, max_batch=1)
+    x = gen.normal((1228, HD64.d_model), 1.0, 77, 1, device=cuda_device, dtype=torch.bfloat16)
+    want = B.aded_debug_gemm(model, 0, 0, x)
+    assert B.aded_model_poll_status(model) == 0
+    for _ in range(2):
+        B.aded_debug_wait_timeout(model, 2, 2_000_000)
+        assert B.aded_model_poll_status(model) == 8
+        assert B.aded_model_poll_status(model) == 0
+    for _ in range(3):
+        assert torch.equal(B.aded_debug_gemm(model, 0, 0, x), want)
+    assert B.aded_model_poll_status(model) == 0
+    with pytest.raises(B.AdedError):
+        B.aded_debug_wait_timeout(B.aded_model_create(HD64, w, max_rows=128, max_batch=1), 2, 2_000_000)
+
+
 def test_quotient_of_the_swiglu_epilogue(cuda_device):
     """Every float of the range in which the epilogue divides without the operator: the same quotient, bit for bit."""
     from paper_2407_12021_b200 import binding as B
