@@ -973,7 +973,7 @@ __device__ __forceinline__ McLookup mc_lookup(const TgView& t, int a, int b, int
 // overflow or lose bits on the way takes the operator.
 __device__ __forceinline__ double mc_div(double a, int n, double rcp) {
     const unsigned hi = (unsigned)__double2hiint(a) & 0x7FFFFFFFu;
-    if (hi - 0x06000000u >= 0x78000000u) return a == 0.0 ? a : __ddiv_rn(a, (double)n);      // (zero, |a| < 2^-927, > 2^992, infinite, NaN)
+    if (hi - 0x06000000u >= 0x78000000u) return a == 0.0 ? a : __ddiv_rn(a, (double)n);      // (zero, |a| < 2^-927, |a| >= 2^993, infinite, NaN)
     const double d = -(double)n;
     double q = __dmul_rn(a, rcp);
     q = __fma_rn(__fma_rn(d, q, a), rcp, q);
