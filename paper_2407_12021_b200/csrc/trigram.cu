@@ -620,18 +620,22 @@ constexpr int DRAFT_MAX_FILLER = 4 * ADED_MAX_NODES;
 // Filler pass over a tree held in shared memory (tok, par, dep; kid[p][0 .. nkid[p]) the child tokens of node p), by one warp:
 // nodes are visited round-robin, a visited node with depth < max_depth and fewer than k children gets the next filler token
 // none of its children holds.  Returns the new node count (every lane); *fail when the filler runs out, holds a token outside the
-// vocabulary, or no node has room.  The steps depend on one another, so each is kept short: the nodes with room wait in two lists
-// (`turn`, [2][ADED_MAX_NODES]: of this round, to which new nodes are added, and of the next), and the lanes compare a token with all
-// children at once.  (A thread that visited every node took 28 us for 50 of 97 nodes.)
+// vocabulary, or no node has room.  The nodes with room wait in two lists (`turn`, [2][ADED_MAX_NODES]: of this round, to which new
+// nodes are added, and of the next).  Up to 32 of them are served at once, a token each; the first whose token does not fit ends
+// the step, as those behind it would have got other tokens.  The last one of a round goes on with its child, which is next in turn and has
+// no children, the child with its own, and so on: a chain, a lane per link.
+// Latency of the steps.  draft_tree for a context without continuations (all nodes are filler), us: a thread that visited every node; a warp
+// with a token per step; this.  128 nodes, depth 8, k = 8: 30, 35, 9; 97 nodes, depth 4, k = 4: 31, 28, 11; a chain of 128: 24, 35, 6.
 __device__ __forceinline__ int draft_fill(int32_t* tok, int32_t* par, int32_t* dep, int32_t* nkid, int32_t* kid, int n, int n_nodes,
                                           int max_depth, int k, const int32_t* fill, int n_filler, int vocab, int lane, int16_t* turn, bool* fail) {
+    const unsigned below = (1u << lane) - 1u;
     int16_t *now = turn, *then = turn + ADED_MAX_NODES;
     int n_now = 0, n_then = 0, at = 0;
     for (int i0 = 0; i0 < n; i0 += 32) {
         const int i = i0 + lane;
         const bool room = i < n && dep[i] < max_depth && nkid[i] < k;
         const unsigned m = __ballot_sync(0xffffffffu, room);
-        if (room) now[n_now + __popc(m & ((1u << lane) - 1u))] = (int16_t)i;
+        if (room) now[n_now + __popc(m & below)] = (int16_t)i;
         n_now += __popc(m);
     }
     __syncwarp();
@@ -643,30 +647,44 @@ __device__ __forceinline__ int draft_fill(int32_t* tok, int32_t* par, int32_t* d
             then = x;
             n_now = n_then;
             n_then = at = 0;
-            if (n_now == 0) { *fail = true; break; }
         }
-        const int p = now[at++];
-        const int nk = nkid[p], depth = dep[p] + 1, child = lane < ADED_DRAFT_MAX_K ? kid[p * ADED_DRAFT_MAX_K + lane] : 0;
-        int32_t f = -1;
-        for (; pos < n_filler; ++pos) {
-            f = fill[pos];
-            if (!__any_sync(0xffffffffu, lane < nk && child == f)) break;
+        const bool chain = n_now - at == 1;
+        const int served = min(min(32, chain ? max_depth - dep[now[at]] : n_now - at), min(n_nodes - n, n_filler - pos));
+        if (served <= 0) { *fail = true; break; }                 // no node has room, or no token is left
+        int p = 0, f = 0, nk = 0, depth = 0;
+        bool clash = false;
+        if (lane < served) {
+            const bool link = chain && lane > 0;                  // (the parent is the lane before)
+            p = link ? n + lane - 1 : now[at + lane];
+            f = fill[pos + lane];
+            nk = link ? 0 : nkid[p];
+            depth = link ? dep[now[at]] + 1 + lane : dep[p] + 1;
+            for (int j = 0; j < nk; ++j) clash |= kid[p * ADED_DRAFT_MAX_K + j] == f;
         }
-        if (pos >= n_filler || f < 0 || f >= vocab) { *fail = true; break; }
-        ++pos;
-        if (lane == 0) {
+        const unsigned clashes = __ballot_sync(0xffffffffu, clash), stops = clashes | __ballot_sync(0xffffffffu, lane < served && (f < 0 || f >= vocab));
+        const int fit = stops ? __ffs((int)stops) - 1 : served;
+        const bool mine = lane < fit, last = !chain || lane == fit - 1, deeper = mine && last && depth < max_depth, again = mine && nk + 1 < k;
+        const unsigned deeper_m = __ballot_sync(0xffffffffu, deeper), again_m = __ballot_sync(0xffffffffu, again);
+        if (mine) {
+            const int c = n + lane;
             kid[p * ADED_DRAFT_MAX_K + nk] = f;
             nkid[p] = nk + 1;
-            tok[n] = f;
-            par[n] = p;
-            dep[n] = depth;
-            nkid[n] = 0;
-            if (depth < max_depth) now[n_now] = (int16_t)n;
-            if (nk + 1 < k) then[n_then] = (int16_t)p;
+            tok[c] = f;
+            par[c] = p;
+            dep[c] = depth;
+            if (last) nkid[c] = 0;
+            if (deeper) now[n_now + __popc(deeper_m & below)] = (int16_t)c;
+            if (again) then[n_then + __popc(again_m & below)] = (int16_t)p;
         }
-        n_now += depth < max_depth;
-        n_then += nk + 1 < k;
-        ++n;
+        n_now += __popc(deeper_m);
+        n_then += __popc(again_m);
+        n += fit;
+        at += chain ? min(fit, 1) : fit;
+        pos += fit;
+        if (stops) {
+            if (!(clashes >> fit & 1u)) { *fail = true; break; }   // (a token outside the vocabulary)
+            ++pos;                                                // a child holds it: this node gets the next one
+        }
         __syncwarp();
     }
     return n;

@@ -71,6 +71,36 @@ def test_filler_edge_cases(cuda_device):
             _tree_gpu(B, t, 0, 1, *bad)
 
 
+@pytest.mark.parametrize("vocab", [9, 20, 3000])
+@pytest.mark.parametrize("n_nodes,max_depth,k", [(2, 1, 1), (33, 2, 8), (34, 2, 8), (66, 3, 4), (73, 2, 8), (128, 3, 8), (128, 8, 2), (128, 127, 1), (128, 127, 8), (128, 40, 3), (128, 7, 3)])
+def test_trees_that_are_mostly_filler(cuda_device, vocab, n_nodes, max_depth, k):
+    """Rounds of fewer and of more than 32 nodes with room, chains shorter and longer than 32, small vocabularies in which tokens meet a child
+    that holds them, a filler that is just long enough or one token short, and one with a bad token in its last place or in the middle."""
+    from paper_2407_12021_b200 import binding as B
+    toks = gen.zipf_tokens(40, vocab, 5, 1)
+    st = TrigramStore()
+    st.update(toks.tolist())
+    t = B.aded_trigram_create(vocab, log2_buckets=10, overflow_buckets=64)
+    B.aded_trigram_update(t, toks.cuda())
+    for start in ((vocab - 1, vocab - 2), (int(toks[3]), int(toks[4]))):
+        filler = gen.zipf_tokens(4 * 128, vocab, 6, start[0]).tolist()
+        want = od.draft_tree(st, *start, n_nodes, max_depth, k, filler=filler)
+        assert _tree_gpu(B, t, *start, n_nodes, max_depth, k, filler=filler) == want
+        used = 0                                        # as many tokens as it takes
+        while used < len(filler):
+            try:
+                od.draft_tree(st, *start, n_nodes, max_depth, k, filler=filler[:used])
+                break
+            except ValueError:
+                used += 1
+        assert _tree_gpu(B, t, *start, n_nodes, max_depth, k, filler=filler[:used] + [vocab]) == want
+        assert B.aded_trigram_poll_status(t) == 0
+        if used > 0:
+            for bad in (filler[:used - 1] + [vocab], filler[:used // 2] + [-3] + filler[used // 2:-1], filler[:used - 1] if used > 1 else [-1]):
+                assert _tree_gpu(B, t, *start, n_nodes, max_depth, k, filler=bad)[0][0] == -1
+                assert B.aded_trigram_poll_status(t) == 1
+
+
 def _decode_setup(cuda_device, seed):
     shape = gen.TINY
     w = gen.model_weights(shape, seed)
