@@ -1087,7 +1087,12 @@ k_mcts_draft(TgView t, const __grid_constant__ McParams p, const int32_t* __rest
     // look up ahead: a level's contexts, by several warps each while they are few (the first may have thousands of continuations)
     for (int lo = 0, level = 0; level < p.length; ++level) {
         const int hi = s_count, n_ctx = hi - lo;
-        if (n_ctx <= 0) break;
+        // A level takes as long as its longest context does, once per MC_WARPS of them; the search meets one of its contexts per iteration.
+        // Cold, table of 2,000,000 tokens, three contexts, us: all levels / these / a search by one warp alone.  1 iteration, k = 8: 94, 92, 106 /
+        // 41, 70, 22 / 47, 69, 25.  2 iterations, k = 4: 66, 51, 74 / 74, 49, 72 / 64, 92, 39; k = 8: 104, 93, 111 / 62, 57, 29 / 68, 88, 25.
+        // 4 iterations, k = 8, sentences of 8: 114, 101, 117 against 211, 189, 209 (these are all levels).
+        const int waves = (n_ctx + MC_WARPS - 1) / MC_WARPS;
+        if (n_ctx <= 0 || (level > 0 && (p.iterations == 1 || waves > p.iterations))) break;
         const bool deeper = level + 1 < p.length && hi + n_ctx * p.k <= MC_AHEAD;
         auto append = [&](int b, const McLookup& lk) {
             if (!deeper || lk.n == 0) return;

@@ -65,6 +65,22 @@ def test_hot_context_with_a_long_chain_and_bad_arguments(cuda_device):
             B.aded_mcts_draft(t, H.i32([1, 2]), bad[0], bad[1], bad[2], bad[3], torch.zeros(2000, device="cuda"))
 
 
+@pytest.mark.parametrize("iters", [1, 2, 3, 4, 5])
+def test_short_searches(cuda_device, iters):
+    """Searches too short for some levels of contexts to be looked up ahead of them."""
+    from paper_2407_12021_b200 import binding as B
+    toks = gen.zipf_tokens(4000, 60, 8, 1)
+    st = TrigramStore()
+    st.update(toks.tolist())
+    t = B.aded_trigram_create(60, log2_buckets=12, overflow_buckets=2048)
+    B.aded_trigram_update(t, toks.cuda())
+    for length, n, k in ((1, 5, 8), (4, 24, 8), (4, 5, 4), (8, 8, 8), (8, 4, 2), (3, 3, 1)):
+        for at in (7, 300, 1500):
+            u = gen.uniform01(iters * length, 8, 10 * length + k).numpy().astype(np.float32)
+            _compare(B, t, st, int(toks[at]), int(toks[at + 1]), iters, length, n, k, u)
+    assert B.aded_trigram_poll_status(t) == 0
+
+
 @pytest.mark.parametrize("start", [(-1, -1), (-1, 3), (3, -1), (60, 60), (2 ** 31 - 1, -2 ** 31)])
 def test_contexts_outside_the_vocabulary_have_no_continuations(cuda_device, start):
     """Also right after a search that filled the kernel's shared memory; (-1, -1) is the key of its empty slots."""
