@@ -317,15 +317,21 @@ k_tg_topk(TgView t, const int32_t* __restrict__ ctx, int q, int k, int per_block
 // now.  Measured, 2^20 queries on the table of a 16-million-token text, us: k = 2, 4, 8: 151, 188, 253 before; 92, 100, 124 now
 // (mark 46, lead 48, copy 14 under ncu, 57 + 93 + 32 before).
 // Taken from the number of queries on from where it is the faster one, which depends on how long contexts are and so on how
-// much text the table holds, of which its size is what a call knows (topk_bulk_min).  k = 4, the per-block kernel against this, us:
-//   home buckets                      2^11        2^12        2^13        2^14        2^15        2^16 queries
-//   2^18 (text of 10^5 tokens)      13 /  22    14 /  20    16 /  21    19 /  21    27 /  22    28 /  23
-//   2^19          2 x 10^5          15 /  24    17 /  24    20 /  23    24 /  23    32 /  24
-//   2^20          4 x 10^5          23 /  25    26 /  26    31 /  25    37 /  24    45 /  26
-//   2^21          8 x 10^5          27 /  28    31 /  28    42 /  30    48 /  28    60 /  28
-//   2^25        1.6 x 10^7         117 /  43   120 /  42   149 /  43   170 /  42   193 /  44
+// much text the table holds (topk_text).  k = 4, the per-block kernel against this, us, everything in L2 / a cold one, for a text of
+// independent Zipf tokens and for one in which every other token is followed by its usual successor (longer contexts, asked for more often):
+//   text             queries   Zipf               usual successors
+//   10^5              2^15     25/29 -> 23/30     25/29 -> 22/28
+//   2 x 10^5          2^15     29/35 -> 25/33     31/35 -> 24/32
+//   4 x 10^5          2^13     23/27 -> 27/34     29/34 -> 25/32
+//                     2^14     28/33 -> 27/34     37/40 -> 25/30
+//   10^6              2^12     25/29 -> 31/38     36/39 -> 28/36
+//                     2^13     33/37 -> 32/39     43/47 -> 28/34
+//   4 x 10^6          2^12     33/37 -> 41/48     65/68 -> 36/46
+//                     2^13     54/57 -> 40/46     81/86 -> 36/44
+//   1.6 x 10^7        2^12     91/94 -> 52/60     125/122 -> 42/52
+// (k = 2 gains less, k = 8 and 24 more.)
 constexpr int MARK_OWN = -2, MARK_PROBES = 16;
-static int topk_bulk_min(uint32_t n_home) { return n_home >= 1u << 21 ? 1 << 12 : n_home >= 1u << 20 ? 1 << 13 : n_home >= 1u << 19 ? 1 << 15 : 1 << 16; }
+static int topk_bulk_min(uint64_t text) { return text > 1u << 19 ? 1 << 12 : text > 1u << 18 ? 1 << 13 : text > 1u << 16 ? 1 << 15 : 1 << 16; }
 __device__ __forceinline__ int mark_leader(int q) { return MARK_OWN - 1 - q; }       // (its own inverse)
 
 // One thread's list: the first k of `key` (in order; eight of them, none beyond) as a row.  `vec`: the words of a row that one store takes.
@@ -1377,6 +1383,7 @@ struct aded_trigram {
     unsigned long long* stats_dev;
     int32_t* step_i;     // decoding step: see STEP_SENT
     mutable bool search_prepared;   // the tree search's shared-memory limit has been raised on this device
+    uint64_t counted;    // windows and entries given to update and import since the table was empty (a decoding step's few are left out)
 };
 
 using namespace aded;
@@ -1386,8 +1393,16 @@ static constexpr size_t TG_STAGE = 1 << 16;
 static constexpr int STEP_SENT = 0, STEP_REAL = 1, STEP_FILL = 2;
 static constexpr int STEP_INTS = STEP_FILL + DRAFT_MAX_FILLER;
 
+// Tokens of text that the table holds, as far as a call knows without asking the device: what it was given, but no more than its home buckets
+// are meant for (half as many).  By its size alone, a table of 2^24 buckets that held 10^5 tokens took 21 us instead of 10 for 4096 lookups.
+static uint64_t topk_text(const aded_trigram* t) {
+    const uint64_t room = t->view.n_home / 2;
+    return t->counted < room ? t->counted : room;
+}
+
 // An empty table: home buckets and index.  The pool needs no clearing: see tg_place.
 static aded_status tg_reset(aded_trigram* t, cudaStream_t st) {
+    t->counted = 0;
     const size_t buckets = (size_t)t->view.n_home + (t->view.chain ? t->view.n_over : 0);     // (chain buckets follow the home buckets)
     static_assert(sizeof(TgIndexSlot) == sizeof(uint4), "a slot per store");
     const size_t parts = buckets * (sizeof(Bucket) / sizeof(uint4)), slots = t->view.index ? (size_t)(t->view.index_mask + 1) : 0;
@@ -1484,6 +1499,7 @@ aded_status aded_trigram_update(aded_trigram* t, const int32_t* tokens_dev, int3
     if (!t || n < 0 || (n > 0 && !tokens_dev)) return ADED_ERR_INVALID_ARG;
     if (n < 3) return ADED_OK;
     const int windows = n - 2;
+    t->counted += (uint64_t)windows;
     note_launch();
     if (windows >= BULK_MIN)
         k_tg_update_bulk<<<(unsigned)(((int64_t)windows + BULK_WINDOWS - 1) / BULK_WINDOWS), BULK_THREADS, (BULK_WINDOWS + 2 + 2 * BULK_SLOTS) * sizeof(int32_t),
@@ -1519,7 +1535,7 @@ aded_status aded_trigram_topk(const aded_trigram* t, const int32_t* ctx_dev, int
     // As many queries per block as fill the device's block slots once (three blocks per SM).
     const int wave = ws_grid_limit(t->device) / 2 * 3;
     int per_block = (int)(((int64_t)q + wave - 1) / wave);
-    if (q >= topk_bulk_min(t->view.n_home) && k >= 2) {
+    if (q >= topk_bulk_min(topk_text(t)) && k >= 2) {
         uint32_t slots = 1;
         while ((uint64_t)slots * 2 < (uint64_t)q) slots *= 2;
         const int deferred = (int)((slots + k - 1) / k);             // rows whose counts the hash table lies in
@@ -1705,6 +1721,7 @@ aded_status aded_trigram_export(const aded_trigram* t, uint32_t min_count, int32
 aded_status aded_trigram_import(aded_trigram* t, const int32_t* keys_dev, const uint32_t* counts_dev, uint64_t n, void* stream) {
     if (!t || (n > 0 && (!keys_dev || !counts_dev))) return ADED_ERR_INVALID_ARG;
     if (n == 0) return ADED_OK;
+    t->counted += n;
     note_launch();
     k_tg_import<<<(unsigned int)((n + 255) / 256), 256, 0, static_cast<cudaStream_t>(stream)>>>(t->view, keys_dev, counts_dev, n);
     ADED_CUDA_TRY(cudaGetLastError());

@@ -501,7 +501,7 @@ def test_export_with_more_long_contexts_than_a_block_shares(cuda_device, entries
 
 @pytest.mark.parametrize("k,offset", [(2, 0), (2, 1), (3, 0), (4, 0), (4, 1), (4, 2), (6, 0), (8, 0), (12, 0), (32, 0)])
 def test_grouped_lookups_of_a_large_table(cuda_device, k, offset):
-    """Tables of many home buckets group from 4096 queries on.  Rows that are answered in the first kernel and rows whose counts its hash
+    """Tables of much text group from 4096 queries on.  Rows that are answered in the first kernel and rows whose counts its hash
     table takes, contexts of every size on both sides of what a thread, a warp and a block look up, repeated within and across the first
     kernel's blocks, absent and invalid ones, rows of one, two and four words per store: all as the same lookups in small calls."""
     from paper_2407_12021_b200 import binding as B
@@ -512,6 +512,10 @@ def test_grouped_lookups_of_a_large_table(cuda_device, k, offset):
         span = [tok for c in range(n) for tok in (2900 + i, i, (c * 7 + i) % vocab)] + [tok for c in range(0, n, 3) for tok in (2900 + i, i, (c * 7 + i) % vocab)]
         B.aded_trigram_update(t, torch.tensor(span, dtype=torch.int32, device="cuda"))
     B.aded_trigram_update(t, gen.zipf_tokens(20000, 300, 71, 1).cuda())
+    launched = B.aded_launch_count()
+    B.aded_trigram_topk(t, torch.zeros((4096, 2), dtype=torch.int32, device="cuda"), k, *(torch.zeros((4096, k), dtype=torch.int32, device="cuda") for _ in range(2)))
+    assert B.aded_launch_count() - launched == 1           # little text: one kernel
+    B.aded_trigram_update(t, torch.full((600_000,), 299, dtype=torch.int32, device="cuda"))
     g = torch.Generator().manual_seed(72)
     for q in (4096, 5001):
         ctx = torch.stack([gen.zipf_tokens(q, 300, 73, 1), gen.zipf_tokens(q, 300, 74, 1)], dim=1)
@@ -527,7 +531,9 @@ def test_grouped_lookups_of_a_large_table(cuda_device, k, offset):
             return [f[offset:].view(n, k) for f in flat] + [torch.full((n,), -5, dtype=torch.int32, device="cuda")]
 
         tok, cnt, total = rows(q)
+        launched = B.aded_launch_count()
         B.aded_trigram_topk(t, ctx, k, tok, cnt, total)
+        assert B.aded_launch_count() - launched == 3
         for a in range(0, q, 1000):
             part = ctx[a:a + 1000].contiguous()
             want = rows(part.shape[0])
