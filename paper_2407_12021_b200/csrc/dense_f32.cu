@@ -171,8 +171,12 @@ __global__ void __launch_bounds__(F32_THREADS) k_gemm_f32(const __grid_constant_
 }
 
 // Rotary embedding, K/V write and tree attention of one (row, head) per block of four warps, from the QKV result.  As k_tree_attn_plain:
-// per chunk of keys a thread per key for the scores, then the threads as (key group, four columns) for the product with V.
-constexpr int F32_ATTN_THREADS = 128, F32_CHUNK = 512;
+// per chunk of keys a thread per key for the scores, then the threads as (key group, four columns) for the product with V.  Cached keys and
+// the tree's are separate loops: with a choice between them in each step the loads of a step waited for the one before.  The tree's few
+// are unrolled by four only (all of it: 255 registers with heads of 128, two blocks per SM instead of three).  us per pass, back to
+// back, 2 layers of 3 heads of 128, 3000 positions, 1 / 16 / 33 / 64 / 128 rows: rotary kernel and k_tree_attn_plain 268, 306, 354, 525, 560;
+// with the choice and without f32_attn_smem 281, 331, 494, 520, 542; now 263, 309, 295, 401, 541.
+constexpr int F32_ATTN_THREADS = 128, F32_CHUNK = 512, F32_ATTN_SMEM = 227 * 1024;
 template <int HD>
 __global__ void __launch_bounds__(F32_ATTN_THREADS) k_attn_rope_f32(
         const float* __restrict__ qkv, const float* __restrict__ cs, const float* __restrict__ sn, float* __restrict__ q, float* __restrict__ out,
@@ -224,34 +228,38 @@ __global__ void __launch_bounds__(F32_ATTN_THREADS) k_attn_rope_f32(
     float mx = -INFINITY, sum = 0.f;                 // running maximum (all threads) and this thread's share of the sum
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int c0 = 0; c0 < n; c0 += F32_CHUNK) {
-        const int here = min(F32_CHUNK, n - c0);
+        const int here = min(F32_CHUNK, n - c0), cached = max(0, min(here, L - c0));      // the first `cached` of them lie in the cache
         float m = -INFINITY;
-        for (int i = tid; i < here; i += F32_ATTN_THREADS) {
+        int i = tid;
+        for (; i < cached; i += F32_ATTN_THREADS) {
             float4 e = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (c0 + i < L) {
-                const float* kr = kbase + (size_t)(c0 + i) * HD;
+            const float* kr = kbase + (size_t)(c0 + i) * HD;
 #pragma unroll
-                for (int j = 0; j < QUADS; ++j) {
-                    const float4 kv = *reinterpret_cast<const float4*>(kr + 4 * j), qv = *reinterpret_cast<const float4*>(s_q + 4 * j);
-                    e.x = fmaf(qv.x, kv.x, e.x); e.y = fmaf(qv.y, kv.y, e.y); e.z = fmaf(qv.z, kv.z, e.z); e.w = fmaf(qv.w, kv.w, e.w);
-                }
-            } else {
-                const int node = s_anc[c0 + i - L];
-                const float *kr = tree + (size_t)node * 3 * d + d, *c = tree_cs + node * HALF, *s = tree_sn + node * HALF;
-#pragma unroll
-                for (int j = 0; j < HALF; j += 4) {
-                    const float4 k0 = *reinterpret_cast<const float4*>(kr + j), k1 = *reinterpret_cast<const float4*>(kr + HALF + j);
-                    const float4 c4 = *reinterpret_cast<const float4*>(c + j), s4 = *reinterpret_cast<const float4*>(s + j);
-                    const float4 q0 = *reinterpret_cast<const float4*>(s_q + j), q1 = *reinterpret_cast<const float4*>(s_q + HALF + j);
-                    e.x = fmaf(q0.x, k0.x * c4.x - k1.x * s4.x, fmaf(q1.x, k1.x * c4.x + k0.x * s4.x, e.x));
-                    e.y = fmaf(q0.y, k0.y * c4.y - k1.y * s4.y, fmaf(q1.y, k1.y * c4.y + k0.y * s4.y, e.y));
-                    e.z = fmaf(q0.z, k0.z * c4.z - k1.z * s4.z, fmaf(q1.z, k1.z * c4.z + k0.z * s4.z, e.z));
-                    e.w = fmaf(q0.w, k0.w * c4.w - k1.w * s4.w, fmaf(q1.w, k1.w * c4.w + k0.w * s4.w, e.w));
-                }
+            for (int j = 0; j < QUADS; ++j) {
+                const float4 kv = *reinterpret_cast<const float4*>(kr + 4 * j), qv = *reinterpret_cast<const float4*>(s_q + 4 * j);
+                e.x = fmaf(qv.x, kv.x, e.x); e.y = fmaf(qv.y, kv.y, e.y); e.z = fmaf(qv.z, kv.z, e.z); e.w = fmaf(qv.w, kv.w, e.w);
             }
             const float s = ((e.x + e.y) + (e.z + e.w)) * scale;
             s_p[i] = s;
             m = fmaxf(m, s);
+        }
+        for (; i < here; i += F32_ATTN_THREADS) {
+            float4 e = make_float4(0.f, 0.f, 0.f, 0.f);
+            const int node = s_anc[c0 + i - L];
+            const float *kr = tree + (size_t)node * 3 * d + d, *c = tree_cs + node * HALF, *s = tree_sn + node * HALF;
+#pragma unroll 4
+            for (int j = 0; j < HALF; j += 4) {
+                const float4 k0 = *reinterpret_cast<const float4*>(kr + j), k1 = *reinterpret_cast<const float4*>(kr + HALF + j);
+                const float4 c4 = *reinterpret_cast<const float4*>(c + j), s4 = *reinterpret_cast<const float4*>(s + j);
+                const float4 q0 = *reinterpret_cast<const float4*>(s_q + j), q1 = *reinterpret_cast<const float4*>(s_q + HALF + j);
+                e.x = fmaf(q0.x, k0.x * c4.x - k1.x * s4.x, fmaf(q1.x, k1.x * c4.x + k0.x * s4.x, e.x));
+                e.y = fmaf(q0.y, k0.y * c4.y - k1.y * s4.y, fmaf(q1.y, k1.y * c4.y + k0.y * s4.y, e.y));
+                e.z = fmaf(q0.z, k0.z * c4.z - k1.z * s4.z, fmaf(q1.z, k1.z * c4.z + k0.z * s4.z, e.z));
+                e.w = fmaf(q0.w, k0.w * c4.w - k1.w * s4.w, fmaf(q1.w, k1.w * c4.w + k0.w * s4.w, e.w));
+            }
+            const float sc = ((e.x + e.y) + (e.z + e.w)) * scale;
+            s_p[i] = sc;
+            m = fmaxf(m, sc);
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
@@ -270,13 +278,15 @@ __global__ void __launch_bounds__(F32_ATTN_THREADS) k_attn_rope_f32(
         }
         __syncthreads();
         acc.x *= corr; acc.y *= corr; acc.z *= corr; acc.w *= corr;
-#pragma unroll 4
-        for (int i = group; i < here; i += GROUPS) {
-            const float* vr = c0 + i < L ? vbase + (size_t)(c0 + i) * HD : tree + (size_t)s_anc[c0 + i - L] * 3 * d + 2 * d;
+        auto add_v = [&](const float* vr, float pr) {
             const float4 vv = *reinterpret_cast<const float4*>(vr + 4 * quad);
-            const float pr = s_p[i];
             acc.x = fmaf(pr, vv.x, acc.x); acc.y = fmaf(pr, vv.y, acc.y); acc.z = fmaf(pr, vv.z, acc.z); acc.w = fmaf(pr, vv.w, acc.w);
-        }
+        };
+        i = group;
+#pragma unroll 4
+        for (; i < cached; i += GROUPS) add_v(vbase + (size_t)(c0 + i) * HD, s_p[i]);
+#pragma unroll 4
+        for (; i < here; i += GROUPS) add_v(tree + (size_t)s_anc[c0 + i - L] * 3 * d + 2 * d, s_p[i]);
         __syncthreads();
     }
 #pragma unroll
@@ -319,9 +329,10 @@ bool f32_prepare(const aded_model* m) {
                reinterpret_cast<uintptr_t>(w.norm1) | reinterpret_cast<uintptr_t>(w.norm2);
     if (low % 16 || f32_smem<16, 32>(c.d_model > c.d_ffn ? c.d_model : c.d_ffn) > F32_SMEM) return false;
     bool ok = true;
-    auto set = [&](auto* f) { ok = ok && cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, F32_SMEM) == cudaSuccess; };
+    auto set = [&](auto* f, int bytes = F32_SMEM) { ok = ok && cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess; };
     set(k_gemm_f32<16, 32, F32_QKV>); set(k_gemm_f32<16, 32, F32_SWIGLU>); set(k_gemm_f32<16, 32, F32_HEAD>); set(k_gemm_f32<16, 32, F32_ADD>);
     set(k_gemm_f32<16, 16, F32_ADD>);
+    set(k_attn_rope_f32<64>, F32_ATTN_SMEM - 12 * 1024); set(k_attn_rope_f32<128>, F32_ATTN_SMEM - 12 * 1024);
     set(k_gemm_f32<32, 32, F32_QKV>); set(k_gemm_f32<32, 32, F32_SWIGLU>); set(k_gemm_f32<32, 32, F32_HEAD>); set(k_gemm_f32<32, 32, F32_ADD>);
     return ok;
 }
@@ -362,9 +373,19 @@ void launch_f32_qkv(aded_model* m, int layer, int rows, cudaStream_t st) {
     const int d = m->cfg.d_model;
     f32_project(m, F32_QKV, m->h, m->layers[layer].wqkv, m->layers[layer].norm1, m->y32, rows, 3 * d, d, TK_GEMM_QKV, st);
 }
+// Shared memory that a block of the attention asks for and does not use: as much as keeps more blocks from an SM than it must take.  The
+// blocks start while the QKV projection still holds SMs, and would crowd onto the others (2 layers of 4 heads of 64, 3000 positions, 33 rows:
+// 307 us without, 184 with this).  Where they are few for the SMs that are left they spread anyway, and waiting for a whole SM would cost
+// 2 us (16 rows of that shape at 64 positions: 67 without, 69 with); beyond what an SM holds by registers there is nothing to keep apart.
+static size_t f32_attn_smem(const aded_model* m, int rows) {
+    const int sms = ws_grid_limit(m->device) / 2, blocks = rows * m->cfg.n_heads, per_sm = (blocks + sms - 1) / sms;
+    const int bm = f32_block_rows(m, rows), projection = (3 * m->cfg.d_model + 31) / 32 * ((rows + bm - 1) / bm);
+    if (per_sm > (m->cfg.head_dim == 128 ? 3 : 4) || 3 * blocks <= 2 * (sms - projection)) return 0;
+    return F32_ATTN_SMEM / per_sm - 12 * 1024;        // (beside the 5 KB that it uses and what the device keeps)
+}
 void launch_f32_attention(aded_model* m, aded_kv* kv, int layer, int rows, cudaStream_t st) {
     const int H = m->cfg.n_heads;
-    launch_k(m->cfg.head_dim == 128 ? k_attn_rope_f32<128> : k_attn_rope_f32<64>, dim3(rows, H), dim3(F32_ATTN_THREADS), 0, st, m->y32, m->rope_cos, m->rope_sin,
+    launch_k(m->cfg.head_dim == 128 ? k_attn_rope_f32<128> : k_attn_rope_f32<64>, dim3(rows, H), dim3(F32_ATTN_THREADS), f32_attn_smem(m, rows), st, m->y32, m->rope_cos, m->rope_sin,
              (float*)m->q, (float*)m->attn, kv->base_dev, kv->cap_dev, kv->len_dev, m->rows.seq, m->rows.local, m->rows.anc, layer, H,
              1.f / sqrtf((float)m->cfg.head_dim), m->status);
 }

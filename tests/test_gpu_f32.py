@@ -40,6 +40,28 @@ def test_one_tree(cuda_device, shape, nodes):
     H.compare_cache(shape, sess, cache, 39, cpu["accept_len"], range(shape.n_layers), "after verify")
 
 
+@pytest.mark.parametrize("shape", ["hd64", "hd128"])
+@pytest.mark.parametrize("context,nodes", [(1, 128), (127, 17), (385, 33), (500, 40), (511, 16), (512, 33), (513, 64), (1020, 20), (1024, 128), (1500, 50)])
+def test_cached_and_tree_keys_around_the_chunks(cuda_device, shape, context, nodes):
+    """The attention goes through 512 keys at a time, the cached ones first: chunks that end with the cache, hold both kinds, or the tree's
+    alone; blocks that share an SM and blocks that must not."""
+    shape = SHAPES[shape]
+    w = gen.model_weights(shape, 87)
+    sess = H.GpuSession(shape, H.weights_to(w, cuda_device), capacity=context + nodes)
+    arch, ow = ov.arch_from_shape(shape), ov.Weights(w, keep=True)
+    cache = ov.Cache(arch)
+    for layer in range(shape.n_layers):
+        k, v = (gen.normal((shape.n_heads, context, shape.head_dim), 1.0, 88, 2 * layer + e) for e in range(2))
+        sess.B.aded_kv_load(sess.kv, 0, layer, k.to(cuda_device), v.to(cuda_device))
+        cache.load(layer, k, v)
+    tokens, parents = gen.make_tree(nodes, min(12, nodes - 1), 40, shape.vocab, 89 + nodes)
+    cpu = ov.verify(arch, ow, cache, tokens, parents)
+    gpu = sess.verify(tokens, parents)
+    assert gpu["status"] == 0
+    H.compare_step(shape, gpu, cpu, tokens, parents, "tree")
+    H.compare_cache(shape, sess, cache, 0, context + cpu["accept_len"], range(shape.n_layers), "after verify")
+
+
 @pytest.mark.parametrize("sizes", [(20, 60, 68), (21, 60, 68), (1, 128, 128, 40)])
 def test_batch_on_both_sides_of_the_line(cuda_device, sizes):
     """148 rows of the 4096-token vocabulary are the last that go the short way, 149 the first that do not: each sequence as in a call of its
