@@ -884,8 +884,8 @@ __global__ void k_tg_stats(TgView t, unsigned long long* out) {
 // k-ary tree of continuations below the root's, which is small near the root: all warps of the block look up its first MC_AHEAD
 // contexts, level by level, before the search begins (85 contexts are all there are for sentences of 4 and k = 4).  Ranking the
 // sentences and laying out the result are the block's work too.
-// Measured, 150 iterations, sentences of 4, 24 of them, k = 4, table of 200,000 tokens, with the pass between two steps around it
-// (compaction, table update): 385 us with a warp for everything, 188 with this (search 125, looking up ahead 25, and what the kernel's own code costs to fetch).
+// Measured, 150 iterations, sentences of 4, 24 of them, k = 4, the kernel alone with a cold L2, six contexts, us: a warp for everything
+// 269 to 389, this 133 to 164 (table of 200,000 tokens); 373 to 492 and 158 to 201 (2,000,000).  Of that the look-ahead is about 25.
 constexpr int MC_MAX_ITER = 160, MC_MAX_K = ADED_DRAFT_MAX_K, MC_MAX_LEN = 8;
 constexpr int MC_MAX_NODES = 1 + MC_MAX_ITER * MC_MAX_K;
 constexpr int MC_WARPS = 16, MC_THREADS = MC_WARPS * 32;
